@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C-ABI CUDA library (``libskipkv.so``): argument marshalling only.
+"""Thin binding of the C-ABI CUDA library (``libskipkv.so``): argument marshalling only, by the extension ``_native.so``
+for the calls of the hot path and by ctypes for the set-up calls.
 
 Every function has the name and argument order of its C counterpart in ``include/skipkv.h``
 and takes ``torch`` CUDA tensors (used purely as device memory) whose ``data_ptr()`` is
@@ -16,6 +17,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libskipkv.so")
 _lib = None
+_native = None          # the extension module, once loaded
 
 ERRORS = {-1: "SKIPKV_ERR_INVALID_ARG", -2: "SKIPKV_ERR_UNSUPPORTED", -3: "SKIPKV_ERR_WORKSPACE",
           -4: "SKIPKV_ERR_CUDA", -5: "SKIPKV_ERR_TIMEOUT"}
@@ -58,6 +60,21 @@ def lib():
             getattr(_lib, name).restype = C.c_int
         _lib.skipkv_last_cuda_error.restype = C.c_char_p
     return _lib
+
+
+def _load_native():
+    """Load the extension with the hot entry points; like the library it has no fallback."""
+    global _native
+    lib()
+    path = os.path.join(os.path.dirname(LIB_PATH), "_native.so")
+    if not os.path.exists(path):
+        raise RuntimeError(f"{path} is missing: build it with `python -m paper_2512_07993_b200.build` (there is no CPU fallback)")
+    import importlib.util
+    spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    _native = mod
+    return mod
 
 
 def _ptr(t: Optional[torch.Tensor], dtype=None):
@@ -119,34 +136,32 @@ def skipkv_status(ws: torch.Tensor, stream=None, raise_on_error=True) -> int:
 
 def skipkv_score(shape, params, K, q_win, kv_len, sent_off, n_sent, tok_imp, sent_imp, sent_red, sent_lam,
                  sent_score, ws, stream=None) -> None:
-    _check(lib().skipkv_score(C.byref(shape), C.byref(params), _ptr(K, torch.bfloat16), _ptr(q_win, torch.bfloat16),
-                              _ptr(kv_len, torch.int32), _ptr(sent_off, torch.int32), _ptr(n_sent, torch.int32),
-                              _ptr(tok_imp, torch.float32), _ptr(sent_imp, torch.float32),
-                              _ptr(sent_red, torch.float32), _ptr(sent_lam, torch.float32),
-                              _ptr(sent_score, torch.float32), _ptr(ws), _stream(stream)), "skipkv_score")
+    rc = (_native or _load_native()).skipkv_score(shape, params, K, q_win, kv_len, sent_off, n_sent, tok_imp, sent_imp,
+                                                  sent_red, sent_lam, sent_score, ws, stream)
+    if rc:
+        _check(rc, "skipkv_score")
 
 
 def skipkv_select(shape, params, sent_score, sent_off, n_sent, keep, kept_idx, n_kept, new_len, ws,
                   stream=None) -> None:
-    _check(lib().skipkv_select(C.byref(shape), C.byref(params), _ptr(sent_score, torch.float32),
-                               _ptr(sent_off, torch.int32), _ptr(n_sent, torch.int32), _ptr(keep, torch.uint8),
-                               _ptr(kept_idx, torch.int32), _ptr(n_kept, torch.int32), _ptr(new_len, torch.int32),
-                               _ptr(ws), _stream(stream)), "skipkv_select")
+    rc = (_native or _load_native()).skipkv_select(shape, params, sent_score, sent_off, n_sent, keep, kept_idx, n_kept,
+                                                   new_len, ws, stream)
+    if rc:
+        _check(rc, "skipkv_select")
 
 
 def skipkv_compact(shape, K, V, keep, sent_off, sent_id, n_sent, kv_len, index_map, ws, stream=None) -> None:
-    _check(lib().skipkv_compact(C.byref(shape), _ptr(K, torch.bfloat16), _ptr(V, torch.bfloat16),
-                                _ptr(keep, torch.uint8), _ptr(sent_off, torch.int32), _ptr(sent_id, torch.int32),
-                                _ptr(n_sent, torch.int32), _ptr(kv_len, torch.int32), _ptr(index_map, torch.int32),
-                                _ptr(ws), _stream(stream)), "skipkv_compact")
+    rc = (_native or _load_native()).skipkv_compact(shape, K, V, keep, sent_off, sent_id, n_sent, kv_len, index_map, ws,
+                                                    stream)
+    if rc:
+        _check(rc, "skipkv_compact")
 
 
 def skipkv_decode_attn(shape, q, K, V, kv_len, out, hidden, steer_vec, alpha, flag, ws, stream=None) -> None:
-    _check(lib().skipkv_decode_attn(C.byref(shape), _ptr(q, torch.bfloat16), _ptr(K, torch.bfloat16),
-                                    _ptr(V, torch.bfloat16), _ptr(kv_len, torch.int32), _ptr(out, torch.bfloat16),
-                                    _ptr(hidden, torch.bfloat16), _ptr(steer_vec, torch.bfloat16),
-                                    _ptr(alpha, torch.float32), _ptr(flag, torch.uint8), _ptr(ws),
-                                    _stream(stream)), "skipkv_decode_attn")
+    rc = (_native or _load_native()).skipkv_decode_attn(shape, q, K, V, kv_len, out, hidden, steer_vec, alpha, flag, ws,
+                                                        stream)
+    if rc:
+        _check(rc, "skipkv_decode_attn")
 
 
 def skipkv_set_wait_limit(ws, polls: int, stream=None) -> None:
@@ -158,143 +173,115 @@ def skipkv_wait_probe(ws, stream=None) -> None:
 
 
 def skipkv_steer(batch, d_model, hidden, steer_vec, alpha, flag, stream=None) -> None:
-    _check(lib().skipkv_steer(C.c_int32(batch), C.c_int32(d_model), _ptr(hidden, torch.bfloat16),
-                              _ptr(steer_vec, torch.bfloat16), _ptr(alpha, torch.float32), _ptr(flag, torch.uint8),
-                              _stream(stream)), "skipkv_steer")
+    rc = (_native or _load_native()).skipkv_steer(batch, d_model, hidden, steer_vec, alpha, flag, stream)
+    if rc:
+        _check(rc, "skipkv_steer")
 
 
 def skipkv_append(shape, K, V, k_new, v_new, kv_len, ws, stream=None) -> None:
-    _check(lib().skipkv_append(C.byref(shape), _ptr(K, torch.bfloat16), _ptr(V, torch.bfloat16),
-                               _ptr(k_new, torch.bfloat16), _ptr(v_new, torch.bfloat16), _ptr(kv_len, torch.int32),
-                               _ptr(ws), _stream(stream)), "skipkv_append")
+    rc = (_native or _load_native()).skipkv_append(shape, K, V, k_new, v_new, kv_len, ws, stream)
+    if rc:
+        _check(rc, "skipkv_append")
 
 
 def skipkv_table_step(batch, d_model, max_gen_sent, hidden_last, flag, acc, acc_count, emb, n_gen_sent, closed,
                       lam_table, tau, eps, status=None, stream=None) -> None:
-    _check(lib().skipkv_table_step(C.c_int32(batch), C.c_int32(d_model), C.c_int32(max_gen_sent),
-                                   _ptr(hidden_last, torch.bfloat16), _ptr(flag, torch.uint8),
-                                   _ptr(acc, torch.float32), _ptr(acc_count, torch.int32), _ptr(emb, torch.float32),
-                                   _ptr(n_gen_sent, torch.int32), _ptr(closed, torch.int32),
-                                   _ptr(lam_table, torch.float32), C.c_float(tau), C.c_float(eps),
-                                   _ptr(status, torch.int32), _stream(stream)), "skipkv_table_step")
+    rc = (_native or _load_native()).skipkv_table_step(batch, d_model, max_gen_sent, hidden_last, flag, acc, acc_count, emb,
+                                                       n_gen_sent, closed, lam_table, tau, eps, status, stream)
+    if rc:
+        _check(rc, "skipkv_table_step")
 
 
 def skipkv_score_table(shape, params, K, q_win, kv_len, sent_off, sent_id, n_sent, lam_table, table_len, tok_imp,
                        sent_imp, sent_red, sent_lam, sent_score, ws, stream=None) -> None:
-    _check(lib().skipkv_score_table(C.byref(shape), C.byref(params), _ptr(K, torch.bfloat16),
-                                    _ptr(q_win, torch.bfloat16), _ptr(kv_len, torch.int32),
-                                    _ptr(sent_off, torch.int32), _ptr(sent_id, torch.int32),
-                                    _ptr(n_sent, torch.int32), _ptr(lam_table, torch.float32),
-                                    C.c_int32(table_len), _ptr(tok_imp, torch.float32),
-                                    _ptr(sent_imp, torch.float32), _ptr(sent_red, torch.float32),
-                                    _ptr(sent_lam, torch.float32), _ptr(sent_score, torch.float32), _ptr(ws),
-                                    _stream(stream)), "skipkv_score_table")
+    rc = (_native or _load_native()).skipkv_score_table(shape, params, K, q_win, kv_len, sent_off, sent_id, n_sent,
+                                                        lam_table, table_len, tok_imp, sent_imp, sent_red, sent_lam,
+                                                        sent_score, ws, stream)
+    if rc:
+        _check(rc, "skipkv_score_table")
 
 
 def skipkv_select_fill(shape, params, sent_score, tok_imp, sent_off, n_sent, keep, tok_keep, kept_idx, n_kept, new_len,
                        ws, stream=None) -> None:
-    _check(lib().skipkv_select_fill(C.byref(shape), C.byref(params), _ptr(sent_score, torch.float32),
-                                    _ptr(tok_imp, torch.float32), _ptr(sent_off, torch.int32),
-                                    _ptr(n_sent, torch.int32), _ptr(keep, torch.uint8), _ptr(tok_keep, torch.uint8),
-                                    _ptr(kept_idx, torch.int32), _ptr(n_kept, torch.int32),
-                                    _ptr(new_len, torch.int32), _ptr(ws), _stream(stream)), "skipkv_select_fill")
+    rc = (_native or _load_native()).skipkv_select_fill(shape, params, sent_score, tok_imp, sent_off, n_sent, keep,
+                                                        tok_keep, kept_idx, n_kept, new_len, ws, stream)
+    if rc:
+        _check(rc, "skipkv_select_fill")
 
 
 def skipkv_select_fill_red(shape, params, sent_score, tok_imp, tok_red, sent_off, n_sent, keep, tok_keep, kept_idx,
                            n_kept, new_len, ws, stream=None) -> None:
-    _check(lib().skipkv_select_fill_red(C.byref(shape), C.byref(params), _ptr(sent_score, torch.float32),
-                                        _ptr(tok_imp, torch.float32), _ptr(tok_red, torch.float32),
-                                        _ptr(sent_off, torch.int32), _ptr(n_sent, torch.int32), _ptr(keep, torch.uint8),
-                                        _ptr(tok_keep, torch.uint8), _ptr(kept_idx, torch.int32),
-                                        _ptr(n_kept, torch.int32), _ptr(new_len, torch.int32), _ptr(ws),
-                                        _stream(stream)), "skipkv_select_fill_red")
+    rc = (_native or _load_native()).skipkv_select_fill_red(shape, params, sent_score, tok_imp, tok_red, sent_off, n_sent,
+                                                            keep, tok_keep, kept_idx, n_kept, new_len, ws, stream)
+    if rc:
+        _check(rc, "skipkv_select_fill_red")
 
 
 def skipkv_compact_fill(shape, K, V, keep, tok_keep, sent_off, sent_id, n_sent, kv_len, index_map, ws,
                         stream=None) -> None:
-    _check(lib().skipkv_compact_fill(C.byref(shape), _ptr(K, torch.bfloat16), _ptr(V, torch.bfloat16),
-                                     _ptr(keep, torch.uint8), _ptr(tok_keep, torch.uint8),
-                                     _ptr(sent_off, torch.int32), _ptr(sent_id, torch.int32),
-                                     _ptr(n_sent, torch.int32), _ptr(kv_len, torch.int32),
-                                     _ptr(index_map, torch.int32), _ptr(ws), _stream(stream)), "skipkv_compact_fill")
+    rc = (_native or _load_native()).skipkv_compact_fill(shape, K, V, keep, tok_keep, sent_off, sent_id, n_sent, kv_len,
+                                                         index_map, ws, stream)
+    if rc:
+        _check(rc, "skipkv_compact_fill")
 
 
 def skipkv_token_redundancy(shape, params, K, kv_len, tok_red, ws, stream=None) -> None:
-    _check(lib().skipkv_token_redundancy(C.byref(shape), C.byref(params), _ptr(K, torch.bfloat16),
-                                         _ptr(kv_len, torch.int32), _ptr(tok_red, torch.float32), _ptr(ws),
-                                         _stream(stream)), "skipkv_token_redundancy")
+    rc = (_native or _load_native()).skipkv_token_redundancy(shape, params, K, kv_len, tok_red, ws, stream)
+    if rc:
+        _check(rc, "skipkv_token_redundancy")
 
 
 def skipkv_append_step(shape, K, V, k_new, v_new, kv_len, sent_off, sent_id, n_sent, new_sent, gen_id, q_win, q, slot,
                        ws, stream=None) -> None:
-    _check(lib().skipkv_append_step(C.byref(shape), _ptr(K, torch.bfloat16), _ptr(V, torch.bfloat16),
-                                    _ptr(k_new, torch.bfloat16), _ptr(v_new, torch.bfloat16),
-                                    _ptr(kv_len, torch.int32), _ptr(sent_off, torch.int32),
-                                    _ptr(sent_id, torch.int32), _ptr(n_sent, torch.int32),
-                                    _ptr(new_sent, torch.uint8), _ptr(gen_id, torch.int32),
-                                    _ptr(q_win, torch.bfloat16), _ptr(q, torch.bfloat16), C.c_int32(slot), _ptr(ws),
-                                    _stream(stream)), "skipkv_append_step")
+    rc = (_native or _load_native()).skipkv_append_step(shape, K, V, k_new, v_new, kv_len, sent_off, sent_id, n_sent,
+                                                        new_sent, gen_id, q_win, q, slot, ws, stream)
+    if rc:
+        _check(rc, "skipkv_append_step")
 
 
 def skipkv_decode_attn_paged(shape, q, K_pages, V_pages, block_table, max_pages, kv_len, out, hidden, steer_vec, alpha,
                              flag, ws, stream=None) -> None:
-    _check(lib().skipkv_decode_attn_paged(C.byref(shape), _ptr(q, torch.bfloat16), _ptr(K_pages, torch.bfloat16),
-                                          _ptr(V_pages, torch.bfloat16), _ptr(block_table, torch.int32),
-                                          C.c_int32(max_pages), _ptr(kv_len, torch.int32), _ptr(out, torch.bfloat16),
-                                          _ptr(hidden, torch.bfloat16), _ptr(steer_vec, torch.bfloat16),
-                                          _ptr(alpha, torch.float32), _ptr(flag, torch.uint8), _ptr(ws),
-                                          _stream(stream)), "skipkv_decode_attn_paged")
+    rc = (_native or _load_native()).skipkv_decode_attn_paged(shape, q, K_pages, V_pages, block_table, max_pages, kv_len,
+                                                              out, hidden, steer_vec, alpha, flag, ws, stream)
+    if rc:
+        _check(rc, "skipkv_decode_attn_paged")
 
 
 def skipkv_score_paged(shape, params, K_pages, block_table, max_pages, q_win, kv_len, sent_off, n_sent, tok_imp,
                        sent_imp, sent_red, sent_lam, sent_score, ws, stream=None) -> None:
-    _check(lib().skipkv_score_paged(C.byref(shape), C.byref(params), _ptr(K_pages, torch.bfloat16),
-                                    _ptr(block_table, torch.int32), C.c_int32(max_pages),
-                                    _ptr(q_win, torch.bfloat16), _ptr(kv_len, torch.int32),
-                                    _ptr(sent_off, torch.int32), _ptr(n_sent, torch.int32),
-                                    _ptr(tok_imp, torch.float32), _ptr(sent_imp, torch.float32),
-                                    _ptr(sent_red, torch.float32), _ptr(sent_lam, torch.float32),
-                                    _ptr(sent_score, torch.float32), _ptr(ws), _stream(stream)),
-           "skipkv_score_paged")
+    rc = (_native or _load_native()).skipkv_score_paged(shape, params, K_pages, block_table, max_pages, q_win, kv_len,
+                                                        sent_off, n_sent, tok_imp, sent_imp, sent_red, sent_lam, sent_score,
+                                                        ws, stream)
+    if rc:
+        _check(rc, "skipkv_score_paged")
 
 
 def skipkv_compact_paged(shape, K_pages, V_pages, block_table, max_pages, keep, sent_off, sent_id, n_sent, kv_len,
                          index_map, ws, stream=None) -> None:
-    _check(lib().skipkv_compact_paged(C.byref(shape), _ptr(K_pages, torch.bfloat16), _ptr(V_pages, torch.bfloat16),
-                                      _ptr(block_table, torch.int32), C.c_int32(max_pages),
-                                      _ptr(keep, torch.uint8), _ptr(sent_off, torch.int32),
-                                      _ptr(sent_id, torch.int32), _ptr(n_sent, torch.int32),
-                                      _ptr(kv_len, torch.int32), _ptr(index_map, torch.int32), _ptr(ws),
-                                      _stream(stream)), "skipkv_compact_paged")
+    rc = (_native or _load_native()).skipkv_compact_paged(shape, K_pages, V_pages, block_table, max_pages, keep, sent_off,
+                                                          sent_id, n_sent, kv_len, index_map, ws, stream)
+    if rc:
+        _check(rc, "skipkv_compact_paged")
 
 
 def skipkv_decode_step_paged(shape, q, k_new, v_new, K_pages, V_pages, block_table, max_pages, kv_len_in, kv_len_out,
                              sent_off, sent_id, n_sent, new_sent, gen_id, q_win, slot, out, hidden, steer_vec, alpha,
                              flag, ws, stream=None) -> None:
-    _check(lib().skipkv_decode_step_paged(C.byref(shape), _ptr(q, torch.bfloat16), _ptr(k_new, torch.bfloat16),
-                                          _ptr(v_new, torch.bfloat16), _ptr(K_pages, torch.bfloat16),
-                                          _ptr(V_pages, torch.bfloat16), _ptr(block_table, torch.int32),
-                                          C.c_int32(max_pages), _ptr(kv_len_in, torch.int32),
-                                          _ptr(kv_len_out, torch.int32), _ptr(sent_off, torch.int32),
-                                          _ptr(sent_id, torch.int32), _ptr(n_sent, torch.int32),
-                                          _ptr(new_sent, torch.uint8), _ptr(gen_id, torch.int32),
-                                          _ptr(q_win, torch.bfloat16), C.c_int32(slot), _ptr(out, torch.bfloat16),
-                                          _ptr(hidden, torch.bfloat16), _ptr(steer_vec, torch.bfloat16),
-                                          _ptr(alpha, torch.float32), _ptr(flag, torch.uint8), _ptr(ws),
-                                          _stream(stream)), "skipkv_decode_step_paged")
+    rc = (_native or _load_native()).skipkv_decode_step_paged(shape, q, k_new, v_new, K_pages, V_pages, block_table,
+                                                              max_pages, kv_len_in, kv_len_out, sent_off, sent_id, n_sent,
+                                                              new_sent, gen_id, q_win, slot, out, hidden, steer_vec, alpha,
+                                                              flag, ws, stream)
+    if rc:
+        _check(rc, "skipkv_decode_step_paged")
 
 
 def skipkv_decode_step(shape, q, k_new, v_new, K, V, kv_len_in, kv_len_out, sent_off, sent_id, n_sent, new_sent, gen_id,
                        q_win, slot, out, hidden, steer_vec, alpha, flag, ws, stream=None) -> None:
-    _check(lib().skipkv_decode_step(C.byref(shape), _ptr(q, torch.bfloat16), _ptr(k_new, torch.bfloat16),
-                                    _ptr(v_new, torch.bfloat16), _ptr(K, torch.bfloat16), _ptr(V, torch.bfloat16),
-                                    _ptr(kv_len_in, torch.int32), _ptr(kv_len_out, torch.int32),
-                                    _ptr(sent_off, torch.int32), _ptr(sent_id, torch.int32),
-                                    _ptr(n_sent, torch.int32), _ptr(new_sent, torch.uint8),
-                                    _ptr(gen_id, torch.int32), _ptr(q_win, torch.bfloat16), C.c_int32(slot),
-                                    _ptr(out, torch.bfloat16), _ptr(hidden, torch.bfloat16),
-                                    _ptr(steer_vec, torch.bfloat16), _ptr(alpha, torch.float32),
-                                    _ptr(flag, torch.uint8), _ptr(ws), _stream(stream)), "skipkv_decode_step")
+    rc = (_native or _load_native()).skipkv_decode_step(shape, q, k_new, v_new, K, V, kv_len_in, kv_len_out, sent_off,
+                                                        sent_id, n_sent, new_sent, gen_id, q_win, slot, out, hidden,
+                                                        steer_vec, alpha, flag, ws, stream)
+    if rc:
+        _check(rc, "skipkv_decode_step")
 
 
 def skipkv_decode_attn_static(shape, q, K, V, kv_len, out, hidden, steer_vec, alpha, flag, status=None,
@@ -303,12 +290,10 @@ def skipkv_decode_attn_static(shape, q, K, V, kv_len, out, hidden, steer_vec, al
 
     For callers that cannot allocate device memory.  ``status`` is an optional one-element
     uint32-sized (int32) device tensor that receives the status bits."""
-    _check(lib().skipkv_decode_attn_static(C.byref(shape), _ptr(q, torch.bfloat16), _ptr(K, torch.bfloat16),
-                                           _ptr(V, torch.bfloat16), _ptr(kv_len, torch.int32),
-                                           _ptr(out, torch.bfloat16), _ptr(hidden, torch.bfloat16),
-                                           _ptr(steer_vec, torch.bfloat16), _ptr(alpha, torch.float32),
-                                           _ptr(flag, torch.uint8), _ptr(status, torch.int32), _stream(stream)),
-           "skipkv_decode_attn_static")
+    rc = (_native or _load_native()).skipkv_decode_attn_static(shape, q, K, V, kv_len, out, hidden, steer_vec, alpha, flag,
+                                                               status, stream)
+    if rc:
+        _check(rc, "skipkv_decode_attn_static")
 
 
 class DeviceLayer:

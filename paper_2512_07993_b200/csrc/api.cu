@@ -29,6 +29,26 @@ int num_sms() {
     return cached;
 }
 
+struct SmemAllowed { const void* kernel; int dev; };
+static thread_local SmemAllowed g_allowed[64];
+static thread_local int g_n_allowed = 0;
+
+cudaError_t allow_max_smem(const void* kernel) {
+    int dev = 0;
+    if (cudaError_t e = cudaGetDevice(&dev)) return e;
+    for (int i = 0; i < g_n_allowed; ++i)
+        if (g_allowed[i].kernel == kernel && g_allowed[i].dev == dev) return cudaSuccess;
+    cudaFuncAttributes fa{};
+    if (cudaError_t e = cudaFuncGetAttributes(&fa, kernel)) return e;
+    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - int(fa.sharedSizeBytes)))
+        return e;
+    if (g_n_allowed == 64) g_n_allowed = 0;              // more kernels x devices than entries: start over
+    g_allowed[g_n_allowed++] = SmemAllowed{kernel, dev};
+    return cudaSuccess;
+}
+
+void forget_max_smem() { g_n_allowed = 0; }
+
 // cuTensorMapEncodeTiled is looked up through the runtime so the library does not link libcuda.
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,

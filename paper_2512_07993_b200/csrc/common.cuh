@@ -92,6 +92,10 @@ int check_shape(const skipkv_shape* s);          // SKIPKV_OK or an error code
 int cuda_fail(cudaError_t e);                    // records the message, returns SKIPKV_ERR_CUDA
 void set_error_text(const char* msg);            // text returned by skipkv_last_cuda_error
 int num_sms();
+// Allow `kernel` all the dynamic shared memory an SM has on the current device.  Every launch of a kernel wants the same
+// attribute value, so it is set once per thread, kernel and device instead of on every call.
+cudaError_t allow_max_smem(const void* kernel);
+void forget_max_smem();                          // after a failed launch: the attributes of a device may have been reset
 
 #define SKIPKV_CUDA(expr)                                            \
     do {                                                             \
@@ -110,7 +114,8 @@ int num_sms();
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// host: launch `kernel` on `st` as a programmatic dependent of the kernel enqueued before it
+// host: launch `kernel` on `st` as a programmatic dependent of the kernel enqueued before it; more than 48 KB of dynamic
+// shared memory is asked for as needed
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                     Args... args) {
@@ -124,7 +129,16 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    if (smem > 48 * 1024)
+        if (cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(kernel))) return e;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    if (e == cudaErrorInvalidValue && smem > 48 * 1024) {            // the device was reset since the attribute was set
+        forget_max_smem();
+        (void)cudaGetLastError();
+        if (cudaError_t e2 = allow_max_smem(reinterpret_cast<const void*>(kernel))) return e2;
+        e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    }
+    return e;
 }
 
 __device__ __forceinline__ size_t slab_row0(const int64_t* slab_off, const int32_t* cap, int Hk, int b, int h) {

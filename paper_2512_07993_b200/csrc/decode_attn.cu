@@ -587,11 +587,9 @@ static int decode_impl(const skipkv_shape* shape, const void* q, const void* K, 
         set_error_text("skipkv_decode_attn: batch * n_kv_heads too large for the shared-memory tile table");
         return SKIPKV_ERR_UNSUPPORTED;
     }
-    // set on every call: the attribute belongs to the current device's context, which a cached value would not track
     const bool exact = (shape->n_q_heads / shape->n_kv_heads) % 4 != 0;
     auto kern = step.k_new ? (exact ? decode_attn_kernel<true, true> : decode_attn_kernel<true, false>)
                            : (exact ? decode_attn_kernel<false, true> : decode_attn_kernel<false, false>);
-    SKIPKV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     int grid = num_sms() * kCtasPerSm;
     if (grid > L.dec_max_ctas) grid = L.dec_max_ctas;
     SKIPKV_CUDA(launch_dependent(
@@ -740,7 +738,7 @@ extern "C" int skipkv_decode_attn_static(const skipkv_shape* shape, const void* 
                         size_t(slabs + 1) * 4;
     unsigned char* base = nullptr;
     if (int rc = static_setup(dev, &base)) return rc;
-    SKIPKV_CUDA(cudaFuncSetAttribute(decode_attn_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    SKIPKV_CUDA(allow_max_smem(reinterpret_cast<const void*>(decode_attn_kernel<false, false>)));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // The array keeps whatever the previous call left: the status word and the arrival counters
     // must start at zero (the partial records are fully written before they are read).

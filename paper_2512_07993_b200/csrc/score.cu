@@ -965,7 +965,6 @@ template <int kSweep, int kN>
 static int launch_sweep(const CUtensorMap& mapK, const CUtensorMap& mapQ, const SweepArgs& a, int grid, size_t smem,
                         cudaStream_t st) {
     auto kern = score_sweep_kernel<kSweep, kN>;
-    SKIPKV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     SKIPKV_CUDA(launch_dependent(kern, dim3(grid), dim3(kSweep == 1 ? kSw1Threads : kSw2Threads), smem, st, mapK, mapQ, a));
     return SKIPKV_OK;
 }
@@ -1051,8 +1050,6 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         if (gsmem > 227 * 1024) return SKIPKV_ERR_UNSUPPORTED;
         const long long max_items = (long long)L.slabs * ((shape->max_sent + 127) / 128);
         const int ggrid = int(max_items < (long long)grid ? max_items : (long long)grid);
-        SKIPKV_CUDA(cudaFuncSetAttribute(score_gram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(gsmem)));
-        SKIPKV_CUDA(cudaFuncSetAttribute(score_gram_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(gsmem)));
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<1>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,
                                      shape->max_sent, n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
                                      sent_score, ext, reinterpret_cast<const Header*>(w + L.header)));

@@ -154,7 +154,6 @@ extern "C" int skipkv_table_step(int32_t batch, int32_t d_model, int32_t max_gen
                                  int(max_gen_sent), static_cast<const __nv_bfloat16*>(hidden_last), flag, acc, acc_count,
                                  emb, n_gen_sent, closed, lam_table, eps, status));
     const size_t smem = size_t(d_model) * 4;
-    SKIPKV_CUDA(cudaFuncSetAttribute(table_pss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     const dim3 grid((max_gen_sent + kPssRows - 1) / kPssRows, batch);
     SKIPKV_CUDA(launch_dependent(table_pss_kernel, grid, dim3(kPssThreads), smem, st, int(d_model), int(max_gen_sent),
                                  static_cast<const float*>(emb), static_cast<const int32_t*>(closed), lam_table, tau));

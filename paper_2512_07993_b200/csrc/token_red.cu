@@ -336,8 +336,6 @@ extern "C" int skipkv_token_redundancy(const skipkv_shape* shape, const skipkv_p
     const long long max_items = (long long)L.slabs * ((shape->max_cap + 127) / 128);
     int grid = num_sms();
     if (max_items < grid) grid = int(max_items);
-    SKIPKV_CUDA(cudaFuncSetAttribute(token_red_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    SKIPKV_CUDA(cudaFuncSetAttribute(token_red_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     SKIPKV_CUDA(launch_dependent(token_red_kernel<1>, dim3(grid), dim3(kTrThreads), smem, st, mapK, int(L.slabs), Hk,
                                  int(shape->max_cap), shape->slab_off, shape->cap, kv_len, static_cast<const float*>(inv_norm),
                                  z, tok_red, hdr));
