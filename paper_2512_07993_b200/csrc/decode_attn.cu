@@ -1,25 +1,27 @@
 // skipkv_decode_attn: GQA decode attention over the ragged, compacted cache (the attention
 // equation of paper Section 4.1 with one query per head), with the steering add of Section 4.2
-// performed by the tail of the same launch.
+// performed by the same launch.
 //
-// The step is HBM bound: every live K and V row is read exactly once.  Design:
-//  * Work = 128-row tiles enumerated over all (sequence, head) slabs.  The tile list is cut into
-//    equal contiguous ranges, one per persistent CTA, so CTAs are balanced whatever the ragged
-//    lengths are; a CTA's range may cross slab boundaries, each (CTA, slab) intersection gives
-//    one partial result (running max, sum, 128-wide accumulator per head).
-//  * K and V tiles are streamed into a shared-memory ring with bulk asynchronous copies (each
-//    tile is one contiguous block of the slab) signalled through mbarriers, issued two tiles
-//    ahead by one elected lane; sixteen warps work on 8 rows of a tile each.  (512 threads in one
-//    CTA per SM leave 128 registers per thread, which the mapping below needs; the ring of
-//    3 x 64 KB keeps 128 KB of loads in flight per SM.)
-//  * Consumer mapping: a half-warp per row, 8 channels (16 bytes) per lane.  The four heads of
-//    the group share every K/V load.  fp32 arithmetic with packed two-wide FMAs; the 16 partial
-//    dot products a lane holds for 4 rows x 4 heads are reduced with a 15-shuffle butterfly
-//    that leaves one finished logit per lane.
-//  * Softmax is online in base 2 (the log2(e)/sqrt(d) factor is folded into q).
-//  * The last CTA to deliver a partial for a slab (self-resetting counter in the workspace)
-//    merges that slab's partials and writes the bf16 output.
-//  * Every wait is bounded; on expiry the status word is flagged and the kernel drains.
+// The step is HBM bound: every live K and V row is read exactly once, 512 bytes per token and slab, and what a call
+// costs beyond that is latency: a decode step is a chain of launches (one per layer) over caches of a few thousand rows.
+// Design:
+//  * Work = 64-row tiles enumerated over all (sequence, head) slabs.  The tile list is cut into equal contiguous
+//    ranges, one per CTA (one CTA per SM), so CTAs are balanced whatever the ragged lengths are; a CTA's range may
+//    cross slab boundaries, each (CTA, slab) intersection gives one partial result (max, sum, 128 accumulators per head).
+//  * Four warps, each with its own 16 rows of every tile and its own ring of asynchronous 16-byte copies: no barrier and
+//    no mbarrier in the stream.  Copies (not bulk copies) because the rows are written to shared memory with their
+//    16-byte pieces permuted (piece c of row r at c ^ (r & 7)), which makes the matrix loads free of bank conflicts, and
+//    because rows past the slab's end are zero-filled and the row being appended can come from another pointer.
+//    Three stages of 8 KB per warp keep 64 KB in flight per SM while 32 KB are worked on.
+//  * Math on the tensor cores (mma.sync m16n8k16: one query row per head is far below a tcgen05 tile): S = Q K^T with the
+//    group's heads as the first rows of the A operand, then P V with the probabilities as bf16 high parts in rows 0..7
+//    and their remainders in rows 8..15, so that nothing is lost against fp32 probabilities to 2^-17.  The cost does not
+//    depend on the group size: 5 heads per group used to be bound by packed FMAs (768 us over the un-evicted stress cache).
+//  * Little shared memory and few threads, so that the CTAs of the next launch are resident while this one streams: a
+//    programmatic dependent launch derives its tile schedule and starts its first tiles towards L2 before the launch
+//    ahead of it has finished, and only then waits.  What it read early is checked afterwards (see "schedule").
+//  * Softmax is online in base 2 with a warp-uniform lazy rescale.
+//  * The last CTA to deliver a partial for a slab (self-resetting counter in the workspace) merges that slab's partials.
 #include <cstdio>
 #include <mutex>
 
@@ -28,34 +30,62 @@
 
 namespace skipkv {
 
-// Measured on the headline workload (166 MB of live rows, calls back to back): one CTA of 512 threads per SM with
-// 128-row tiles takes 45.8 us per call, two CTAs of 256 threads with 64-row tiles 46.9 us (178.7 against 174.3 us over
-// the un-evicted cache): the second CTA does not hide the fixed part of a call, because both CTAs of an SM reach their
-// set-up and their merge at the same time.
-constexpr int kTileRows = 128;
-constexpr int kTileBytes = kTileRows * kRowBytes;         // 32 KB for K, same for V
+constexpr int kDecWarps = 4;
+constexpr int kDecThreads = kDecWarps * 32;
+constexpr int kWarpRows = 16;                             // rows of a tile that one warp works on
+constexpr int kTileRows = kDecWarps * kWarpRows;          // 64
 constexpr int kPageRows = 128;                            // paged cache: rows per page
-constexpr int kPageBytes = kPageRows * kRowBytes;
-constexpr int kTilesPerPage = kPageRows / kTileRows;
 constexpr int kStages = 3;
-constexpr int kConsWarps = 16;
-constexpr int kDecThreads = kConsWarps * 32;
-constexpr int kCtasPerSm = 1;
+constexpr int kStageBytes = 2 * kWarpRows * kRowBytes;    // one warp's K rows, then its V rows
+constexpr int kRingBytes = kDecWarps * kStages * kStageBytes;
+constexpr int kPrefetchTiles = 6;                         // tiles a CTA starts towards L2 before it may read the cache
 constexpr int kPartStride = 130;                          // global record: 128 accumulators + max + sum
 constexpr int kWpStride = 132;                            // same record in shared memory, 16-byte aligned rows
 constexpr int kMaxDecSlabs = 8192;
+constexpr int kDecMaxGrid = 256;                          // the merge keeps (max, sum) of every partial in wpart
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// 16 bytes global -> shared, asynchronously; src_bytes = 0 writes zeros and reads nothing
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes) {
+    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
+
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+// D[16 x 8] += A[16 x 16] B[16 x 8], bf16 operands, fp32 accumulators
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// two probabilities as bf16 high parts and as the bf16 remainders
+__device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x - bf16lo(hi), y - bf16hi(hi));
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
 
 // Optional fusion of the per-step bookkeeping into the decode launch (k_new == nullptr: plain decode attention).
-// The tile schedule covers the rows already cached; the CTA that owns a slab's last tile writes the new K/V row into
-// the cache, folds it into the attention as a one-row tile after the last streamed tile, and updates the slab's range
-// list and length when it flushes the segment.  A slab that was empty is handled with the zero-length slabs.  Lengths are read from kv_len and written to kv_len_out (a different buffer), so CTAs that
-// start late still derive the same tile schedule.
+// The tile schedule covers the cached rows and the new one, which is read from k_new / v_new; the CTA that owns a slab's
+// last tile also writes the new row into the cache and updates the slab's range list and length.  Lengths are read from
+// kv_len and written to kv_len_out (a different buffer), so CTAs that start late still derive the same tile schedule.
 struct StepArgs {
     const uint4* k_new;          // [batch][Hk][16]
     const uint4* v_new;
@@ -69,504 +99,383 @@ struct StepArgs {
     int window, slot, max_sent;
 };
 
-struct DecSmem {
-    uint64_t full[kStages];
-    uint64_t empty[kStages];
-    int abort_flag;
-    int is_last;
-    uint32_t wsum[kDecThreads / 32];
-    int step_n_sent, step_starts;          // fused step: range-list inputs of the slab whose tail this CTA holds
-};
-
-__device__ __forceinline__ void consumer_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kConsWarps * 32) : "memory"); }
-
-// One consumer warp, 8 rows [row_base, row_base+8) of a tile, the kH (1..4) heads of the warp's head group: the
-// multiply-adds are done for those heads only, the reduction always runs over four head slots.
-template <bool kGuard, int kH>
-__device__ __forceinline__ void tile_rows_h(const uint8_t* Ks, const uint8_t* Vs, int row_base, int rows, int lane,
-                                          const float2 (&q2)[4][4], float2 (&acc)[4][4], float& m_run,
-                                          float& l_run) {
-    const int half = lane >> 4, l16 = lane & 15;
-    const uint4* Kp = reinterpret_cast<const uint4*>(Ks + size_t(row_base + half) * kRowBytes) + l16;
-    const uint4* Vp = reinterpret_cast<const uint4*>(Vs + size_t(row_base + half) * kRowBytes) + l16;
-    float part[16];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint4 kk = Kp[i * 32];                     // row_base + 2i + half
-        const float2 k0 = bf16x2_to_f2(kk.x), k1 = bf16x2_to_f2(kk.y), k2 = bf16x2_to_f2(kk.z),
-                     k3 = bf16x2_to_f2(kk.w);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            if (h < kH) {
-                float2 a = __fmul2_rn(q2[h][0], k0);
-                a = __ffma2_rn(q2[h][1], k1, a);
-                a = __ffma2_rn(q2[h][2], k2, a);
-                a = __ffma2_rn(q2[h][3], k3, a);
-                part[i * 4 + h] = a.x + a.y;
-            } else {
-                part[i * 4 + h] = 0.f;
-            }
-        }
-    }
-    // butterfly over the 16 lanes of a half-warp: lane l16 ends with the full sum of part[l16]
-    const bool u8 = lane & 8, u4 = lane & 4, u2 = lane & 2, u1 = lane & 1;
-    float r8[8], r4[4], r2[2];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const float mine = u8 ? part[k + 8] : part[k], send = u8 ? part[k] : part[k + 8];
-        r8[k] = mine + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float mine = u4 ? r8[k + 4] : r8[k], send = u4 ? r8[k] : r8[k + 4];
-        r4[k] = mine + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float mine = u2 ? r4[k + 2] : r4[k], send = u2 ? r4[k] : r4[k + 2];
-        r2[k] = mine + __shfl_xor_sync(0xffffffffu, send, 2);
-    }
-    float s;
-    {
-        const float mine = u1 ? r2[1] : r2[0], send = u1 ? r2[0] : r2[1];
-        s = mine + __shfl_xor_sync(0xffffffffu, send, 1);
-    }
-    // this lane's logit: row row_base + 2*(l16>>2) + half, head l16 & 3
-    if (kGuard) {
-        if (row_base + 2 * (l16 >> 2) + half >= rows) s = -INFINITY;
-    }
-    float bm = s;
-    bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 4));
-    bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 8));
-    bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 16));
-    const float m_new = fmaxf(m_run, bm);
-    if (__any_sync(0xffffffffu, m_new > m_run)) {
-        const float sc = ex2(m_run - m_new);             // first block: 2^(-inf) = 0
-        l_run *= sc;
-#pragma unroll
-        for (int h = 0; h < kH; ++h) {
-            const float sh = __shfl_sync(0xffffffffu, sc, h);
-            const float2 s2 = make_float2(sh, sh);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[h][c] = __fmul2_rn(acc[h][c], s2);
-        }
-        m_run = m_new;
-    }
-    const float p = ex2(s - m_run);
-    l_run += p;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        uint4 vv = Vp[i * 32];
-        if (kGuard) {
-            if (row_base + 2 * i + half >= rows) vv = make_uint4(0u, 0u, 0u, 0u);   // stale shared memory
-        }
-        const float2 v0 = bf16x2_to_f2(vv.x), v1 = bf16x2_to_f2(vv.y), v2 = bf16x2_to_f2(vv.z),
-                     v3 = bf16x2_to_f2(vv.w);
-#pragma unroll
-        for (int h = 0; h < kH; ++h) {
-            const float ph = __shfl_sync(0xffffffffu, p, (lane & 16) | (i * 4 + h));
-            const float2 pp = make_float2(ph, ph);
-            acc[h][0] = __ffma2_rn(pp, v0, acc[h][0]);
-            acc[h][1] = __ffma2_rn(pp, v1, acc[h][1]);
-            acc[h][2] = __ffma2_rn(pp, v2, acc[h][2]);
-            acc[h][3] = __ffma2_rn(pp, v3, acc[h][3]);
-        }
-    }
-}
-
-template <bool kGuard, bool kExact>
-__device__ __forceinline__ void tile_rows(int heads, const uint8_t* Ks, const uint8_t* Vs, int row_base, int rows, int lane,
-                                          const float2 (&q2)[4][4], float2 (&acc)[4][4], float& m_run, float& l_run) {
-    if (!kExact) {
-        tile_rows_h<kGuard, 4>(Ks, Vs, row_base, rows, lane, q2, acc, m_run, l_run);
-        return;
-    }
-    switch (heads) {                                         // the same for every thread of a warp
-        case 4: tile_rows_h<kGuard, 4>(Ks, Vs, row_base, rows, lane, q2, acc, m_run, l_run); break;
-        case 3: tile_rows_h<kGuard, 3>(Ks, Vs, row_base, rows, lane, q2, acc, m_run, l_run); break;
-        case 2: tile_rows_h<kGuard, 2>(Ks, Vs, row_base, rows, lane, q2, acc, m_run, l_run); break;
-        default: tile_rows_h<kGuard, 1>(Ks, Vs, row_base, rows, lane, q2, acc, m_run, l_run); break;
-    }
-}
-
-// kExact: head groups of equal size with the multiply-adds of a warp limited to its group's heads (for group sizes
-// that are not a multiple of four; a separate instance, so that the common four-heads-per-group kernel carries one
-// copy of the row code, not four).
 // kStep: the launch also performs the per-step bookkeeping described at StepArgs (a separate instance, so that
 // plain decode attention carries none of it).
-template <bool kStep, bool kExact>
-__global__ void __launch_bounds__(kDecThreads, kCtasPerSm)
-decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, const int64_t* slab_off, const int32_t* cap,
+template <bool kStep>
+__global__ void __launch_bounds__(kDecThreads, 2)
+decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows, const int64_t* slab_off, const int32_t* cap,
                    const __nv_bfloat16* q, const uint8_t* K, const uint8_t* V, const int32_t* kv_len,
                    __nv_bfloat16* out, uint32_t* status, uint32_t* dec_cnt, float* dec_part, int d_model,
                    __nv_bfloat16* hidden, const __nv_bfloat16* steer_vec, const float* alpha, const uint8_t* flag,
-                   const int32_t* block_table, int max_pages, StepArgs step, const uint32_t* wait_limit) {
-    extern __shared__ __align__(1024) uint8_t dsm[];
-    uint8_t* ring = dsm;                                                     // kStages x (K tile, V tile)
-    float* wpart = reinterpret_cast<float*>(dsm + kStages * 2 * kTileBytes);  // [warps][4 heads][132]
-    DecSmem* sm = reinterpret_cast<DecSmem*>(wpart + kConsWarps * 4 * kWpStride);
-    int* pref = reinterpret_cast<int*>(sm + 1);                              // [n_slabs + 1] tile prefix
+                   const int32_t* block_table, int max_pages, StepArgs step) {
+    extern __shared__ __align__(128) uint8_t dsm[];
+    const int n = Hq / Hk;                                                   // heads per group
+    float* wpart = reinterpret_cast<float*>(dsm + kRingBytes);               // [warps][n heads][132]
+    int* pref = reinterpret_cast<int*>(wpart + kDecWarps * n * kWpStride);   // [n_slabs + 1] tile prefix
+    uint32_t* lens = reinterpret_cast<uint32_t*>(pref + n_slabs + 1);        // [n_slabs] 2 * rows to attend to + (a row is appended)
+    __shared__ uint32_t s_wsum[kDecWarps];
+    __shared__ int s_last;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    pdl_trigger();
-    // live rows of slab s; with a block table (paged cache) a slab cannot exceed its max_pages pages of kPageRows rows
+    const int G = gridDim.x, cta = blockIdx.x;
+    // rows slab s has room for; with a block table (paged cache) no more than its max_pages pages
     auto room = [&](int s) { return block_table ? min(cap[s / Hk], max_pages * kPageRows) : cap[s / Hk]; };
-    auto old_len = [&](int s) { return min(max(kv_len[s], 0), room(s)); };     // rows before this launch
+    auto slab_len = [&](int s) {
+        const int r = room(s), old = min(max(kv_len[s], 0), r);
+        const uint32_t app = kStep && old < r ? 1u : 0u;
+        return (uint32_t(old) + app) * 2u + app;
+    };
     // cache row of token t of slab s (contiguous slabs, or through the block table)
     auto phys_row = [&](int s, int t) {
         return block_table ? size_t(max(block_table[size_t(s) * max_pages + t / kPageRows], 0)) * kPageRows + size_t(t % kPageRows)
                            : slab_row0(slab_off, cap, Hk, s / Hk, s % Hk) + size_t(t);
     };
-    // rows streamed through the tile ring; with the fused step the row being appended is folded in separately
-    auto live = [&](int s) { return old_len(s); };
-    const int n = Hq / Hk;                     // heads per group
-    const int NG = (n + 3) / 4;                // head groups (1 or 2) of H0 heads each, the last one possibly smaller:
-    const int H0 = kExact ? (n + NG - 1) / NG : 4;   // exact: 5 heads are 3 + 2, not 4 + 1, and no warp multiplies for absent heads
-    const int G = gridDim.x, cta = blockIdx.x;
 
-    if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(&sm->full[s], 1); mbar_init(&sm->empty[s], kConsWarps); }
-        sm->abort_flag = 0;
-        sm->is_last = 0;
-        mbar_fence_init();
-    }
-    if (kStep) {
-        // the step's small inputs are read in the middle of the stream: start them towards L2 now (L2 is the point of
-        // coherence, so this is safe before the wait below)
-        const size_t row_bytes = size_t(n_slabs) * kRowBytes;
-        for (size_t o = size_t(cta * kDecThreads + tid) * 128; o < row_bytes; o += size_t(G) * kDecThreads * 128) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(step.k_new) + o));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(step.v_new) + o));
-        }
-        if (tid * 32 < n_slabs) asm volatile("prefetch.global.L2 [%0];" ::"l"(step.n_sent + tid * 32));
-    }
-    pdl_wait();                                          // inputs (and the workspace) may come from the kernel before
-    // polls a wait makes before it gives up: the workspace's setting, or the default without a workspace
-    uint32_t limit = kDefaultWaitLimit;
-    if (wait_limit) { const uint32_t v = *reinterpret_cast<const volatile uint32_t*>(wait_limit); if (v) limit = v; }
-    // tile prefix over slabs (its first barrier also publishes the barrier inits)
-    cta_prefix<kDecThreads>(n_slabs, [&](int s) { return (live(s) + kTileRows - 1) / kTileRows; }, pref, sm->wsum);
-    const int Ttot = pref[n_slabs];
-    const int per_cta = max(1, (Ttot + G - 1) / G);
-    const int t_begin = min(cta * per_cta, Ttot), t_end = min(t_begin + per_cta, Ttot);
-
-    // slab holding tile t_begin: largest s with pref[s] <= t_begin and a non-empty slab
-    int slab0 = 0;
-    if (t_begin < t_end) {
-        int lo = 0, hi = n_slabs - 1;
+    // ---- schedule.  The lengths may be written by the launch ahead of this one, but mostly they are older (another layer
+    // ran in between).  So the tile schedule is derived from what they are now, the first tiles of this CTA are started
+    // towards L2 (the point of coherence, so a row that is still being written is not read too early), and after the wait
+    // the lengths are read once more: only if one of them changed is the schedule derived again.
+    const int s_per = (n_slabs + kDecThreads - 1) / kDecThreads;
+    const int s_lo = min(tid * s_per, n_slabs), s_hi = min(s_lo + s_per, n_slabs);
+    for (int s = s_lo; s < s_hi; ++s) lens[s] = slab_len(s);
+    auto tiles_of = [&](int s) { return (int(lens[s] >> 1) + kTileRows - 1) / kTileRows; };
+    cta_prefix<kDecThreads>(n_slabs, tiles_of, pref, s_wsum);
+    // CTA c has the tiles [c T / Ge, (c + 1) T / Ge) of the T tiles, Ge = the CTAs that have work
+    int T, Ge, t_begin, t_end, slab0;
+    auto derive = [&]() {
+        T = pref[n_slabs];
+        Ge = min(G, T);
+        t_begin = cta < Ge ? int((long long)cta * T / Ge) : T;
+        t_end = cta < Ge ? int((long long)(cta + 1) * T / Ge) : T;
+        int lo = 0, hi = n_slabs - 1;                     // slab holding tile t_begin: the last s with pref[s] <= t_begin
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
             if (pref[mid] <= t_begin) lo = mid; else hi = mid - 1;
         }
         slab0 = lo;
+    };
+    derive();
+    if (tid < 2 * kPrefetchTiles && t_begin + (tid >> 1) < t_end) {
+        const int t = t_begin + (tid >> 1);
+        int s = slab0;
+        while (pref[s + 1] <= t) ++s;
+        const int r0 = (t - pref[s]) * kTileRows;
+        const int rows = min(kTileRows, int(lens[s] >> 1) - int(lens[s] & 1u) - r0);     // without the row not yet written
+        const long long row = (long long)phys_row(s, r0);
+        if (rows > 0 && row >= 0 && row + rows <= total_rows)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(((tid & 1) ? V : K) + size_t(row) * kRowBytes),
+                         "r"(rows * kRowBytes) : "memory");
+    }
+    pdl_wait();                                           // inputs (and the workspace) may come from the kernel before
+    {
+        int changed = 0;
+        for (int s = s_lo; s < s_hi; ++s) {
+            const uint32_t v = slab_len(s);
+            if (v != lens[s]) { lens[s] = v; changed = 1; }
+        }
+        if (__syncthreads_or(changed)) {
+            cta_prefix<kDecThreads>(n_slabs, tiles_of, pref, s_wsum);
+            derive();
+        }
     }
 
-    {
-        const int hg = warp % NG;                       // head group of this warp
-        const int Hg = min(H0, n - hg * H0);            // its heads
-        const int rb = warp / NG;                       // row block: rows [rb*NG*8, (rb+1)*NG*8) of each tile
-        const int half = lane >> 4, l16 = lane & 15;
-        const float qscale = 1.4426950408889634f * rsqrtf(float(kHeadDim));
-        float2 q2[4][4], acc[4][4];
-        float m_run = -INFINITY, l_run = 0.f;
-        bool aborted = false;
-
-        // ---- copy issue (thread 0 only): the CTA's k-th tile goes to stage k % kStages.  The cursor
-        // walks the slab parts of this CTA's tile range; divisions and table reads happen once per part.
-        const bool is_producer = (tid == 0);
-        int p_slab = slab0, p_t = t_begin, p_rows_left = 0, p_stage = 0, p_j = 0;
-        uint32_t p_phase = 0;                           // parity of the previous use of p_stage (first lap: no wait)
-        bool p_first_lap = true;
-        const uint8_t *p_K = K, *p_V = V;
-        auto issue_next = [&]() {
-            if (p_t >= t_end) return;
-            if (p_rows_left <= 0) {
+    // ---- copies: this warp's 16 rows of the CTA's k-th tile go to stage k % kStages.  The cursor walks the slab parts of
+    // the tile range; divisions and table reads happen once per part.
+    const uint32_t ring = smem_u32(dsm) + warp * kStages * kStageBytes;
+    const int c_col = lane & 15, c_half = lane >> 4;
+    int p_t = t_begin, p_slab = slab0, p_end = t_begin, p_r0 = 0, p_rows = 0, p_stage = 0;
+    size_t p_row0 = 0;
+    bool p_app = false;
+    auto issue_next = [&]() {
+        if (p_t < t_end) {
+            if (p_end <= p_t) {
                 while (pref[p_slab + 1] <= p_t) ++p_slab;
-                const int j = p_t - pref[p_slab];
-                if (!block_table) {
-                    const size_t off =
-                        (slab_row0(slab_off, cap, Hk, p_slab / Hk, p_slab % Hk) + size_t(j) * kTileRows) * kRowBytes;
-                    p_K = K + off;
-                    p_V = V + off;
-                }
-                p_j = j;
-                p_rows_left = live(p_slab) - j * kTileRows;
+                p_end = pref[p_slab + 1];
+                p_r0 = (p_t - pref[p_slab]) * kTileRows + warp * kWarpRows;
+                p_rows = int(lens[p_slab] >> 1);
+                p_app = kStep && (lens[p_slab] & 1u);
+                if (!block_table) p_row0 = slab_row0(slab_off, cap, Hk, p_slab / Hk, p_slab % Hk);
             }
-            if (block_table) {                          // paged cache: tile j of the slab lies in page block_table[slab][j / tiles per page]
-                const size_t off = size_t(max(block_table[size_t(p_slab) * max_pages + p_j / kTilesPerPage], 0)) * kPageBytes +
-                                   size_t(p_j % kTilesPerPage) * kTileBytes;
-                p_K = K + off;
-                p_V = V + off;
-            }
-            if (!p_first_lap) {
-                if (sm->abort_flag || !mbar_wait(&sm->empty[p_stage], p_phase, limit)) {
-                    if (!sm->abort_flag) atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
-                    sm->abort_flag = 1;
-                    return;
-                }
-            }
-            const uint32_t bytes = uint32_t(min(kTileRows, p_rows_left)) * kRowBytes;
-            uint8_t* dstK = ring + size_t(p_stage) * 2 * kTileBytes;
-            mbar_expect_tx(&sm->full[p_stage], 2 * bytes);
-            bulk_g2s(dstK, p_K, bytes, &sm->full[p_stage]);
-            bulk_g2s(dstK + kTileBytes, p_V, bytes, &sm->full[p_stage]);
-            p_K += kTileBytes;
-            p_V += kTileBytes;
-            p_rows_left -= kTileRows;
-            ++p_t;
-            ++p_j;
-            if (++p_stage == kStages) {
-                p_stage = 0;
-                if (p_first_lap) p_first_lap = false; else p_phase ^= 1u;
-            }
-        };
-        if (is_producer)
-            for (int k = 0; k < kStages - 1; ++k) issue_next();
-        // ------------------------------------------------------------------ steering add
-        // Independent of the attention (its own tensor), so it runs here, behind the wait for the first tiles
-        // whose copies were just issued, instead of lengthening the tail of the launch.
-        if (hidden != nullptr) {
-            const int vec_per_row = d_model / 8, total = batch * vec_per_row;
-            for (int i = cta * kDecThreads + tid; i < total; i += G * kDecThreads)
-                steer_vec8(i, vec_per_row, hidden, steer_vec, alpha, flag);
-        }
-        // fused step: this step's queries take their slot of the observation window
-        if (kStep && step.q_win != nullptr) {
-            const int total = batch * Hq * 16;
-            for (int i = cta * kDecThreads + tid; i < total; i += G * kDecThreads)
-                step.q_win[(size_t(i >> 4) * step.window + step.slot) * 16 + (i & 15)] = reinterpret_cast<const uint4*>(q)[i];
-        }
-        // fused step: new length and range list of a slab after the append (all consumer threads call this together)
-        auto step_tables = [&](int slab_, int b_, bool appended, int S0, int starts_sentence) {
-            const int len = old_len(slab_);
-            const int new_len = appended ? len + 1 : len;
-            int32_t* so = step.sent_off + size_t(slab_) * (step.max_sent + 1);
-            const bool table_ok = S0 >= 0 && S0 <= step.max_sent;
-            int S = S0;
-            bool full_list = false;
-            if (appended && table_ok && (S0 == 0 || starts_sentence)) {
-                if (S0 < step.max_sent) S = S0 + 1; else full_list = true;   // full list: the token joins the last sentence
-            }
-            if (tid == 0) {
-                step.kv_len_out[slab_] = new_len;
-                if (appended && table_ok && S != S0) {
-                    if (S0 == 0) so[0] = 0;
-                    step.sent_id[size_t(slab_) * step.max_sent + S0] = step.gen_id[b_];
-                    step.n_sent[slab_] = S;
-                }
-                if (!appended || !table_ok || full_list) atomicOr(status, SKIPKV_STATUS_BAD_TABLE);
-            }
-            if (appended && table_ok)
-                for (int i = S + tid; i <= step.max_sent; i += kConsWarps * 32) so[i] = new_len;
-        };
-
-        int slab = slab0, t = t_begin, c_stage = 0;
-        uint32_t c_phase = 0;
-        while (t < t_end) {
-            // ---------------------------------------------------------- one (CTA, slab) segment
-            while (pref[slab + 1] <= t) ++slab;
-            const int seg_end = min(t_end, pref[slab + 1]);
-            const int b = slab / Hk, h = slab % Hk;
-            int rows_left = live(slab) - (t - pref[slab]) * kTileRows;
-            const bool seg_append = kStep && old_len(slab) < room(slab);   // fused step: a row joins this slab
-            // fused step, this CTA holds the slab's last tile: fetch what the tail of the segment will need now, so
-            // that the loads are long complete when they are used
-            const bool own_tail = kStep && seg_end == pref[slab + 1];
-            if (own_tail) {
-                // the row being appended: into the cache, and staged as a one-row tile (K at byte 0, V at byte 2048 of
-                // the merge buffer, which is idle until the flush) for the fold-in after the last streamed tile
-                if (seg_append && warp == kConsWarps - 1) {
-                    const int part = lane >> 4, c = lane & 15;
-                    const uint4 val = (part ? step.v_new : step.k_new)[size_t(slab) * 16 + c];
-                    reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(wpart) + part * 2048)[c] = val;
-                    const size_t row = phys_row(slab, old_len(slab));
-                    reinterpret_cast<uint4*>(const_cast<uint8_t*>(part ? V : K))[row * 16 + c] = val;
-                }
-                if (tid == kDecThreads - 33) { sm->step_n_sent = step.n_sent[slab]; sm->step_starts = step.new_sent[b]; }
-            }
+            const int rows = p_rows - p_r0;               // rows of this warp's part, may be <= 0 or > 16
+            if (rows > 0) {
+                size_t row = p_row0 + size_t(p_r0);
+                if (block_table)
+                    row = size_t(max(block_table[size_t(p_slab) * max_pages + p_r0 / kPageRows], 0)) * kPageRows + size_t(p_r0 % kPageRows);
+                const size_t off = (row + size_t(c_half)) * kRowBytes + size_t(c_col) * 16;
+                const uint8_t *kp = K + off, *vp = V + off;
+                const uint32_t dst = ring + p_stage * kStageBytes + c_half * kRowBytes;
+                const int last = rows - 1;                // the appended row, where there is one
+                if (rows > kWarpRows || (rows == kWarpRows && !p_app)) {
 #pragma unroll
-            for (int hh = 0; hh < 4; ++hh) {
-                const int hl = hg * H0 + hh;
-                uint4 qq = make_uint4(0u, 0u, 0u, 0u);
-                if (hh < Hg)
-                    qq = reinterpret_cast<const uint4*>(q + (size_t(b) * Hq + size_t(h) * n + hl) * kHeadDim)[l16];
-                const float2 s2 = make_float2(qscale, qscale);
-                q2[hh][0] = __fmul2_rn(bf16x2_to_f2(qq.x), s2);
-                q2[hh][1] = __fmul2_rn(bf16x2_to_f2(qq.y), s2);
-                q2[hh][2] = __fmul2_rn(bf16x2_to_f2(qq.z), s2);
-                q2[hh][3] = __fmul2_rn(bf16x2_to_f2(qq.w), s2);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[hh][c] = make_float2(0.f, 0.f);
-            }
-            m_run = -INFINITY;
-            l_run = 0.f;
-            for (; t < seg_end; ++t, rows_left -= kTileRows) {
-                if (is_producer) issue_next();                  // keeps kStages-1 tiles in flight
-                if (!aborted) {
-                    if (!mbar_wait(&sm->full[c_stage], c_phase, limit) || sm->abort_flag) {
-                        if (!sm->abort_flag) atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
-                        sm->abort_flag = 1;
-                        aborted = true;
+                    for (int i = 0; i < kWarpRows / 2; ++i) {
+                        const uint32_t d = dst + i * 2 * kRowBytes + ((c_col ^ ((2 * i + c_half) & 7)) << 4);
+                        cp_async16(d, kp + i * 2 * kRowBytes);
+                        cp_async16(d + kWarpRows * kRowBytes, vp + i * 2 * kRowBytes);
                     }
-                }
-                if (!aborted) {
-                    const uint8_t* Ks = ring + size_t(c_stage) * 2 * kTileBytes;
-                    const uint8_t* Vs = Ks + kTileBytes;
-                    if (rows_left >= kTileRows) {
-                        for (int sub = 0; sub < NG; ++sub)
-                            tile_rows<false, kExact>(Hg, Ks, Vs, (rb * NG + sub) * 8, kTileRows, lane, q2, acc, m_run, l_run);
-                    } else {
-                        for (int sub = 0; sub < NG; ++sub) {
-                            const int row_base = (rb * NG + sub) * 8;
-                            if (row_base >= rows_left) break;
-                            tile_rows<true, kExact>(Hg, Ks, Vs, row_base, rows_left, lane, q2, acc, m_run, l_run);
-                        }
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm->empty[c_stage]);
-                }
-                if (++c_stage == kStages) { c_stage = 0; c_phase ^= 1u; }
-            }
-
-            // ---------------------------------------------------------- fused step: this CTA held the slab's last tile
-            if (own_tail && seg_append) {
-                consumer_bar();                            // the staged row is visible
-                if (warp < NG && !aborted)                 // one warp per head group folds the row into its running state
-                    tile_rows<true, kExact>(Hg, reinterpret_cast<const uint8_t*>(wpart), reinterpret_cast<const uint8_t*>(wpart) + 2048, 0, 1,
-                                    lane, q2, acc, m_run, l_run);
-                consumer_bar();                            // before the flush reuses the buffer
-            }
-            if (own_tail) {
-                consumer_bar();                            // the values parked at the start of the segment are visible
-                step_tables(slab, b, seg_append, sm->step_n_sent, sm->step_starts);
-            }
-            // ---------------------------------------------------------- flush this (CTA, slab) segment
-            // halves of the warp hold different rows: add them; finish the sum of p
-#pragma unroll
-            for (int hh = 0; hh < 4; ++hh)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    acc[hh][c].x += __shfl_xor_sync(0xffffffffu, acc[hh][c].x, 16);
-                    acc[hh][c].y += __shfl_xor_sync(0xffffffffu, acc[hh][c].y, 16);
-                }
-            l_run += __shfl_xor_sync(0xffffffffu, l_run, 4);
-            l_run += __shfl_xor_sync(0xffffffffu, l_run, 8);
-            l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);
-            float* wp = wpart + size_t(warp) * 4 * kWpStride;
-            if (half == 0) {
-#pragma unroll
-                for (int hh = 0; hh < 4; ++hh) {
-                    float4* dst = reinterpret_cast<float4*>(wp + hh * kWpStride + l16 * 8);
-                    dst[0] = make_float4(acc[hh][0].x, acc[hh][0].y, acc[hh][1].x, acc[hh][1].y);
-                    dst[1] = make_float4(acc[hh][2].x, acc[hh][2].y, acc[hh][3].x, acc[hh][3].y);
-                }
-            }
-            if (lane < 4) {
-                wp[lane * kWpStride + 128] = m_run;
-                wp[lane * kWpStride + 129] = l_run;
-            }
-            consumer_bar();
-            // merge the warps of each head group; thread -> (head, channel) pairs
-            const int fc = pref[slab] / per_cta, lc = (pref[slab + 1] - 1) / per_cta;
-            const int n_part = lc - fc + 1;
-            __nv_bfloat16* o = out + (size_t(b) * Hq + size_t(h) * n) * kHeadDim;
-            float* rec = dec_part + size_t(cta + slab) * n * kPartStride;
-            for (int idx = tid; idx < n * kHeadDim; idx += kConsWarps * 32) {
-                const int hl = idx / kHeadDim, c = idx % kHeadDim;
-                const int g2 = hl / H0, hh = hl % H0;
-                float M = -INFINITY;
-                for (int w = g2; w < kConsWarps; w += NG) M = fmaxf(M, wpart[(w * 4 + hh) * kWpStride + 128]);
-                float L = 0.f, A = 0.f;
-                for (int w = g2; w < kConsWarps; w += NG) {
-                    const float* p = wpart + (w * 4 + hh) * kWpStride;
-                    const float e = ex2(p[128] - M);
-                    L += p[129] * e;
-                    A += p[c] * e;
-                }
-                if (n_part == 1) {
-                    o[idx] = __float2bfloat16_rn(L > 0.f ? A / L : 0.f);
                 } else {
-                    rec[hl * kPartStride + c] = A;
-                    if (c == 0) { rec[hl * kPartStride + 128] = M; rec[hl * kPartStride + 129] = L; }
-                }
-            }
-            if (n_part > 1) {
-                consumer_bar();                            // every thread's record stores are ordered before ...
-                if (tid == 0) {
-                    __threadfence();                       // ... this fence, which publishes them with the arrival below
-                    const uint32_t old = atomicAdd(dec_cnt + slab, 1u);
-                    const int last = (old == uint32_t(n_part - 1)) ? 1 : 0;
-                    if (last) dec_cnt[slab] = 0u;          // self-resetting for the next launch
-                    sm->is_last = last;
-                }
-                consumer_bar();
-                if (sm->is_last) {
-                    __threadfence();
-                    const float* r0 = dec_part + size_t(fc + slab) * n * kPartStride;
-                    for (int idx = tid; idx < n * kHeadDim; idx += kConsWarps * 32) {
-                        const int hl = idx / kHeadDim, c = idx % kHeadDim;
-                        // four records per round: their loads are all in flight before the first is used
-                        float M = -INFINITY, L = 0.f, A = 0.f;
-                        for (int p0 = 0; p0 < n_part; p0 += 4) {
-                            float mm[4], ll[4], aa[4];
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                const float* rp = r0 + (size_t(min(p0 + k, n_part - 1)) * n + hl) * kPartStride;
-                                mm[k] = (p0 + k < n_part) ? __ldcg(rp + 128) : -INFINITY;
-                                ll[k] = __ldcg(rp + 129);
-                                aa[k] = __ldcg(rp + c);
-                            }
-                            float Mn = M;
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) Mn = fmaxf(Mn, mm[k]);
-                            const float keep = ex2(M - Mn);              // first round: 2^(-inf) = 0
-                            L *= keep; A *= keep;
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                const float e = ex2(mm[k] - Mn);         // absent records: 2^(-inf) = 0
-                                L = fmaf(ll[k], e, L);
-                                A = fmaf(aa[k], e, A);
-                            }
-                            M = Mn;
+                    for (int i = 0; i < kWarpRows / 2; ++i) {
+                        const int r = 2 * i + c_half;
+                        const uint32_t d = dst + i * 2 * kRowBytes + ((c_col ^ (r & 7)) << 4);
+                        const void *ks = kp + i * 2 * kRowBytes, *vs = vp + i * 2 * kRowBytes;
+                        if (kStep && p_app && r == last) {
+                            ks = step.k_new + size_t(p_slab) * 16 + c_col;
+                            vs = step.v_new + size_t(p_slab) * 16 + c_col;
                         }
-                        o[idx] = __float2bfloat16_rn(L > 0.f ? A / L : 0.f);
+                        const int bytes = r <= last ? 16 : 0;
+                        cp_async16(d, bytes ? ks : K, bytes);
+                        cp_async16(d + kWarpRows * kRowBytes, bytes ? vs : V, bytes);
                     }
                 }
             }
-            consumer_bar();                                // wpart and is_last reusable
+            p_r0 += kTileRows;
+            ++p_t;
+            if (++p_stage == kStages) p_stage = 0;
         }
-        // after an abort copies may still be in flight: they must land before the CTA retires
-        if (is_producer && sm->abort_flag)
-            for (int st = 0; st < kStages; ++st) { mbar_wait(&sm->full[st], 0u, 1u << 16); mbar_wait(&sm->full[st], 1u, 1u << 16); }
-        // slabs with no live row: zeros (owned round-robin)
-        for (int s = cta; s < n_slabs; s += G) {
-            if (live(s) > 0) continue;
-            const int b = s / Hk, h = s % Hk;
-            __nv_bfloat16* o = out + (size_t(b) * Hq + size_t(h) * n) * kHeadDim;
-            if (kStep && room(s) > 0) {
-                // fused step on an empty slab: the appended row is its only row, so every head's output is that value row
-                const __nv_bfloat16* vrow = reinterpret_cast<const __nv_bfloat16*>(step.v_new) + size_t(s) * kHeadDim;
-                for (int idx = tid; idx < n * kHeadDim; idx += kConsWarps * 32) o[idx] = vrow[idx % kHeadDim];
-                if (tid < 32) {
-                    const int part = tid >> 4, c = tid & 15;
-                    const size_t row = phys_row(s, 0);
-                    reinterpret_cast<uint4*>(const_cast<uint8_t*>(part ? V : K))[row * 16 + c] =
-                        (part ? step.v_new : step.k_new)[size_t(s) * 16 + c];
-                }
-                const int S0 = step.n_sent[s], starts = step.new_sent[b];
-                consumer_bar();                            // every thread has read n_sent before it changes
-                step_tables(s, b, true, S0, starts);
-            } else {
-                for (int idx = tid; idx < n * kHeadDim; idx += kConsWarps * 32) o[idx] = __float2bfloat16_rn(0.f);
-                if (kStep) step_tables(s, b, false, 0, 0);  // no room: unchanged, reported
+        cp_async_commit();                                // empty groups keep the count
+    };
+#pragma unroll
+    for (int k = 0; k < kStages - 1; ++k) issue_next();
+    // The next launch's CTAs may start when every CTA has come here: early enough to have their schedule and their first
+    // tiles ready, and not so early that what they start towards L2 is evicted by this launch's stream.
+    bool triggered = false;
+    auto maybe_trigger = [&](int tiles_left) {
+        if (!triggered && tiles_left <= kPrefetchTiles) { triggered = true; pdl_trigger(); }
+    };
+    maybe_trigger(t_end - t_begin);
+
+    // ---- steering add: independent of the attention (its own tensor), behind the copies just issued
+    if (hidden != nullptr) {
+        const int vec_per_row = d_model / 8, total = batch * vec_per_row;
+        for (int i = cta * kDecThreads + tid; i < total; i += G * kDecThreads)
+            steer_vec8(i, vec_per_row, hidden, steer_vec, alpha, flag);
+    }
+    // fused step: this step's queries take their slot of the observation window
+    if (kStep && step.q_win != nullptr) {
+        const int total = batch * Hq * 16;
+        for (int i = cta * kDecThreads + tid; i < total; i += G * kDecThreads)
+            step.q_win[(size_t(i >> 4) * step.window + step.slot) * 16 + (i & 15)] = reinterpret_cast<const uint4*>(q)[i];
+    }
+    // fused step: new length and range list of a slab after the append (every thread has read n_sent before any calls this)
+    auto step_tables = [&](int slab_, int b_, int new_len, bool appended, int S0, int starts_sentence) {
+        int32_t* so = step.sent_off + size_t(slab_) * (step.max_sent + 1);
+        const bool table_ok = S0 >= 0 && S0 <= step.max_sent;
+        int S = S0;
+        bool full_list = false;
+        if (appended && table_ok && (S0 == 0 || starts_sentence)) {
+            if (S0 < step.max_sent) S = S0 + 1; else full_list = true;   // full list: the token joins the last sentence
+        }
+        if (tid == 0) {
+            step.kv_len_out[slab_] = new_len;
+            if (appended && table_ok && S != S0) {
+                if (S0 == 0) so[0] = 0;
+                step.sent_id[size_t(slab_) * step.max_sent + S0] = step.gen_id[b_];
+                step.n_sent[slab_] = S;
+            }
+            if (!appended || !table_ok || full_list) atomicOr(status, SKIPKV_STATUS_BAD_TABLE);
+        }
+        if (appended && table_ok)
+            for (int i = S + tid; i <= step.max_sent; i += kDecThreads) so[i] = new_len;
+    };
+
+    const int g = lane >> 2, qd = lane & 3;               // mma fragments: row (head) g, columns 2 qd and 2 qd + 1
+    const float qscale = 1.4426950408889634f * rsqrtf(float(kHeadDim));
+    // this lane's row address offsets inside a stage for the matrix loads (K: token octets by the upper bit, V: by the lower)
+    const int lm = lane >> 3, k_row = (lane & 7) + (lm >> 1) * 8, v_row = (lane & 7) + (lm & 1) * 8;
+    const uint32_t k_base = ring + k_row * kRowBytes, v_base = ring + (kWarpRows + v_row) * kRowBytes;
+    const int k_x = lm & 1, v_x = lm >> 1, sw = lane & 7;
+
+    int slab = slab0, t = t_begin, c_stage = 0;
+    while (t < t_end) {
+        // -------------------------------------------------------------- one (CTA, slab) segment
+        while (pref[slab + 1] <= t) ++slab;
+        const int seg_end = min(t_end, pref[slab + 1]);
+        const int b = slab / Hk, h = slab % Hk;
+        const int n_rows = int(lens[slab] >> 1);
+        const bool appended = kStep && (lens[slab] & 1u);
+        const bool own_tail = kStep && seg_end == pref[slab + 1];
+        int step_S0 = 0, step_starts = 0;
+        if (own_tail) {
+            step_S0 = step.n_sent[slab]; step_starts = step.new_sent[b];
+            if (appended && warp == kDecWarps - 1) {      // the row being appended goes into the cache
+                const size_t row = phys_row(slab, n_rows - 1);
+                reinterpret_cast<uint4*>(const_cast<uint8_t*>(c_half ? V : K))[row * 16 + c_col] =
+                    (c_half ? step.v_new : step.k_new)[size_t(slab) * 16 + c_col];
             }
         }
+        uint32_t qa[8][2];
+        {
+            const uint32_t* qp = reinterpret_cast<const uint32_t*>(q + (size_t(b) * Hq + size_t(h) * n + min(g, n - 1)) * kHeadDim) + qd;
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                qa[ks][0] = g < n ? qp[ks * 8] : 0u;
+                qa[ks][1] = g < n ? qp[ks * 8 + 4] : 0u;
+            }
+        }
+        float acc[16][4];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) { acc[j][0] = 0.f; acc[j][1] = 0.f; acc[j][2] = 0.f; acc[j][3] = 0.f; }
+        float m_run = -INFINITY, l_run = 0.f;
+        int rows_left = n_rows - (t - pref[slab]) * kTileRows - warp * kWarpRows;     // of this warp's part of the tile
+        for (; t < seg_end; ++t, rows_left -= kTileRows) {
+            cp_async_wait<kStages - 2>();
+            __syncwarp();                                 // every lane's pieces have landed; the stage before is read out
+            issue_next();
+            maybe_trigger(t_end - t);
+            if (rows_left > 0) {
+                const uint32_t stage = c_stage * kStageBytes;
+                float s[2][4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { s[0][k] = 0.f; s[1][k] = 0.f; }
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks) {
+                    uint32_t kb[4];
+                    ldmatrix4(k_base + stage + (((2 * ks + k_x) ^ sw) << 4), kb);
+                    mma16816(s[0], qa[ks][0], 0u, qa[ks][1], 0u, kb[0], kb[1]);
+                    mma16816(s[1], qa[ks][0], 0u, qa[ks][1], 0u, kb[2], kb[3]);
+                }
+                // this lane's logits: head g, tokens 2 qd, 2 qd + 1, 8 + 2 qd, 9 + 2 qd
+                float x0 = s[0][0] * qscale, x1 = s[0][1] * qscale, x2 = s[1][0] * qscale, x3 = s[1][1] * qscale;
+                if (rows_left < kWarpRows) {
+                    if (2 * qd >= rows_left) x0 = -INFINITY;
+                    if (2 * qd + 1 >= rows_left) x1 = -INFINITY;
+                    if (2 * qd + 8 >= rows_left) x2 = -INFINITY;
+                    if (2 * qd + 9 >= rows_left) x3 = -INFINITY;
+                }
+                float bm = fmaxf(fmaxf(x0, x1), fmaxf(x2, x3));
+                bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
+                bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
+                const float m_new = fmaxf(m_run, bm);
+                if (__any_sync(0xffffffffu, m_new > m_run)) {
+                    const float sc = ex2(m_run - m_new);  // first rows: 2^(-inf) = 0
+                    l_run *= sc;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) { acc[j][0] *= sc; acc[j][1] *= sc; acc[j][2] *= sc; acc[j][3] *= sc; }
+                    m_run = m_new;
+                }
+                const float p0 = ex2(x0 - m_run), p1 = ex2(x1 - m_run), p2 = ex2(x2 - m_run), p3 = ex2(x3 - m_run);
+                l_run += (p0 + p1) + (p2 + p3);
+                uint32_t a0, a1, a2, a3;
+                split_bf16(p0, p1, a0, a1);
+                split_bf16(p2, p3, a2, a3);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    uint32_t vb[4];
+                    ldmatrix4_trans(v_base + stage + (((2 * j + v_x) ^ sw) << 4), vb);
+                    mma16816(acc[2 * j], a0, a1, a2, a3, vb[0], vb[1]);
+                    mma16816(acc[2 * j + 1], a0, a1, a2, a3, vb[2], vb[3]);
+                }
+            }
+            if (++c_stage == kStages) c_stage = 0;
+        }
+
+        // -------------------------------------------------------------- flush this (CTA, slab) segment
+        l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+        l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+        if (g < n) {
+            float* wp = wpart + (size_t(warp) * n + g) * kWpStride;
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                *reinterpret_cast<float2*>(wp + j * 8 + 2 * qd) = make_float2(acc[j][0] + acc[j][2], acc[j][1] + acc[j][3]);
+            if (qd == 0) { wp[128] = m_run; wp[129] = l_run; }
+        }
+        __syncthreads();
+        if (own_tail) step_tables(slab, b, n_rows, appended, step_S0, step_starts);
+        // merge the warps; thread -> channel
+        const int fc = int(((long long)(pref[slab] + 1) * Ge - 1) / T), lc = int(((long long)pref[slab + 1] * Ge - 1) / T);
+        const int n_part = lc - fc + 1;
+        __nv_bfloat16* o = out + (size_t(b) * Hq + size_t(h) * n) * kHeadDim;
+        float* rec = dec_part + size_t(cta + slab) * n * kPartStride;
+        for (int hl = 0; hl < n; ++hl) {
+            float M = -INFINITY, L = 0.f, A = 0.f;
+#pragma unroll
+            for (int w = 0; w < kDecWarps; ++w) M = fmaxf(M, wpart[(w * n + hl) * kWpStride + 128]);
+#pragma unroll
+            for (int w = 0; w < kDecWarps; ++w) {
+                const float* p = wpart + (w * n + hl) * kWpStride;
+                const float e = ex2(p[128] - M);
+                L = fmaf(p[129], e, L);
+                A = fmaf(p[tid], e, A);
+            }
+            if (n_part == 1) {
+                o[hl * kHeadDim + tid] = __float2bfloat16_rn(A / L);
+            } else {
+                rec[hl * kPartStride + tid] = A;
+                if (tid == 0) { rec[hl * kPartStride + 128] = M; rec[hl * kPartStride + 129] = L; }
+            }
+        }
+        __syncthreads();                                   // every thread's record stores are ordered before the arrival; wpart is free
+        if (n_part > 1) {
+            if (tid == 0) {
+                __threadfence();
+                const uint32_t old = atomicAdd(dec_cnt + slab, 1u);
+                const int last = (old == uint32_t(n_part - 1)) ? 1 : 0;
+                if (last) dec_cnt[slab] = 0u;              // self-resetting for the next launch
+                s_last = last;
+            }
+            __syncthreads();
+            if (s_last) {
+                __threadfence();
+                const float* r0 = dec_part + size_t(fc + slab) * n * kPartStride;
+                // (max, sum) of every partial, then each partial's weight, per head
+                float* wm = wpart;                         // [n_part * n]
+                float* wl = wpart + kDecMaxGrid * n;
+                for (int i = tid; i < n_part * n; i += kDecThreads) {
+                    wm[i] = __ldcg(r0 + size_t(i) * kPartStride + 128);
+                    wl[i] = __ldcg(r0 + size_t(i) * kPartStride + 129);
+                }
+                __syncthreads();
+                for (int hl = warp; hl < n; hl += kDecWarps) {
+                    float M = -INFINITY, L = 0.f;
+                    for (int p = lane; p < n_part; p += 32) M = fmaxf(M, wm[p * n + hl]);
+#pragma unroll
+                    for (int d = 16; d; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
+                    for (int p = lane; p < n_part; p += 32) L = fmaf(wl[p * n + hl], ex2(wm[p * n + hl] - M), L);
+#pragma unroll
+                    for (int d = 16; d; d >>= 1) L += __shfl_xor_sync(0xffffffffu, L, d);
+                    const float inv = 1.f / L;
+                    for (int p = lane; p < n_part; p += 32) wm[p * n + hl] = ex2(wm[p * n + hl] - M) * inv;
+                }
+                __syncthreads();
+                float A[kMaxGroup];
+#pragma unroll
+                for (int hl = 0; hl < kMaxGroup; ++hl) A[hl] = 0.f;
+                for (int p0 = 0; p0 < n_part; p0 += 4) {   // four records per round: their loads are in flight together
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int p = min(p0 + k, n_part - 1);
+                        const float on = p0 + k < n_part ? 1.f : 0.f;
+#pragma unroll
+                        for (int hl = 0; hl < kMaxGroup; ++hl)
+                            if (hl < n) A[hl] = fmaf(__ldcg(r0 + (size_t(p) * n + hl) * kPartStride + tid), on * wm[p * n + hl], A[hl]);
+                    }
+                }
+#pragma unroll
+                for (int hl = 0; hl < kMaxGroup; ++hl)
+                    if (hl < n) o[hl * kHeadDim + tid] = __float2bfloat16_rn(A[hl]);
+                __syncthreads();                           // wpart reusable
+            }
+        }
+    }
+    cp_async_wait<0>();
+    if (!triggered) pdl_trigger();
+    // slabs with no row to attend to: zeros (owned round-robin); in the fused step they have no room: unchanged, reported
+    for (int s = cta; s < n_slabs; s += G) {
+        if (lens[s] >> 1) continue;
+        const int b = s / Hk, h = s % Hk;
+        __nv_bfloat16* o = out + (size_t(b) * Hq + size_t(h) * n) * kHeadDim;
+        for (int idx = tid; idx < n * kHeadDim; idx += kDecThreads) o[idx] = __float2bfloat16_rn(0.f);
+        if (kStep) step_tables(s, b, 0, false, 0, 0);
     }
 }
 
 }  // namespace skipkv
 
 using namespace skipkv;
+
+static size_t dec_smem_bytes(int slabs, int group) {
+    return size_t(kRingBytes) + size_t(kDecWarps) * group * kWpStride * 4 + size_t(2 * slabs + 1) * 4;
+}
 
 static int decode_impl(const skipkv_shape* shape, const void* q, const void* K, const void* V, const int32_t* kv_len,
                        void* out, void* hidden, const void* steer_vec, const float* alpha, const uint8_t* flag,
@@ -581,25 +490,20 @@ static int decode_impl(const skipkv_shape* shape, const void* q, const void* K, 
     const WsLayout L = make_layout(*shape);
     if (L.slabs > kMaxDecSlabs) return SKIPKV_ERR_UNSUPPORTED;
     uint8_t* w = static_cast<uint8_t*>(ws);
-    const size_t smem = size_t(kStages) * 2 * kTileBytes + size_t(kConsWarps) * 4 * kWpStride * 4 + sizeof(DecSmem) +
-                        size_t(L.slabs + 1) * 4;
+    const size_t smem = dec_smem_bytes(L.slabs, L.group);
     if (smem > 227 * 1024) {                         // the per-slab tile table no longer fits beside the tile ring
         set_error_text("skipkv_decode_attn: batch * n_kv_heads too large for the shared-memory tile table");
         return SKIPKV_ERR_UNSUPPORTED;
     }
-    const bool exact = (shape->n_q_heads / shape->n_kv_heads) % 4 != 0;
-    auto kern = step.k_new ? (exact ? decode_attn_kernel<true, true> : decode_attn_kernel<true, false>)
-                           : (exact ? decode_attn_kernel<false, true> : decode_attn_kernel<false, false>);
-    int grid = num_sms() * kCtasPerSm;
-    if (grid > L.dec_max_ctas) grid = L.dec_max_ctas;
+    const int grid = num_sms() < kDecMaxGrid ? num_sms() : kDecMaxGrid;
     SKIPKV_CUDA(launch_dependent(
-        kern, dim3(grid), dim3(kDecThreads), smem, static_cast<cudaStream_t>(stream), int(shape->batch),
-        int(shape->n_q_heads), int(shape->n_kv_heads), int(L.slabs), shape->slab_off, shape->cap,
-        static_cast<const __nv_bfloat16*>(q), static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len,
-        static_cast<__nv_bfloat16*>(out), &reinterpret_cast<Header*>(w + L.header)->status,
-        reinterpret_cast<uint32_t*>(w + L.dec_cnt), reinterpret_cast<float*>(w + L.dec_part), int(shape->d_model),
-        static_cast<__nv_bfloat16*>(hidden), static_cast<const __nv_bfloat16*>(steer_vec), alpha, flag, block_table,
-        max_pages, step, static_cast<const uint32_t*>(&reinterpret_cast<Header*>(w + L.header)->wait_limit)));
+        step.k_new ? decode_attn_kernel<true> : decode_attn_kernel<false>, dim3(grid), dim3(kDecThreads), smem,
+        static_cast<cudaStream_t>(stream), int(shape->batch), int(shape->n_q_heads), int(shape->n_kv_heads), int(L.slabs),
+        static_cast<long long>(shape->total_rows), shape->slab_off, shape->cap, static_cast<const __nv_bfloat16*>(q),
+        static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len, static_cast<__nv_bfloat16*>(out),
+        &reinterpret_cast<Header*>(w + L.header)->status, reinterpret_cast<uint32_t*>(w + L.dec_cnt),
+        reinterpret_cast<float*>(w + L.dec_part), int(shape->d_model), static_cast<__nv_bfloat16*>(hidden),
+        static_cast<const __nv_bfloat16*>(steer_vec), alpha, flag, block_table, max_pages, step));
     return SKIPKV_OK;
 }
 
@@ -680,7 +584,7 @@ extern "C" int skipkv_decode_step_paged(const skipkv_shape* shape, const void* q
 namespace skipkv {
 
 constexpr int kStaticMaxSlabs = SKIPKV_STATIC_MAX_SLABS;
-constexpr int kStaticMaxCtas = 256;
+constexpr int kStaticMaxCtas = kDecMaxGrid;
 constexpr size_t kStaticCntOff = 256;                                      // after the status word
 constexpr size_t kStaticPartOff = kStaticCntOff + size_t(kStaticMaxSlabs) * 4;
 constexpr size_t kStaticBytes =
@@ -734,25 +638,22 @@ extern "C" int skipkv_decode_attn_static(const skipkv_shape* shape, const void* 
         set_error_text("skipkv_decode_attn_static: device ordinal beyond 63");
         return SKIPKV_ERR_UNSUPPORTED;
     }
-    const size_t smem = size_t(kStages) * 2 * kTileBytes + size_t(kConsWarps) * 4 * kWpStride * 4 + sizeof(DecSmem) +
-                        size_t(slabs + 1) * 4;
+    const size_t smem = dec_smem_bytes(slabs, shape->n_q_heads / shape->n_kv_heads);
     unsigned char* base = nullptr;
     if (int rc = static_setup(dev, &base)) return rc;
-    SKIPKV_CUDA(allow_max_smem(reinterpret_cast<const void*>(decode_attn_kernel<false, false>)));
+    SKIPKV_CUDA(allow_max_smem(reinterpret_cast<const void*>(decode_attn_kernel<false>)));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // The array keeps whatever the previous call left: the status word and the arrival counters
     // must start at zero (the partial records are fully written before they are read).
     SKIPKV_CUDA(cudaMemsetAsync(base, 0, kStaticPartOff, st));
-    int grid = num_sms() * kCtasPerSm;
-    if (grid > kStaticMaxCtas) grid = kStaticMaxCtas;
+    const int grid = num_sms() < kStaticMaxCtas ? num_sms() : kStaticMaxCtas;
     uint32_t* status_word = status ? status : reinterpret_cast<uint32_t*>(base);
-    decode_attn_kernel<false, false><<<grid, kDecThreads, smem, st>>>(
-        shape->batch, shape->n_q_heads, shape->n_kv_heads, slabs, shape->slab_off, shape->cap,
-        static_cast<const __nv_bfloat16*>(q), static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len,
+    decode_attn_kernel<false><<<grid, kDecThreads, smem, st>>>(
+        shape->batch, shape->n_q_heads, shape->n_kv_heads, slabs, static_cast<long long>(shape->total_rows), shape->slab_off,
+        shape->cap, static_cast<const __nv_bfloat16*>(q), static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len,
         static_cast<__nv_bfloat16*>(out), status_word, reinterpret_cast<uint32_t*>(base + kStaticCntOff),
         reinterpret_cast<float*>(base + kStaticPartOff), shape->d_model, static_cast<__nv_bfloat16*>(hidden),
-        static_cast<const __nv_bfloat16*>(steer_vec), alpha, flag, static_cast<const int32_t*>(nullptr), 0, StepArgs{},
-        static_cast<const uint32_t*>(nullptr));
+        static_cast<const __nv_bfloat16*>(steer_vec), alpha, flag, static_cast<const int32_t*>(nullptr), 0, StepArgs{});
     SKIPKV_CUDA(cudaGetLastError());
     return SKIPKV_OK;
 }
