@@ -38,11 +38,13 @@ constexpr int kPageRows = 128;                            // paged cache: rows p
 constexpr int kStages = 3;
 constexpr int kStageBytes = 2 * kWarpRows * kRowBytes;    // one warp's K rows, then its V rows
 constexpr int kRingBytes = kDecWarps * kStages * kStageBytes;
-constexpr int kPrefetchTiles = 6;                         // tiles a CTA starts towards L2 before it may read the cache
-constexpr int kPartStride = 130;                          // global record: 128 accumulators + max + sum
-constexpr int kWpStride = 132;                            // same record in shared memory, 16-byte aligned rows
+constexpr int kPrefetchTiles = 3;                         // tiles a CTA starts towards L2 before it may read the cache
+constexpr int kTriggerTiles = 2;                          // tiles a CTA still has when it lets the next launch's CTAs start
+constexpr int kPartStride = kDecPartStride;               // record of one head: 128 accumulators, max, sum (16-byte aligned rows)
+constexpr int kWpStride = 132;                            // the same in shared memory
+constexpr int kMergeAhead = 12;                           // partials whose accumulators the merge requests before it knows their weights
 constexpr int kMaxDecSlabs = 8192;
-constexpr int kDecMaxGrid = 256;                          // the merge keeps (max, sum) of every partial in wpart
+constexpr int kDecMaxGrid = 256;
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -166,7 +168,20 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(((tid & 1) ? V : K) + size_t(row) * kRowBytes),
                          "r"(rows * kRowBytes) : "memory");
     }
+    if (kStep) {                                          // the rows being appended are read in the middle of the stream
+        const size_t bytes = size_t(n_slabs) * kRowBytes;
+        for (size_t o = size_t(cta * kDecThreads + tid) * 128; o < bytes; o += size_t(G) * kDecThreads * 128) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(step.k_new) + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(step.v_new) + o));
+        }
+    }
     pdl_wait();                                           // inputs (and the workspace) may come from the kernel before
+    // row of token 0 of the first slab (paged: the page of this warp's first rows), requested together with the lengths
+    auto first_row = [&](int s, int r) {
+        return block_table ? size_t(max(block_table[size_t(s) * max_pages + r / kPageRows], 0)) : slab_row0(slab_off, cap, Hk, s / Hk, s % Hk);
+    };
+    auto first_r0 = [&]() { return min((t_begin - pref[slab0]) * kTileRows + warp * kWarpRows, max(int(lens[slab0] >> 1) - 1, 0)); };
+    size_t row_first = t_begin < t_end ? first_row(slab0, first_r0()) : 0;
     {
         int changed = 0;
         for (int s = s_lo; s < s_hi; ++s) {
@@ -176,6 +191,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
         if (__syncthreads_or(changed)) {
             cta_prefix<kDecThreads>(n_slabs, tiles_of, pref, s_wsum);
             derive();
+            row_first = t_begin < t_end ? first_row(slab0, first_r0()) : 0;
         }
     }
 
@@ -194,13 +210,14 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
                 p_r0 = (p_t - pref[p_slab]) * kTileRows + warp * kWarpRows;
                 p_rows = int(lens[p_slab] >> 1);
                 p_app = kStep && (lens[p_slab] & 1u);
-                if (!block_table) p_row0 = slab_row0(slab_off, cap, Hk, p_slab / Hk, p_slab % Hk);
+                if (!block_table) p_row0 = p_t == t_begin ? row_first : slab_row0(slab_off, cap, Hk, p_slab / Hk, p_slab % Hk);
             }
             const int rows = p_rows - p_r0;               // rows of this warp's part, may be <= 0 or > 16
             if (rows > 0) {
                 size_t row = p_row0 + size_t(p_r0);
                 if (block_table)
-                    row = size_t(max(block_table[size_t(p_slab) * max_pages + p_r0 / kPageRows], 0)) * kPageRows + size_t(p_r0 % kPageRows);
+                    row = (p_t == t_begin ? row_first : size_t(max(block_table[size_t(p_slab) * max_pages + p_r0 / kPageRows], 0))) * kPageRows +
+                          size_t(p_r0 % kPageRows);
                 const size_t off = (row + size_t(c_half)) * kRowBytes + size_t(c_col) * 16;
                 const uint8_t *kp = K + off, *vp = V + off;
                 const uint32_t dst = ring + p_stage * kStageBytes + c_half * kRowBytes;
@@ -240,20 +257,20 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     // tiles ready, and not so early that what they start towards L2 is evicted by this launch's stream.
     bool triggered = false;
     auto maybe_trigger = [&](int tiles_left) {
-        if (!triggered && tiles_left <= kPrefetchTiles) { triggered = true; pdl_trigger(); }
+        if (!triggered && tiles_left <= kTriggerTiles) { triggered = true; pdl_trigger(); }
     };
     maybe_trigger(t_end - t_begin);
 
-    // ---- steering add: independent of the attention (its own tensor), behind the copies just issued
-    if (hidden != nullptr) {
-        const int vec_per_row = d_model / 8, total = batch * vec_per_row;
-        for (int i = cta * kDecThreads + tid; i < total; i += G * kDecThreads)
-            steer_vec8(i, vec_per_row, hidden, steer_vec, alpha, flag);
-    }
-    // fused step: this step's queries take their slot of the observation window
-    if (kStep && step.q_win != nullptr) {
-        const int total = batch * Hq * 16;
-        for (int i = cta * kDecThreads + tid; i < total; i += G * kDecThreads)
+    // ---- steering add and (fused step) this step's queries into their slot of the observation window: both independent of
+    // the attention.  Done while the copies just issued are on their way: every load of an item is independent of the
+    // others, and consecutive warps' shares lie in different CTAs.
+    {
+        const int side0 = (warp * G + cta) * 32 + lane, side_step = G * kDecThreads;
+        const int vec_per_row = d_model / 8, steer_total = hidden != nullptr ? batch * vec_per_row : 0;
+        for (int i = side0; i < steer_total; i += side_step)
+            steer_store(i, vec_per_row, hidden, steer_load(i, vec_per_row, hidden, steer_vec, alpha, flag));
+        const int qwin_total = kStep && step.q_win != nullptr ? batch * Hq * 16 : 0;
+        for (int i = side0; i < qwin_total; i += side_step)
             step.q_win[(size_t(i >> 4) * step.window + step.slot) * 16 + (i & 15)] = reinterpret_cast<const uint4*>(q)[i];
     }
     // fused step: new length and range list of a slab after the append (every thread has read n_sent before any calls this)
@@ -380,7 +397,6 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
             if (qd == 0) { wp[128] = m_run; wp[129] = l_run; }
         }
         __syncthreads();
-        if (own_tail) step_tables(slab, b, n_rows, appended, step_S0, step_starts);
         // merge the warps; thread -> channel
         const int fc = int(((long long)(pref[slab] + 1) * Ge - 1) / T), lc = int(((long long)pref[slab + 1] * Ge - 1) / T);
         const int n_part = lc - fc + 1;
@@ -401,7 +417,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
                 o[hl * kHeadDim + tid] = __float2bfloat16_rn(A / L);
             } else {
                 rec[hl * kPartStride + tid] = A;
-                if (tid == 0) { rec[hl * kPartStride + 128] = M; rec[hl * kPartStride + 129] = L; }
+                if (tid == 0) *reinterpret_cast<float2*>(rec + hl * kPartStride + 128) = make_float2(M, L);
             }
         }
         __syncthreads();                                   // every thread's record stores are ordered before the arrival; wpart is free
@@ -416,46 +432,57 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
             __syncthreads();
             if (s_last) {
                 __threadfence();
+                // The launch waits for this merge, so all its loads go out together: a warp takes a head, a lane a partial
+                // for the weights (max, sum) and four channels for the accumulators, the first kMergeAhead of which are
+                // requested before the weights are known.  (In rounds of four behind the weights, 18 partials took 7 us.)
                 const float* r0 = dec_part + size_t(fc + slab) * n * kPartStride;
-                // (max, sum) of every partial, then each partial's weight, per head
-                float* wm = wpart;                         // [n_part * n]
-                float* wl = wpart + kDecMaxGrid * n;
-                for (int i = tid; i < n_part * n; i += kDecThreads) {
-                    wm[i] = __ldcg(r0 + size_t(i) * kPartStride + 128);
-                    wl[i] = __ldcg(r0 + size_t(i) * kPartStride + 129);
-                }
-                __syncthreads();
                 for (int hl = warp; hl < n; hl += kDecWarps) {
+                    auto record = [&](int p) { return r0 + (size_t(min(p, n_part - 1)) * n + hl) * kPartStride; };
+                    float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
                     float M = -INFINITY, L = 0.f;
-                    for (int p = lane; p < n_part; p += 32) M = fmaxf(M, wm[p * n + hl]);
+                    for (int p0 = 0; p0 < n_part; p0 += 32) {
+                        const float2 ml = __ldcg(reinterpret_cast<const float2*>(record(p0 + lane) + 128));
+                        float4 a[kMergeAhead];
 #pragma unroll
-                    for (int d = 16; d; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
-                    for (int p = lane; p < n_part; p += 32) L = fmaf(wl[p * n + hl], ex2(wm[p * n + hl] - M), L);
+                        for (int k = 0; k < kMergeAhead; ++k)
+                            if (p0 + k < n_part) a[k] = __ldcg(reinterpret_cast<const float4*>(record(p0 + k)) + lane);
+                        const bool on = p0 + lane < n_part;
+                        float mx = on ? ml.x : -INFINITY;
 #pragma unroll
-                    for (int d = 16; d; d >>= 1) L += __shfl_xor_sync(0xffffffffu, L, d);
-                    const float inv = 1.f / L;
-                    for (int p = lane; p < n_part; p += 32) wm[p * n + hl] = ex2(wm[p * n + hl] - M) * inv;
-                }
-                __syncthreads();
-                float A[kMaxGroup];
+                        for (int d = 16; d; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+                        const float Mn = fmaxf(M, mx), keep = ex2(M - Mn);          // first round: 2^(-inf) = 0
+                        const float w = on ? ex2(ml.x - Mn) : 0.f;
+                        float ls = on ? ml.y * w : 0.f;
 #pragma unroll
-                for (int hl = 0; hl < kMaxGroup; ++hl) A[hl] = 0.f;
-                for (int p0 = 0; p0 < n_part; p0 += 4) {   // four records per round: their loads are in flight together
+                        for (int d = 16; d; d >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, d);
+                        L = fmaf(L, keep, ls);
+                        M = Mn;
+                        A.x *= keep; A.y *= keep; A.z *= keep; A.w *= keep;
+                        const int cnt = min(32, n_part - p0);
+                        for (int k0 = 0; k0 < cnt; k0 += kMergeAhead) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int p = min(p0 + k, n_part - 1);
-                        const float on = p0 + k < n_part ? 1.f : 0.f;
+                            for (int k = 0; k < kMergeAhead; ++k) {
+                                if (k0 + k < cnt) {
+                                    const float wk = __shfl_sync(0xffffffffu, w, k0 + k);
+                                    A.x = fmaf(a[k].x, wk, A.x); A.y = fmaf(a[k].y, wk, A.y);
+                                    A.z = fmaf(a[k].z, wk, A.z); A.w = fmaf(a[k].w, wk, A.w);
+                                }
+                            }
+                            if (k0 + kMergeAhead < cnt) {
 #pragma unroll
-                        for (int hl = 0; hl < kMaxGroup; ++hl)
-                            if (hl < n) A[hl] = fmaf(__ldcg(r0 + (size_t(p) * n + hl) * kPartStride + tid), on * wm[p * n + hl], A[hl]);
+                                for (int k = 0; k < kMergeAhead; ++k)
+                                    if (k0 + kMergeAhead + k < cnt) a[k] = __ldcg(reinterpret_cast<const float4*>(record(p0 + k0 + kMergeAhead + k)) + lane);
+                            }
+                        }
                     }
+                    const float inv = 1.f / L;
+                    __nv_bfloat16* oi = o + hl * kHeadDim + lane * 4;
+                    oi[0] = __float2bfloat16_rn(A.x * inv); oi[1] = __float2bfloat16_rn(A.y * inv);
+                    oi[2] = __float2bfloat16_rn(A.z * inv); oi[3] = __float2bfloat16_rn(A.w * inv);
                 }
-#pragma unroll
-                for (int hl = 0; hl < kMaxGroup; ++hl)
-                    if (hl < n) o[hl * kHeadDim + tid] = __float2bfloat16_rn(A[hl]);
-                __syncthreads();                           // wpart reusable
             }
         }
+        if (own_tail) step_tables(slab, b, n_rows, appended, step_S0, step_starts);
     }
     cp_async_wait<0>();
     if (!triggered) pdl_trigger();

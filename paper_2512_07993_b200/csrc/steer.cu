@@ -10,7 +10,7 @@ __global__ void steer_kernel(int batch, int d_model, __nv_bfloat16* hidden, cons
     const int vec_per_row = d_model / 8;
     const int total = batch * vec_per_row;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x)
-        steer_vec8(i, vec_per_row, hidden, v, alpha, flag);
+        steer_store(i, vec_per_row, hidden, steer_load(i, vec_per_row, hidden, v, alpha, flag));
 }
 
 __global__ void append_kernel(int batch, int Hk, const int64_t* slab_off, const int32_t* cap, uint4* K, uint4* V,
