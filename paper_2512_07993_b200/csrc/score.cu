@@ -961,6 +961,176 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// Everything after the sweeps for slabs of at most 128 sentences (caches near a budget of a few thousand tokens): one CTA
+// per slab pools its sentences, puts the pooled keys' high and low parts into shared memory as operand tiles, multiplies
+// them once, and takes the row sums, the penalties, the redundancy and the scores from the one accumulator, whose
+// exponentials stay in registers between the two uses.  Nothing but latency bounds these slabs: the three kernels this
+// replaces (pooling and two Gram passes, for any number of sentences) took 22 us for 8 slabs and 28 us for 80, each
+// waiting for the one before it to drain.
+// ---------------------------------------------------------------------------------------
+constexpr int kSmallThreads = 256;
+constexpr int kSmallSent = 128;
+constexpr int kSmallBatch = 8;          // sentences of a warp whose loads are in flight together
+struct SmallCtl {
+    uint64_t done;
+    uint32_t tmem_base;
+    alignas(16) float imp[kSmallSent], sum[2][kSmallSent], mx[2][kSmallSent], invz[kSmallSent];
+};
+constexpr size_t kSmallSmem = 1024 + 2 * size_t(kOpBytes) + sizeof(SmallCtl);
+
+__global__ void __launch_bounds__(kSmallThreads)
+score_small_kernel(int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len, const int32_t* sent_off,
+                   const int32_t* n_sent, float eps, float sigma, float tau, const float* tok_imp_ws, const float* vsum,
+                   float* sent_imp, float* sent_red, float* sent_lam, float* sent_score, LamTable ext, const Header* hdr) {
+    extern __shared__ uint8_t small_smem_raw[];
+    const uint32_t raw = smem_u32(small_smem_raw);
+    uint8_t* hi_t = small_smem_raw + (((raw + 1023u) & ~1023u) - raw);
+    uint8_t* lo_t = hi_t + kOpBytes;
+    SmallCtl* ctl = reinterpret_cast<SmallCtl*>(lo_t + kOpBytes);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int slab = blockIdx.x;
+    pdl_trigger();
+    if (tid == 0) { mbar_init(&ctl->done, 1); mbar_fence_init(); }
+    if (warp == 1) tmem_alloc(&ctl->tmem_base, 128);
+    pdl_wait();
+    const int S = min(max(n_sent[slab], 0), max_sent), N = min(max(kv_len[slab], 0), cap[slab / Hk]);
+    const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
+    const float* ti_p = tok_imp_ws + size_t(slab) * max_cap;
+    // ---- pooling: 16 rows per warp, kSmallBatch at a time; rows past the last sentence are zeros
+#pragma unroll 1
+    for (int b = 0; b < 16; b += kSmallBatch) {
+        const int i0 = warp * 16 + b, cnt = min(kSmallBatch, S - i0);
+        const int off = lane <= cnt ? so[i0 + lane] : 0;
+        float4 v[kSmallBatch];
+#pragma unroll
+        for (int u = 0; u < kSmallBatch; ++u)
+            v[u] = u < cnt ? reinterpret_cast<const float4*>(vsum + (size_t(slab) * max_sent + i0 + u) * kHeadDim)[lane]
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+        float ti[kSmallBatch];
+        int beg[kSmallBatch], end[kSmallBatch];
+#pragma unroll
+        for (int u = 0; u < kSmallBatch; ++u) {
+            beg[u] = max(__shfl_sync(0xffffffffu, off, u), 0);
+            end[u] = min(__shfl_sync(0xffffffffu, off, u + 1), N);
+            if (u >= cnt) end[u] = beg[u];
+            const int t = beg[u] + lane;                 // most sentences have at most 64 tokens: two loads, all in flight
+            ti[u] = t < end[u] ? ti_p[t] : 0.f;
+            if (t + 32 < end[u]) ti[u] += ti_p[t + 32];
+        }
+#pragma unroll
+        for (int u = 0; u < kSmallBatch; ++u)
+            for (int t = beg[u] + lane + 64; t < end[u]; t += 32) ti[u] += ti_p[t];
+#pragma unroll
+        for (int u = 0; u < kSmallBatch; ++u) {
+            const int n = end[u] - beg[u], r = i0 + u;
+            const float inv_len = n > 0 ? 1.f / float(n) : 0.f;
+            float4 x = n > 0 ? v[u] : make_float4(0.f, 0.f, 0.f, 0.f);
+            x.x *= inv_len; x.y *= inv_len; x.z *= inv_len; x.w *= inv_len;
+            float nn = x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w, ts = ti[u];
+#pragma unroll
+            for (int d = 16; d; d >>= 1) {
+                nn += __shfl_xor_sync(0xffffffffu, nn, d);
+                ts += __shfl_xor_sync(0xffffffffu, ts, d);
+            }
+            const float inv = 1.f / (sqrtf(nn) + eps);
+            const float y[4] = {x.x * inv, x.y * inv, x.z * inv, x.w * inv};
+            uint32_t hi[4], lo[4];                       // bf16 bit patterns
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const __nv_bfloat16 h = __float2bfloat16_rn(y[c]);
+                hi[c] = __bfloat16_as_ushort(h);
+                lo[c] = __bfloat16_as_ushort(__float2bfloat16_rn(y[c] - __bfloat162float(h)));
+            }
+            // channels 4 lane .. 4 lane + 3 of row r, as a tiled copy with the 128-byte swizzle would place them
+            const int at = (lane >> 4) * kOpHalfBytes + r * 128 + ((((lane & 15) >> 1) ^ (r & 7)) << 4) + (lane & 1) * 8;
+            *reinterpret_cast<uint2*>(hi_t + at) = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
+            *reinterpret_cast<uint2*>(lo_t + at) = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
+            if (lane == 0 && u < cnt) {
+                const float imp = n > 0 ? ts * inv_len : 0.f;
+                ctl->imp[r] = imp;
+                sent_imp[size_t(slab) * max_sent + r] = imp;
+            }
+        }
+    }
+    fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    if (tid == 0) {
+        const uint32_t a = smem_u32(hi_t), b = smem_u32(lo_t);
+        umma_tile_128x128x128(tmem_base, a, a, false);
+        umma_tile_128x128x128(tmem_base, a, b, true);
+        umma_tile_128x128x128(tmem_base, b, a, true);
+        umma_commit(&ctl->done);
+    }
+    const bool ok = mbar_wait(&ctl->done, 0u, load_wait_limit(hdr));
+    if (!ok && lane == 0) atomicOr(const_cast<uint32_t*>(&hdr->status), SKIPKV_STATUS_COPY_TIMEOUT);
+    tc_fence_after();
+    // ---- thread: row i, 64 columns; two warps share a row
+    const int half = warp >> 2, i = (warp & 3) * 32 + lane;
+    const uint32_t taddr = tmem_base + (uint32_t((warp & 3) * 32) << 16) + half * 64;
+    float e[64];
+    float sum = 0.f, mx = -INFINITY;
+#pragma unroll
+    for (int ch = 0; ch < 2; ++ch) {
+        float v[32];
+        if (half * 64 + ch * 32 < S) {                   // (the same for the whole warp)
+            tmem_ld32(taddr + ch * 32, v);
+        } else {
+#pragma unroll
+            for (int jj = 0; jj < 32; ++jj) v[jj] = 0.f;
+        }
+#pragma unroll
+        for (int jj = 0; jj < 32; ++jj) {
+            const int j = half * 64 + ch * 32 + jj;
+            const bool on = j < S && j != i;
+            e[ch * 32 + jj] = on ? ex2f(v[jj] * kLog2e) : 0.f;
+            sum += e[ch * 32 + jj];
+            if (on && j > i) mx = fmaxf(mx, v[jj]);
+        }
+    }
+    ctl->sum[half][i] = sum;
+    ctl->mx[half][i] = mx;
+    tc_fence_before();
+    __syncthreads();
+    if (half == 0) {
+        const float z = ctl->sum[0][i] + ctl->sum[1][i];
+        ctl->invz[i] = (i < S && z > 0.f) ? 1.f / z : 0.f;
+    }
+    __syncthreads();
+    float red = 0.f;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        const float4 iz = *reinterpret_cast<const float4*>(&ctl->invz[half * 64 + q * 4]);
+        red = fmaf(e[q * 4], iz.x, red);
+        red = fmaf(e[q * 4 + 1], iz.y, red);
+        red = fmaf(e[q * 4 + 2], iz.z, red);
+        red = fmaf(e[q * 4 + 3], iz.w, red);
+    }
+    if (half == 1) ctl->sum[1][i] = red;
+    __syncthreads();
+    if (half == 0 && i < S && ok) {
+        const size_t o = size_t(slab) * max_sent + i;
+        float lam = fmaxf(ctl->mx[0][i], ctl->mx[1][i]);
+        if (ext.table) {                                 // penalty from the generation-space table through Phi
+            const int g = ext.sent_id[o];
+            lam = (g >= 0 && g < ext.table_len) ? ext.table[size_t(slab / Hk) * ext.table_len + g] : 0.f;
+        } else {
+            lam = (lam > tau) ? lam : 0.f;
+        }
+        red = (red + ctl->sum[1][i]) / float(S);
+        sent_lam[o] = lam;
+        sent_red[o] = red;
+        sent_score[o] = sigma * ctl->imp[i] - (1.f - sigma) * red - lam;
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 128);
+    }
+}
+
 template <int kSweep, int kN>
 static int launch_sweep(const CUtensorMap& mapK, const CUtensorMap& mapQ, const SweepArgs& a, int grid, size_t smem,
                         cudaStream_t st) {
@@ -1039,6 +1209,14 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         default: break;
     }
     if (rc) return rc;
+    // one tile of sentences per slab: one kernel instead of three, with the operands in shared memory throughout
+    if (shape->max_sent <= kSmallSent) {
+        SKIPKV_CUDA(launch_dependent(score_small_kernel, dim3(L.slabs), dim3(kSmallThreads), kSmallSmem, st, Hk, int(shape->max_sent),
+                                     int(shape->max_cap), shape->cap, kv_len, sent_off, n_sent, params->eps, params->sigma,
+                                     params->tau, static_cast<const float*>(sc_tok), static_cast<const float*>(vsum), sent_imp,
+                                     sent_red, sent_lam, sent_score, ext, reinterpret_cast<const Header*>(w + L.header)));
+        return SKIPKV_OK;
+    }
     {
         dim3 pgrid((shape->max_sent + 7) / 8, L.slabs);
         SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, Hk, shape->max_sent, shape->max_cap,

@@ -41,3 +41,31 @@ def test_decode_rows_around_warp_and_tile_edges(hq):
         out = D.out.float().cpu().numpy().astype(np.float64)
         err = np.abs(out - o64) / np.abs(o64).max(axis=-1, keepdims=True)
         assert np.isfinite(out).all() and err.max() <= 2e-2 and np.sqrt((err ** 2).mean()) < 2e-3
+
+
+def check_scores(B, L, D, rtol=1e-3):
+    cfg = L["cfg"]
+    D.score()
+    torch.cuda.synchronize()
+    assert D.status() == 0
+    ref = oracle.score_batch(oshape(L), W.bf16_bits(L["K"]), W.bf16_bits(L["q_win"]), L["kv_len"], L["sent_off"], L["n_sent"],
+                             float(np.float32(0.1)), float(np.float32(0.95)), float(np.float32(1e-6)), want_tok_imp=True)
+    live = np.arange(L["max_sent"])[None, None, :] < L["n_sent"][:, :, None]
+    for name, got in (("imp", D.sent_imp), ("red", D.sent_red), ("lam", D.sent_lam), ("score", D.sent_score)):
+        g, r = got.cpu().numpy()[live].astype(np.float64), np.asarray(ref[name], np.float64)[live]
+        assert (np.abs(g - r) <= rtol * np.abs(r) + 1e-7).all(), (name, np.abs(g - r).max())
+    tok = D.tok_imp.cpu().numpy()
+    for b in range(cfg.batch):
+        for h in range(cfg.n_kv_heads):
+            rows = W.slab_rows(L, b, h)
+            n = int(L["kv_len"][b, h])
+            g, r = tok[rows][:n].astype(np.float64), np.asarray(ref["tok_imp"], np.float64)[rows][:n]
+            assert (np.abs(g - r) <= rtol * np.abs(r)).all(), ("tok_imp", b, h)
+
+
+@pytest.mark.parametrize("sentences", [[1, 2, 31, 33], [63, 64, 65, 128], [127, 129, 5, 1], [256, 257, 300]])
+def test_score_sentence_counts_around_a_tile(sentences):
+    """Up to 128 sentences per slab: one kernel behind the sweeps; more: the blocked kernels."""
+    B, L, D = layer([5 * n for n in sentences], sent_lo=5, sent_hi=5, dup_rate=0.3, seed=500 + sentences[0])
+    assert int(L["n_sent"].max()) == max(sentences)
+    check_scores(B, L, D)
