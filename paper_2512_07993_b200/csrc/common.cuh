@@ -35,7 +35,8 @@ struct WsLayout {
     size_t cp_run_dst;     // int32  [slabs][max_sent+1]  first destination token; [nruns] = new_len
     size_t dec_cnt;        // uint32 [slabs]              partials that arrived (self-resetting)
     size_t dec_part;       // float  [max_ctas + slabs][group][kDecPartStride]
-    size_t sc_part;        // float2 [(max_ctas + slabs) * 4][sc_rb * 128]  (max, sum) of a CTA's part of a slab
+    size_t sc_cnt;         // uint32 [slabs]              tiles whose log-sum-exp records are written (zero between calls)
+    size_t sc_part;        // float2 [max_ctas + slabs][sc_ra * 128]  (reference, sum) of a CTA's part of a slab
     size_t sc_tokimp;      // float  [slabs][max_cap]
     size_t sc_vsum;        // float  [slabs][max_sent][128]  per-sentence sums of key rows
     size_t sc_vbar_hi;     // bf16   [slabs][max_sent][128]  normalised mean key, high part
@@ -46,8 +47,9 @@ struct WsLayout {
     size_t tr_z;           // float  [slabs][max_cap]  token redundancy: row sums of exp(G)
     size_t total;
     int slabs, group, qrows, dec_max_ctas;
-    int sc_wb;             // window positions per query block: floor(128 / group)
-    int sc_rb;             // query blocks per group: ceil(window / sc_wb)
+    int sc_wb;             // window positions per block of query rows of the scoring sweeps: 32 or 16
+    int sc_rb;             // blocks: ceil(window / sc_wb)
+    int sc_ra;             // the same rows in blocks of 128
 };
 
 constexpr int kDecPartStride = 132;    // decode partial of one head: 128 accumulators, max, sum, padding
@@ -62,8 +64,13 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     L.slabs = s.batch * s.n_kv_heads;
     L.group = s.n_q_heads / s.n_kv_heads;
     L.qrows = L.group * s.window;
-    L.sc_wb = 128 / (L.group > 0 ? L.group : 1);
+    // scoring sweeps: a block of query rows is sc_wb window positions x group heads.  32 positions where the accumulators of
+    // such a block (32 * group columns) leave room for three of them, and where that does not pad the window to more rows.
+    const int n = L.group > 0 ? L.group : 1;
+    const int r32 = (s.window + 31) / 32 * 32 * n;
+    L.sc_wb = (s.window > 16 && n <= 5 && r32 <= kMaxQRows) ? 32 : 16;
     L.sc_rb = (s.window + L.sc_wb - 1) / L.sc_wb;
+    L.sc_ra = (L.sc_rb * L.sc_wb * n + 127) / 128;
     L.dec_max_ctas = kDecMaxCtas;
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align256(o + bytes); return r; };
@@ -75,8 +82,9 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     L.cp_run_src = take(slabs * ms * 4);
     L.cp_run_dst = take(slabs * (ms + 1) * 4);
     L.dec_cnt = take(slabs * 4);
+    L.sc_cnt = take(slabs * 4);
     L.dec_part = take((size_t(L.dec_max_ctas) + slabs) * L.group * kDecPartStride * 4);
-    L.sc_part = take((size_t(L.dec_max_ctas) + slabs) * 4 * size_t(L.sc_rb) * 128 * 8);
+    L.sc_part = take((size_t(L.dec_max_ctas) + slabs) * size_t(L.sc_ra) * 128 * 8);
     L.sc_tokimp = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);
     L.sc_vsum = take(slabs * ms * kHeadDim * 4);
     L.sc_vbar_hi = take(slabs * ms * kHeadDim * 2);
@@ -117,7 +125,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // host: launch `kernel` on `st` as a programmatic dependent of the kernel enqueued before it; more than 48 KB of dynamic
 // shared memory is asked for as needed
-template <typename... KArgs, typename... Args>
+template <bool kCooperative = false, typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                     Args... args) {
     cudaLaunchConfig_t cfg{};
@@ -125,11 +133,13 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = kCooperative ? 2 : 1;
     if (smem > 48 * 1024)
         if (cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(kernel))) return e;
     cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
@@ -250,8 +260,12 @@ __device__ __forceinline__ void cta_prefix(int n, F count, int* pref, uint32_t* 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int per = (n + kThreads - 1) / kThreads;
     const int s0 = min(tid * per, n), s1 = min(s0 + per, n);
-    uint32_t local = 0;
-    for (int s = s0; s < s1; ++s) local += uint32_t(count(s));
+    uint32_t local = 0, first = 0;
+    for (int s = s0; s < s1; ++s) {
+        const uint32_t c = uint32_t(count(s));
+        if (s == s0) first = c;
+        local += c;
+    }
     uint32_t inc = local;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -260,12 +274,13 @@ __device__ __forceinline__ void cta_prefix(int n, F count, int* pref, uint32_t* 
     }
     if (lane == 31) wsum[warp] = inc;
     __syncthreads();
-    uint32_t base = 0;
-    for (int w = 0; w < warp; ++w) base += wsum[w];
+    uint32_t base = (lane < warp) ? wsum[lane] : 0u;      // at most 32 warps
+#pragma unroll
+    for (int d = 16; d; d >>= 1) base += __shfl_xor_sync(0xffffffffu, base, d);
     uint32_t run = base + inc - local;
     for (int s = s0; s < s1; ++s) {
         pref[s] = int(run);
-        run += uint32_t(count(s));
+        run += s == s0 ? first : uint32_t(count(s));
     }
     if (tid == kThreads - 1) pref[n] = int(run);
     __syncthreads();

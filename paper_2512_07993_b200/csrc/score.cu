@@ -1,11 +1,12 @@
 // skipkv_score: sentence scores per (sequence, KV head) slab (paper Section 4.1).
 //
-//   sweep 1   log-sum-exp of every window-query row over the slab's tokens
-//             (tensor cores: logits = Q_group x K_tile^T, one thread per query row)
-//   sweep 2   tok_imp[t] = (1/alpha) sum_w max_q 2^(s_q[w][t] - lse_q[w])   (max before exp: exp is monotone)
-//             (tensor cores: logits = K_tile x Q_group^T, one thread per token), and in the same pass
+//   sweeps    (one launch) pass A: log-sum-exp of every window-query row over the slab's tokens
+//             (tensor cores: logits = Q_rows x K_tile^T, one thread per query row);
+//             pass B: tok_imp[t] = (1/alpha) sum_w max_q 2^(s_q[w][t] - lse_q[w])   (max before exp: exp is monotone)
+//             (tensor cores: logits - lse = [K_tile, 1] x [Q_block, -lse]^T, one thread per token), and in the same pass
 //             the per-sentence sums of the key rows as a second product on the tile already in shared
 //             memory: K_tile^T x (0/1 matrix token -> sentence slot)
+//   up to 128 sentences per slab: one kernel for the rest, else
 //   pool      per sentence: mean tok_imp, mean key, normalisation, split into bf16 high and low parts
 //   gram x2   pairwise cosine G on the tensor cores (three bf16 products: hi.hi + hi.lo + lo.hi);
 //             pass 1: Z_i = sum_{j!=i} e^{G_ij} and lam_i = max_{j>i} G_ij;
@@ -14,17 +15,16 @@
 // Logits are kept in base 2: s = (q.k) * log2(e)/sqrt(d).  |G| <= 1 so the row softmax of G
 // needs no max subtraction.
 //
-// Both sweeps are persistent, warp-specialised kernels, one CTA per SM: a TMA warp streams
-// 128-token key tiles (and the group's query block) into shared memory, one thread issues
-// tcgen05.mma into a ring of tensor-memory accumulators (four in sweep 1, three in sweep 2), several
-// warpgroups of epilogue warps take the tiles round-robin, and (sweep 2) one more warpgroup writes the 0/1
+// The sweeps are a persistent, warp-specialised kernel, one CTA per SM: a TMA warp streams 128-token key tiles (and the
+// group's query rows) into shared memory, one thread issues tcgen05.mma into a ring of tensor-memory accumulators,
+// warpgroups of epilogue warps take the tiles round-robin, and (pass B) one more warpgroup writes the 0/1
 // matrices of the pooling product and reads out the pooled sums while one thread of a further warp issues
 // that product.  Work is the list of 128-token tiles over all slabs cut into equal contiguous ranges, so
 // ragged slabs balance.
 //
-// Query rows of a group are staged as blocks of WB = floor(128/n) window positions x n heads
-// (row q*WB + w of a block), so that the n heads of a window position sit at a fixed column
-// stride for the max over heads.
+// Query rows of a group are staged as blocks of WB window positions x n heads (row q*WB + w of a block), so that the n
+// heads of a window position sit at a fixed column stride for the max over heads; pass A takes the same rows in
+// blocks of 128.
 #include <cstddef>
 
 #include "common.cuh"
@@ -32,55 +32,57 @@
 
 namespace skipkv {
 
-constexpr int kAccBufs = 4;             // tensor-memory accumulators of 128 columns
-constexpr int kMaxRB = 4;               // query blocks per group
-constexpr int kSwMaxStages = 6;
-constexpr int kSw1Groups = 4;           // epilogue warpgroups of sweep 1
-constexpr int kSw2Groups = 2;           // epilogue warpgroups of sweep 2
-constexpr int kSw2Bufs = 3;             // sweep 2: accumulators of the logits (the columns after them hold the pooled sums)
-constexpr int kPoolWarps = 4;           // sweep 2: the warpgroup that writes the indicator matrices and drains the pooled sums
+// ---------------------------------------------------------------------------------------
+// Both sweeps over the keys in one persistent launch.  A CTA goes through its range of tiles twice:
+//   pass A   log-sum-exp of every window-query row over the CTA's part of each slab -> one record per (CTA, slab)
+//   pass B   importance of every token and the per-sentence key sums
+// Between the two it waits, slab by slab, until every CTA that shares the slab has left its record (a counter of tiles);
+// nobody waits for anything but pass A of CTAs that are all resident (one per SM), and the waits are bounded anyway.
+// As two launches the second started its first tile 6 us after the first had drained.  Pass A runs backwards through the
+// range, so that pass B finds the tiles read last in L2 -- or, where the range fits into the ring, still in shared memory.
+// ---------------------------------------------------------------------------------------
+constexpr int kStagesMax = 6;
+constexpr int kAGroups = 4;             // pass A: epilogue warpgroups = accumulators of 128 columns
+constexpr int kBGroups = 3;             // pass B: epilogue warpgroups = accumulators of up to 160 columns
+constexpr int kBAccCols = 160;
 constexpr int kIndRing = 2;             // indicator matrices in flight (the pooled sums have two accumulators of their own)
 constexpr int kIndSlots = 16;           // sentence slots of one indicator matrix
 constexpr int kIndBytes = kIndSlots * 128 * 2;   // [16 slots][128 tokens] bf16 as two 64-token halves, 128-byte swizzle
-constexpr uint32_t kPoolCol = kSw2Bufs * 128;    // tensor-memory column of the first pooled-sum accumulator (16 columns each)
-constexpr int kSw1Threads = (2 + 4 * kSw1Groups) * 32;        // TMA warp, MMA warp, epilogue warps
-constexpr int kSw2Threads = (2 + 4 * kSw2Groups + kPoolWarps + 1) * 32;   // + the thread that issues the pooling products
+constexpr uint32_t kPoolCol = kBGroups * kBAccCols;   // tensor-memory column of the first pooled-sum accumulator (16 columns each)
+constexpr int kPoolWarps = 4;
+constexpr int kSweepThreads = (2 + 4 * kAGroups + 1) * 32;    // TMA warp, MMA warp, 16 epilogue warps, issuer of the pooling products
+constexpr int kMaxBlocksA = 5;          // blocks of 128 query rows
+constexpr int kExtRow = 32;             // bytes of a row of the extra K step (16 bf16)
 constexpr float kLog2e = 1.4426950408889634f;
 
-__device__ __forceinline__ float ex2f(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 struct SweepCtl {                       // barriers and small shared state, after the tile buffers
-    uint64_t full[kSwMaxStages], empty[kSwMaxStages];
+    uint64_t full[kStagesMax], empty[kStagesMax];
     uint64_t qfull, qempty;
     // "accumulator ready" barriers are per epilogue warpgroup (a ring of 4 per group, indexed by the group's own item
     // count), so every barrier has one consumer that sees its phases in order; a barrier per accumulator would be
     // waited on by different groups in turn, and a group polling for a later phase could pass on an earlier one.
-    uint64_t tfull[4][4], tempty[kAccBufs];
-    uint32_t tmem_base;
-    int abort_flag;
-    // sweep 2, ring of indicator matrices: written by the four pooling warps -> multiplied by the MMA thread -> drained by
-    // the pooling warps
+    uint64_t tfull_a[kAGroups][4], tempty_a[kAGroups], tfull_b[kBGroups][4], tempty_b[kBGroups];
+    uint64_t extfull, extempty;         // pass B: the rows' -lse as operand columns
+    // ring of indicator matrices: written by the four pooling warps -> multiplied by their issuer -> read out by the pooling warps
     uint64_t ifull[kIndRing], iempty[kIndRing];
     uint64_t pfull[2];                  // the last product of a run of tiles into accumulator i has completed
     uint64_t issued_done[2];            // after a failed wait: every product of the MMA thread (0) / the pooling issuer (1) has retired
+    uint32_t tmem_base;
+    int abort_flag;
     int ind_flags[kIndRing];            // 1: the tile has another matrix after this one, 2: joins the open run, 4: closes a run
     uint32_t wsum[32];
-    alignas(16) float neg_lse[kSw2Groups][kMaxRB * 128];   // sweep 2: one copy per epilogue warpgroup (read as float4)
 };
-static_assert(offsetof(SweepCtl, neg_lse) % 16 == 0, "neg_lse is read with 16-byte loads");
 
 struct SweepArgs {
-    int Hq, Hk, window, n_slabs, max_cap, max_sent, RB, WB, stages;
+    int Hq, Hk, window, n_slabs, max_cap, max_sent, stages;
+    int WB, RB, N, R, RA;               // window positions per block of pass B, its blocks, their rows N = WB * n; all rows R = RB * N; blocks of pass A
     const int64_t* slab_off;
     const int32_t* cap;
     const int32_t* kv_len;
     const int32_t* sent_off;
     const int32_t* n_sent;
-    float2* sc_part;                    // [(cta + slab) * kSw1Groups + warpgroup][RB * 128] (max, sum)
+    float2* rec;                        // [cta + slab][RA * 128] (reference, sum) of a CTA's part of a slab
+    uint32_t* lse_cnt;                  // [slabs] tiles whose records are written; zero at the start
     float* tok_imp_user;
     float* tok_imp_ws;
     float* vsum;                        // [slabs][max_sent][128] sums of key rows
@@ -90,9 +92,47 @@ struct SweepArgs {
     int max_pages;
 };
 
-// ---- sweep 1 epilogue: one accumulator (128 tokens) folded into the running (max, sum) of a row
-// (The loop over the four 32-column pieces is kept rolled, here and in imp_fold for four heads per group: the epilogue
-// code is fetched again for every tile, and unrolled it stalls on instruction fetch more than the loop costs.)
+__device__ __forceinline__ float ex2f(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// Bounded wait of one thread until *p reaches `want`; gives up like role_wait.
+static __device__ __noinline__ bool flag_wait(const uint32_t* p, uint32_t want, uint32_t limit, int* abort_flag, uint32_t* status) {
+    for (uint32_t i = 0; i < limit; ++i) {
+        if (ld_acquire(p) >= want) return true;
+        if (i > 16) __nanosleep(32);
+        if ((i & 255) == 255 && *reinterpret_cast<volatile int*>(abort_flag)) return false;
+    }
+    atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
+    *reinterpret_cast<volatile int*>(abort_flag) = 1;
+    return false;
+}
+
+// D[128 x n] (+)= A[128 x 128] * B[n x 128]^T.  Both operands are two halves of 64 channels, a_half / b_half bytes apart.
+__device__ __forceinline__ void umma_tile(uint32_t tmem_d, uint32_t a_smem, uint32_t a_half, uint32_t b_smem, uint32_t b_half, uint32_t idesc) {
+    const uint64_t da = umma_desc_sw128(a_smem), db = umma_desc_sw128(b_smem);
+#pragma unroll
+    for (int half = 0; half < 2; ++half)
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+            umma_bf16(tmem_d, da + uint64_t(half * (a_half >> 4) + ks * 2), db + uint64_t(half * (b_half >> 4) + ks * 2), idesc, (half || ks) ? 1u : 0u);
+}
+// Descriptor of a K-major operand of 16 columns, rows 32 bytes apart, 32-byte swizzle (groups of 8 rows 256 bytes apart).
+__device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
+    return uint64_t((smem_addr >> 4) & 0x3fffu) | (uint64_t(1) << 16) | (uint64_t(256 >> 4) << 32) | (uint64_t(1) << 46) | (uint64_t(6) << 61);
+}
+__device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
+
+// ---- pass A epilogue: one accumulator (128 tokens) folded into a row's sum of 2^(logit - m).  The reference m is the
+// largest logit of the row's first 32 tokens; it stays, whatever comes later, as long as a chunk's sum is below 2^60 --
+// no running maximum and no rescaling in the common case.  A chunk beyond that is folded again under a larger reference.
 template <bool kMasked>
 __device__ __forceinline__ void lse_fold(uint32_t taddr, int valid, float scale, float& m, float& l) {
     const int nch = kMasked ? (valid + 31) >> 5 : 4;
@@ -105,102 +145,73 @@ __device__ __forceinline__ void lse_fold(uint32_t taddr, int valid, float scale,
             for (int j = 0; j < 32; ++j)
                 if (ch * 32 + j >= valid) v[j] = -INFINITY;
         }
-        float c0 = fmaxf(v[0], v[1]), c1 = fmaxf(v[2], v[3]);
+        auto chunk_max = [&]() {
+            float c0 = fmaxf(v[0], v[1]), c1 = fmaxf(v[2], v[3]);
 #pragma unroll
-        for (int j = 4; j < 32; j += 2) { c0 = fmaxf(c0, v[j]); c1 = fmaxf(c1, v[j + 1]); }
-        const float m_new = fmaxf(m, fmaxf(c0, c1) * scale);
-        const float neg = -m_new;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+            for (int j = 4; j < 32; j += 4) { c0 = max3(c0, v[j], v[j + 1]); c1 = max3(c1, v[j + 2], v[j + 3]); }
+            return fmaxf(c0, c1) * scale;
+        };
+        auto chunk_sum = [&]() {
+            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+            const float neg = -m;
 #pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-            s0 += ex2f(fmaf(v[j + 0], scale, neg));
-            s1 += ex2f(fmaf(v[j + 1], scale, neg));
-            s2 += ex2f(fmaf(v[j + 2], scale, neg));
-            s3 += ex2f(fmaf(v[j + 3], scale, neg));
+            for (int j = 0; j < 32; j += 4) {
+                s0 += ex2f(fmaf(v[j + 0], scale, neg));
+                s1 += ex2f(fmaf(v[j + 1], scale, neg));
+                s2 += ex2f(fmaf(v[j + 2], scale, neg));
+                s3 += ex2f(fmaf(v[j + 3], scale, neg));
+            }
+            return (s0 + s1) + (s2 + s3);
+        };
+        if (m == -INFINITY) m = chunk_max();
+        float s = chunk_sum();
+        if (!(s < 1.15e18f)) {
+            const float m_new = fmaxf(m, chunk_max());
+            l *= ex2f(m - m_new);
+            m = m_new;
+            s = chunk_sum();
         }
-        l = l * ex2f(m - m_new) + ((s0 + s1) + (s2 + s3));      // first chunk: 2^(-inf) = 0
-        m = m_new;
+        l += s;
     }
 }
 
-// ---- sweep 2 epilogue: one accumulator (this thread's token x one query block) added to the token's total
-template <int kN>
-__device__ __forceinline__ float imp_fold(uint32_t taddr, const float* neg_lse, int wvalid, float scale) {
-    constexpr int WB = 128 / kN;
-    if constexpr (kN == 4) {
-        float b4[32];
+// ---- pass B epilogue: one accumulator (this thread's token x one block of kWB window positions x n heads, a head's
+// positions in consecutive columns) added to the token's total.  The logits come less the row's log-sum-exp, so the
+// maximum over the heads needs no further arithmetic, and one exponential per window position follows it.
+template <int kWB>
+__device__ __forceinline__ float imp_fold(uint32_t taddr, int n, int wvalid, float scale) {
+    float t0 = 0.f, t1 = 0.f;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) b4[j] = -INFINITY;
+    for (int c = 0; c < kWB; c += 16) {
+        if (c >= wvalid) break;
+        float best[16];
+        tmem_ld16(taddr + c, best);
+        int q = 1;
 #pragma unroll 1
-        for (int q = 0; q < 4; ++q) {
-            float v[32];
-            tmem_ld32(taddr + q * 32, v);
+        for (; q + 1 < n; q += 2) {
+            float x[16], y[16];
+            tmem_ld16(taddr + q * kWB + c, x);
+            tmem_ld16(taddr + (q + 1) * kWB + c, y);
 #pragma unroll
-            for (int j4 = 0; j4 < 32; j4 += 4) {
-                const float4 nl = *reinterpret_cast<const float4*>(neg_lse + q * 32 + j4);
-                b4[j4 + 0] = fmaxf(b4[j4 + 0], fmaf(v[j4 + 0], scale, nl.x));
-                b4[j4 + 1] = fmaxf(b4[j4 + 1], fmaf(v[j4 + 1], scale, nl.y));
-                b4[j4 + 2] = fmaxf(b4[j4 + 2], fmaf(v[j4 + 2], scale, nl.z));
-                b4[j4 + 3] = fmaxf(b4[j4 + 3], fmaf(v[j4 + 3], scale, nl.w));
-            }
+            for (int w = 0; w < 16; ++w) best[w] = max3(best[w], x[w], y[w]);
         }
-        float t0 = 0.f, t1 = 0.f;
+        if (q < n) {
+            float x[16];
+            tmem_ld16(taddr + q * kWB + c, x);
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-            t0 += (j < wvalid) ? ex2f(b4[j]) : 0.f;
-            t1 += (j + 1 < wvalid) ? ex2f(b4[j + 1]) : 0.f;
+            for (int w = 0; w < 16; ++w) best[w] = fmaxf(best[w], x[w]);
         }
-        return t0 + t1;
-    }
-    if constexpr (kN > 4) {
-        // WB <= 25 window positions per head: one load of 32 columns per head, starting at the head's first column
-        // (the columns read past its last position are not used), in a rolled loop like the four-head case
-        float best[WB];
+        const int left = wvalid - c;
 #pragma unroll
-        for (int w = 0; w < WB; ++w) best[w] = -INFINITY;
-#pragma unroll 1
-        for (int q = 0; q < kN; ++q) {
-            float v[32];
-            tmem_ld32(taddr + q * WB, v);
-            const float* nl = neg_lse + q * WB;
-#pragma unroll
-            for (int w = 0; w < WB; ++w) best[w] = fmaxf(best[w], fmaf(v[w], scale, nl[w]));
-        }
-        float t0 = 0.f, t1 = 0.f;
-#pragma unroll
-        for (int w = 0; w < WB; w += 2) {
-            t0 += (w < wvalid) ? ex2f(best[w]) : 0.f;
-            if (w + 1 < WB) t1 += (w + 1 < wvalid) ? ex2f(best[w + 1]) : 0.f;
-        }
-        return t0 + t1;
-    }
-    float best[WB];
-    float total = 0.f;
-#pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-        if (ch * 32 >= kN * WB) break;
-        float v[32];
-        tmem_ld32(taddr + ch * 32, v);
-#pragma unroll
-        for (int j4 = 0; j4 < 32; j4 += 4) {
-            const float4 nl = *reinterpret_cast<const float4*>(neg_lse + ch * 32 + j4);
-            const float nls[4] = {nl.x, nl.y, nl.z, nl.w};
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                const int c = ch * 32 + j4 + jj;
-                if (c < kN * WB) {
-                    const int q = c / WB, w = c % WB;
-                    const float x = fmaf(v[j4 + jj], scale, nls[jj]);
-                    best[w] = (q == 0) ? x : fmaxf(best[w], x);
-                    if (q == kN - 1) total += (w < wvalid) ? ex2f(best[w]) : 0.f;
-                }
-            }
+        for (int w = 0; w < 16; w += 2) {
+            t0 += (w < left) ? ex2f(best[w] * scale) : 0.f;
+            t1 += (w + 1 < left) ? ex2f(best[w + 1] * scale) : 0.f;
         }
     }
-    return total;
+    return t0 + t1;
 }
 
-// ---- sweep 2: pooled key sums on the tensor cores
+// ---- pass B: pooled key sums on the tensor cores
 // Pooling product of one staged tile: D[128 channels x 16 slots] = K_tile^T x Ind^T.  A = the tile as the TMA load
 // wrote it ([token][channel], two 64-channel halves, 128-byte swizzle) read as an MN-major operand: 64 channels x 8
 // tokens per swizzle atom, atoms 1024 bytes apart along the tokens and a half (16 KB) apart along the channels.
@@ -217,20 +228,6 @@ __device__ __forceinline__ void umma_pool(uint32_t tmem_d, uint32_t tile_smem, u
         umma_bf16(tmem_d, da, db, kIdescPool, (accumulate || ks) ? 1u : 0u);
     }
 }
-// 16 consecutive fp32 columns of this thread's tensor-memory lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 // One 16-byte piece of an indicator matrix: tokens 8c .. 8c + 7 of slot row j; ones (bf16 1.0) for the tokens
 // [lo, hi), zeros elsewhere.
 __device__ __forceinline__ void indicator_piece(uint8_t* ind, int j, int c, int lo, int hi) {
@@ -244,23 +241,24 @@ __device__ __forceinline__ void indicator_piece(uint8_t* ind, int j, int c, int 
     *reinterpret_cast<uint4*>(ind + (c >> 3) * (kIndBytes / 2) + j * 128 + (((c & 7) ^ (j & 7)) << 4)) = val;
 }
 
-template <int kSweep, int kN>
-__global__ void __launch_bounds__(kSweep == 1 ? kSw1Threads : kSw2Threads, 1)
-score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapQ,
-                   const SweepArgs a) {
+template <int kWB>
+__global__ void __launch_bounds__(kSweepThreads, 1)
+score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapQ, const SweepArgs a) {
     extern __shared__ uint8_t sweep_smem_raw[];
-    constexpr int kThreads = kSweep == 1 ? kSw1Threads : kSw2Threads;
-    constexpr int kGroups = kSweep == 1 ? kSw1Groups : kSw2Groups;
     const uint32_t raw = smem_u32(sweep_smem_raw);
-    uint8_t* tiles = sweep_smem_raw + (((raw + 1023u) & ~1023u) - raw);          // 1024-byte aligned
-    uint8_t* qbuf = tiles + size_t(a.stages) * kOpBytes;
-    uint8_t* indb = qbuf + size_t(a.RB) * kOpBytes;                              // sweep 2: the indicator matrices
-    SweepCtl* ctl = reinterpret_cast<SweepCtl*>(indb + (kSweep == 2 ? kIndRing * kIndBytes : 0));
+    uint8_t* qbuf = sweep_smem_raw + (((raw + 1023u) & ~1023u) - raw);           // [2 halves][R rows][128 bytes]
+    const uint32_t q_half = uint32_t(a.R) * 128u;
+    uint8_t* tiles = qbuf + size_t(a.R) * kRowBytes;                             // (R is a multiple of 16: 1024-byte aligned)
+    uint8_t* indb = tiles + size_t(a.stages) * kOpBytes;                         // pass B: the indicator matrices
+    uint8_t* onesb = indb + kIndRing * kIndBytes;                                // pass B: the keys' side of the extra K step
+    uint8_t* extb = onesb + 128 * kExtRow;                                       // pass B: the queries' side; pass A: [4 groups][RA * 128] (m, l)
+    SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + size_t(a.RA) * 128 * kExtRow);
     int* pref = reinterpret_cast<int*>(ctl + 1);                                 // [n_slabs + 1] tile prefix
+    int* rowb = pref + a.n_slabs + 1;                                            // [n_slabs] cache row of a slab's first token
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, cta = blockIdx.x;
-    const int n_slabs = a.n_slabs, Hk = a.Hk, RB = a.RB;
+    const int n_slabs = a.n_slabs, Hk = a.Hk;
     pdl_trigger();
     auto live = [&](int s) {
         const int room = a.block_table ? min(a.cap[s / Hk], a.max_pages * 128) : a.cap[s / Hk];
@@ -268,15 +266,19 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     };
 
     if (tid == 0) {
-        for (int s = 0; s < kSwMaxStages; ++s) {
-            mbar_init(&ctl->full[s], 1);
-            mbar_init(&ctl->empty[s], kSweep == 1 ? 1 : 2);      // commit of the logits (+ commit of the tile's last pooling product)
-        }
+        for (int s = 0; s < kStagesMax; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 2); }
         mbar_init(&ctl->qfull, 1);
         mbar_init(&ctl->qempty, 1);
-        for (int b = 0; b < kAccBufs; ++b) mbar_init(&ctl->tempty[b], 4);
-        for (int g = 0; g < 4; ++g)
-            for (int j = 0; j < 4; ++j) mbar_init(&ctl->tfull[g][j], 1);
+        for (int g = 0; g < kAGroups; ++g) {
+            mbar_init(&ctl->tempty_a[g], 4);
+            for (int j = 0; j < 4; ++j) mbar_init(&ctl->tfull_a[g][j], 1);
+        }
+        for (int g = 0; g < kBGroups; ++g) {
+            mbar_init(&ctl->tempty_b[g], 4);
+            for (int j = 0; j < 4; ++j) mbar_init(&ctl->tfull_b[g][j], 1);
+        }
+        mbar_init(&ctl->extfull, 4);
+        mbar_init(&ctl->extempty, 1);
         for (int i = 0; i < kIndRing; ++i) { mbar_init(&ctl->ifull[i], kPoolWarps); mbar_init(&ctl->iempty[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&ctl->pfull[i], 1); mbar_init(&ctl->issued_done[i], 1); }
         ctl->abort_flag = 0;
@@ -285,73 +287,79 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         tmap_prefetch(&mapQ);
     }
     if (warp == 1) tmem_alloc(&ctl->tmem_base, 512);
-    // the lengths may come from the kernel before this call (and, in sweep 2, the records from sweep 1): the set-up
-    // above touched nothing that another kernel writes
-    pdl_wait();
+    // every key row of the extra K step is 1 in the columns that carry a query row's -lse (three bf16 pieces, half of each
+    // in either 8-column piece of the row, so that a swizzle that exchanges the two makes no difference)
+    if (tid < 256) *reinterpret_cast<uint4*>(onesb + tid * 16) = make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);
+    fence_proxy_async_smem();
+    pdl_wait();                                          // the lengths may come from the kernel before this call
     const uint32_t limit = load_wait_limit(a.hdr);
     tc_fence_before();
-    cta_prefix<kThreads>(n_slabs, [&](int s) { return (live(s) + 127) >> 7; }, pref, ctl->wsum);   // also publishes the set-up
+    for (int s = tid; s < n_slabs; s += kSweepThreads)
+        rowb[s] = a.block_table ? 0 : int(slab_row0(a.slab_off, a.cap, Hk, s / Hk, s % Hk));
+    cta_prefix<kSweepThreads>(n_slabs, [&](int s) { return (live(s) + 127) >> 7; }, pref, ctl->wsum);   // also publishes the set-up
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    const int Ttot = pref[n_slabs];
-    const int per_cta = max(1, (Ttot + G - 1) / G);
-    const int t_begin = min(cta * per_cta, Ttot), t_end = min(t_begin + per_cta, Ttot);
+    const int T = pref[n_slabs], Ge = min(G, T);         // CTA c has the tiles [c T / Ge, (c + 1) T / Ge)
+    const int t_begin = cta < Ge ? int((long long)cta * T / Ge) : T, t_end = cta < Ge ? int((long long)(cta + 1) * T / Ge) : T;
     const int ntl = t_end - t_begin;
-    int slab0 = 0;
-    if (ntl > 0) {
+    auto slab_of = [&](int t) {                          // last slab that starts at or before tile t
         int lo = 0, hi = n_slabs - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (pref[mid] <= t_begin) lo = mid; else hi = mid - 1;
+            if (pref[mid] <= t) lo = mid; else hi = mid - 1;
         }
-        slab0 = lo;
-    }
+        return lo;
+    };
+    auto owner = [&](int t) { return int(((long long)(t + 1) * Ge - 1) / T); };
+    const bool resident = ntl <= a.stages;               // the range fits into the ring: pass B reads it where pass A left it
     const float scale = kLog2e * rsqrtf(float(kHeadDim));
     const int n = a.Hq / Hk;
+    const uint32_t ext_smem = smem_u32(extb);
 
-    if (kSweep == 1 && warp < 2 && lane != 0) {
-        // the 62 otherwise idle lanes of the TMA and MMA warps clear the per-sentence key sums that sweep 2 accumulates
-        const size_t total = size_t(n_slabs) * a.max_sent * (kHeadDim / 4);        // float4 words
-        const size_t per = (total + G - 1) / G, w0 = min(size_t(cta) * per, total), w1 = min(w0 + per, total);
-        float4* v4 = reinterpret_cast<float4*>(a.vsum);
-        for (size_t i = w0 + size_t(warp * 31 + lane - 1); i < w1; i += 62) v4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    if (ntl > 0) {
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0 && ntl > 0) {
+        if (lane == 0) {
             // what depends on the slab only is kept in registers: between "stage free" and the next copy's issue nothing
             // waits on shared or global memory
-            int slab = slab0, stage = 0, issued = 0, slab_begin = 0, slab_end = 0;
-            long long row0 = 0;
+            int stage = 0;
             uint32_t lap = 0, qlap = 0;
             bool ok = true;
-            for (int t = t_begin; t < t_end && ok; ++t) {
-                if (t == t_begin || slab_end <= t) {
-                    while (pref[slab + 1] <= t) ++slab;
-                    slab_begin = pref[slab]; slab_end = pref[slab + 1];
-                    row0 = a.block_table ? 0 : (long long)slab_row0(a.slab_off, a.cap, Hk, slab / Hk, slab % Hk);
-                    if (qlap > 0) ok = role_wait(&ctl->qempty, (qlap - 1) & 1u, limit, &ctl->abort_flag, a.status);
-                    if (!ok) break;
-                    const int b = slab / Hk, h = slab % Hk;
-                    mbar_expect_tx(&ctl->qfull, uint32_t(RB) * 2u * 128u * uint32_t(a.WB * n));
-                    for (int k = 0; k < RB; ++k) {
-                        tma_load_3d(qbuf + size_t(k) * kOpBytes, &mapQ, 0, k * a.WB, b * a.Hq + h * n, &ctl->qfull);
-                        tma_load_3d(qbuf + size_t(k) * kOpBytes + kOpHalfBytes, &mapQ, 64, k * a.WB, b * a.Hq + h * n,
-                                    &ctl->qfull);
-                    }
-                    ++qlap;
-                }
-                const long long row =
-                    a.block_table ? (long long)max(a.block_table[size_t(slab) * a.max_pages + (t - slab_begin)], 0) * 128
-                                  : row0 + (long long)(t - slab_begin) * 128;
+            auto load_q = [&](int slab) {
+                if (qlap > 0) ok = role_wait(&ctl->qempty, (qlap - 1) & 1u, limit, &ctl->abort_flag, a.status);
+                if (!ok) return;
+                const int b = slab / Hk, h = slab % Hk;
+                mbar_expect_tx(&ctl->qfull, uint32_t(a.R) * kRowBytes);
+                for (int k = 0; k < a.RB; ++k)
+                    for (int half = 0; half < 2; ++half)
+                        tma_load_3d(qbuf + size_t(half) * q_half + size_t(k) * a.N * 128, &mapQ, half * 64, k * kWB, b * a.Hq + h * n, &ctl->qfull);
+                ++qlap;
+            };
+            auto load_tile = [&](int slab, int j, int row0) {
+                const int row = a.block_table ? max(a.block_table[size_t(slab) * a.max_pages + j], 0) * 128 : row0 + j * 128;
                 if (lap > 0) ok = role_wait(&ctl->empty[stage], (lap - 1) & 1u, limit, &ctl->abort_flag, a.status);
-                if (!ok) break;
+                if (!ok) return;
                 uint8_t* dst = tiles + size_t(stage) * kOpBytes;
                 mbar_expect_tx(&ctl->full[stage], kOpBytes);
-                tma_load_2d(dst, &mapK, 0, int(row), &ctl->full[stage]);
-                tma_load_2d(dst + kOpHalfBytes, &mapK, 64, int(row), &ctl->full[stage]);
-                ++issued;
+                tma_load_2d(dst, &mapK, 0, row, &ctl->full[stage]);
+                tma_load_2d(dst + kOpHalfBytes, &mapK, 64, row, &ctl->full[stage]);
                 if (++stage == a.stages) { stage = 0; ++lap; }
+            };
+            for (int pass = 0; pass < 2 && ok; ++pass) {
+                const int t_first = pass == 0 && !resident ? t_end - 1 : t_begin;
+                int slab = slab_of(t_first), lo = 0, hi = 0, row0 = 0;          // tiles [lo, hi) belong to the slab
+                for (int i = 0; i < ntl && ok; ++i) {
+                    const int t = pass == 0 && !resident ? t_end - 1 - i : t_begin + i;
+                    if (i == 0 || t >= hi || t < lo) {
+                        while (pref[slab + 1] <= t) ++slab;
+                        while (pref[slab] > t) --slab;
+                        lo = pref[slab]; hi = pref[slab + 1];
+                        row0 = rowb[slab];
+                        load_q(slab);
+                        if (!ok) break;
+                    }
+                    if (pass == 0 || !resident) load_tile(slab, t - lo, row0);
+                }
             }
             if (!ok) {
                 // copies already issued must land before the CTA retires
@@ -362,14 +370,19 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0 && ntl > 0) {
-            int slab = slab0, stage = 0, it = 0, slab_end = 0;
-            uint32_t lap = 0, qlap = 0;
-            bool ok = true;
-            for (int t = t_begin; t < t_end && ok; ++t) {
-                if (t == t_begin || slab_end <= t) {
+        bool ok = true;
+        uint32_t qlap = 0;
+        int load_no = 0;                                 // tiles of the ring so far: stage load_no % stages, lap load_no / stages
+        if (lane == 0) {
+            int stage = 0, it = 0, slab = slab_of(resident ? t_begin : t_end - 1), lo = 0, hi = 0;
+            uint32_t lap = 0;
+            const uint32_t q0 = smem_u32(qbuf);
+            for (int i = 0; i < ntl && ok; ++i) {
+                const int t = resident ? t_begin + i : t_end - 1 - i;
+                if (i == 0 || t >= hi || t < lo) {
                     while (pref[slab + 1] <= t) ++slab;
-                    slab_end = pref[slab + 1];
+                    while (pref[slab] > t) --slab;
+                    lo = pref[slab]; hi = pref[slab + 1];
                     ok = role_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     ++qlap;
@@ -377,23 +390,59 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 ok = role_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
                 if (!ok) break;
                 const uint32_t k_smem = smem_u32(tiles + size_t(stage) * kOpBytes);
-                for (int k = 0; k < RB && ok; ++k, ++it) {
-                    constexpr int kBufs = kSweep == 1 ? kAccBufs : kSw2Bufs;
-                    const int buf = it % kBufs, use = it / kBufs;
-                    if (use > 0) ok = role_wait(&ctl->tempty[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
+                for (int k = 0; k < a.RA && ok; ++k, ++it) {
+                    const int buf = it & (kAGroups - 1), use = it / kAGroups;
+                    if (use > 0) ok = role_wait(&ctl->tempty_a[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t q_smem = smem_u32(qbuf + size_t(k) * kOpBytes);
-                    if (kSweep == 1) umma_tile_128x128x128(tmem_base + buf * 128, q_smem, k_smem, false);
-                    else             umma_tile_128x128x128(tmem_base + buf * 128, k_smem, q_smem, false);
-                    {
-                        const int ti = t - t_begin, gj = (ti / kGroups) * RB + k;     // the owning group's item count
-                        umma_commit(&ctl->tfull[ti % kGroups][gj & 3]);
-                    }
+                    umma_tile(tmem_base + buf * 128, q0 + uint32_t(k) * kOpHalfBytes, q_half, k_smem, kOpHalfBytes, kIdescBf16M128N128);
+                    const int gj = (i / kAGroups) * a.RA + k;        // the owning group's item count
+                    umma_commit(&ctl->tfull_a[i % kAGroups][gj & 3]);
                 }
-                if (t + 1 == t_end || slab_end <= t + 1) umma_commit(&ctl->qempty);
-                umma_commit(&ctl->empty[stage]);
+                const int t_next = resident ? t + 1 : t - 1;
+                if (i + 1 == ntl || t_next >= hi || t_next < lo) umma_commit(&ctl->qempty);
+                if (!resident) { umma_commit(&ctl->empty[stage]); umma_commit(&ctl->empty[stage]); }
                 if (++stage == a.stages) { stage = 0; ++lap; }
+            }
+            load_no = resident ? 0 : ntl;
+            if (!ok) { umma_commit(&ctl->issued_done[0]); mbar_wait(&ctl->issued_done[0], 0u, 1u << 18); }
+        }
+        __syncwarp();
+        tc_fence_before();
+        named_bar_sync(1, kSweepThreads - 32);           // every accumulator of pass A has been read
+        tc_fence_after();
+        if (lane == 0 && ok) {
+            int it = 0, slab = slab_of(t_begin), hi = 0;
+            uint32_t elap = 0;
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t(a.N) >> 3) << 17) | ((128u >> 4) << 24);
+            const uint64_t d_ones = umma_desc_sw32(smem_u32(onesb));
+            for (int i = 0; i < ntl && ok; ++i, ++load_no) {
+                const int t = t_begin + i;
+                if (i == 0 || t >= hi) {
+                    while (pref[slab + 1] <= t) ++slab;
+                    hi = pref[slab + 1];
+                    ok = role_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status) &&
+                         role_wait(&ctl->extfull, elap & 1u, limit, &ctl->abort_flag, a.status);
+                    if (!ok) break;
+                    ++qlap; ++elap;
+                }
+                const int stage = load_no % a.stages;
+                ok = role_wait(&ctl->full[stage], uint32_t(load_no / a.stages) & 1u, limit, &ctl->abort_flag, a.status);
+                if (!ok) break;
+                const uint32_t k_smem = smem_u32(tiles + size_t(stage) * kOpBytes);
+                for (int k = 0; k < a.RB && ok; ++k, ++it) {
+                    const int buf = it % kBGroups, use = it / kBGroups;
+                    if (use > 0) ok = role_wait(&ctl->tempty_b[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d = tmem_base + buf * kBAccCols;
+                    umma_tile(d, k_smem, kOpHalfBytes, smem_u32(qbuf) + uint32_t(k * a.N) * 128u, q_half, idesc);
+                    umma_bf16(d, d_ones, umma_desc_sw32(ext_smem + uint32_t(k * a.N) * kExtRow), idesc, 1u);      // - lse
+                    const int gj = (i / kBGroups) * a.RB + k;
+                    umma_commit(&ctl->tfull_b[i % kBGroups][gj & 3]);
+                }
+                if (i + 1 == ntl || hi <= t + 1) { umma_commit(&ctl->qempty); umma_commit(&ctl->extempty); }
+                umma_commit(&ctl->empty[stage]);
             }
             if (!ok) {
                 // nobody will wait for the products still in flight: let them retire before the tensor memory is released
@@ -401,96 +450,156 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 mbar_wait(&ctl->issued_done[0], 0u, 1u << 18);
             }
         }
-    } else if (warp < 2 + 4 * kGroups) {
-        // ------------------------------------------------------------------ epilogue warpgroups
-        const int g = (warp - 2) >> 2;                       // warpgroup: tiles t_begin + g, + g + kGroups, ...
+    } else {
+        // ------------------------------------------------------------------ pass A: epilogue warpgroups (and the clearing warp)
         const int quarter = warp & 3;                        // tensor-memory lanes this warp may read
-        const int row = quarter * 32 + lane;
-        const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16);
         bool ok = true;
-        int slab = slab0, tl = g;
-        if (kSweep == 1) {
-            for (int seg_t = t_begin; seg_t < t_end;) {
-                while (pref[slab + 1] <= seg_t) ++slab;
-                const int seg_end = min(t_end, pref[slab + 1]);
-                const int N = live(slab);
-                float m[kMaxRB], l[kMaxRB];
+        {
+            const int g = (warp - 2) >> 2;                   // warpgroup (warp 18: 4, clears the key sums)
+            const int row = quarter * 32 + lane;
+            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16);
+            float2* part = reinterpret_cast<float2*>(extb);  // [group][RA * 128]
+            int i = g;                                       // tiles of this warpgroup: i, i + 4, ... in the order of the pass
+            int slab = slab_of(resident ? t_begin : t_end - 1);
+            for (int done = 0; done < ntl;) {
+                // one segment: the tiles of a slab that this CTA has
+                const int t_cur = resident ? t_begin + done : t_end - 1 - done;
+                while (pref[slab + 1] <= t_cur) ++slab;
+                while (pref[slab] > t_cur) --slab;
+                const int lo = max(pref[slab], t_begin), hi = min(pref[slab + 1], t_end), seg_end = done + (hi - lo);
+                const int fc = owner(pref[slab]), lc = owner(pref[slab + 1] - 1);
+                if (g < kAGroups) {
+                    const int N = live(slab);
+                    float m[kMaxBlocksA], l[kMaxBlocksA];
 #pragma unroll
-                for (int k = 0; k < kMaxRB; ++k) { m[k] = -INFINITY; l[k] = 0.f; }
-                for (; t_begin + tl < seg_end; tl += kGroups) {
-                    const int t = t_begin + tl;
-                    const int valid = min(128, N - (t - pref[slab]) * 128);
+                    for (int k = 0; k < kMaxBlocksA; ++k) { m[k] = -INFINITY; l[k] = 0.f; }
+                    for (; i < seg_end; i += kAGroups) {
+                        const int t = resident ? t_begin + i : t_end - 1 - i;
+                        const int valid = min(128, N - (t - pref[slab]) * 128);
 #pragma unroll
-                    for (int k = 0; k < kMaxRB; ++k) {
-                        if (k < RB && ok) {
-                            const int it = tl * RB + k, buf = it & (kAccBufs - 1);
-                            const int gj = (tl / kGroups) * RB + k;
-                            ok = role_wait(&ctl->tfull[g][gj & 3], uint32_t(gj >> 2) & 1u, limit, &ctl->abort_flag, a.status);
-                            ok = __all_sync(0xffffffffu, ok);
-                            if (ok) {
-                                tc_fence_after();
-                                if (valid == 128) lse_fold<false>(lane_addr + buf * 128, valid, scale, m[k], l[k]);
-                                else              lse_fold<true>(lane_addr + buf * 128, valid, scale, m[k], l[k]);
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(&ctl->tempty[buf]);
+                        for (int k = 0; k < kMaxBlocksA; ++k) {
+                            if (k < a.RA && ok) {
+                                const int buf = (i * a.RA + k) & (kAGroups - 1), gj = (i / kAGroups) * a.RA + k;
+                                ok = role_wait(&ctl->tfull_a[g][gj & 3], uint32_t(gj >> 2) & 1u, limit, &ctl->abort_flag, a.status);
+                                ok = __all_sync(0xffffffffu, ok);
+                                if (ok) {
+                                    tc_fence_after();
+                                    if (k * 128 + quarter * 32 < a.R) {          // (the last block may hold fewer rows)
+                                        if (valid == 128) lse_fold<false>(lane_addr + buf * 128, valid, scale, m[k], l[k]);
+                                        else              lse_fold<true>(lane_addr + buf * 128, valid, scale, m[k], l[k]);
+                                    }
+                                    tc_fence_before();
+                                    __syncwarp();
+                                    if (lane == 0) mbar_arrive(&ctl->tempty_a[buf]);
+                                }
                             }
                         }
                     }
-                }
-                float2* rec = a.sc_part + (size_t(cta + slab) * kSw1Groups + g) * (size_t(RB) * 128);
 #pragma unroll
-                for (int k = 0; k < kMaxRB; ++k)
-                    if (k < RB) rec[k * 128 + row] = make_float2(m[k], l[k]);
-                seg_t = seg_end;
+                    for (int k = 0; k < kMaxBlocksA; ++k)
+                        if (k < a.RA) part[(g * a.RA + k) * 128 + row] = make_float2(m[k], l[k]);
+                } else {
+                    // this CTA's share of the slab's key sums, which pass B accumulates
+                    const int S = min(max(a.n_sent[slab], 0), a.max_sent), P = lc - fc + 1, p = cta - fc;
+                    float4* v4 = reinterpret_cast<float4*>(a.vsum + size_t(slab) * a.max_sent * kHeadDim);
+                    const int w1 = int((long long)S * 32 * (p + 1) / P);
+                    for (int w = int((long long)S * 32 * p / P) + lane; w < w1; w += 32) v4[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                named_bar_sync(2, (4 * kAGroups + 1) * 32);
+                if (g == 0) {                                // the four groups' parts -> one record per CTA and slab
+                    float2* rec = a.rec + size_t(cta + slab) * (size_t(a.RA) * 128);
+                    for (int k = 0; k < a.RA; ++k) {
+                        float2 x[kAGroups];
+                        float M = -INFINITY, L = 0.f;
+#pragma unroll
+                        for (int q = 0; q < kAGroups; ++q) { x[q] = part[(q * a.RA + k) * 128 + row]; M = fmaxf(M, x[q].x); }
+#pragma unroll
+                        for (int q = 0; q < kAGroups; ++q) L += x[q].y > 0.f ? x[q].y * ex2f(x[q].x - M) : 0.f;
+                        rec[k * 128 + row] = make_float2(M, L);
+                    }
+                    named_bar_sync(3, 128);
+                    if (tid == 64 && ok) { __threadfence(); atomicAdd(a.lse_cnt + slab, uint32_t(hi - lo)); }
+                }
+                named_bar_sync(4, (4 * kAGroups + 1) * 32);  // the parts have been read
+                done = seg_end;
             }
-        } else {
-            float* nl = ctl->neg_lse[g];
-            const int wt = tid - 64 - g * 128;              // thread index inside the warpgroup
-            int N = 0;
+        }
+        tc_fence_before();
+        named_bar_sync(1, kSweepThreads - 32);               // every accumulator of pass A has been read
+        tc_fence_after();
+        const int load0 = resident ? 0 : ntl;                // the ring's tiles before pass B
+        if (warp < 10 || (warp >= 14 && warp < 18)) {
+            // -------------------------------------------------------------- pass B: importance, a thread per token
+            const int g = warp < 10 ? (warp - 2) >> 2 : 2;
+            const int row = quarter * 32 + lane;
+            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16);
+            int slab = slab_of(t_begin), seg_first = t_begin, N = 0;
+            uint32_t ext_no = 0;                             // slabs begun so far
             size_t row0 = 0;
             bool have = false;
-            for (; tl < ntl; tl += kGroups) {
-                const int t = t_begin + tl;
+            for (int i = 0; i < ntl; ++i) {
+                const int t = t_begin + i;
                 if (!have || pref[slab + 1] <= t) {
                     while (pref[slab + 1] <= t) ++slab;
                     have = true;
+                    seg_first = t;
                     N = live(slab);
-                    row0 = a.block_table ? size_t(slab) * a.max_pages * 128 : slab_row0(a.slab_off, a.cap, Hk, slab / Hk, slab % Hk);
-                    // log-sum-exp of every query row of this slab from the sweep-1 records
-                    const int fc = pref[slab] / per_cta, lc = (pref[slab + 1] - 1) / per_cta;
-                    const float2* r0 = a.sc_part + size_t(fc + slab) * kSw1Groups * (size_t(RB) * 128);
-                    const int n_part = (lc - fc + 1) * kSw1Groups;
-                    named_bar_sync(2 + g, 128);              // previous readers of nl are done
-                    for (int k = 0; k < RB; ++k) {
-                        float M = -INFINITY;
-                        for (int p = 0; p < n_part; ++p) M = fmaxf(M, r0[size_t(p) * RB * 128 + k * 128 + wt].x);
-                        float L = 0.f;
-                        for (int p = 0; p < n_part; ++p) {
-                            const float2 pr = r0[size_t(p) * RB * 128 + k * 128 + wt];
-                            if (pr.y > 0.f) L += pr.y * ex2f(pr.x - M);
+                    row0 = a.block_table ? size_t(slab) * a.max_pages * 128 : size_t(rowb[slab]);
+                    ++ext_no;
+                }
+                if (i % kBGroups != g) continue;
+                if (t == seg_first) {
+                    // the group of a slab's first tile prepares the slab: log-sum-exp of its query rows from the records of
+                    // all its CTAs, negated, in units of raw logits, as three bf16 pieces of the extra K step
+                    const int fc = owner(pref[slab]), lc = owner(pref[slab + 1] - 1);
+                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(pref[slab + 1] - pref[slab]), limit, &ctl->abort_flag, a.status);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                    if (ok && ext_no > 1) ok = role_wait(&ctl->extempty, (ext_no - 2) & 1u, limit, &ctl->abort_flag, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (ok) {
+                        const float2* r0 = a.rec + size_t(fc + slab) * (size_t(a.RA) * 128);
+                        const int n_part = lc - fc + 1;
+                        for (int r = row; r < a.R; r += 128) {
+                            float M = -INFINITY, L = 0.f;
+                            for (int p0 = 0; p0 < n_part; p0 += 8) {         // eight records per round: their loads are in flight together
+                                float2 x[8];
+#pragma unroll
+                                for (int p = 0; p < 8; ++p)
+                                    x[p] = p0 + p < n_part ? __ldcg(r0 + size_t(p0 + p) * (a.RA * 128) + r) : make_float2(-INFINITY, 0.f);
+                                float mx = M;
+#pragma unroll
+                                for (int p = 0; p < 8; ++p) mx = fmaxf(mx, x[p].x);
+                                L *= M == -INFINITY ? 0.f : ex2f(M - mx);
+                                M = mx;
+#pragma unroll
+                                for (int p = 0; p < 8; ++p) L += x[p].y > 0.f ? x[p].y * ex2f(x[p].x - M) : 0.f;
+                            }
+                            const float v = L > 0.f ? -0.5f * (M + log2f(L)) / scale : 0.f;
+                            const __nv_bfloat16 b0 = __float2bfloat16_rn(v);
+                            const float v1 = v - __bfloat162float(b0);
+                            const __nv_bfloat16 b1 = __float2bfloat16_rn(v1), b2 = __float2bfloat16_rn(v1 - __bfloat162float(b1));
+                            const uint4 piece = make_uint4(uint32_t(__bfloat16_as_ushort(b0)) | (uint32_t(__bfloat16_as_ushort(b1)) << 16),
+                                                           uint32_t(__bfloat16_as_ushort(b2)), 0u, 0u);
+                            *reinterpret_cast<uint4*>(extb + size_t(r) * kExtRow) = piece;
+                            *reinterpret_cast<uint4*>(extb + size_t(r) * kExtRow + 16) = piece;
                         }
-                        nl[k * 128 + wt] = (L > 0.f) ? -(M + log2f(L)) : 0.f;
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&ctl->extfull);
                     }
-                    named_bar_sync(2 + g, 128);
                 }
                 float total = 0.f;
-#pragma unroll
-                for (int k = 0; k < kMaxRB; ++k) {
-                    if (k < RB && ok) {
-                        const int it = tl * RB + k, buf = it % kSw2Bufs;
-                        const int gj = (tl / kGroups) * RB + k;
-                        ok = role_wait(&ctl->tfull[g][gj & 3], uint32_t(gj >> 2) & 1u, limit, &ctl->abort_flag, a.status);
-                        ok = __all_sync(0xffffffffu, ok);
-                        if (ok) {
-                            tc_fence_after();
-                            total += imp_fold<kN>(lane_addr + buf * 128, nl + k * 128,
-                                                  min(128 / kN, a.window - k * (128 / kN)), scale);
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(&ctl->tempty[buf]);
-                        }
-                    }
+                for (int k = 0; k < a.RB; ++k) {
+                    const int buf = (i * a.RB + k) % kBGroups, gj = (i / kBGroups) * a.RB + k;
+                    if (!ok) break;
+                    ok = role_wait(&ctl->tfull_b[g][gj & 3], uint32_t(gj >> 2) & 1u, limit, &ctl->abort_flag, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+                    total += imp_fold<kWB>(lane_addr + buf * kBAccCols, n, min(kWB, a.window - k * kWB), scale);
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&ctl->tempty_b[buf]);
                 }
                 const int tok = (t - pref[slab]) * 128 + row;
                 if (ok && tok < N) {
@@ -499,173 +608,176 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     if (a.tok_imp_user) a.tok_imp_user[row0 + tok] = v;
                 }
             }
-        }
-    } else if (kSweep == 2 && warp < 2 + 4 * kGroups + kPoolWarps) {
-        // ------------------------------------------------------------------ per-sentence sums of the key rows
-        // The sums are a product on the tensor cores: (tile^T: channel x token) x (indicator: token x sentence slot).
-        // A run of consecutive tiles whose sentences all fall among the 16 sentences B .. B + 15 shares one accumulator
-        // (slot j = sentence B + j; the products of the run accumulate), so the sums are read out and added to global
-        // memory once per run, about every fifth tile.  Each of the four warps writes a quarter of a tile's matrix and
-        // arrives; one thread of a fifth warp issues the product; when a tile opens a new run the four warps read out the
-        // run before it (a thread owns one channel) while the new one is being multiplied.  A tile that touches more
-        // than 16 sentences (empty ones count) gets several matrices, each a run of its own.
-        // Every warp keeps, one entry per lane, the sentence offsets B .. B + 31 of the current run (entries past the
-        // table read as "never starts"), fetched from global memory when a run opens: loads from shared memory wait
-        // several hundred cycles here (the tensor core streams its operands from it), so the per-tile work touches
-        // shared memory only to write the matrix.
-        constexpr int kNever = 0x7fffffff;
-        const int gw = warp - (2 + 4 * kGroups);                // warp of the group: slots 4 gw .. 4 gw + 3 of a matrix
-        const int gtid = tid - (2 + 4 * kGroups) * 32;
-        const int quarter = warp & 3;                           // tensor-memory lanes this warp may read
-        const int ch = quarter * 32 + lane;
-        const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + kPoolCol;
-        int slab = slab0, S = 0, N = 0, first = 0;
-        int ic = 0;                                             // indicator matrices written so far
-        int run = -1, B = 0, w = kNever;                        // current run: index, sentence of slot 0, offsets B + lane
-        uint32_t run_held = 0;                                  // its slots that hold tokens so far
-        int run_slab = 0;
-        const int32_t* so = a.sent_off;
-        bool ok = true, have = false;
-        // 32-way search for the last sentence that starts at or before token `tok`, one probe per lane
-        auto holder = [&](int tok) {
-            int lo = 0, len = S;
-            while (len > 32) {
-                const int stride = (len + 31) >> 5;
-                const int pidx = lo + lane * stride;
-                const bool le = pidx < lo + len && so[pidx] <= tok;
-                const int adv = max(__popc(__ballot_sync(0xffffffffu, le)) - 1, 0) * stride;
-                len = min(stride, len - adv);
-                lo += adv;
-            }
-            const bool le = lane < len && so[lo + lane] <= tok;
-            return lo + max(__popc(__ballot_sync(0xffffffffu, le)) - 1, 0);
-        };
-        // read out run r (accumulator r & 1) and add it to the sums
-        auto drain = [&](int r, int r_slab, int r_B, uint32_t r_held) {
-            ok = role_wait(&ctl->pfull[r & 1], uint32_t(r >> 1) & 1u, limit, &ctl->abort_flag, a.status);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) return;
-            tc_fence_after();
-            float v[kIndSlots];
-            tmem_ld16(lane_addr + uint32_t(r & 1) * kIndSlots, v);
-            tc_fence_before();
-            float* dst = a.vsum + (size_t(r_slab) * a.max_sent + r_B) * kHeadDim + ch;
+        } else if (warp < 14) {
+            // -------------------------------------------------------------- pass B: per-sentence sums of the key rows
+            // The sums are a product on the tensor cores: (tile^T: channel x token) x (indicator: token x sentence slot).
+            // A run of consecutive tiles whose sentences all fall among the 16 sentences B .. B + 15 shares one accumulator
+            // (slot j = sentence B + j; the products of the run accumulate), so the sums are read out and added to global
+            // memory once per run, about every fifth tile.  Each of the four warps writes a quarter of a tile's matrix and
+            // arrives; one thread of a fifth warp issues the product; when a tile opens a new run the four warps read out the
+            // run before it (a thread owns one channel) while the new one is being multiplied.  A tile that touches more
+            // than 16 sentences (empty ones count) gets several matrices, each a run of its own.
+            // Every warp keeps, one entry per lane, the sentence offsets B .. B + 31 of the current run (entries past the
+            // table read as "never starts"), fetched from global memory when a run opens: loads from shared memory wait
+            // several hundred cycles here (the tensor core streams its operands from it), so the per-tile work touches
+            // shared memory only to write the matrix.
+            constexpr int kNever = 0x7fffffff;
+            const int gw = warp - 10;                               // warp of the group: slots 4 gw .. 4 gw + 3 of a matrix
+            const int gtid = tid - 320;
+            const int ch = quarter * 32 + lane;
+            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + kPoolCol;
+            int slab = slab_of(t_begin), S = 0, N = 0, first = 0;
+            int ic = 0;                                             // indicator matrices written so far
+            int run = -1, B = 0, w = kNever;                        // current run: index, sentence of slot 0, offsets B + lane
+            uint32_t run_held = 0;                                  // its slots that hold tokens so far
+            int run_slab = 0;
+            const int32_t* so = a.sent_off;
+            bool have = false;
+            // 32-way search for the last sentence that starts at or before token `tok`, one probe per lane
+            auto holder = [&](int tok) {
+                int lo = 0, len = S;
+                while (len > 32) {
+                    const int stride = (len + 31) >> 5;
+                    const int pidx = lo + lane * stride;
+                    const bool le = pidx < lo + len && so[pidx] <= tok;
+                    const int adv = max(__popc(__ballot_sync(0xffffffffu, le)) - 1, 0) * stride;
+                    len = min(stride, len - adv);
+                    lo += adv;
+                }
+                const bool le = lane < len && so[lo + lane] <= tok;
+                return lo + max(__popc(__ballot_sync(0xffffffffu, le)) - 1, 0);
+            };
+            // read out run r (accumulator r & 1) and add it to the sums
+            auto drain = [&](int r, int r_slab, int r_B, uint32_t r_held) {
+                ok = role_wait(&ctl->pfull[r & 1], uint32_t(r >> 1) & 1u, limit, &ctl->abort_flag, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) return;
+                tc_fence_after();
+                float v[kIndSlots];
+                tmem_ld16(lane_addr + uint32_t(r & 1) * kIndSlots, v);
+                tc_fence_before();
+                float* dst = a.vsum + (size_t(r_slab) * a.max_sent + r_B) * kHeadDim + ch;
 #pragma unroll
-            for (int j = 0; j < kIndSlots; ++j)
-                if (r_held & (1u << j)) atomicAdd(dst + size_t(j) * kHeadDim, v[j]);
-        };
-        for (int tl = 0; tl < ntl && ok; ++tl) {
-            const int t = t_begin + tl;
-            const bool fresh = !have || pref[slab + 1] <= t;
-            if (fresh) {
-                while (pref[slab + 1] <= t) ++slab;
-                have = true;
-                so = a.sent_off + size_t(slab) * (a.max_sent + 1);
-                S = min(max(a.n_sent[slab], 0), a.max_sent);
-                N = live(slab);
-            }
-            const int tok0 = (t - pref[slab]) * 128, valid = min(128, N - tok0), tok_end = tok0 + valid;
-            const int stage = tl % a.stages;
-            if (fresh) first = tok0 > 0 ? holder(tok0) : 0;     // (a slab that opens with empty sentences: they get slots)
-            // every warp follows every tile's arrival (in order, so it sees each phase of the stage's barrier)
-            ok = role_wait(&ctl->full[stage], uint32_t(tl / a.stages) & 1u, limit, &ctl->abort_flag, a.status);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            if (valid < 128) {
-                // a zero in the indicator does not silence a NaN or an infinity in a dead row: clear the rows past the
-                // slab's end in the staged tile (the logits of those rows are never read)
-                uint8_t* tile = tiles + size_t(stage) * kOpBytes;
-                for (int u = valid * 8 + gtid; u < 128 * 8; u += kPoolWarps * 32) {
-                    *reinterpret_cast<uint4*>(tile + u * 16) = make_uint4(0u, 0u, 0u, 0u);
-                    *reinterpret_cast<uint4*>(tile + kOpHalfBytes + u * 16) = make_uint4(0u, 0u, 0u, 0u);
-                }
-            }
-            int cur = first;                                    // first sentence of the tile not yet in a matrix
-            int more = 0;
-            do {
-                // can the tile (from sentence cur on) join the open run?  its last sentence must be below B + 16
-                bool join = false;
-                if (run >= 0 && !fresh && cur >= B && cur - B < kIndSlots) {
-                    const int touching = __popc(__ballot_sync(0xffffffffu, lane > cur - B && B + lane < S && w < tok_end));
-                    join = cur + touching - B < kIndSlots;
-                }
-                const int r_prev = run, p_slab = run_slab, p_B = B;
-                const uint32_t p_held = run_held;
-                if (!join) {                                    // open a run at sentence cur
-                    ++run; B = cur; run_slab = slab; run_held = 0;
-                    w = (B + lane <= S) ? so[B + lane] : kNever;
-                }
-                // tile-relative start of the sentences B + lane, clamped to the tile; slot j holds [cl(j), cl(j + 1))
-                const int cl = min(max(min(w, tok_end) - tok0, 0), valid);
-                const int cl_next = __shfl_down_sync(0xffffffffu, cl, 1);
-                const uint32_t held = __ballot_sync(0xffffffffu, lane < kIndSlots && B + lane < S && cl_next > cl);
-                const int s_next = __shfl_sync(0xffffffffu, w, kIndSlots);           // start of the sentence after slot 15
-                more = (B + kIndSlots < S && s_next < tok_end) ? 1 : 0;
-                const int is = ic & (kIndRing - 1);
-                if (ic >= kIndRing) {                           // the product that read this buffer last has completed
-                    ok = role_wait(&ctl->iempty[is], uint32_t(ic / kIndRing - 1) & 1u, limit, &ctl->abort_flag, a.status);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                }
-                {
-                    const int j = 4 * gw + (lane >> 3);         // this thread's slot row and its two pieces
-                    const int lo = __shfl_sync(0xffffffffu, cl, j), hi = __shfl_sync(0xffffffffu, cl, j + 1);
-                    const bool is_sent = (held >> j) & 1u;
-                    indicator_piece(indb + size_t(is) * kIndBytes, j, (lane & 7) * 2, is_sent ? lo : 0, is_sent ? hi : 0);
-                    indicator_piece(indb + size_t(is) * kIndBytes, j, (lane & 7) * 2 + 1, is_sent ? lo : 0, is_sent ? hi : 0);
-                }
-                fence_proxy_async_smem();                       // the matrix (and cleared rows) are read by the tensor core
-                tc_fence_before();                              // and this warp's reads of the accumulators came first
-                __syncwarp();
-                if (lane == 0) {
-                    if (gw == 0) ctl->ind_flags[is] = more | (join ? 2 : 0) | ((!join && r_prev >= 0) ? 4 : 0);
-                    mbar_arrive(&ctl->ifull[is]);
-                }
-                run_held |= held;
-                ++ic;
-                if (!join && r_prev >= 0) {                     // the run before, while the new one is being multiplied
-                    drain(r_prev, p_slab, p_B, p_held);
-                    if (!ok) break;
-                }
-                cur = B + kIndSlots;
-            } while (more);
-            // the next tile starts in the last sentence of the run's window that starts at or before its first token
-            const int n_le = __popc(__ballot_sync(0xffffffffu, B + lane < S && w <= tok0 + 128));
-            first = (n_le == 32 && B + 32 < S) ? holder(tok0 + 128) : B + max(n_le - 1, 0);
-        }
-        if (ok && run >= 0) drain(run, run_slab, B, run_held);  // the issuer closes the last run when its tiles are done
-    } else if (kSweep == 2) {
-        // ------------------------------------------------------------------ issuer of the pooling products
-        // (its own thread: an issue blocks for the length of the product, and every look at shared memory costs the
-        // thread that issues the logits a few hundred cycles)
-        if (lane == 0 && ntl > 0) {
-            const uint32_t indb_u32 = smem_u32(indb);
-            bool ok = true;
-            int pc = 0, run = -1;
+                for (int j = 0; j < kIndSlots; ++j)
+                    if (r_held & (1u << j)) atomicAdd(dst + size_t(j) * kHeadDim, v[j]);
+            };
             for (int tl = 0; tl < ntl && ok; ++tl) {
-                const int stage = tl % a.stages;
-                int flags = 0;
-                do {
-                    const int is = pc & (kIndRing - 1);
-                    ok = role_wait(&ctl->ifull[is], uint32_t(pc / kIndRing) & 1u, limit, &ctl->abort_flag, a.status);
+                const int t = t_begin + tl;
+                const bool fresh = !have || pref[slab + 1] <= t;
+                if (fresh) {
+                    while (pref[slab + 1] <= t) ++slab;
+                    have = true;
+                    so = a.sent_off + size_t(slab) * (a.max_sent + 1);
+                    S = min(max(a.n_sent[slab], 0), a.max_sent);
+                    N = live(slab);
+                    // every CTA of the slab has cleared its share of the sums (and left its record)
+                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(pref[slab + 1] - pref[slab]), limit, &ctl->abort_flag, a.status);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                     if (!ok) break;
-                    flags = *reinterpret_cast<volatile int*>(&ctl->ind_flags[is]);       // 1: more, 2: joins the run, 4: closes one
-                    tc_fence_after();
-                    if (flags & 4) umma_commit(&ctl->pfull[run & 1]);                    // everything of the run before is issued
-                    if (!(flags & 2)) ++run;
-                    umma_pool(tmem_base + kPoolCol + uint32_t(run & 1) * kIndSlots, smem_u32(tiles + size_t(stage) * kOpBytes),
-                              indb_u32 + uint32_t(is) * kIndBytes, (flags & 2) != 0);
-                    umma_commit(&ctl->iempty[is]);
-                    ++pc;
-                } while (flags & 1);
-                if (ok) umma_commit(&ctl->empty[stage]);
+                }
+                const int tok0 = (t - pref[slab]) * 128, valid = min(128, N - tok0), tok_end = tok0 + valid;
+                const int stage = (load0 + tl) % a.stages;
+                if (fresh) first = tok0 > 0 ? holder(tok0) : 0;     // (a slab that opens with empty sentences: they get slots)
+                // every warp follows every tile's arrival (in order, so it sees each phase of the stage's barrier)
+                ok = role_wait(&ctl->full[stage], uint32_t((load0 + tl) / a.stages) & 1u, limit, &ctl->abort_flag, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (valid < 128) {
+                    // a zero in the indicator does not silence a NaN or an infinity in a dead row: clear the rows past the
+                    // slab's end in the staged tile (the logits of those rows are never read)
+                    uint8_t* tile = tiles + size_t(stage) * kOpBytes;
+                    for (int u = valid * 8 + gtid; u < 128 * 8; u += kPoolWarps * 32) {
+                        *reinterpret_cast<uint4*>(tile + u * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        *reinterpret_cast<uint4*>(tile + kOpHalfBytes + u * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                }
+                int cur = first;                                    // first sentence of the tile not yet in a matrix
+                int more = 0;
+                do {
+                    // can the tile (from sentence cur on) join the open run?  its last sentence must be below B + 16
+                    bool join = false;
+                    if (run >= 0 && !fresh && cur >= B && cur - B < kIndSlots) {
+                        const int touching = __popc(__ballot_sync(0xffffffffu, lane > cur - B && B + lane < S && w < tok_end));
+                        join = cur + touching - B < kIndSlots;
+                    }
+                    const int r_prev = run, p_slab = run_slab, p_B = B;
+                    const uint32_t p_held = run_held;
+                    if (!join) {                                    // open a run at sentence cur
+                        ++run; B = cur; run_slab = slab; run_held = 0;
+                        w = (B + lane <= S) ? so[B + lane] : kNever;
+                    }
+                    // tile-relative start of the sentences B + lane, clamped to the tile; slot j holds [cl(j), cl(j + 1))
+                    const int cl = min(max(min(w, tok_end) - tok0, 0), valid);
+                    const int cl_next = __shfl_down_sync(0xffffffffu, cl, 1);
+                    const uint32_t held = __ballot_sync(0xffffffffu, lane < kIndSlots && B + lane < S && cl_next > cl);
+                    const int s_next = __shfl_sync(0xffffffffu, w, kIndSlots);           // start of the sentence after slot 15
+                    more = (B + kIndSlots < S && s_next < tok_end) ? 1 : 0;
+                    const int is = ic & (kIndRing - 1);
+                    if (ic >= kIndRing) {                           // the product that read this buffer last has completed
+                        ok = role_wait(&ctl->iempty[is], uint32_t(ic / kIndRing - 1) & 1u, limit, &ctl->abort_flag, a.status);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                    }
+                    {
+                        const int j = 4 * gw + (lane >> 3);         // this thread's slot row and its two pieces
+                        const int lo = __shfl_sync(0xffffffffu, cl, j), hi = __shfl_sync(0xffffffffu, cl, j + 1);
+                        const bool is_sent = (held >> j) & 1u;
+                        indicator_piece(indb + size_t(is) * kIndBytes, j, (lane & 7) * 2, is_sent ? lo : 0, is_sent ? hi : 0);
+                        indicator_piece(indb + size_t(is) * kIndBytes, j, (lane & 7) * 2 + 1, is_sent ? lo : 0, is_sent ? hi : 0);
+                    }
+                    fence_proxy_async_smem();                       // the matrix (and cleared rows) are read by the tensor core
+                    tc_fence_before();                              // and this warp's reads of the accumulators came first
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (gw == 0) ctl->ind_flags[is] = more | (join ? 2 : 0) | ((!join && r_prev >= 0) ? 4 : 0);
+                        mbar_arrive(&ctl->ifull[is]);
+                    }
+                    run_held |= held;
+                    ++ic;
+                    if (!join && r_prev >= 0) {                     // the run before, while the new one is being multiplied
+                        drain(r_prev, p_slab, p_B, p_held);
+                        if (!ok) break;
+                    }
+                    cur = B + kIndSlots;
+                } while (more);
+                // the next tile starts in the last sentence of the run's window that starts at or before its first token
+                const int n_le = __popc(__ballot_sync(0xffffffffu, B + lane < S && w <= tok0 + 128));
+                first = (n_le == 32 && B + 32 < S) ? holder(tok0 + 128) : B + max(n_le - 1, 0);
             }
-            if (ok && run >= 0) umma_commit(&ctl->pfull[run & 1]);
-            if (!ok) {
-                umma_commit(&ctl->issued_done[1]);
-                mbar_wait(&ctl->issued_done[1], 0u, 1u << 18);
+            if (ok && run >= 0) drain(run, run_slab, B, run_held);  // the issuer closes the last run when its tiles are done
+        } else {
+            // -------------------------------------------------------------- pass B: issuer of the pooling products
+            // (its own thread: an issue blocks for the length of the product, and every look at shared memory costs the
+            // thread that issues the logits a few hundred cycles)
+            if (lane == 0) {
+                const uint32_t indb_u32 = smem_u32(indb);
+                int pc = 0, run = -1;
+                for (int tl = 0; tl < ntl && ok; ++tl) {
+                    const int stage = (load0 + tl) % a.stages;
+                    int flags = 0;
+                    do {
+                        const int is = pc & (kIndRing - 1);
+                        ok = role_wait(&ctl->ifull[is], uint32_t(pc / kIndRing) & 1u, limit, &ctl->abort_flag, a.status);
+                        if (!ok) break;
+                        flags = *reinterpret_cast<volatile int*>(&ctl->ind_flags[is]);       // 1: more, 2: joins the run, 4: closes one
+                        tc_fence_after();
+                        if (flags & 4) umma_commit(&ctl->pfull[run & 1]);                    // everything of the run before is issued
+                        if (!(flags & 2)) ++run;
+                        umma_pool(tmem_base + kPoolCol + uint32_t(run & 1) * kIndSlots, smem_u32(tiles + size_t(stage) * kOpBytes),
+                                  indb_u32 + uint32_t(is) * kIndBytes, (flags & 2) != 0);
+                        umma_commit(&ctl->iempty[is]);
+                        ++pc;
+                    } while (flags & 1);
+                    if (ok) umma_commit(&ctl->empty[stage]);
+                }
+                if (ok && run >= 0) umma_commit(&ctl->pfull[run & 1]);
+                if (!ok) {
+                    umma_commit(&ctl->issued_done[1]);
+                    mbar_wait(&ctl->issued_done[1], 0u, 1u << 18);
+                }
             }
         }
+    }
     }
     tc_fence_before();
     __syncthreads();
@@ -679,12 +791,13 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
 // pooling: one warp per sentence, 4 channels per lane; writes the normalised mean key as bf16 hi + lo
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-score_pool_kernel(int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len,
+score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len,
                   const int32_t* sent_off, const int32_t* n_sent, float eps, const float* tok_imp_ws,
                   const float* vsum, float* sent_imp, __nv_bfloat16* vbar_hi, __nv_bfloat16* vbar_lo) {
     pdl_trigger();
     pdl_wait();
     const int slab = blockIdx.y;
+    if (blockIdx.x == 0 && threadIdx.x == 0) lse_cnt[slab] = 0u;            // for the next call's sweeps
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int S = min(n_sent[slab], max_sent);
@@ -980,7 +1093,7 @@ struct SmallCtl {
 constexpr size_t kSmallSmem = 1024 + 2 * size_t(kOpBytes) + sizeof(SmallCtl);
 
 __global__ void __launch_bounds__(kSmallThreads)
-score_small_kernel(int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len, const int32_t* sent_off,
+score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len, const int32_t* sent_off,
                    const int32_t* n_sent, float eps, float sigma, float tau, const float* tok_imp_ws, const float* vsum,
                    float* sent_imp, float* sent_red, float* sent_lam, float* sent_score, LamTable ext, const Header* hdr) {
     extern __shared__ uint8_t small_smem_raw[];
@@ -994,6 +1107,7 @@ score_small_kernel(int Hk, int max_sent, int max_cap, const int32_t* cap, const 
     if (tid == 0) { mbar_init(&ctl->done, 1); mbar_fence_init(); }
     if (warp == 1) tmem_alloc(&ctl->tmem_base, 128);
     pdl_wait();
+    if (tid == 0) lse_cnt[slab] = 0u;                    // for the next call's sweeps
     const int S = min(max(n_sent[slab], 0), max_sent), N = min(max(kv_len[slab], 0), cap[slab / Hk]);
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
     const float* ti_p = tok_imp_ws + size_t(slab) * max_cap;
@@ -1131,14 +1245,6 @@ score_small_kernel(int Hk, int max_sent, int max_cap, const int32_t* cap, const 
     }
 }
 
-template <int kSweep, int kN>
-static int launch_sweep(const CUtensorMap& mapK, const CUtensorMap& mapQ, const SweepArgs& a, int grid, size_t smem,
-                        cudaStream_t st) {
-    auto kern = score_sweep_kernel<kSweep, kN>;
-    SKIPKV_CUDA(launch_dependent(kern, dim3(grid), dim3(kSweep == 1 ? kSw1Threads : kSw2Threads), smem, st, mapK, mapQ, a));
-    return SKIPKV_OK;
-}
-
 }  // namespace skipkv
 
 using namespace skipkv;
@@ -1174,44 +1280,26 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
 
     SweepArgs a{};
     a.Hq = Hq; a.Hk = Hk; a.window = shape->window; a.n_slabs = L.slabs; a.max_cap = shape->max_cap;
-    a.max_sent = shape->max_sent; a.RB = L.sc_rb; a.WB = L.sc_wb;
+    a.max_sent = shape->max_sent;
+    a.WB = L.sc_wb; a.RB = L.sc_rb; a.N = L.sc_wb * n; a.R = a.RB * a.N; a.RA = L.sc_ra;
     a.slab_off = shape->slab_off; a.cap = shape->cap; a.kv_len = kv_len; a.sent_off = sent_off; a.n_sent = n_sent;
-    a.sc_part = reinterpret_cast<float2*>(w + L.sc_part);
+    a.rec = reinterpret_cast<float2*>(w + L.sc_part); a.lse_cnt = reinterpret_cast<uint32_t*>(w + L.sc_cnt);
     a.tok_imp_user = tok_imp; a.tok_imp_ws = sc_tok; a.vsum = vsum; a.status = status;
     a.hdr = reinterpret_cast<const Header*>(w + L.header);
     a.block_table = block_table; a.max_pages = max_pages;
     const size_t max_smem = 227 * 1024;
-    const size_t fixed1 = 1024 + size_t(a.RB) * kOpBytes + sizeof(SweepCtl) + size_t(L.slabs + 1) * 4;
-    if (fixed1 + kOpBytes > max_smem) return SKIPKV_ERR_UNSUPPORTED;
-    SweepArgs a1 = a, a2 = a;
-    a1.stages = int((max_smem - fixed1) / kOpBytes);
-    if (a1.stages > kSwMaxStages) a1.stages = kSwMaxStages;
-    // sweep 2 also holds the indicator matrices of its pooling product
-    const size_t fixed2 = fixed1 + size_t(kIndRing) * kIndBytes;
-    if (fixed2 + kOpBytes > max_smem) return SKIPKV_ERR_UNSUPPORTED;
-    a2.stages = int((max_smem - fixed2) / kOpBytes);
-    if (a2.stages > kSwMaxStages) a2.stages = kSwMaxStages;
-    const size_t smem1 = fixed1 + size_t(a1.stages) * kOpBytes, smem2 = fixed2 + size_t(a2.stages) * kOpBytes;
+    const size_t fixed = 1024 + size_t(a.R) * kRowBytes + size_t(kIndRing) * kIndBytes + 128 * kExtRow + size_t(a.RA) * 128 * kExtRow +
+                         sizeof(SweepCtl) + size_t(2 * L.slabs + 1) * 4;
+    if (fixed + kOpBytes > max_smem) return SKIPKV_ERR_UNSUPPORTED;
+    a.stages = int((max_smem - fixed) / kOpBytes);
+    if (a.stages > kStagesMax) a.stages = kStagesMax;
     int grid = num_sms();
     if (grid > L.dec_max_ctas) grid = L.dec_max_ctas;
-
-    if (int rc = launch_sweep<1, 1>(mapK, mapQ, a1, grid, smem1, st)) return rc;
-    int rc = SKIPKV_ERR_UNSUPPORTED;
-    switch (n) {
-        case 1: rc = launch_sweep<2, 1>(mapK, mapQ, a2, grid, smem2, st); break;
-        case 2: rc = launch_sweep<2, 2>(mapK, mapQ, a2, grid, smem2, st); break;
-        case 3: rc = launch_sweep<2, 3>(mapK, mapQ, a2, grid, smem2, st); break;
-        case 4: rc = launch_sweep<2, 4>(mapK, mapQ, a2, grid, smem2, st); break;
-        case 5: rc = launch_sweep<2, 5>(mapK, mapQ, a2, grid, smem2, st); break;
-        case 6: rc = launch_sweep<2, 6>(mapK, mapQ, a2, grid, smem2, st); break;
-        case 7: rc = launch_sweep<2, 7>(mapK, mapQ, a2, grid, smem2, st); break;
-        case 8: rc = launch_sweep<2, 8>(mapK, mapQ, a2, grid, smem2, st); break;
-        default: break;
-    }
-    if (rc) return rc;
+    SKIPKV_CUDA(launch_dependent<true>(L.sc_wb == 32 ? score_sweep_kernel<32> : score_sweep_kernel<16>, dim3(grid), dim3(kSweepThreads),
+                                 fixed + size_t(a.stages) * kOpBytes, st, mapK, mapQ, a));
     // one tile of sentences per slab: one kernel instead of three, with the operands in shared memory throughout
     if (shape->max_sent <= kSmallSent) {
-        SKIPKV_CUDA(launch_dependent(score_small_kernel, dim3(L.slabs), dim3(kSmallThreads), kSmallSmem, st, Hk, int(shape->max_sent),
+        SKIPKV_CUDA(launch_dependent(score_small_kernel, dim3(L.slabs), dim3(kSmallThreads), kSmallSmem, st, a.lse_cnt, Hk, int(shape->max_sent),
                                      int(shape->max_cap), shape->cap, kv_len, sent_off, n_sent, params->eps, params->sigma,
                                      params->tau, static_cast<const float*>(sc_tok), static_cast<const float*>(vsum), sent_imp,
                                      sent_red, sent_lam, sent_score, ext, reinterpret_cast<const Header*>(w + L.header)));
@@ -1219,7 +1307,7 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     }
     {
         dim3 pgrid((shape->max_sent + 7) / 8, L.slabs);
-        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, Hk, shape->max_sent, shape->max_cap,
+        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, shape->max_cap,
                                      shape->cap, kv_len, sent_off, n_sent, params->eps, sc_tok, vsum, sent_imp, vbar_hi,
                                      vbar_lo));
     }
