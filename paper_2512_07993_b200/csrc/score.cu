@@ -50,7 +50,7 @@ constexpr int kIndSlots = 16;           // sentence slots of one indicator matri
 constexpr int kIndBytes = kIndSlots * 128 * 2;   // [16 slots][128 tokens] bf16 as two 64-token halves, 128-byte swizzle
 constexpr uint32_t kPoolCol = kBGroups * kBAccCols;   // tensor-memory column of the first pooled-sum accumulator (16 columns each)
 constexpr int kPoolWarps = 4;
-constexpr int kSweepThreads = (2 + 4 * kAGroups + 1) * 32;    // TMA warp, MMA warp, 16 epilogue warps, issuer of the pooling products
+constexpr int kSweepThreads = (2 + 4 * kAGroups + 2) * 32;    // TMA warp, MMA warp, 16 epilogue warps, issuer of the pooling products, second MMA warp
 constexpr int kMaxBlocksA = 5;          // blocks of 128 query rows
 constexpr int kExtRow = 32;             // bytes of a row of the extra K step (16 bf16)
 constexpr float kLog2e = 1.4426950408889634f;
@@ -58,15 +58,16 @@ constexpr float kLog2e = 1.4426950408889634f;
 struct SweepCtl {                       // barriers and small shared state, after the tile buffers
     uint64_t full[kStagesMax], empty[kStagesMax];
     uint64_t qfull, qempty;
-    // "accumulator ready" barriers are per epilogue warpgroup (a ring of 4 per group, indexed by the group's own item
-    // count), so every barrier has one consumer that sees its phases in order; a barrier per accumulator would be
-    // waited on by different groups in turn, and a group polling for a later phase could pass on an earlier one.
-    uint64_t tfull_a[kAGroups][4], tempty_a[kAGroups], tfull_b[kBGroups][4], tempty_b[kBGroups];
+    // accumulator i belongs to epilogue warpgroup i (a product of a tile and a block of query rows goes to product number % groups)
+    uint64_t tfull_a[kAGroups], tempty_a[kAGroups], tfull_b[kBGroups];
+    uint64_t tempty_b[2 * kBGroups];    // by product number: a product waits for the one kBGroups before it, which is the other MMA warp's, and
+                                        // with twice as many barriers as accumulators each has one waiter that sees all its phases
+    uint64_t tokfull[4];                // pass B, several blocks per tile: the shares of a tile's tokens from all blocks but the last
     uint64_t extfull, extempty;         // pass B: the rows' -lse as operand columns
     // ring of indicator matrices: written by the four pooling warps -> multiplied by their issuer -> read out by the pooling warps
     uint64_t ifull[kIndRing], iempty[kIndRing];
     uint64_t pfull[2];                  // the last product of a run of tiles into accumulator i has completed
-    uint64_t issued_done[2];            // after a failed wait: every product of the MMA thread (0) / the pooling issuer (1) has retired
+    uint64_t issued_done[3];            // after a failed wait: every product of the MMA warps (0, 1) / the pooling issuer (2) has retired
     uint32_t tmem_base;
     int abort_flag;
     int ind_flags[kIndRing];            // 1: the tile has another matrix after this one, 2: joins the open run, 4: closes a run
@@ -253,7 +254,8 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     uint8_t* onesb = indb + kIndRing * kIndBytes;                                // pass B: the keys' side of the extra K step
     uint8_t* extb = onesb + 128 * kExtRow;                                       // pass B: the queries' side; pass A: [4 groups][RA * 128] (m, l)
     SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + size_t(a.RA) * 128 * kExtRow);
-    int* pref = reinterpret_cast<int*>(ctl + 1);                                 // [n_slabs + 1] tile prefix
+    float* tokp = reinterpret_cast<float*>(ctl + 1);                             // [4 tiles][RB - 1][128] shares of a tile's tokens
+    int* pref = reinterpret_cast<int*>(tokp + 4 * (a.RB - 1) * 128);             // [n_slabs + 1] tile prefix
     int* rowb = pref + a.n_slabs + 1;                                            // [n_slabs] cache row of a slab's first token
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -266,21 +268,17 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     };
 
     if (tid == 0) {
-        for (int s = 0; s < kStagesMax; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 2); }
+        for (int s = 0; s < kStagesMax; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], a.RB > 1 ? 3 : 2); }
         mbar_init(&ctl->qfull, 1);
-        mbar_init(&ctl->qempty, 1);
-        for (int g = 0; g < kAGroups; ++g) {
-            mbar_init(&ctl->tempty_a[g], 4);
-            for (int j = 0; j < 4; ++j) mbar_init(&ctl->tfull_a[g][j], 1);
-        }
-        for (int g = 0; g < kBGroups; ++g) {
-            mbar_init(&ctl->tempty_b[g], 4);
-            for (int j = 0; j < 4; ++j) mbar_init(&ctl->tfull_b[g][j], 1);
-        }
+        mbar_init(&ctl->qempty, 2);
+        for (int g = 0; g < kAGroups; ++g) { mbar_init(&ctl->tfull_a[g], 1); mbar_init(&ctl->tempty_a[g], 4); }
+        for (int g = 0; g < kBGroups; ++g) { mbar_init(&ctl->tfull_b[g], 1); mbar_init(&ctl->tempty_b[g], 4); mbar_init(&ctl->tempty_b[kBGroups + g], 4); }
+        for (int i = 0; i < 4; ++i) mbar_init(&ctl->tokfull[i], a.RB > 1 ? 4 * (a.RB - 1) : 1);
         mbar_init(&ctl->extfull, 4);
-        mbar_init(&ctl->extempty, 1);
+        mbar_init(&ctl->extempty, 2);
         for (int i = 0; i < kIndRing; ++i) { mbar_init(&ctl->ifull[i], kPoolWarps); mbar_init(&ctl->iempty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&ctl->pfull[i], 1); mbar_init(&ctl->issued_done[i], 1); }
+        for (int i = 0; i < 2; ++i) mbar_init(&ctl->pfull[i], 1);
+        for (int i = 0; i < 3; ++i) mbar_init(&ctl->issued_done[i], 1);
         ctl->abort_flag = 0;
         mbar_fence_init();
         tmap_prefetch(&mapK);
@@ -315,6 +313,11 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     const float scale = kLog2e * rsqrtf(float(kHeadDim));
     const int n = a.Hq / Hk;
     const uint32_t ext_smem = smem_u32(extb);
+    // Pass A, last block of at most 64 rows: on every second tile its rows take the upper tensor-memory lanes, so that the
+    // exponentials spread over all four schedulers.  (Which tiles an epilogue group gets its last block from has one parity
+    // for each group when there are 2, 3 or 5 blocks.)
+    const bool can_shift = a.RA > 1 && a.RA != 4 && a.R - (a.RA - 1) * 128 <= 64;
+    auto shifted = [&](int i) { return can_shift && (i & 1); };
 
     if (ntl > 0) {
     if (warp == 0) {
@@ -368,15 +371,19 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 mbar_wait(&ctl->qfull, 1u, 1u << 16);
             }
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer
+    } else if (warp == 1 || warp == 19) {
+        // ------------------------------------------------------------------ MMA warps
+        // Two of them take the products in turn.  An issue blocks until the tensor core has taken the product, and a look
+        // at a barrier in between (115 cycles and more) leaves it idle; with two issuers one waits while the other's
+        // product runs (measured without epilogue: 817 against 579 cycles per 128 x 128 x 128 product, 512 the least).
+        const int mine = warp == 1 ? 0 : 1;
         bool ok = true;
         uint32_t qlap = 0;
-        int load_no = 0;                                 // tiles of the ring so far: stage load_no % stages, lap load_no / stages
+        const uint32_t q0 = smem_u32(qbuf);
         if (lane == 0) {
             int stage = 0, it = 0, slab = slab_of(resident ? t_begin : t_end - 1), lo = 0, hi = 0;
             uint32_t lap = 0;
-            const uint32_t q0 = smem_u32(qbuf);
+            const int n_empty = a.RB > 1 ? 3 : 2;        // arrivals that free a stage
             for (int i = 0; i < ntl && ok; ++i) {
                 const int t = resident ? t_begin + i : t_end - 1 - i;
                 if (i == 0 || t >= hi || t < lo) {
@@ -387,36 +394,41 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     if (!ok) break;
                     ++qlap;
                 }
+                // (both warps follow every tile's arrival, so that they see each phase of a stage's barrier)
                 ok = role_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
-                if (!ok) break;
-                const uint32_t k_smem = smem_u32(tiles + size_t(stage) * kOpBytes);
+                bool here = false;                       // this warp has a product of the tile
                 for (int k = 0; k < a.RA && ok; ++k, ++it) {
+                    if ((it & 1) != mine) continue;
+                    here = true;
                     const int buf = it & (kAGroups - 1), use = it / kAGroups;
                     if (use > 0) ok = role_wait(&ctl->tempty_a[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     tc_fence_after();
-                    umma_tile(tmem_base + buf * 128, q0 + uint32_t(k) * kOpHalfBytes, q_half, k_smem, kOpHalfBytes, kIdescBf16M128N128);
-                    const int gj = (i / kAGroups) * a.RA + k;        // the owning group's item count
-                    umma_commit(&ctl->tfull_a[i % kAGroups][gj & 3]);
+                    const int r = k + 1 == a.RA && shifted(i) ? a.R - 128 : k * 128;       // first query row
+                    umma_tile(tmem_base + buf * 128, q0 + uint32_t(r) * 128u, q_half, smem_u32(tiles + size_t(stage) * kOpBytes),
+                              kOpHalfBytes, kIdescBf16M128N128);
+                    umma_commit(&ctl->tfull_a[buf]);
                 }
                 const int t_next = resident ? t + 1 : t - 1;
                 if (i + 1 == ntl || t_next >= hi || t_next < lo) umma_commit(&ctl->qempty);
-                if (!resident) { umma_commit(&ctl->empty[stage]); umma_commit(&ctl->empty[stage]); }
+                if (!resident && here) {                 // one warp: all arrivals; two: the second one of the tile makes up the number
+                    const int c = a.RA == 1 ? n_empty : (((it - 1) & 1) == mine ? n_empty - 1 : 1);
+                    for (int e = 0; e < c; ++e) umma_commit(&ctl->empty[stage]);
+                }
                 if (++stage == a.stages) { stage = 0; ++lap; }
             }
-            load_no = resident ? 0 : ntl;
-            if (!ok) { umma_commit(&ctl->issued_done[0]); mbar_wait(&ctl->issued_done[0], 0u, 1u << 18); }
+            if (!ok) { umma_commit(&ctl->issued_done[mine]); mbar_wait(&ctl->issued_done[mine], 0u, 1u << 18); }
         }
         __syncwarp();
         tc_fence_before();
         named_bar_sync(1, kSweepThreads - 32);           // every accumulator of pass A has been read
         tc_fence_after();
         if (lane == 0 && ok) {
-            int it = 0, slab = slab_of(t_begin), hi = 0;
-            uint32_t elap = 0;
+            int it = 0, slab = slab_of(t_begin), hi = 0, stage = resident ? 0 : ntl % a.stages;
+            uint32_t elap = 0, lap = resident ? 0u : uint32_t(ntl / a.stages);
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t(a.N) >> 3) << 17) | ((128u >> 4) << 24);
             const uint64_t d_ones = umma_desc_sw32(smem_u32(onesb));
-            for (int i = 0; i < ntl && ok; ++i, ++load_no) {
+            for (int i = 0; i < ntl && ok; ++i) {
                 const int t = t_begin + i;
                 if (i == 0 || t >= hi) {
                     while (pref[slab + 1] <= t) ++slab;
@@ -426,28 +438,28 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     if (!ok) break;
                     ++qlap; ++elap;
                 }
-                const int stage = load_no % a.stages;
-                ok = role_wait(&ctl->full[stage], uint32_t(load_no / a.stages) & 1u, limit, &ctl->abort_flag, a.status);
-                if (!ok) break;
-                const uint32_t k_smem = smem_u32(tiles + size_t(stage) * kOpBytes);
+                ok = role_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
+                bool here = false;
                 for (int k = 0; k < a.RB && ok; ++k, ++it) {
-                    const int buf = it % kBGroups, use = it / kBGroups;
-                    if (use > 0) ok = role_wait(&ctl->tempty_b[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
+                    if ((it & 1) != mine) continue;
+                    here = true;
+                    const int buf = it % kBGroups, before = it - kBGroups;
+                    if (before >= 0) ok = role_wait(&ctl->tempty_b[before % (2 * kBGroups)], uint32_t(before / (2 * kBGroups)) & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d = tmem_base + buf * kBAccCols;
-                    umma_tile(d, k_smem, kOpHalfBytes, smem_u32(qbuf) + uint32_t(k * a.N) * 128u, q_half, idesc);
+                    umma_tile(d, smem_u32(tiles + size_t(stage) * kOpBytes), kOpHalfBytes, q0 + uint32_t(k * a.N) * 128u, q_half, idesc);
                     umma_bf16(d, d_ones, umma_desc_sw32(ext_smem + uint32_t(k * a.N) * kExtRow), idesc, 1u);      // - lse
-                    const int gj = (i / kBGroups) * a.RB + k;
-                    umma_commit(&ctl->tfull_b[i % kBGroups][gj & 3]);
+                    umma_commit(&ctl->tfull_b[buf]);
                 }
                 if (i + 1 == ntl || hi <= t + 1) { umma_commit(&ctl->qempty); umma_commit(&ctl->extempty); }
-                umma_commit(&ctl->empty[stage]);
+                if (here) umma_commit(&ctl->empty[stage]);
+                if (++stage == a.stages) { stage = 0; ++lap; }
             }
             if (!ok) {
                 // nobody will wait for the products still in flight: let them retire before the tensor memory is released
-                umma_commit(&ctl->issued_done[0]);
-                mbar_wait(&ctl->issued_done[0], 0u, 1u << 18);
+                umma_commit(&ctl->issued_done[mine]);
+                mbar_wait(&ctl->issued_done[mine], 0u, 1u << 18);
             }
         }
     } else {
@@ -457,9 +469,11 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         {
             const int g = (warp - 2) >> 2;                   // warpgroup (warp 18: 4, clears the key sums)
             const int row = quarter * 32 + lane;
-            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16);
+            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + g * 128;
             float2* part = reinterpret_cast<float2*>(extb);  // [group][RA * 128]
-            int i = g;                                       // tiles of this warpgroup: i, i + 4, ... in the order of the pass
+            const bool g_shifted = can_shift && (a.RA == 2 ? g == 3 : (g & 1) != 0);
+            const int rem = a.R - (a.RA - 1) * 128;          // rows of the last block
+            int it = g, ti = g / a.RA, tk = g - ti * a.RA;   // this group's next product: its number, tile (in the order of the pass) and block
             int slab = slab_of(resident ? t_begin : t_end - 1);
             for (int done = 0; done < ntl;) {
                 // one segment: the tiles of a slab that this CTA has
@@ -473,27 +487,31 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     float m[kMaxBlocksA], l[kMaxBlocksA];
 #pragma unroll
                     for (int k = 0; k < kMaxBlocksA; ++k) { m[k] = -INFINITY; l[k] = 0.f; }
-                    for (; i < seg_end; i += kAGroups) {
-                        const int t = resident ? t_begin + i : t_end - 1 - i;
+                    for (; ti < seg_end; it += kAGroups) {
+                        const int t = resident ? t_begin + ti : t_end - 1 - ti;
                         const int valid = min(128, N - (t - pref[slab]) * 128);
-#pragma unroll
-                        for (int k = 0; k < kMaxBlocksA; ++k) {
-                            if (k < a.RA && ok) {
-                                const int buf = (i * a.RA + k) & (kAGroups - 1), gj = (i / kAGroups) * a.RA + k;
-                                ok = role_wait(&ctl->tfull_a[g][gj & 3], uint32_t(gj >> 2) & 1u, limit, &ctl->abort_flag, a.status);
-                                ok = __all_sync(0xffffffffu, ok);
-                                if (ok) {
-                                    tc_fence_after();
-                                    if (k * 128 + quarter * 32 < a.R) {          // (the last block may hold fewer rows)
-                                        if (valid == 128) lse_fold<false>(lane_addr + buf * 128, valid, scale, m[k], l[k]);
-                                        else              lse_fold<true>(lane_addr + buf * 128, valid, scale, m[k], l[k]);
-                                    }
-                                    tc_fence_before();
-                                    __syncwarp();
-                                    if (lane == 0) mbar_arrive(&ctl->tempty_a[buf]);
-                                }
-                            }
+                        if (ok) {
+                            ok = role_wait(&ctl->tfull_a[g], uint32_t(it / kAGroups) & 1u, limit, &ctl->abort_flag, a.status);
+                            ok = __all_sync(0xffffffffu, ok);
                         }
+                        if (ok) {
+                            tc_fence_after();
+                            // (the last block may hold fewer rows than lanes)
+                            if (tk + 1 < a.RA || (g_shifted ? quarter * 32 + 31 >= 128 - rem : quarter * 32 < rem)) {
+                                float mk = m[0], lk = l[0];
+#pragma unroll
+                                for (int k = 1; k < kMaxBlocksA; ++k) if (tk == k) { mk = m[k]; lk = l[k]; }
+                                if (valid == 128) lse_fold<false>(lane_addr, valid, scale, mk, lk);
+                                else              lse_fold<true>(lane_addr, valid, scale, mk, lk);
+#pragma unroll
+                                for (int k = 0; k < kMaxBlocksA; ++k) if (tk == k) { m[k] = mk; l[k] = lk; }
+                            }
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&ctl->tempty_a[g]);
+                        }
+                        tk += kAGroups;
+                        while (tk >= a.RA) { tk -= a.RA; ++ti; }
                     }
 #pragma unroll
                     for (int k = 0; k < kMaxBlocksA; ++k)
@@ -512,7 +530,11 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                         float2 x[kAGroups];
                         float M = -INFINITY, L = 0.f;
 #pragma unroll
-                        for (int q = 0; q < kAGroups; ++q) { x[q] = part[(q * a.RA + k) * 128 + row]; M = fmaxf(M, x[q].x); }
+                        for (int q = 0; q < kAGroups; ++q) {
+                            const bool sh = k + 1 == a.RA && can_shift && (a.RA == 2 ? q == 3 : (q & 1) != 0);
+                            x[q] = part[(q * a.RA + k) * 128 + (sh ? min(row + 128 - rem, 127) : row)];
+                            M = fmaxf(M, x[q].x);
+                        }
 #pragma unroll
                         for (int q = 0; q < kAGroups; ++q) L += x[q].y > 0.f ? x[q].y * ex2f(x[q].x - M) : 0.f;
                         rec[k * 128 + row] = make_float2(M, L);
@@ -533,26 +555,30 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             const int g = warp < 10 ? (warp - 2) >> 2 : 2;
             const int row = quarter * 32 + lane;
             const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16);
-            int slab = slab_of(t_begin), seg_first = t_begin, N = 0;
+            // (what depends on the slab only is kept in registers: while the tensor core streams its operands every look at
+            // shared memory takes a hundred cycles and more)
+            int slab = slab_of(t_begin), lo = 0, hi = 0, N = 0;         // the slab's tiles are [lo, hi)
             uint32_t ext_no = 0;                             // slabs begun so far
-            size_t row0 = 0;
-            bool have = false;
-            for (int i = 0; i < ntl; ++i) {
-                const int t = t_begin + i;
-                if (!have || pref[slab + 1] <= t) {
+            float *imp_ws = nullptr, *imp_user = nullptr;
+            const float inv_window = 1.f / float(a.window);
+            int ti = 0, tk = 0;
+            for (int it = 0; it < ntl * a.RB; ++it) {
+                const int t = t_begin + ti, i = ti, k = tk;
+                if (++tk == a.RB) { tk = 0; ++ti; }
+                if (t >= hi) {
                     while (pref[slab + 1] <= t) ++slab;
-                    have = true;
-                    seg_first = t;
+                    lo = pref[slab]; hi = pref[slab + 1];
                     N = live(slab);
-                    row0 = a.block_table ? size_t(slab) * a.max_pages * 128 : size_t(rowb[slab]);
+                    imp_ws = a.tok_imp_ws + size_t(slab) * a.max_cap;
+                    imp_user = a.tok_imp_user ? a.tok_imp_user + (a.block_table ? size_t(slab) * a.max_pages * 128 : size_t(rowb[slab])) : nullptr;
                     ++ext_no;
                 }
-                if (i % kBGroups != g) continue;
-                if (t == seg_first) {
-                    // the group of a slab's first tile prepares the slab: log-sum-exp of its query rows from the records of
+                if (it % kBGroups != g) continue;
+                if (k == 0 && t == max(lo, t_begin)) {
+                    // the group of a slab's first product prepares the slab: log-sum-exp of its query rows from the records of
                     // all its CTAs, negated, in units of raw logits, as three bf16 pieces of the extra K step
-                    const int fc = owner(pref[slab]), lc = owner(pref[slab + 1] - 1);
-                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(pref[slab + 1] - pref[slab]), limit, &ctl->abort_flag, a.status);
+                    const int fc = owner(lo), lc = owner(hi - 1);
+                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(hi - lo), limit, &ctl->abort_flag, a.status);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                     if (ok && ext_no > 1) ok = role_wait(&ctl->extempty, (ext_no - 2) & 1u, limit, &ctl->abort_flag, a.status);
                     ok = __all_sync(0xffffffffu, ok);
@@ -588,24 +614,32 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                         if (lane == 0) mbar_arrive(&ctl->extfull);
                     }
                 }
-                float total = 0.f;
-                for (int k = 0; k < a.RB; ++k) {
-                    const int buf = (i * a.RB + k) % kBGroups, gj = (i / kBGroups) * a.RB + k;
-                    if (!ok) break;
-                    ok = role_wait(&ctl->tfull_b[g][gj & 3], uint32_t(gj >> 2) & 1u, limit, &ctl->abort_flag, a.status);
+                if (ok) {
+                    ok = role_wait(&ctl->tfull_b[g], uint32_t(it / kBGroups) & 1u, limit, &ctl->abort_flag, a.status);
                     ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                    tc_fence_after();
-                    total += imp_fold<kWB>(lane_addr + buf * kBAccCols, n, min(kWB, a.window - k * kWB), scale);
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->tempty_b[buf]);
                 }
-                const int tok = (t - pref[slab]) * 128 + row;
-                if (ok && tok < N) {
-                    const float v = total / float(a.window);
-                    a.tok_imp_ws[size_t(slab) * a.max_cap + tok] = v;
-                    if (a.tok_imp_user) a.tok_imp_user[row0 + tok] = v;
+                if (!ok) continue;
+                tc_fence_after();
+                float total = imp_fold<kWB>(lane_addr + g * kBAccCols, n, min(kWB, a.window - k * kWB), scale);
+                float* share = tokp + (i & 3) * (a.RB - 1) * 128 + row;
+                if (k + 1 < a.RB) {
+                    share[k * 128] = total;                  // another group adds the shares up, in the order of the blocks
+                } else if (a.RB > 1) {
+                    ok = role_wait(&ctl->tokfull[i & 3], uint32_t(i >> 2) & 1u, limit, &ctl->abort_flag, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    for (int q = a.RB - 2; q >= 0; --q) total += share[q * 128];
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (k + 1 < a.RB) mbar_arrive(&ctl->tokfull[i & 3]);
+                    mbar_arrive(&ctl->tempty_b[it % (2 * kBGroups)]);
+                }
+                const int tok = (t - lo) * 128 + row;
+                if (k + 1 == a.RB && ok && tok < N) {
+                    const float v = total * inv_window;
+                    imp_ws[tok] = v;
+                    if (imp_user) imp_user[tok] = v;
                 }
             }
         } else if (warp < 14) {
@@ -628,11 +662,14 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + kPoolCol;
             int slab = slab_of(t_begin), S = 0, N = 0, first = 0;
             int ic = 0;                                             // indicator matrices written so far
-            int run = -1, B = 0, w = kNever;                        // current run: index, sentence of slot 0, offsets B + lane
+            int run = -1, B = 0, w = kNever, w1 = kNever;           // current run: index, sentence of slot 0, offsets B + lane and B + lane + 1
+            int wj = kNever, wj1 = kNever;                          // and the offsets of this thread's slot row
+            const int sj = 4 * gw + (lane >> 3);                    // the slot row, of which this thread writes two pieces
+            int lo = 0, hi = 0, stage = load0 % a.stages;           // the slab's tiles are [lo, hi)
+            uint32_t lap = uint32_t(load0 / a.stages);
             uint32_t run_held = 0;                                  // its slots that hold tokens so far
             int run_slab = 0;
             const int32_t* so = a.sent_off;
-            bool have = false;
             // 32-way search for the last sentence that starts at or before token `tok`, one probe per lane
             auto holder = [&](int tok) {
                 int lo = 0, len = S;
@@ -663,23 +700,22 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             };
             for (int tl = 0; tl < ntl && ok; ++tl) {
                 const int t = t_begin + tl;
-                const bool fresh = !have || pref[slab + 1] <= t;
+                const bool fresh = t >= hi;
                 if (fresh) {
                     while (pref[slab + 1] <= t) ++slab;
-                    have = true;
+                    lo = pref[slab]; hi = pref[slab + 1];
                     so = a.sent_off + size_t(slab) * (a.max_sent + 1);
                     S = min(max(a.n_sent[slab], 0), a.max_sent);
                     N = live(slab);
                     // every CTA of the slab has cleared its share of the sums (and left its record)
-                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(pref[slab + 1] - pref[slab]), limit, &ctl->abort_flag, a.status);
+                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(hi - lo), limit, &ctl->abort_flag, a.status);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                     if (!ok) break;
                 }
-                const int tok0 = (t - pref[slab]) * 128, valid = min(128, N - tok0), tok_end = tok0 + valid;
-                const int stage = (load0 + tl) % a.stages;
+                const int tok0 = (t - lo) * 128, valid = min(128, N - tok0), tok_end = tok0 + valid;
                 if (fresh) first = tok0 > 0 ? holder(tok0) : 0;     // (a slab that opens with empty sentences: they get slots)
                 // every warp follows every tile's arrival (in order, so it sees each phase of the stage's barrier)
-                ok = role_wait(&ctl->full[stage], uint32_t((load0 + tl) / a.stages) & 1u, limit, &ctl->abort_flag, a.status);
+                ok = role_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (valid < 128) {
@@ -705,13 +741,14 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     if (!join) {                                    // open a run at sentence cur
                         ++run; B = cur; run_slab = slab; run_held = 0;
                         w = (B + lane <= S) ? so[B + lane] : kNever;
+                        w1 = (B + lane + 1 <= S) ? so[B + lane + 1] : kNever;
+                        wj = (B + sj <= S) ? so[B + sj] : kNever;
+                        wj1 = (B + sj + 1 <= S) ? so[B + sj + 1] : kNever;
                     }
-                    // tile-relative start of the sentences B + lane, clamped to the tile; slot j holds [cl(j), cl(j + 1))
-                    const int cl = min(max(min(w, tok_end) - tok0, 0), valid);
-                    const int cl_next = __shfl_down_sync(0xffffffffu, cl, 1);
-                    const uint32_t held = __ballot_sync(0xffffffffu, lane < kIndSlots && B + lane < S && cl_next > cl);
-                    const int s_next = __shfl_sync(0xffffffffu, w, kIndSlots);           // start of the sentence after slot 15
-                    more = (B + kIndSlots < S && s_next < tok_end) ? 1 : 0;
+                    // tile-relative starts of sentences, clamped to the tile; slot j holds the tokens from its start to the next one's
+                    auto clamped = [&](int off) { return min(max(min(off, tok_end) - tok0, 0), valid); };
+                    const uint32_t held = __ballot_sync(0xffffffffu, lane < kIndSlots && B + lane < S && clamped(w1) > clamped(w));
+                    more = __any_sync(0xffffffffu, lane == kIndSlots && B + kIndSlots < S && w < tok_end) ? 1 : 0;    // does slot 15 leave some?
                     const int is = ic & (kIndRing - 1);
                     if (ic >= kIndRing) {                           // the product that read this buffer last has completed
                         ok = role_wait(&ctl->iempty[is], uint32_t(ic / kIndRing - 1) & 1u, limit, &ctl->abort_flag, a.status);
@@ -719,11 +756,10 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                         if (!ok) break;
                     }
                     {
-                        const int j = 4 * gw + (lane >> 3);         // this thread's slot row and its two pieces
-                        const int lo = __shfl_sync(0xffffffffu, cl, j), hi = __shfl_sync(0xffffffffu, cl, j + 1);
-                        const bool is_sent = (held >> j) & 1u;
-                        indicator_piece(indb + size_t(is) * kIndBytes, j, (lane & 7) * 2, is_sent ? lo : 0, is_sent ? hi : 0);
-                        indicator_piece(indb + size_t(is) * kIndBytes, j, (lane & 7) * 2 + 1, is_sent ? lo : 0, is_sent ? hi : 0);
+                        const bool is_sent = (held >> sj) & 1u;
+                        const int from = is_sent ? clamped(wj) : 0, to = is_sent ? clamped(wj1) : 0;
+                        indicator_piece(indb + size_t(is) * kIndBytes, sj, (lane & 7) * 2, from, to);
+                        indicator_piece(indb + size_t(is) * kIndBytes, sj, (lane & 7) * 2 + 1, from, to);
                     }
                     fence_proxy_async_smem();                       // the matrix (and cleared rows) are read by the tensor core
                     tc_fence_before();                              // and this warp's reads of the accumulators came first
@@ -743,6 +779,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 // the next tile starts in the last sentence of the run's window that starts at or before its first token
                 const int n_le = __popc(__ballot_sync(0xffffffffu, B + lane < S && w <= tok0 + 128));
                 first = (n_le == 32 && B + 32 < S) ? holder(tok0 + 128) : B + max(n_le - 1, 0);
+                if (++stage == a.stages) { stage = 0; ++lap; }
             }
             if (ok && run >= 0) drain(run, run_slab, B, run_held);  // the issuer closes the last run when its tiles are done
         } else {
@@ -751,9 +788,8 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             // thread that issues the logits a few hundred cycles)
             if (lane == 0) {
                 const uint32_t indb_u32 = smem_u32(indb);
-                int pc = 0, run = -1;
+                int pc = 0, run = -1, stage = load0 % a.stages;
                 for (int tl = 0; tl < ntl && ok; ++tl) {
-                    const int stage = (load0 + tl) % a.stages;
                     int flags = 0;
                     do {
                         const int is = pc & (kIndRing - 1);
@@ -769,11 +805,12 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                         ++pc;
                     } while (flags & 1);
                     if (ok) umma_commit(&ctl->empty[stage]);
+                    if (++stage == a.stages) stage = 0;
                 }
                 if (ok && run >= 0) umma_commit(&ctl->pfull[run & 1]);
                 if (!ok) {
-                    umma_commit(&ctl->issued_done[1]);
-                    mbar_wait(&ctl->issued_done[1], 0u, 1u << 18);
+                    umma_commit(&ctl->issued_done[2]);
+                    mbar_wait(&ctl->issued_done[2], 0u, 1u << 18);
                 }
             }
         }
@@ -1289,14 +1326,22 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     a.block_table = block_table; a.max_pages = max_pages;
     const size_t max_smem = 227 * 1024;
     const size_t fixed = 1024 + size_t(a.R) * kRowBytes + size_t(kIndRing) * kIndBytes + 128 * kExtRow + size_t(a.RA) * 128 * kExtRow +
-                         sizeof(SweepCtl) + size_t(2 * L.slabs + 1) * 4;
+                         sizeof(SweepCtl) + size_t(a.RB - 1) * 4 * 128 * 4 + size_t(2 * L.slabs + 1) * 4;
     if (fixed + kOpBytes > max_smem) return SKIPKV_ERR_UNSUPPORTED;
     a.stages = int((max_smem - fixed) / kOpBytes);
     if (a.stages > kStagesMax) a.stages = kStagesMax;
     int grid = num_sms();
     if (grid > L.dec_max_ctas) grid = L.dec_max_ctas;
-    SKIPKV_CUDA(launch_dependent<true>(L.sc_wb == 32 ? score_sweep_kernel<32> : score_sweep_kernel<16>, dim3(grid), dim3(kSweepThreads),
-                                 fixed + size_t(a.stages) * kOpBytes, st, mapK, mapQ, a));
+    // Cooperative: the CTAs wait for one another between the passes, so they have to be resident together whatever else
+    // runs on the GPU.  Where the context may use fewer SMs than the device has, a smaller grid does.
+    cudaError_t le = cudaErrorCooperativeLaunchTooLarge;
+    for (; grid >= 1 && le == cudaErrorCooperativeLaunchTooLarge; grid /= 2) {
+        le = launch_dependent<true>(L.sc_wb == 32 ? score_sweep_kernel<32> : score_sweep_kernel<16>, dim3(grid), dim3(kSweepThreads),
+                                    fixed + size_t(a.stages) * kOpBytes, st, mapK, mapQ, a);
+        if (le == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();
+        else break;
+    }
+    SKIPKV_CUDA(le);
     // one tile of sentences per slab: one kernel instead of three, with the operands in shared memory throughout
     if (shape->max_sent <= kSmallSent) {
         SKIPKV_CUDA(launch_dependent(score_small_kernel, dim3(L.slabs), dim3(kSmallThreads), kSmallSmem, st, a.lse_cnt, Hk, int(shape->max_sent),
