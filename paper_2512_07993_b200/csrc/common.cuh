@@ -28,10 +28,12 @@ constexpr uint32_t kDefaultWaitLimit = 1u << 22;
 
 struct WsLayout {
     size_t header;
-    size_t cp_nseg;        // int32  [slabs]              segments per stream
-    size_t cp_loaded;      // uint32 [2*slabs]            segments whose loads are complete
+    size_t cp_len;         // int32  [slabs]              rows after the compaction
+    size_t cp_loaded;      // uint32 [2*slabs][cp_segs]   1: the segment's source rows have been read
+    size_t cp_seg_run;     // int32  [slabs][cp_segs]     first run that reaches into the segment
+    size_t cp_seg_dep;     // int32  [slabs][cp_segs]     destination row of the first survivor at or behind the segment's first row
     size_t cp_nruns;       // int32  [slabs]
-    size_t cp_run_src;     // int32  [slabs][max_sent]    first source token of a run
+    size_t cp_run_src;     // int32  [slabs][max_sent]    first source token of a run (~: its index entries are already written)
     size_t cp_run_dst;     // int32  [slabs][max_sent+1]  first destination token; [nruns] = new_len
     size_t dec_cnt;        // uint32 [slabs]              partials that arrived (self-resetting)
     size_t dec_part;       // float  [max_ctas + slabs][group][kDecPartStride]
@@ -42,7 +44,6 @@ struct WsLayout {
     size_t sc_vbar_hi;     // bf16   [slabs][max_sent][128]  normalised mean key, high part
     size_t sc_vbar_lo;     // bf16   [slabs][max_sent][128]  and the rounding remainder
     size_t sc_z;           // float  [slabs][max_sent]
-    size_t cp_part;        // int32  [slabs][1 + 3*kMaxPartial]  partly kept sentences: count, then (begin, end, dst)
     size_t tr_inv;         // float  [slabs][max_cap]  token redundancy: 1 / (|K_t| + eps)
     size_t tr_z;           // float  [slabs][max_cap]  token redundancy: row sums of exp(G)
     size_t total;
@@ -50,11 +51,13 @@ struct WsLayout {
     int sc_wb;             // window positions per block of query rows of the scoring sweeps: 32 or 16
     int sc_rb;             // blocks: ceil(window / sc_wb)
     int sc_ra;             // the same rows in blocks of 128
+    int cp_segs;           // segments of kSegRows rows a slab can have (and a few more: paged slabs end on whole pages)
 };
 
 constexpr int kDecPartStride = 132;    // decode partial of one head: 128 accumulators, max, sum, padding
 constexpr int kDecMaxCtas = 1024;     // upper bound of the persistent grids
 constexpr int kMaxQueryBlocks = 4;
+constexpr int kSegRows = 128;         // rows per segment of the compaction
 constexpr int kMaxPartial = 4;        // partly kept sentences per slab that one compaction call can carry
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -76,8 +79,11 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     auto take = [&](size_t bytes) { size_t r = o; o = align256(o + bytes); return r; };
     const size_t slabs = L.slabs, ms = s.max_sent > 0 ? s.max_sent : 1;
     L.header = take(sizeof(Header));
-    L.cp_nseg = take(slabs * 4);
-    L.cp_loaded = take(slabs * 2 * 4);
+    L.cp_segs = (s.max_cap > 0 ? s.max_cap : 1) / kSegRows + 3;
+    L.cp_len = take(slabs * 4);
+    L.cp_loaded = take(slabs * 2 * size_t(L.cp_segs) * 4);
+    L.cp_seg_run = take(slabs * size_t(L.cp_segs) * 4);
+    L.cp_seg_dep = take(slabs * size_t(L.cp_segs) * 4);
     L.cp_nruns = take(slabs * 4);
     L.cp_run_src = take(slabs * ms * 4);
     L.cp_run_dst = take(slabs * (ms + 1) * 4);
@@ -90,7 +96,6 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     L.sc_vbar_hi = take(slabs * ms * kHeadDim * 2);
     L.sc_vbar_lo = take(slabs * ms * kHeadDim * 2);
     L.sc_z = take(slabs * ms * 4);
-    L.cp_part = take(slabs * (1 + 3 * kMaxPartial) * 4);
     L.tr_inv = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);
     L.tr_z = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);
     L.total = o;

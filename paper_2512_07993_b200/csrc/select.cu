@@ -1,15 +1,15 @@
 // skipkv_select: which sentences survive under the KV budget (paper Section 4.1: evict in
 // increasing order of the final score until the cache meets budget B), at sentence granularity.
 //
-// One CTA per (sequence, head) slab.  Each sentence becomes a 64-bit key
-//     [ 1 bit: not protected | 32 bits: ~orderable(score) | 31 bits: sentence index ]
-// so an ascending sort yields: protected-tail sentences in index order, then the rest by score
-// descending with ties broken by the lower index (exact fp32 comparison, -0 == +0).  The keys
-// are sorted with a block-wide bitonic network in shared memory, the sentence lengths are
-// prefix-summed in rank order, and a sentence survives iff its inclusive running total is
-// within the budget.  Because lengths are non-negative the running total is monotone, so this
-// is exactly "the longest rank prefix that fits; stop at the first sentence that does not".
-// skipkv_select_fill then lets that first sentence keep its most important tokens, so that exactly B survive.
+// One CTA per (sequence, head) slab.  The ranking is: protected-tail sentences in index order, then the rest by score
+// descending with ties broken by the lower index (exact fp32 comparison, -0 == +0); a sentence survives iff its inclusive
+// running total of lengths in rank order is within the budget.  Lengths are non-negative, so the total is monotone and
+// this is exactly "the longest rank prefix that fits; stop at the first sentence that does not": nothing has to be sorted,
+// only the score has to be found at which the total crosses the budget.  It is found digit by digit (8 bits at a time,
+// from the top): a histogram of lengths over the sentences that share the digits so far, and the bin in which the
+// running total crosses; sentences of exactly that score are then taken in index order.  One barrier per digit (every warp
+// scans the histogram itself).  A bitonic sort of 1024 keys took 55 rounds and 14 us per call; this takes 4 digits.
+// skipkv_select_fill then lets the first sentence that does not fit keep its most important tokens, so that exactly B survive.
 #include "common.cuh"
 
 namespace skipkv {
@@ -22,10 +22,9 @@ __device__ __forceinline__ uint32_t orderable(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u); // ascending in f
 }
 
-// exclusive scan over P = blockDim.x * per values held per thread as a running block; generic helper:
-// each thread passes its local total, gets the exclusive offset of its first element.
+// each thread passes its local total, gets the exclusive offset of its first element
 __device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t* wsum, uint32_t& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t inc = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -34,10 +33,12 @@ __device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t* wsum, uint3
     }
     if (lane == 31) wsum[warp] = inc;
     __syncthreads();
-    uint32_t base = 0, t = 0;
-    for (int w = 0; w < nw; ++w) {
-        if (w == warp) base = t;
-        t += wsum[w];
+    const uint32_t w = lane < kSelThreads / 32 ? wsum[lane] : 0u;
+    uint32_t base = lane < warp ? w : 0u, t = w;
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        base += __shfl_xor_sync(0xffffffffu, base, d);
+        t += __shfl_xor_sync(0xffffffffu, t, d);
     }
     total = t;
     __syncthreads();
@@ -57,24 +58,30 @@ struct FillArgs {
     int Hk, max_cap, from_rows;
 };
 
+constexpr int kFillStage = 1024;        // tokens of a cut sentence whose order keys are staged in shared memory
+
 __global__ void __launch_bounds__(kSelThreads)
-select_kernel(int max_sent, int P, int budget, int protect_tail, const float* sent_score, const int32_t* sent_off,
+select_kernel(int max_sent, int budget, int protect_tail, const float* sent_score, const int32_t* sent_off,
               const int32_t* n_sent, uint8_t* keep, int32_t* kept_idx, int32_t* n_kept, int32_t* new_len,
               FillArgs fill, uint32_t* status) {
     extern __shared__ __align__(16) uint8_t sel_smem[];
-    uint64_t* keys = reinterpret_cast<uint64_t*>(sel_smem);             // [P]
-    uint8_t* flags = reinterpret_cast<uint8_t*>(keys + P);             // [P] keep flag by sentence index
-    __shared__ uint32_t wsum[kSelThreads / 32];
+    uint32_t* keys = reinterpret_cast<uint32_t*>(sel_smem);            // [max_sent] ascending in rank; a thread touches its own only
+    int* lens = reinterpret_cast<int*>(keys + max_sent);               // [max_sent] length, negative - 1 if protected
+    __shared__ uint32_t hist[4][256], wsum[kSelThreads / 32];
+    __shared__ uint32_t s_forced;
     __shared__ int s_cut, s_slack;
+    __shared__ float s_key[kFillStage];
     pdl_trigger();
+    const int slab = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    for (int i = tid; i < 4 * 256; i += kSelThreads) (&hist[0][0])[i] = 0u;
+    if (tid == 0) { s_forced = 0u; s_cut = -1; s_slack = 0; }
     pdl_wait();                                          // inputs may come from the kernel before
-    const int slab = blockIdx.x, tid = threadIdx.x;
     const float* score = sent_score + size_t(slab) * max_sent;
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
     uint8_t* kp = keep + size_t(slab) * max_sent;
     int32_t* ki = kept_idx ? kept_idx + size_t(slab) * max_sent : nullptr;
     int S = n_sent[slab];
-    if (S < 0 || S > max_sent || S > P) {
+    if (S < 0 || S > max_sent) {
         if (tid == 0) atomicOr(status, SKIPKV_STATUS_BAD_TABLE);
         S = 0;
     }
@@ -92,53 +99,75 @@ select_kernel(int max_sent, int P, int budget, int protect_tail, const float* se
         return;
     }
 
-    for (int i = tid; i < P; i += kSelThreads) {
-        uint64_t k = ~0ull;
-        if (i < S) {
-            const int b = so[i], e = so[i + 1];
-            const bool forced = protect_tail > 0 && e > total - protect_tail && e > b;
-            const uint64_t hi = forced ? 0ull : (0x100000000ull | uint64_t(~orderable(score[i])));
-            k = (hi << 31) | uint64_t(uint32_t(i));
-        }
+    __syncthreads();                                     // the histograms are clear
+    const int per = (S + kSelThreads - 1) / kSelThreads, i0 = min(tid * per, S), i1 = min(i0 + per, S);   // this thread's sentences
+    for (int i = i0; i < i1; ++i) {
+        const int b = so[i], e = so[i + 1];
+        const bool forced = protect_tail > 0 && e > total - protect_tail && e > b;
+        const uint32_t k = ~orderable(score[i]);
         keys[i] = k;
-        flags[i] = 0;
+        lens[i] = forced ? -(e - b) - 1 : e - b;
+        if (forced) atomicAdd(&s_forced, uint32_t(e - b));
+        else if (e > b) atomicAdd(&hist[0][k >> 24], uint32_t(e - b));
     }
-    if (tid == 0) { s_cut = -1; s_slack = 0; }
     __syncthreads();
-    // bitonic sort, ascending.  Thread p of a pass owns the compare-exchange pair (i, i | j) with
-    // i = ((p & ~(j-1)) << 1) | (p & (j-1)).  For j <= 32 the 32 pairs of a warp stay inside the warp's own
-    // 64-key block, so those steps only need a warp barrier; a block barrier separates them from the wider steps.
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int p = tid; p < (P >> 1); p += kSelThreads) {
-                const int i = ((p & ~(j - 1)) << 1) | (p & (j - 1)), l = i | j;
-                const uint64_t a = keys[i], c = keys[l];
-                const bool up = (i & k) == 0;
-                if ((a > c) == up) { keys[i] = c; keys[l] = a; }
+    const uint32_t forced_len = s_forced;
+    const bool only_forced = forced_len > uint32_t(budget);      // then the protected sentences alone, in index order
+    uint32_t room = only_forced ? uint32_t(budget) : uint32_t(budget) - forced_len;    // left for the sentences of score `cross`
+    uint32_t cross = 0;
+    if (!only_forced) {
+#pragma unroll 1
+        for (int d = 0; d < 4; ++d) {
+            // bin in which the running total exceeds the room: 8 bins per lane, every warp for itself
+            const int shift = 24 - 8 * d;
+            uint32_t h[8], mine = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) { h[q] = hist[d][lane * 8 + q]; mine += h[q]; }
+            uint32_t inc = mine;
+#pragma unroll
+            for (int s = 1; s < 32; s <<= 1) {
+                const uint32_t x = __shfl_up_sync(0xffffffffu, inc, s);
+                if (lane >= s) inc += x;
             }
-            if (j > 32 || j == 1) __syncthreads(); else __syncwarp();
+            const int src = __ffs(__ballot_sync(0xffffffffu, inc > room)) - 1;     // (the total exceeds the room: some lane's does)
+            uint32_t before = inc - mine, bin = uint32_t(lane) * 8u;
+#pragma unroll
+            for (int q = 0; q < 7; ++q)
+                if (before + h[q] <= room && bin == uint32_t(lane) * 8u + q) { before += h[q]; ++bin; }
+            bin = __shfl_sync(0xffffffffu, bin, src);
+            room -= __shfl_sync(0xffffffffu, before, src);
+            cross |= bin << shift;
+            if (d < 3) {
+                for (int i = i0; i < i1; ++i)
+                    if (lens[i] > 0 && ((keys[i] ^ cross) >> shift) == 0u) atomicAdd(&hist[d + 1][(keys[i] >> (shift - 8)) & 255u], uint32_t(lens[i]));
+                __syncthreads();
+            }
         }
     }
-    // running total of lengths in rank order; each thread owns a contiguous block of ranks
-    const int per = (P + kSelThreads - 1) / kSelThreads;
-    const int r0 = tid * per, r1 = min(r0 + per, S);
-    uint32_t local = 0;
-    for (int r = r0; r < r1; ++r) {
-        const int i = int(keys[r] & 0x7fffffffu);
-        local += uint32_t(so[i + 1] - so[i]);
+    // sentences at the crossing are taken in index order; the first of them that does not fit is the cut one
+    auto at_cross = [&](int i) { return only_forced ? lens[i] < 0 : (lens[i] >= 0 && keys[i] == cross); };
+    auto length = [&](int i) { return uint32_t(lens[i] < 0 ? -lens[i] - 1 : lens[i]); };
+    uint32_t local = 0, all;
+    for (int i = i0; i < i1; ++i) local += at_cross(i) ? length(i) : 0u;
+    uint32_t run = block_excl(local, wsum, all);
+    uint32_t cnt = 0, kept_tokens = 0;
+    for (int i = i0; i < i1; ++i) {
+        bool k;
+        if (at_cross(i)) {
+            const uint32_t before = run;
+            run += length(i);
+            k = run <= room;
+            if (!k && before < room) { s_cut = i; s_slack = int(room - before); }      // one sentence only
+        } else {
+            k = !only_forced && (lens[i] < 0 || keys[i] < cross);
+        }
+        kept_tokens += k ? length(i) : 0u;
+        keys[i] = k ? 1u : 0u;
     }
-    uint32_t tot;
-    uint32_t run = block_excl(local, wsum, tot);
-    uint32_t kept_tokens = 0;
-    for (int r = r0; r < r1; ++r) {
-        const int i = int(keys[r] & 0x7fffffffu);
-        const uint32_t before = run;
-        run += uint32_t(so[i + 1] - so[i]);
-        if (run <= uint32_t(budget)) { flags[i] = 1; kept_tokens = run; }
-        else if (fill.tok_keep && before < uint32_t(budget)) { s_cut = i; s_slack = budget - int(before); }  // one rank only
-    }
-    __syncthreads();
-    if (fill.tok_keep && s_cut >= 0) {
+    uint32_t sum_tokens;
+    block_excl(kept_tokens, wsum, sum_tokens);           // (its barriers also publish the cut)
+    const bool filled = fill.tok_keep && s_cut >= 0;
+    if (filled) {
         const int c = s_cut, slack = s_slack;
         const int cb = so[c], len = so[c + 1] - cb;
         const int b = slab / fill.Hk, h = slab % fill.Hk;
@@ -151,45 +180,37 @@ select_kernel(int max_sent, int P, int budget, int protect_tail, const float* se
             const float i = __ldg(imp + u);
             return red ? __fsub_rn(__fmul_rn(fill.sigma, i), __fmul_rn(w_red, __ldg(red + u))) : i;
         };
+        const bool staged = len <= kFillStage;
+        if (staged) {
+            for (int u = tid; u < len; u += kSelThreads) s_key[u] = key(u);
+            __syncthreads();
+        }
         for (int t = tid; t < len; t += kSelThreads) {   // rank by counting: tokens that come before t in the order
-            const float mine = key(t);
+            const float mine = staged ? s_key[t] : key(t);
             int rank = 0;
-            for (int u = 0; u < len; ++u) {
-                const float other = key(u);
-                rank += (other > mine || (other == mine && u < t)) ? 1 : 0;
+            if (staged) {
+                for (int u = 0; u < len; ++u) { const float other = s_key[u]; rank += (other > mine || (other == mine && u < t)) ? 1 : 0; }
+            } else {
+                for (int u = 0; u < len; ++u) { const float other = key(u); rank += (other > mine || (other == mine && u < t)) ? 1 : 0; }
             }
             tk[t] = rank < slack ? 1 : 0;
         }
-        if (tid == 0) flags[c] = 2;
-        __syncthreads();
     }
-    const bool filled = fill.tok_keep && s_cut >= 0;
     // outputs in sentence-index order
-    const int per_i = (max(S, 1) + kSelThreads - 1) / kSelThreads;
-    const int i0 = tid * per_i, i1 = min(i0 + per_i, S);
-    uint32_t cnt = 0;
-    for (int i = i0; i < i1; ++i) cnt += flags[i] ? 1u : 0u;
+    for (int i = i0; i < i1; ++i) cnt += (keys[i] || (filled && i == s_cut)) ? 1u : 0u;
     uint32_t nk;
     uint32_t pos = block_excl(cnt, wsum, nk);
     for (int i = i0; i < i1; ++i) {
-        kp[i] = flags[i];
-        if (flags[i] && ki) ki[pos] = i;
-        pos += flags[i] ? 1u : 0u;
+        const uint8_t f = keys[i] ? 1 : (filled && i == s_cut ? 2 : 0);
+        kp[i] = f;
+        if (f && ki) ki[pos] = i;
+        pos += f ? 1u : 0u;
     }
     for (int i = S + tid; i < max_sent; i += kSelThreads) kp[i] = 0;
     if (ki) for (int i = int(nk) + tid; i < max_sent; i += kSelThreads) ki[i] = -1;
-    // the largest kept running total is the new length
-    uint32_t m = kept_tokens;
-#pragma unroll
-    for (int d = 16; d; d >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
-    __syncthreads();
-    if ((tid & 31) == 0) wsum[tid >> 5] = m;
-    __syncthreads();
     if (tid == 0) {
-        uint32_t mm = 0;
-        for (int w = 0; w < kSelThreads / 32; ++w) mm = max(mm, wsum[w]);
         if (n_kept) n_kept[slab] = int(nk);
-        if (new_len) new_len[slab] = filled ? budget : int(mm);
+        if (new_len) new_len[slab] = filled ? budget : int(sum_tokens);
     }
 }
 
@@ -204,13 +225,11 @@ static int select_impl(const skipkv_shape* shape, const skipkv_params* params, c
     if (!params || !sent_score || !sent_off || !n_sent || !keep) return SKIPKV_ERR_INVALID_ARG;
     if (params->budget < 0 || params->protect_tail < 0) return SKIPKV_ERR_INVALID_ARG;
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255)) return SKIPKV_ERR_WORKSPACE;
-    int P = 32;
-    while (P < shape->max_sent) P <<= 1;
-    const size_t smem = size_t(P) * 9;
-    if (smem > 200 * 1024) return SKIPKV_ERR_UNSUPPORTED;     // max_sent beyond ~22k sentences per slab
+    const size_t smem = size_t(shape->max_sent) * 8;
+    if (shape->max_sent > 16384) return SKIPKV_ERR_UNSUPPORTED;
     const int slabs = shape->batch * shape->n_kv_heads;
     SKIPKV_CUDA(launch_dependent(select_kernel, dim3(slabs), dim3(kSelThreads), smem, static_cast<cudaStream_t>(stream),
-                                 shape->max_sent, P, params->budget, params->protect_tail, sent_score, sent_off, n_sent, keep,
+                                 shape->max_sent, params->budget, params->protect_tail, sent_score, sent_off, n_sent, keep,
                                  kept_idx, n_kept, new_len, fill, &static_cast<Header*>(ws)->status));
     return SKIPKV_OK;
 }
