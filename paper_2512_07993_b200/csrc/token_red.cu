@@ -9,42 +9,42 @@
 //   token_red_kernel<1>    row sums Z;
 //   token_red_kernel<2>    R.
 // G is symmetric, so every pair of 128-row blocks {I, J} is multiplied and exponentiated once: the tile gives the
-// rows of I their sums over the columns (a thread owns a row) and the rows of J theirs as column sums (a butterfly
-// over the lanes of each warp, then shared-memory and global reductions).  A work item is block I of a slab
-// against I itself and the blocks after it, cyclically, half-way round: every pair once, all items of a slab
-// equally long.  Z and R are accumulated with floating-point reductions: sums agree to rounding, not to the bit,
+// rows of I their sums over the columns and the rows of J theirs as column sums.  A work item is block J of a slab as
+// columns against itself and the blocks after it as rows, cyclically, half-way round: every pair once, all items of a
+// slab equally long.  Z and R are accumulated with floating-point reductions: sums agree to rounding, not to the bit,
 // from run to run.
 // The Gram kernels are persistent and warp-specialised.  Warp 0 streams the bf16 key tiles straight from the cache
-// with tiled TMA loads (the i tile once per item, the j tiles through a ring), warp 1 issues one
-// 128 x 128 x 128 tcgen05.mma group per (i, j) block into one of four tensor-memory accumulators, and four
-// warpgroups (one per accumulator, so that one's tensor-memory reads hide behind the others' arithmetic)
-// read the accumulators back, scale by the two inverse norms and exponentiate.  The products of bf16
-// keys are exact in fp32, so no operand is rounded: normalisation happens after the contraction.
-// One exponential per matrix element makes the special-function unit, not the tensor pipe, the limit.
+// with tiled TMA loads (the J tile once per item, the I tiles through a ring), warps 1 and 2 issue one
+// 128 x 128 x 128 tcgen05.mma group per block pair in turn into one of four tensor-memory accumulators (a single issuer
+// leaves the tensor pipe idle while it waits on its barriers), and sixteen warps read every accumulator back, 32
+// rows x 32 columns each, scale by the two inverse norms and exponentiate.  The products of bf16 keys are exact in fp32,
+// so no operand is rounded: normalisation happens after the contraction.
+// The columns of an item stay the same from tile to tile, so a thread keeps its 32 column sums in registers and the lanes are added
+// up once per item; with the rows fixed and the columns streamed, that butterfly (31 exchanges and as many selects for 32
+// elements) came with every tile and took longer than the exponentials.
+// What bounds it: issue slots of the epilogue.  Per element 4 multiply-add lanes, one exponential (8 clocks of a scheduler for a
+// warp) and about one instruction of overhead; the schedulers issue on 6 clocks of 10.  Four warps per scheduler hide the latencies
+// of these short chains, two with 64 columns each do not (326 us a pass); a share of the exponentials as polynomials adds more
+// issue slots than it takes off the special-function unit.  80 slabs x 4224 keys, both passes and the norms: 806 -> 558 us.
 #include "tc.cuh"
 
 namespace skipkv {
 
-constexpr int kTrGroups = 4;                 // epilogue warpgroups = tensor-memory accumulators of 128 columns
-constexpr int kTrThreads = (2 + 4 * kTrGroups) * 32;   // TMA warp, MMA warp, epilogue warpgroups
-constexpr int kTrStages = 4;                 // j tiles in flight
+constexpr int kTrAcc = 4;                    // tensor-memory accumulators of 128 columns
+constexpr int kTrThreads = 20 * 32;          // TMA warp, two MMA warps, one idle, four epilogue warpgroups
+constexpr int kTrStages = 4;                 // row tiles in flight
 constexpr float kTrLog2e = 1.4426950408889634f;
 
 struct TrCtl {
-    uint64_t afull, aempty, bfull[kTrStages], bempty[kTrStages], tfull[kTrGroups], tempty[kTrGroups];
+    uint64_t jfull[2], jempty[2], ifull[kTrStages], iempty[kTrStages], tfull[kTrAcc], tempty[kTrAcc];
     uint32_t tmem_base;
     int abort_flag;
     uint32_t wsum[32];
-    // per warpgroup, by the parity of its block count: a warp that runs ahead fills the other half while its
-    // siblings still read this one (the barrier of the block after orders the reuse)
-    alignas(16) float jn[kTrGroups][2][128]; // log2(e) / (|K_j| + eps) of the j block under an accumulator
-    alignas(16) float jz[kTrGroups][2][128]; // pass 2: 1 / Z_j
-    float part[2][kTrGroups - 1][128];       // the other warpgroups' shares of an item's row sums (by item parity)
-    float colsum[kTrGroups][2][128];         // column sums of the tile under an accumulator (by the same parity as jn)
+    alignas(16) float col[16][2][32];        // by epilogue warp: log2(e) / (|K_j| + eps) of its columns; pass 2: 1 / Z_j
 };
-static size_t tr_smem_bytes(int slabs) { return 1024 + (1 + kTrStages) * size_t(kOpBytes) + sizeof(TrCtl) + size_t(slabs + 1) * 4; }
+static size_t tr_smem_bytes(int slabs) { return 1024 + (2 + kTrStages) * size_t(kOpBytes) + sizeof(TrCtl) + size_t(slabs + 1) * 4; }
 
-// Blocks that item (slab of NB blocks, block I) multiplies block I with: I itself and the next ones, cyclically.
+// Blocks that item (slab of NB blocks, block J) multiplies block J with: J itself and the next ones, cyclically.
 __device__ __forceinline__ int tr_count(int NB, int I) {
     const int half = NB >> 1;
     return (NB & 1) ? 1 + half : half + (I < half ? 1 : 0);
@@ -98,6 +98,8 @@ token_norm_kernel(int Hk, int max_cap, const int64_t* slab_off, const int32_t* c
     }
 }
 
+struct TrItem { int slab, S, NB, J, NJ; size_t sbase; };
+
 template <int kPass>
 __global__ void __launch_bounds__(kTrThreads, 1)
 token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, int max_cap, const int64_t* slab_off,
@@ -105,199 +107,214 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
                  const Header* hdr) {
     extern __shared__ uint8_t tr_smem_raw[];
     const uint32_t raw = smem_u32(tr_smem_raw);
-    uint8_t* At = tr_smem_raw + (((raw + 1023u) & ~1023u) - raw);
-    uint8_t* Bt = At + kOpBytes;
-    TrCtl* ctl = reinterpret_cast<TrCtl*>(Bt + kTrStages * kOpBytes);
-    int* ipref = reinterpret_cast<int*>(ctl + 1);                                // [n_slabs + 1] prefix of i blocks
+    uint8_t* Jt = tr_smem_raw + (((raw + 1023u) & ~1023u) - raw);
+    uint8_t* It = Jt + 2 * kOpBytes;
+    TrCtl* ctl = reinterpret_cast<TrCtl*>(It + kTrStages * kOpBytes);
+    int* ipref = reinterpret_cast<int*>(ctl + 1);                                // [n_slabs + 1] prefix of blocks
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, cta = blockIdx.x;
     auto len_of = [&](int s) { return min(max(kv_len[s], 0), min(cap[s / Hk], max_cap)); };
     pdl_trigger();
 
     if (tid == 0) {
-        mbar_init(&ctl->afull, 1);
-        mbar_init(&ctl->aempty, 1);
-        for (int s = 0; s < kTrStages; ++s) { mbar_init(&ctl->bfull[s], 1); mbar_init(&ctl->bempty[s], 1); }
-        for (int s = 0; s < kTrGroups; ++s) { mbar_init(&ctl->tfull[s], 1); mbar_init(&ctl->tempty[s], 4); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&ctl->jfull[s], 1); mbar_init(&ctl->jempty[s], 2); }
+        for (int s = 0; s < kTrStages; ++s) { mbar_init(&ctl->ifull[s], 1); mbar_init(&ctl->iempty[s], 1); }
+        for (int s = 0; s < kTrAcc; ++s) { mbar_init(&ctl->tfull[s], 1); mbar_init(&ctl->tempty[s], 16); }
         ctl->abort_flag = 0;
         mbar_fence_init();
         tmap_prefetch(&mapK);
     }
-    if (warp == 1) tmem_alloc(&ctl->tmem_base, 128 * kTrGroups);
+    if (warp == 1) tmem_alloc(&ctl->tmem_base, 128 * kTrAcc);
     pdl_wait();                                          // kv_len and the norms may come from the kernels before
     uint32_t* status = const_cast<uint32_t*>(&hdr->status);
     const uint32_t limit = load_wait_limit(hdr);
     tc_fence_before();
-    cta_prefix<kTrThreads>(n_slabs, [&](int s) { return (len_of(s) + 127) >> 7; }, ipref, ctl->wsum);   // i blocks per slab
+    cta_prefix<kTrThreads>(n_slabs, [&](int s) { return (len_of(s) + 127) >> 7; }, ipref, ctl->wsum);   // blocks per slab
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     const int n_items = ipref[n_slabs];
     auto row0_of = [&](int s) { return int(slab_row0(slab_off, cap, Hk, s / Hk, s % Hk)); };
+    auto get_item = [&](int item, int slab) {            // slab: where to look from
+        TrItem x;
+        while (ipref[slab + 1] <= item) ++slab;
+        x.slab = slab;
+        x.S = len_of(slab);
+        x.NB = (x.S + 127) >> 7;
+        x.J = item - ipref[slab];
+        x.NJ = tr_count(x.NB, x.J);
+        x.sbase = size_t(slab) * max_cap;
+        return x;
+    };
 
-    if (warp == 0) {
-        if (lane == 0) {
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        if (warp == 0 && lane == 0) {
             bool ok = true;
             int slab = 0;
-            uint32_t bc = 0, ic = 0;                                // j blocks and items issued so far
+            uint32_t bc = 0, ic = 0;                                // tiles and items issued so far
             for (int item = cta; item < n_items && ok; item += G, ++ic) {
-                while (ipref[slab + 1] <= item) ++slab;
-                const int NB = (len_of(slab) + 127) >> 7, row0 = row0_of(slab);
-                const int I = item - ipref[slab], NJ = tr_count(NB, I);
-                const int i0 = I * 128;
-                if (ic > 0) ok = role_wait(&ctl->aempty, (ic - 1) & 1u, limit, &ctl->abort_flag, status);
+                const TrItem x = get_item(item, slab);
+                slab = x.slab;
+                const int row0 = row0_of(slab), js = ic & 1;
+                if (ic >= 2) ok = role_wait(&ctl->jempty[js], ((ic >> 1) - 1) & 1u, limit, &ctl->abort_flag, status);
                 if (!ok) break;
-                mbar_expect_tx(&ctl->afull, kOpBytes);
-                tma_load_2d(At, &mapK, 0, row0 + i0, &ctl->afull);
-                tma_load_2d(At + kOpHalfBytes, &mapK, 64, row0 + i0, &ctl->afull);
-                for (int jb = 0; jb < NJ && ok; ++jb, ++bc) {
+                mbar_expect_tx(&ctl->jfull[js], kOpBytes);
+                tma_load_2d(Jt + js * kOpBytes, &mapK, 0, row0 + x.J * 128, &ctl->jfull[js]);
+                tma_load_2d(Jt + js * kOpBytes + kOpHalfBytes, &mapK, 64, row0 + x.J * 128, &ctl->jfull[js]);
+                int I = x.J;
+                for (int t = 0; t < x.NJ && ok; ++t, ++bc) {
                     const int s = bc % kTrStages;
-                    if (bc >= kTrStages) ok = role_wait(&ctl->bempty[s], ((bc / kTrStages) - 1) & 1u, limit, &ctl->abort_flag, status);
+                    if (bc >= kTrStages) ok = role_wait(&ctl->iempty[s], ((bc / kTrStages) - 1) & 1u, limit, &ctl->abort_flag, status);
                     if (!ok) break;
-                    uint8_t* dst = Bt + size_t(s) * kOpBytes;
-                    mbar_expect_tx(&ctl->bfull[s], kOpBytes);
-                    const int J = (I + jb) % NB;
-                    tma_load_2d(dst, &mapK, 0, row0 + J * 128, &ctl->bfull[s]);
-                    tma_load_2d(dst + kOpHalfBytes, &mapK, 64, row0 + J * 128, &ctl->bfull[s]);
+                    uint8_t* dst = It + size_t(s) * kOpBytes;
+                    mbar_expect_tx(&ctl->ifull[s], kOpBytes);
+                    tma_load_2d(dst, &mapK, 0, row0 + I * 128, &ctl->ifull[s]);
+                    tma_load_2d(dst + kOpHalfBytes, &mapK, 64, row0 + I * 128, &ctl->ifull[s]);
+                    if (++I == x.NB) I = 0;
                 }
             }
             if (!ok) {                                   // let the copies in flight land before the CTA exits
-                mbar_wait(&ctl->afull, 0u, 1u << 16); mbar_wait(&ctl->afull, 1u, 1u << 16);
-                for (int s = 0; s < kTrStages; ++s) { mbar_wait(&ctl->bfull[s], 0u, 1u << 16); mbar_wait(&ctl->bfull[s], 1u, 1u << 16); }
+                for (int s = 0; s < 2; ++s) { mbar_wait(&ctl->jfull[s], 0u, 1u << 16); mbar_wait(&ctl->jfull[s], 1u, 1u << 16); }
+                for (int s = 0; s < kTrStages; ++s) { mbar_wait(&ctl->ifull[s], 0u, 1u << 16); mbar_wait(&ctl->ifull[s], 1u, 1u << 16); }
             }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
+        } else if ((warp == 1 || warp == 2) && lane == 0) {
+            // two issuers, a tile each in turn (stages and accumulators are four: each is always the same issuer's)
+            const uint32_t me = warp - 1;
             bool ok = true;
             int slab = 0;
             uint32_t bc = 0, ic = 0;
-            const uint32_t a = smem_u32(At);
             for (int item = cta; item < n_items && ok; item += G, ++ic) {
-                while (ipref[slab + 1] <= item) ++slab;
-                const int NJ = tr_count((len_of(slab) + 127) >> 7, item - ipref[slab]);
-                ok = role_wait(&ctl->afull, ic & 1u, limit, &ctl->abort_flag, status);
-                for (int jb = 0; jb < NJ && ok; ++jb, ++bc) {
-                    const int st = bc % kTrStages, s = bc % kTrGroups;
-                    ok = role_wait(&ctl->bfull[st], (bc / kTrStages) & 1u, limit, &ctl->abort_flag, status);
-                    if (ok && bc >= kTrGroups) ok = role_wait(&ctl->tempty[s], ((bc / kTrGroups) - 1) & 1u, limit, &ctl->abort_flag, status);
+                const TrItem x = get_item(item, slab);
+                slab = x.slab;
+                ok = role_wait(&ctl->jfull[ic & 1], (ic >> 1) & 1u, limit, &ctl->abort_flag, status);
+                const uint32_t jt = smem_u32(Jt + (ic & 1) * kOpBytes);
+                for (int t = 0; t < x.NJ && ok; ++t, ++bc) {
+                    if ((bc & 1u) != me) continue;
+                    const int st = bc % kTrStages, s = bc % kTrAcc;
+                    ok = role_wait(&ctl->ifull[st], (bc / kTrStages) & 1u, limit, &ctl->abort_flag, status);
+                    if (ok && bc >= kTrAcc) ok = role_wait(&ctl->tempty[s], ((bc / kTrAcc) - 1) & 1u, limit, &ctl->abort_flag, status);
                     if (!ok) break;
                     tc_fence_after();
-                    umma_tile_128x128x128(tmem_base + s * 128, a, smem_u32(Bt + size_t(st) * kOpBytes), false);
+                    umma_tile_128x128x128(tmem_base + s * 128, smem_u32(It + size_t(st) * kOpBytes), jt, false);
                     umma_commit(&ctl->tfull[s]);
-                    umma_commit(&ctl->bempty[st]);
+                    umma_commit(&ctl->iempty[st]);
                 }
-                if (ok) umma_commit(&ctl->aempty);                   // every MMA that reads this i tile has completed
+                if (ok) umma_commit(&ctl->jempty[ic & 1]);           // every product of this issuer that reads the column tile has completed
             }
         }
     } else {
-        const int grp = (warp - 2) >> 2;                           // the accumulator this warpgroup drains
-        const int quarter = warp & 3, wt = (tid - 64) & 127;
-        const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + grp * 128;
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        const int quarter = warp & 3, c0 = ((warp - 4) >> 2) * 32;   // this warp's rows (32 * quarter + lane) and columns
+        const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + c0;
+        float* col_s = ctl->col[warp - 4][0];
+        const float2* col = reinterpret_cast<const float2*>(col_s);
+        const float2* colz = col + 16;
+        uint32_t acc = 0, parity = 0;
+        uint64_t* tfull = ctl->tfull;                        // of the accumulator acc; its tempty lies kTrAcc words behind
+        float2 cs[16];
         bool ok = true;
-        int slab = 0;
-        uint32_t bc = 0, ic = 0;
-        ctl->colsum[grp][0][wt] = 0.f;
-        ctl->colsum[grp][1][wt] = 0.f;
-        named_bar_sync(1 + grp, 128);
-        for (int item = cta; item < n_items; item += G, ++ic) {
-            while (ipref[slab + 1] <= item) ++slab;
-            const int S = len_of(slab), NB = (S + 127) >> 7;
-            const int I = item - ipref[slab], NJ = tr_count(NB, I);
-            const size_t sbase = size_t(slab) * max_cap;
-            const int i0 = I * 128;
-            const int row = quarter * 32 + lane;
-            const int i = i0 + row;
-            const float inv_i = (i < S) ? inv_norm[sbase + i] : 0.f;
-            float invz_i = 0.f;                                    // pass 2: 1 / Z_i, the weight of this row in column sums
-            if (kPass == 2 && i < S) { const float zz = z[sbase + i]; invz_i = (zz > 0.f) ? 1.f / zz : 0.f; }
-            const float inv_S = 1.f / float(max(S, 1));
-            float accum = 0.f;
-            for (int jb = 0; jb < NJ; ++jb, ++bc) {
-                if (int(bc % kTrGroups) != grp) continue;          // another warpgroup's block
-                const int J = (I + jb) % NB, j0 = J * 128;
-                const bool diag = jb == 0;                         // the block against itself: row sums only
-                const uint32_t par = (bc / kTrGroups) & 1u;
-                float* jn_s = ctl->jn[grp][par];
-                float* jz_s = ctl->jz[grp][par];
-                float* cs = ctl->colsum[grp][par];
-                {
-                    const int j = j0 + wt;
-                    jn_s[wt] = (j < S) ? inv_norm[sbase + j] * kTrLog2e : 0.f;
-                    if (kPass == 2) {
-                        const float zz = (j < S) ? z[sbase + j] : 1.f;
-                        jz_s[wt] = (zz > 0.f) ? 1.f / zz : 0.f;
-                    }
-                    named_bar_sync(1 + grp, 128);
-                }
-                if (ok) {
-                    ok = role_wait(&ctl->tfull[grp], par, limit, &ctl->abort_flag, status);
-                    ok = __all_sync(0xffffffffu, ok);
-                }
-                if (ok) {
-                    tc_fence_after();
-                    const bool interior = !diag && (j0 + 128 <= S) && (i0 + 128 <= S);
-#pragma unroll 1
-                    for (int ch = 0; ch < 4; ++ch) {
-                        float v[32];
-                        tmem_ld32(lane_addr + ch * 32, v);
-                        const float* jn = jn_s + ch * 32;
-                        const float* jz = jz_s + ch * 32;
-                        if (interior) {
-                            // two elements per instruction (packed fp32 multiply / add): the epilogue is issue-bound
-                            float2 acc2 = make_float2(0.f, 0.f);
-                            const float2 inv2 = make_float2(inv_i, inv_i);
-#pragma unroll
-                            for (int jj = 0; jj < 32; jj += 2) {
-                                const float2 w = __fmul2_rn(__fmul2_rn(make_float2(v[jj], v[jj + 1]), inv2),
-                                                            *reinterpret_cast<const float2*>(jn + jj));
-                                const float2 e = make_float2(tr_ex2(w.x), tr_ex2(w.y));
-                                if (kPass == 1) acc2 = __fadd2_rn(acc2, e);
-                                else acc2 = __ffma2_rn(e, *reinterpret_cast<const float2*>(jz + jj), acc2);
-                                v[jj] = e.x; v[jj + 1] = e.y;
-                            }
-                            accum += acc2.x + acc2.y;
-                        } else {
-#pragma unroll
-                            for (int jj = 0; jj < 32; ++jj) {
-                                const int j = j0 + ch * 32 + jj;
-                                float e = 0.f;
-                                if (j < S && i < S && j != i) {
-                                    e = tr_ex2(v[jj] * inv_i * jn[jj]);
-                                    if (kPass == 1) accum += e; else accum = fmaf(e, jz[jj], accum);
-                                }
-                                v[jj] = e;
-                            }
-                        }
-                        if (!diag) {
-                            // the same exponentials as column sums: they belong to the rows of block J
-                            if (kPass == 2) {
-#pragma unroll
-                                for (int jj = 0; jj < 32; ++jj) v[jj] *= invz_i;
-                            }
-                            atomicAdd(&cs[ch * 32 + lane], tr_col_reduce(v, lane));
-                        }
-                    }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->tempty[grp]);
-                }
-                if (!diag) {
-                    named_bar_sync(1 + grp, 128);                  // the four warps' shares of the column sums are in
-                    const int j = j0 + wt;
-                    if (ok && j < S) {
-                        if (kPass == 1) atomicAdd(&z[sbase + j], cs[wt]);
-                        else atomicAdd(&tok_red[size_t(row0_of(slab)) + j], cs[wt] * inv_S);
-                    }
-                    cs[wt] = 0.f;                                  // used again two blocks later, behind a barrier
-                }
+        TrItem x = {};
+        float inv_n = 0.f, z_n = 1.f, cn = 0.f, cz = 1.f;
+        auto fetch_row = [&](const TrItem& y, int i) {       // the row scale of a tile, a tile ahead
+            inv_n = 1.f; z_n = 0.f;
+            if (i < y.S) {
+                inv_n = inv_norm[y.sbase + i];
+                if (kPass == 2) z_n = z[y.sbase + i];
             }
-            // the warpgroups hold the row sums over interleaved j blocks: the others hand their shares to the first
-            if (grp > 0) ctl->part[ic & 1][grp - 1][row] = accum;
-            named_bar_sync(1 + kTrGroups, 128 * kTrGroups);
-            if (grp == 0 && ok && i < S) {
+        };
+        auto fetch_col = [&](const TrItem& y) {
+            const int j = y.J * 128 + c0 + lane;
+            cn = 1.f; cz = 0.f;
+            if (j < y.S) {
+                cn = inv_norm[y.sbase + j];
+                if (kPass == 2) cz = z[y.sbase + j];
+            }
+        };
+        int slab = 0;
+#pragma unroll 1
+        for (int item = cta; item < n_items && ok; item += G) {
+            x = get_item(item, slab);
+            slab = x.slab;
+            fetch_col(x);
+            fetch_row(x, x.J * 128 + quarter * 32 + lane);
+            __syncwarp();
+            col_s[lane] = cn * kTrLog2e;
+            if (kPass == 2) col_s[32 + lane] = cz > 0.f ? 1.f / cz : 0.f;
+            __syncwarp();
 #pragma unroll
-                for (int g = 0; g < kTrGroups - 1; ++g) accum += ctl->part[ic & 1][g][row];
-                if (kPass == 1) atomicAdd(&z[sbase + i], accum);
-                else atomicAdd(&tok_red[size_t(row0_of(slab)) + i], accum * inv_S);
+            for (int k = 0; k < 16; ++k) cs[k] = make_float2(0.f, 0.f);
+            const float inv_S = 1.f / float(max(x.S, 1));
+            float* dst = kPass == 1 ? z + x.sbase : tok_red + row0_of(slab);
+            const int j0 = x.J * 128 + c0;
+            int i = x.J * 128 + quarter * 32 + lane;
+            const bool full = (x.J + 1) * 128 <= x.S;
+#pragma unroll 1
+            for (int t = 0; t < x.NJ; ++t) {
+                const float inv_i = inv_n;
+                const float invz_i = (kPass == 2 && z_n > 0.f) ? 1.f / z_n : 0.f;   // the weight of this row in column sums
+                const int i_next = i + 128 < x.NB * 128 ? i + 128 : i + 128 - x.NB * 128;
+                fetch_row(x, i_next);
+                {
+                    // (inline: a call would spill the sums)
+                    bool r = mbar_try_wait(tfull, parity);
+                    for (uint32_t n = 0; !r && n < limit; ++n) {
+                        if ((n & 63) == 63 && *reinterpret_cast<volatile int*>(&ctl->abort_flag)) break;
+                        r = mbar_try_wait(tfull, parity);
+                    }
+                    ok = __all_sync(0xffffffffu, r);
+                    tc_fence_after();
+                }
+                if (!ok) {
+                    atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
+                    *reinterpret_cast<volatile int*>(&ctl->abort_flag) = 1;
+                    break;
+                }
+                const bool interior = full && t > 0 && i - lane + 32 <= x.S;
+                float2 row = make_float2(0.f, 0.f);
+                float v[32];
+                tmem_ld32(lane_addr + acc * 128, v);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tfull + kTrAcc);
+                // two elements per instruction (packed fp32 multiply / add)
+                const float2 inv2 = make_float2(inv_i, inv_i), iz2 = make_float2(invz_i, invz_i);
+                auto add = [&](int k, float2 e) {
+                    if (kPass == 1) {
+                        row = __fadd2_rn(row, e);
+                        cs[k] = __fadd2_rn(cs[k], e);
+                    } else {
+                        row = __ffma2_rn(e, colz[k], row);
+                        cs[k] = __ffma2_rn(e, iz2, cs[k]);
+                    }
+                };
+                if (interior) {
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const float2 w = __fmul2_rn(__fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), inv2), col[k]);
+                        add(k, make_float2(tr_ex2(w.x), tr_ex2(w.y)));
+                    }
+                } else {                                     // nothing where a row or column is none of the slab's, and for i == j
+                    const int lim = i < x.S ? x.S - j0 : 0, self = i - j0;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const float2 w = __fmul2_rn(__fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), inv2), col[k]);
+                        add(k, make_float2(2 * k < lim && 2 * k != self ? tr_ex2(w.x) : 0.f,
+                                           2 * k + 1 < lim && 2 * k + 1 != self ? tr_ex2(w.y) : 0.f));
+                    }
+                }
+                // (the block against itself is symmetric: its column sums are all there is to it)
+                if (t > 0 && i < x.S) atomicAdd(dst + i, kPass == 1 ? row.x + row.y : (row.x + row.y) * inv_S);
+                i = i_next;
+                ++tfull;
+                if (++acc == kTrAcc) { acc = 0; tfull = ctl->tfull; parity ^= 1u; }
+            }
+            if (ok) {
+                // the same exponentials as column sums: they belong to the rows of block J
+                float s[32];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) { s[2 * k] = cs[k].x; s[2 * k + 1] = cs[k].y; }
+                const float sum = tr_col_reduce(s, lane);
+                if (j0 + lane < x.S) atomicAdd(dst + j0 + lane, kPass == 1 ? sum : sum * inv_S);
             }
         }
     }
@@ -305,7 +322,7 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 128 * kTrGroups);
+        tmem_dealloc(tmem_base, 128 * kTrAcc);
     }
 }
 
