@@ -825,8 +825,11 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
 }
 
 // ---------------------------------------------------------------------------------------
-// pooling: one warp per sentence, 4 channels per lane; writes the normalised mean key as bf16 hi + lo
+// pooling: a warp takes kPoolRows sentences, 4 channels per lane; writes the normalised mean key as bf16 hi + lo.
+// Bound by DRAM where there are many sentences (512 bytes in and out each): the loads of all the warp's sentences are in flight
+// together, importances of the first 96 tokens included.
 // ---------------------------------------------------------------------------------------
+constexpr int kPoolRows = 4;
 __global__ void __launch_bounds__(256)
 score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len,
                   const int32_t* sent_off, const int32_t* n_sent, float eps, const float* tok_imp_ws,
@@ -836,38 +839,62 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const in
     const int slab = blockIdx.y;
     if (blockIdx.x == 0 && threadIdx.x == 0) lse_cnt[slab] = 0u;            // for the next call's sweeps
     const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int i0 = blockIdx.x * 8 * kPoolRows + (threadIdx.x >> 5);         // and every eighth after it
     const int S = min(n_sent[slab], max_sent);
-    if (i >= S) return;
     const int N = min(max(kv_len[slab], 0), cap[slab / Hk]);
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
-    const int b = max(so[i], 0), e = min(so[i + 1], N);
-    float ti = 0.f;
-    for (int t = b + lane; t < e; t += 32) ti += tok_imp_ws[size_t(slab) * max_cap + t];
-    const float len = float(max(e - b, 1));
-    const size_t o = (size_t(slab) * max_sent + i) * kHeadDim;
-    float4 v = reinterpret_cast<const float4*>(vsum + o)[lane];
-    if (e <= b) v = make_float4(0.f, 0.f, 0.f, 0.f);
-    v.x /= len; v.y /= len; v.z /= len; v.w /= len;
-    float nn = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    const float* imp = tok_imp_ws + size_t(slab) * max_cap;
+    int b[kPoolRows], e[kPoolRows];
+    float4 v[kPoolRows];
 #pragma unroll
-    for (int d = 16; d; d >>= 1) {
-        nn += __shfl_xor_sync(0xffffffffu, nn, d);
-        ti += __shfl_xor_sync(0xffffffffu, ti, d);
+    for (int q = 0; q < kPoolRows; ++q) {
+        const int i = i0 + q * 8;
+        b[q] = e[q] = 0;
+        v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < S) {
+            b[q] = max(so[i], 0);
+            e[q] = min(so[i + 1], N);
+            v[q] = reinterpret_cast<const float4*>(vsum + (size_t(slab) * max_sent + i) * kHeadDim)[lane];
+        }
     }
-    const float inv = 1.f / (sqrtf(nn) + eps);
-    const float x[4] = {v.x * inv, v.y * inv, v.z * inv, v.w * inv};
-    uint32_t hi[4], lo[4];                                   // bf16 bit patterns
+    float first[kPoolRows][3];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(x[c]);
-        const __nv_bfloat16 r = __float2bfloat16_rn(x[c] - __bfloat162float(h));
-        hi[c] = __bfloat16_as_ushort(h);
-        lo[c] = __bfloat16_as_ushort(r);
+    for (int q = 0; q < kPoolRows; ++q)
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            const int t = b[q] + p * 32 + lane;
+            first[q][p] = t < e[q] ? imp[t] : 0.f;
+        }
+#pragma unroll
+    for (int q = 0; q < kPoolRows; ++q) {
+        const int i = i0 + q * 8;
+        if (i >= S) break;
+        float ti = first[q][0] + first[q][1] + first[q][2];
+        for (int t = b[q] + 96 + lane; t < e[q]; t += 32) ti += imp[t];
+        const float len = float(max(e[q] - b[q], 1));
+        if (e[q] <= b[q]) v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float m[4] = {v[q].x / len, v[q].y / len, v[q].z / len, v[q].w / len};
+        float nn = m[0] * m[0] + m[1] * m[1] + m[2] * m[2] + m[3] * m[3];
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            nn += __shfl_xor_sync(0xffffffffu, nn, d);
+            ti += __shfl_xor_sync(0xffffffffu, ti, d);
+        }
+        const float inv = 1.f / (sqrtf(nn) + eps);
+        uint32_t hi[4], lo[4];                               // bf16 bit patterns
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float x = m[c] * inv;
+            const __nv_bfloat16 h = __float2bfloat16_rn(x);
+            const __nv_bfloat16 r = __float2bfloat16_rn(x - __bfloat162float(h));
+            hi[c] = __bfloat16_as_ushort(h);
+            lo[c] = __bfloat16_as_ushort(r);
+        }
+        const size_t o = (size_t(slab) * max_sent + i) * kHeadDim;
+        reinterpret_cast<uint2*>(vbar_hi + o)[lane] = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
+        reinterpret_cast<uint2*>(vbar_lo + o)[lane] = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
+        if (lane == 0) sent_imp[size_t(slab) * max_sent + i] = (e[q] > b[q]) ? ti / len : 0.f;
     }
-    reinterpret_cast<uint2*>(vbar_hi + o)[lane] = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
-    reinterpret_cast<uint2*>(vbar_lo + o)[lane] = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
-    if (lane == 0) sent_imp[size_t(slab) * max_sent + i] = (e > b) ? ti / len : 0.f;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -886,7 +913,7 @@ struct GramCtl {
                                                    // fills the other half while its siblings still read this one
     float part[2][kGramGroups - 1][2][128];   // by item parity: the other groups' (sum, max) shares of a row
 };
-constexpr int kGramThreads = (2 + 4 * kGramGroups) * 32;
+constexpr int kGramThreads = (3 + 4 * kGramGroups) * 32;   // TMA warp, MMA warp, epilogue warpgroups, the other MMA warp
 static size_t gram_smem_bytes(int slabs) { return 1024 + 6 * size_t(kOpBytes) + sizeof(GramCtl) + size_t(slabs + 1) * 4; }
 
 // Optional source of the sentence penalty: the lookup table T of one value per generation-space sentence,
@@ -917,7 +944,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
 
     if (tid == 0) {
         mbar_init(&ctl->afull, 1);
-        mbar_init(&ctl->aempty, 1);
+        mbar_init(&ctl->aempty, 2);
         for (int s = 0; s < 2; ++s) {
             mbar_init(&ctl->bfull[s], 1);
             mbar_init(&ctl->bempty[s], 1);
@@ -974,8 +1001,10 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 for (int s = 0; s < 2; ++s) { mbar_wait(&ctl->bfull[s], 0u, 1u << 16); mbar_wait(&ctl->bfull[s], 1u, 1u << 16); }
             }
         }
-    } else if (warp == 1) {
+    } else if (warp == 1 || warp == kGramThreads / 32 - 1) {
         if (lane == 0) {
+            // a j block each in turn: a stage and an accumulator are always the same issuer's
+            const uint32_t me = warp == 1 ? 0u : 1u;
             bool ok = true;
             int slab = 0;
             uint32_t bc = 0, ic = 0;
@@ -985,6 +1014,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 const int NJ = (sent_of(slab) + 127) >> 7;
                 ok = role_wait(&ctl->afull, ic & 1u, limit, &ctl->abort_flag, status);
                 for (int jb = 0; jb < NJ && ok; ++jb, ++bc) {
+                    if ((bc & 1u) != me) continue;
                     const int s = bc & 1, acc = bc % kGramGroups;
                     ok = role_wait(&ctl->bfull[s], (bc >> 1) & 1u, limit, &ctl->abort_flag, status);
                     if (ok && bc >= kGramGroups) ok = role_wait(&ctl->tempty[acc], ((bc / kGramGroups) - 1) & 1u, limit, &ctl->abort_flag, status);
@@ -998,7 +1028,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                     umma_commit(&ctl->tfull[acc]);
                     umma_commit(&ctl->bempty[s]);
                 }
-                if (ok) umma_commit(&ctl->aempty);                   // every MMA that reads this i block has completed
+                if (ok) umma_commit(&ctl->aempty);                   // every MMA of this issuer that reads this i block has completed
             }
         }
     } else {
@@ -1351,7 +1381,7 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         return SKIPKV_OK;
     }
     {
-        dim3 pgrid((shape->max_sent + 7) / 8, L.slabs);
+        dim3 pgrid((shape->max_sent + 8 * kPoolRows - 1) / (8 * kPoolRows), L.slabs);
         SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, shape->max_cap,
                                      shape->cap, kv_len, sent_off, n_sent, params->eps, sc_tok, vsum, sent_imp, vbar_hi,
                                      vbar_lo));
