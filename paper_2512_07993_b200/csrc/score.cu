@@ -901,11 +901,14 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const in
 // Gram passes on the tensor cores.  Work item = 128 sentences i of one slab against all j in blocks of 128;
 // persistent CTAs take the items round-robin, so barriers, tensor memory and descriptors are set up once and
 // the j-block ring keeps streaming from one item into the next.
+// Bound by shared memory where there are many sentences: the three products of a block pair stream 192 KB of operands in 1536 clocks,
+// the port's 128 bytes per clock, and the next block's 64 KB have to be written through the same port; a pair takes 1940 clocks
+// (2640 with one issuer that waits between its blocks).  128 slabs x 2K sentences: 351 + 396 -> 265 + 275 us.
 // ---------------------------------------------------------------------------------------
 constexpr int kGramGroups = 4;          // epilogue warpgroups = tensor-memory accumulators: one group's tensor-memory
                                        // reads hide behind the arithmetic of the others
 struct GramCtl {
-    uint64_t afull, aempty, bfull[2], bempty[2], tfull[kGramGroups], tempty[kGramGroups];
+    uint64_t afull, aempty, bfull[2][2], bempty[2][2], turn[2], tfull[kGramGroups], tempty[kGramGroups];
     uint32_t tmem_base;
     int abort_flag;
     uint32_t wsum[32];
@@ -946,8 +949,8 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
         mbar_init(&ctl->afull, 1);
         mbar_init(&ctl->aempty, 2);
         for (int s = 0; s < 2; ++s) {
-            mbar_init(&ctl->bfull[s], 1);
-            mbar_init(&ctl->bempty[s], 1);
+            for (int part = 0; part < 2; ++part) { mbar_init(&ctl->bfull[s][part], 1); mbar_init(&ctl->bempty[s][part], 1); }
+            mbar_init(&ctl->turn[s], 1);
         }
         for (int s = 0; s < kGramGroups; ++s) {
             mbar_init(&ctl->tfull[s], 1);
@@ -986,24 +989,28 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 tma_load_2d(At + kOpBytes + kOpHalfBytes, &mapLo, 64, rowbase + i0, &ctl->afull);
                 for (int jb = 0; jb < NJ && ok; ++jb, ++bc) {
                     const int s = bc & 1;
-                    if (bc >= 2) ok = role_wait(&ctl->bempty[s], ((bc >> 1) - 1) & 1u, limit, &ctl->abort_flag, status);
-                    if (!ok) break;
-                    uint8_t* dst = Bt + size_t(s) * 2 * kOpBytes;
-                    mbar_expect_tx(&ctl->bfull[s], 2 * kOpBytes);
-                    tma_load_2d(dst, &mapHi, 0, rowbase + jb * 128, &ctl->bfull[s]);
-                    tma_load_2d(dst + kOpHalfBytes, &mapHi, 64, rowbase + jb * 128, &ctl->bfull[s]);
-                    tma_load_2d(dst + kOpBytes, &mapLo, 0, rowbase + jb * 128, &ctl->bfull[s]);
-                    tma_load_2d(dst + kOpBytes + kOpHalfBytes, &mapLo, 64, rowbase + jb * 128, &ctl->bfull[s]);
+                    for (int part = 1; part >= 0 && ok; --part) {         // low, high: the order in which they are given back
+                        if (bc >= 2) ok = role_wait(&ctl->bempty[s][part], ((bc >> 1) - 1) & 1u, limit, &ctl->abort_flag, status);
+                        if (!ok) break;
+                        uint8_t* dst = Bt + size_t(2 * s + part) * kOpBytes;
+                        const CUtensorMap* map = part ? &mapLo : &mapHi;
+                        mbar_expect_tx(&ctl->bfull[s][part], kOpBytes);
+                        tma_load_2d(dst, map, 0, rowbase + jb * 128, &ctl->bfull[s][part]);
+                        tma_load_2d(dst + kOpHalfBytes, map, 64, rowbase + jb * 128, &ctl->bfull[s][part]);
+                    }
                 }
             }
             if (!ok) {
                 mbar_wait(&ctl->afull, 0u, 1u << 16); mbar_wait(&ctl->afull, 1u, 1u << 16);
-                for (int s = 0; s < 2; ++s) { mbar_wait(&ctl->bfull[s], 0u, 1u << 16); mbar_wait(&ctl->bfull[s], 1u, 1u << 16); }
+                for (int s = 0; s < 2; ++s)
+                    for (int part = 0; part < 2; ++part) { mbar_wait(&ctl->bfull[s][part], 0u, 1u << 16); mbar_wait(&ctl->bfull[s][part], 1u, 1u << 16); }
             }
         }
     } else if (warp == 1 || warp == kGramThreads / 32 - 1) {
         if (lane == 0) {
-            // a j block each in turn: a stage and an accumulator are always the same issuer's
+            // A j block each in turn: a stage and an accumulator are always the same issuer's, and one waits for its operands while the
+            // other's products run.  The turn is handed over a little before a block's last instructions are issued; left to themselves, the
+            // two blocks share the tensor pipe, end together, and then wait for their stages to be filled again together.
             const uint32_t me = warp == 1 ? 0u : 1u;
             bool ok = true;
             int slab = 0;
@@ -1016,17 +1023,21 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 for (int jb = 0; jb < NJ && ok; ++jb, ++bc) {
                     if ((bc & 1u) != me) continue;
                     const int s = bc & 1, acc = bc % kGramGroups;
-                    ok = role_wait(&ctl->bfull[s], (bc >> 1) & 1u, limit, &ctl->abort_flag, status);
+                    ok = role_wait(&ctl->bfull[s][1], (bc >> 1) & 1u, limit, &ctl->abort_flag, status) &&
+                         role_wait(&ctl->bfull[s][0], (bc >> 1) & 1u, limit, &ctl->abort_flag, status);
                     if (ok && bc >= kGramGroups) ok = role_wait(&ctl->tempty[acc], ((bc / kGramGroups) - 1) & 1u, limit, &ctl->abort_flag, status);
+                    if (ok && bc > 0) ok = role_wait(&ctl->turn[me], ((bc >> 1) - (me ? 0u : 1u)) & 1u, limit, &ctl->abort_flag, status);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t b_hi = smem_u32(Bt + size_t(s) * 2 * kOpBytes), b_lo = b_hi + kOpBytes;
                     const uint32_t d = tmem_base + acc * 128;
-                    umma_tile_128x128x128(d, a_hi, b_hi, false);
-                    umma_tile_128x128x128(d, a_hi, b_lo, true);
+                    umma_tile_128x128x128(d, a_hi, b_lo, false);
+                    umma_commit(&ctl->bempty[s][1]);
+                    umma_tile_128x128x128(d, a_hi, b_hi, true);
+                    mbar_arrive(&ctl->turn[me ^ 1u]);
                     umma_tile_128x128x128(d, a_lo, b_hi, true);
                     umma_commit(&ctl->tfull[acc]);
-                    umma_commit(&ctl->bempty[s]);
+                    umma_commit(&ctl->bempty[s][0]);
                 }
                 if (ok) umma_commit(&ctl->aempty);                   // every MMA of this issuer that reads this i block has completed
             }
