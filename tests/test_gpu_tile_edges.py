@@ -69,3 +69,14 @@ def test_score_sentence_counts_around_a_tile(sentences):
     B, L, D = layer([5 * n for n in sentences], sent_lo=5, sent_hi=5, dup_rate=0.3, seed=500 + sentences[0])
     assert int(L["n_sent"].max()) == max(sentences)
     check_scores(B, L, D)
+
+
+@pytest.mark.parametrize("group,window", [(1, 1), (1, 16), (1, 17), (1, 127), (1, 512), (2, 33), (2, 128), (3, 32), (3, 128), (4, 31),
+                                          (4, 96), (5, 17), (5, 64), (6, 16), (6, 64), (7, 48), (7, 72), (8, 15), (8, 49)])
+def test_score_query_blocks(group, window):
+    """Blocks of 32 and of 16 window positions, one to sixteen of them, one and several per row operand, whole and partly
+    filled; slabs of less than a tile, of whole tiles and of many tiles in one CTA's share."""
+    for ctx in ([100, 128, 129, 520], [4100, 9000, 257, 128]):
+        B, L, D = layer([max(c, window) for c in ctx], n_q_heads=2 * group, n_kv_heads=2, window=window, sent_lo=8, sent_hi=40,
+                        dup_rate=0.3, seed=700 + 10 * group + window % 10)
+        check_scores(B, L, D)
