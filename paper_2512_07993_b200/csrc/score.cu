@@ -903,7 +903,8 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const in
 // the j-block ring keeps streaming from one item into the next.
 // Bound by shared memory where there are many sentences: the three products of a block pair stream 192 KB of operands in 1536 clocks,
 // the port's 128 bytes per clock, and the next block's 64 KB have to be written through the same port; a pair takes 1940 clocks
-// (2640 with one issuer that waits between its blocks).  128 slabs x 2K sentences: 351 + 396 -> 265 + 275 us.
+// (2640 with one issuer that waits between its blocks).  128 slabs x 2K sentences: 351 + 396 -> 312 + 350 us
+// back to back, where the clock falls under the power limit.
 // ---------------------------------------------------------------------------------------
 constexpr int kGramGroups = 4;          // epilogue warpgroups = tensor-memory accumulators: one group's tensor-memory
                                        // reads hide behind the arithmetic of the others
@@ -1158,15 +1159,16 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
 // them once, and takes the row sums, the penalties, the redundancy and the scores from the one accumulator, whose
 // exponentials stay in registers between the two uses.  Nothing but latency bounds these slabs: the three kernels this
 // replaces (pooling and two Gram passes, for any number of sentences) took 22 us for 8 slabs and 28 us for 80, each
-// waiting for the one before it to drain.
+// waiting for the one before it to drain.  16 warps, so that all rows' loads are one batch: 22.3 -> 18.2 us a launch (with its
+// wait for the sweep) against 8 warps with two.
 // ---------------------------------------------------------------------------------------
-constexpr int kSmallThreads = 256;
+constexpr int kSmallThreads = 512;
 constexpr int kSmallSent = 128;
-constexpr int kSmallBatch = 8;          // sentences of a warp whose loads are in flight together
+constexpr int kSmallBatch = 8;          // sentences of a warp: their loads are in flight together
 struct SmallCtl {
     uint64_t done;
     uint32_t tmem_base;
-    alignas(16) float imp[kSmallSent], sum[2][kSmallSent], mx[2][kSmallSent], invz[kSmallSent];
+    alignas(16) float imp[kSmallSent], sum[4][kSmallSent], mx[4][kSmallSent], red[4][kSmallSent], invz[kSmallSent];
 };
 constexpr size_t kSmallSmem = 1024 + 2 * size_t(kOpBytes) + sizeof(SmallCtl);
 
@@ -1189,10 +1191,9 @@ score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const i
     const int S = min(max(n_sent[slab], 0), max_sent), N = min(max(kv_len[slab], 0), cap[slab / Hk]);
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
     const float* ti_p = tok_imp_ws + size_t(slab) * max_cap;
-    // ---- pooling: 16 rows per warp, kSmallBatch at a time; rows past the last sentence are zeros
-#pragma unroll 1
-    for (int b = 0; b < 16; b += kSmallBatch) {
-        const int i0 = warp * 16 + b, cnt = min(kSmallBatch, S - i0);
+    // ---- pooling: kSmallBatch rows per warp; rows past the last sentence are zeros
+    {
+        const int i0 = warp * kSmallBatch, cnt = min(kSmallBatch, S - i0);
         const int off = lane <= cnt ? so[i0 + lane] : 0;
         float4 v[kSmallBatch];
 #pragma unroll
@@ -1260,59 +1261,54 @@ score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const i
     const bool ok = mbar_wait(&ctl->done, 0u, load_wait_limit(hdr));
     if (!ok && lane == 0) atomicOr(const_cast<uint32_t*>(&hdr->status), SKIPKV_STATUS_COPY_TIMEOUT);
     tc_fence_after();
-    // ---- thread: row i, 64 columns; two warps share a row
-    const int half = warp >> 2, i = (warp & 3) * 32 + lane;
-    const uint32_t taddr = tmem_base + (uint32_t((warp & 3) * 32) << 16) + half * 64;
-    float e[64];
+    // ---- thread: row i, 32 columns; four warps share a row
+    const int part = warp >> 2, i = (warp & 3) * 32 + lane, c0 = part * 32;
+    float e[32];
     float sum = 0.f, mx = -INFINITY;
-#pragma unroll
-    for (int ch = 0; ch < 2; ++ch) {
-        float v[32];
-        if (half * 64 + ch * 32 < S) {                   // (the same for the whole warp)
-            tmem_ld32(taddr + ch * 32, v);
-        } else {
-#pragma unroll
-            for (int jj = 0; jj < 32; ++jj) v[jj] = 0.f;
-        }
+    if (c0 < S) {                                        // (the same for the whole warp)
+        tmem_ld32(tmem_base + (uint32_t((warp & 3) * 32) << 16) + c0, e);
 #pragma unroll
         for (int jj = 0; jj < 32; ++jj) {
-            const int j = half * 64 + ch * 32 + jj;
+            const int j = c0 + jj;
             const bool on = j < S && j != i;
-            e[ch * 32 + jj] = on ? ex2f(v[jj] * kLog2e) : 0.f;
-            sum += e[ch * 32 + jj];
-            if (on && j > i) mx = fmaxf(mx, v[jj]);
+            if (on && j > i) mx = fmaxf(mx, e[jj]);
+            e[jj] = on ? ex2f(e[jj] * kLog2e) : 0.f;
+            sum += e[jj];
         }
+    } else {
+#pragma unroll
+        for (int jj = 0; jj < 32; ++jj) e[jj] = 0.f;
     }
-    ctl->sum[half][i] = sum;
-    ctl->mx[half][i] = mx;
+    ctl->sum[part][i] = sum;
+    ctl->mx[part][i] = mx;
     tc_fence_before();
     __syncthreads();
-    if (half == 0) {
-        const float z = ctl->sum[0][i] + ctl->sum[1][i];
+    if (part == 0) {
+        const float z = (sum + ctl->sum[1][i]) + (ctl->sum[2][i] + ctl->sum[3][i]);
         ctl->invz[i] = (i < S && z > 0.f) ? 1.f / z : 0.f;
     }
     __syncthreads();
     float red = 0.f;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const float4 iz = *reinterpret_cast<const float4*>(&ctl->invz[half * 64 + q * 4]);
+    for (int q = 0; q < 8; ++q) {
+        const float4 iz = *reinterpret_cast<const float4*>(&ctl->invz[c0 + q * 4]);
         red = fmaf(e[q * 4], iz.x, red);
         red = fmaf(e[q * 4 + 1], iz.y, red);
         red = fmaf(e[q * 4 + 2], iz.z, red);
         red = fmaf(e[q * 4 + 3], iz.w, red);
     }
-    if (half == 1) ctl->sum[1][i] = red;
+    ctl->red[part][i] = red;
     __syncthreads();
-    if (half == 0 && i < S && ok) {
+    if (part == 0 && i < S && ok) {
         const size_t o = size_t(slab) * max_sent + i;
-        float lam = fmaxf(ctl->mx[0][i], ctl->mx[1][i]);
+        float lam = fmaxf(fmaxf(mx, ctl->mx[1][i]), fmaxf(ctl->mx[2][i], ctl->mx[3][i]));
         if (ext.table) {                                 // penalty from the generation-space table through Phi
             const int g = ext.sent_id[o];
             lam = (g >= 0 && g < ext.table_len) ? ext.table[size_t(slab / Hk) * ext.table_len + g] : 0.f;
         } else {
             lam = (lam > tau) ? lam : 0.f;
         }
-        red = (red + ctl->sum[1][i]) / float(S);
+        red = ((red + ctl->red[1][i]) + (ctl->red[2][i] + ctl->red[3][i])) / float(S);
         sent_lam[o] = lam;
         sent_red[o] = red;
         sent_score[o] = sigma * ctl->imp[i] - (1.f - sigma) * red - lam;

@@ -25,7 +25,8 @@
 // What bounds it: issue slots of the epilogue.  Per element 4 multiply-add lanes, one exponential (8 clocks of a scheduler for a
 // warp) and about one instruction of overhead; the schedulers issue on 6 clocks of 10.  Four warps per scheduler hide the latencies
 // of these short chains, two with 64 columns each do not (326 us a pass); a share of the exponentials as polynomials adds more
-// issue slots than it takes off the special-function unit.  80 slabs x 4224 keys, both passes and the norms: 806 -> 558 us.
+// issue slots than it takes off the special-function unit.  80 slabs x 4224 keys, both passes and the norms: 804 -> 617 us
+// back to back (558 in a short burst: the clock falls under the power limit).
 #include "tc.cuh"
 
 namespace skipkv {
