@@ -35,7 +35,7 @@ from paper_2512_07993_b200 import workloads as W  # noqa: E402
 
 METRIC = "SkipKV compress+compact µs/layer and decode-attn HBM GB/s, 32K ctx, batch 10"
 UNIT = "us/layer (score+select+compact); decode-attn GB/s in decode_attn_gbs"
-LAUNCHES_PER_STEP = {"score": 5, "select": 1, "compact": 2, "decode_attn": 1, "decode_attn_full_ctx": 1}   # kernels per layer
+LAUNCHES_PER_STEP = {"score": 4, "select": 1, "compact": 2, "decode_attn": 1, "decode_attn_full_ctx": 1}   # kernels per layer
 
 
 def measured_peaks():
