@@ -40,7 +40,9 @@ struct WsLayout {
     size_t sc_cnt;         // uint32 [slabs]              tiles whose log-sum-exp records are written (zero between calls)
     size_t sc_part;        // float2 [max_ctas + slabs][sc_ra * 128]  (reference, sum) of a CTA's part of a slab
     size_t sc_tokimp;      // float  [slabs][max_cap]
-    size_t sc_vsum;        // float  [slabs][max_sent][128]  per-sentence sums of key rows
+    size_t sc_vsum;        // float  [slabs][max_sent][128]  per-sentence sums of key rows; then partial sums of the Gram passes,
+                           //        [slabs] x sc_vsum_slab floats, of which [4 * blocks][max_sent] are used
+    size_t sc_vsum_slab;
     size_t sc_vbar_hi;     // bf16   [slabs][max_sent][128]  normalised mean key, high part
     size_t sc_vbar_lo;     // bf16   [slabs][max_sent][128]  and the rounding remainder
     size_t sc_z;           // float  [slabs][max_sent]
@@ -92,7 +94,10 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     L.dec_part = take((size_t(L.dec_max_ctas) + slabs) * L.group * kDecPartStride * 4);
     L.sc_part = take((size_t(L.dec_max_ctas) + slabs) * size_t(L.sc_ra) * 128 * 8);
     L.sc_tokimp = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);
-    L.sc_vsum = take(slabs * ms * kHeadDim * 4);
+    // 128 channels per sentence, then four partial sums per sentence and block of 128 sentences: more from 4096 sentences on
+    const size_t sums = (ms + 127) / 128 * 4;
+    L.sc_vsum_slab = ms * (sums > size_t(kHeadDim) ? sums : size_t(kHeadDim));
+    L.sc_vsum = take(slabs * L.sc_vsum_slab * 4);
     L.sc_vbar_hi = take(slabs * ms * kHeadDim * 2);
     L.sc_vbar_lo = take(slabs * ms * kHeadDim * 2);
     L.sc_z = take(slabs * ms * 4);

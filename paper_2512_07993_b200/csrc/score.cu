@@ -833,7 +833,7 @@ constexpr int kPoolRows = 4;
 __global__ void __launch_bounds__(256)
 score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len,
                   const int32_t* sent_off, const int32_t* n_sent, float eps, const float* tok_imp_ws,
-                  const float* vsum, float* sent_imp, __nv_bfloat16* vbar_hi, __nv_bfloat16* vbar_lo) {
+                  const float* vsum, float* sent_imp, __nv_bfloat16* vbar_hi, __nv_bfloat16* vbar_lo, float* sent_lam) {
     pdl_trigger();
     pdl_wait();
     const int slab = blockIdx.y;
@@ -893,32 +893,86 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const in
         const size_t o = (size_t(slab) * max_sent + i) * kHeadDim;
         reinterpret_cast<uint2*>(vbar_hi + o)[lane] = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
         reinterpret_cast<uint2*>(vbar_lo + o)[lane] = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
-        if (lane == 0) sent_imp[size_t(slab) * max_sent + i] = (e[q] > b[q]) ? ti / len : 0.f;
+        if (lane == 0) {
+            const size_t s = size_t(slab) * max_sent + i;
+            sent_imp[s] = (e[q] > b[q]) ? ti / len : 0.f;
+            sent_lam[s] = 0.f;                               // (as bits: below every ordered penalty)
+        }
     }
 }
 
 // ---------------------------------------------------------------------------------------
-// Gram passes on the tensor cores.  Work item = 128 sentences i of one slab against all j in blocks of 128;
-// persistent CTAs take the items round-robin, so barriers, tensor memory and descriptors are set up once and
-// the j-block ring keeps streaming from one item into the next.
-// Bound by shared memory where there are many sentences: the three products of a block pair stream 192 KB of operands in 1536 clocks,
-// the port's 128 bytes per clock, and the next block's 64 KB have to be written through the same port; a pair takes 1940 clocks
-// (2640 with one issuer that waits between its blocks).  128 slabs x 2K sentences: 351 + 396 -> 312 + 350 us
-// back to back, where the clock falls under the power limit.
+// Gram passes on the tensor cores.  G is symmetric: every pair of 128-sentence blocks I <= J of a slab is multiplied and
+// exponentiated once, and gives the rows of I their sums over the columns and the columns of J theirs over the rows (the
+// diagonal pair: column sums only).  Work is the list of pairs, J by J, over all slabs, cut into equal contiguous ranges.
+// Every sentence has four partial sums per block of its slab, each written by one warp: rows by the pair (the four column groups), columns by a
+// range's part of J (the four row groups; the blocks of the part's other pairs get zeros).  The CTA that completes a slab adds them up in
+// order, so the results do not depend on who was first.  They lie where the sums of the keys were, which the pooling was the last to read.
+// The penalty is the maximum over later sentences; only those beyond tau are reported, which are few (pass 1, an integer maximum).
+// Roles as in the token-level kernel: a TMA warp, two MMA warps that take the pairs in turn, sixteen epilogue warps with 32
+// rows x 32 columns of every accumulator each, column sums in registers for as long as J stays.
+// Three shared-memory slots hold a block's high and low parts.  One is J's, the other two take the I blocks in turn; the next J takes
+// the slot that is free next and the old J's goes to the end of the queue, so a change of J costs no drain.
+// Bound by shared memory where there are many sentences: the three products of a pair stream 192 KB of operands in 1536 clocks,
+// the port's 128 bytes per clock, and the next block's 64 KB are written through the same port; under a sustained load the clock falls with the
+// power limit, and half the products is the larger gain.  128 slabs x 2K sentences, the whole scoring call: 2319 -> 2190 us against all pairs twice.
 // ---------------------------------------------------------------------------------------
-constexpr int kGramGroups = 4;          // epilogue warpgroups = tensor-memory accumulators: one group's tensor-memory
-                                       // reads hide behind the arithmetic of the others
+constexpr int kGramAcc = 4;
 struct GramCtl {
-    uint64_t afull, aempty, bfull[2][2], bempty[2][2], turn[2], tfull[kGramGroups], tempty[kGramGroups];
+    uint64_t full[3][2], empty[3][2];        // slot, part: loaded (every use) / given back by the pair that used it as I
+    uint64_t ddone[3];                       // the diagonal pair of the J block in this slot is complete
+    uint64_t turn[2];
+    uint64_t tfull[kGramAcc], tempty[kGramAcc];
     uint32_t tmem_base;
-    int abort_flag;
+    int abort_flag, last;
     uint32_t wsum[32];
-    alignas(16) float invz[kGramGroups][2][128];   // by the parity of the group's block count: a warp that runs ahead
-                                                   // fills the other half while its siblings still read this one
-    float part[2][kGramGroups - 1][2][128];   // by item parity: the other groups' (sum, max) shares of a row
+    alignas(16) float colz[16][32];          // pass 2, by epilogue warp: 1 / Z_j of its columns
 };
-constexpr int kGramThreads = (3 + 4 * kGramGroups) * 32;   // TMA warp, MMA warp, epilogue warpgroups, the other MMA warp
+constexpr int kGramThreads = 20 * 32;        // TMA warp, two MMA warps, one idle, four epilogue warpgroups
 static size_t gram_smem_bytes(int slabs) { return 1024 + 6 * size_t(kOpBytes) + sizeof(GramCtl) + size_t(slabs + 1) * 4; }
+
+// Floats as integers in the same order (0 lies below all of them).
+__device__ __forceinline__ uint32_t ordered_bits(float f) {
+    const uint32_t u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float from_ordered_bits(uint32_t u) { return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u); }
+
+// A CTA's walk over its pairs, and which slot a block is in.  Every role steps through the same sequence.
+struct GramWalk {
+    int slab, S, J, t;                       // pair t of block column J: 0 is the diagonal, t > 0 multiplies block t - 1
+    int left;                                // pairs of the range not yet walked, this one included
+    int jslot, q0, q1, q2;                   // slot of J, and the others in the order in which they are taken
+    bool have_j;
+    __device__ __forceinline__ void start(const int* ipref, int first, int count) {
+        left = count; slab = 0; have_j = false; q0 = 0; q1 = 1; q2 = 2; jslot = 0;
+        if (count <= 0) return;
+        while (ipref[slab + 1] <= first) ++slab;
+        const int p = first - ipref[slab];
+        J = int((sqrtf(8.f * float(p) + 1.f) - 1.f) * 0.5f);
+        while (J > 0 && J * (J + 1) / 2 > p) --J;
+        while ((J + 1) * (J + 2) / 2 <= p) ++J;
+        t = p - J * (J + 1) / 2;
+    }
+    __device__ __forceinline__ int pop() { const int s = q0; q0 = q1; q1 = q2; return s; }
+    __device__ __forceinline__ void take_j() {           // J changes (or the range begins)
+        if (have_j) q2 = jslot;                          // the old one's slot goes to the end of the queue
+        jslot = pop();
+        have_j = true;
+    }
+    __device__ __forceinline__ int take_i() { const int s = pop(); q1 = s; return s; }
+    // on to the next pair: true if it has another J
+    __device__ __forceinline__ bool next(const int* ipref) {
+        --left;
+        if (t++ < J) return false;
+        t = 0; ++J;
+        if (left > 0 && ipref[slab] + J * (J + 1) / 2 >= ipref[slab + 1]) {
+            J = 0;
+            do ++slab; while (ipref[slab + 1] == ipref[slab]);
+        }
+        return true;
+    }
+};
 
 // Optional source of the sentence penalty: the lookup table T of one value per generation-space sentence,
 // [batch][table_len], read through the cache-space sentence's generation-space index (Phi).  table == nullptr:
@@ -934,214 +988,280 @@ template <int kPass>
 __global__ void __launch_bounds__(kGramThreads, 1)
 score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ CUtensorMap mapLo, int n_slabs,
                   int max_sent, const int32_t* n_sent, float sigma, float tau, float* sc_z, const float* sent_imp,
-                  float* sent_red, float* sent_lam, float* sent_score, LamTable ext, const Header* hdr) {
+                  float* sent_red, float* sent_lam, float* sent_score, float* parts, size_t parts_slab, uint32_t* cnt, LamTable ext, const Header* hdr) {
     extern __shared__ uint8_t gram_smem_raw[];
     const uint32_t raw = smem_u32(gram_smem_raw);
-    uint8_t* At = gram_smem_raw + (((raw + 1023u) & ~1023u) - raw);              // hi, lo of the i block
-    uint8_t* Bt = At + 2 * kOpBytes;                                             // 2 stages x (hi, lo) of a j block
-    GramCtl* ctl = reinterpret_cast<GramCtl*>(Bt + 4 * kOpBytes);
-    int* ipref = reinterpret_cast<int*>(ctl + 1);                                // [n_slabs + 1] prefix of i blocks
+    uint8_t* slots = gram_smem_raw + (((raw + 1023u) & ~1023u) - raw);           // 3 x (high, low)
+    GramCtl* ctl = reinterpret_cast<GramCtl*>(slots + 6 * kOpBytes);
+    int* ipref = reinterpret_cast<int*>(ctl + 1);                                // [n_slabs + 1] prefix of pairs
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int G = gridDim.x, cta = blockIdx.x;
     auto sent_of = [&](int s) { return min(max(n_sent[s], 0), max_sent); };
     pdl_trigger();
 
     if (tid == 0) {
-        mbar_init(&ctl->afull, 1);
-        mbar_init(&ctl->aempty, 2);
-        for (int s = 0; s < 2; ++s) {
-            for (int part = 0; part < 2; ++part) { mbar_init(&ctl->bfull[s][part], 1); mbar_init(&ctl->bempty[s][part], 1); }
-            mbar_init(&ctl->turn[s], 1);
+        for (int s = 0; s < 3; ++s) {
+            for (int part = 0; part < 2; ++part) { mbar_init(&ctl->full[s][part], 1); mbar_init(&ctl->empty[s][part], 1); }
+            mbar_init(&ctl->ddone[s], 1);
         }
-        for (int s = 0; s < kGramGroups; ++s) {
-            mbar_init(&ctl->tfull[s], 1);
-            mbar_init(&ctl->tempty[s], 4);
-        }
+        for (int s = 0; s < 2; ++s) mbar_init(&ctl->turn[s], 1);
+        for (int s = 0; s < kGramAcc; ++s) { mbar_init(&ctl->tfull[s], 1); mbar_init(&ctl->tempty[s], 16); }
         ctl->abort_flag = 0;
         mbar_fence_init();
         tmap_prefetch(&mapHi);
         tmap_prefetch(&mapLo);
     }
-    if (warp == 1) tmem_alloc(&ctl->tmem_base, 128 * kGramGroups);
+    if (warp == 1) tmem_alloc(&ctl->tmem_base, 128 * kGramAcc);
     pdl_wait();                                          // n_sent, the pooled keys and the row sums may come from the kernel before
     uint32_t* status = const_cast<uint32_t*>(&hdr->status);
     const uint32_t limit = load_wait_limit(hdr);
     tc_fence_before();
-    cta_prefix<kGramThreads>(n_slabs, [&](int s) { return (sent_of(s) + 127) >> 7; }, ipref, ctl->wsum);   // i blocks per slab
+    cta_prefix<kGramThreads>(n_slabs, [&](int s) { const int nb = (sent_of(s) + 127) >> 7; return nb * (nb + 1) / 2; }, ipref, ctl->wsum);
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    const int n_items = ipref[n_slabs];
+    const long long total = ipref[n_slabs];
+    const int first = int(total * blockIdx.x / gridDim.x), count = int(total * (blockIdx.x + 1) / gridDim.x) - first;
 
-    if (warp == 0) {
-        if (lane == 0) {
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        if (warp == 0 && lane == 0) {
             bool ok = true;
-            int slab = 0;
-            uint32_t bc = 0, ic = 0;                                // j blocks and items issued so far
-            for (int item = cta; item < n_items && ok; item += G, ++ic) {
-                while (ipref[slab + 1] <= item) ++slab;
-                const int S = sent_of(slab), NJ = (S + 127) >> 7, rowbase = slab * max_sent;
-                const int i0 = (item - ipref[slab]) * 128;
-                if (ic > 0) ok = role_wait(&ctl->aempty, (ic - 1) & 1u, limit, &ctl->abort_flag, status);
-                if (!ok) break;
-                mbar_expect_tx(&ctl->afull, 2 * kOpBytes);
-                tma_load_2d(At, &mapHi, 0, rowbase + i0, &ctl->afull);
-                tma_load_2d(At + kOpHalfBytes, &mapHi, 64, rowbase + i0, &ctl->afull);
-                tma_load_2d(At + kOpBytes, &mapLo, 0, rowbase + i0, &ctl->afull);
-                tma_load_2d(At + kOpBytes + kOpHalfBytes, &mapLo, 64, rowbase + i0, &ctl->afull);
-                for (int jb = 0; jb < NJ && ok; ++jb, ++bc) {
-                    const int s = bc & 1;
-                    for (int part = 1; part >= 0 && ok; --part) {         // low, high: the order in which they are given back
-                        if (bc >= 2) ok = role_wait(&ctl->bempty[s][part], ((bc >> 1) - 1) & 1u, limit, &ctl->abort_flag, status);
-                        if (!ok) break;
-                        uint8_t* dst = Bt + size_t(2 * s + part) * kOpBytes;
-                        const CUtensorMap* map = part ? &mapLo : &mapHi;
-                        mbar_expect_tx(&ctl->bfull[s][part], kOpBytes);
-                        tma_load_2d(dst, map, 0, rowbase + jb * 128, &ctl->bfull[s][part]);
-                        tma_load_2d(dst + kOpHalfBytes, map, 64, rowbase + jb * 128, &ctl->bfull[s][part]);
-                    }
-                }
-            }
-            if (!ok) {
-                mbar_wait(&ctl->afull, 0u, 1u << 16); mbar_wait(&ctl->afull, 1u, 1u << 16);
-                for (int s = 0; s < 2; ++s)
-                    for (int part = 0; part < 2; ++part) { mbar_wait(&ctl->bfull[s][part], 0u, 1u << 16); mbar_wait(&ctl->bfull[s][part], 1u, 1u << 16); }
-            }
-        }
-    } else if (warp == 1 || warp == kGramThreads / 32 - 1) {
-        if (lane == 0) {
-            // A j block each in turn: a stage and an accumulator are always the same issuer's, and one waits for its operands while the
-            // other's products run.  The turn is handed over a little before a block's last instructions are issued; left to themselves, the
-            // two blocks share the tensor pipe, end together, and then wait for their stages to be filled again together.
-            const uint32_t me = warp == 1 ? 0u : 1u;
-            bool ok = true;
-            int slab = 0;
-            uint32_t bc = 0, ic = 0;
-            const uint32_t a_hi = smem_u32(At), a_lo = smem_u32(At + kOpBytes);
-            for (int item = cta; item < n_items && ok; item += G, ++ic) {
-                while (ipref[slab + 1] <= item) ++slab;
-                const int NJ = (sent_of(slab) + 127) >> 7;
-                ok = role_wait(&ctl->afull, ic & 1u, limit, &ctl->abort_flag, status);
-                for (int jb = 0; jb < NJ && ok; ++jb, ++bc) {
-                    if ((bc & 1u) != me) continue;
-                    const int s = bc & 1, acc = bc % kGramGroups;
-                    ok = role_wait(&ctl->bfull[s][1], (bc >> 1) & 1u, limit, &ctl->abort_flag, status) &&
-                         role_wait(&ctl->bfull[s][0], (bc >> 1) & 1u, limit, &ctl->abort_flag, status);
-                    if (ok && bc >= kGramGroups) ok = role_wait(&ctl->tempty[acc], ((bc / kGramGroups) - 1) & 1u, limit, &ctl->abort_flag, status);
-                    if (ok && bc > 0) ok = role_wait(&ctl->turn[me], ((bc >> 1) - (me ? 0u : 1u)) & 1u, limit, &ctl->abort_flag, status);
+            uint32_t ipar = 0, lasti = 0, dpar = 0, lastd = 0;         // bits by slot
+            GramWalk w;
+            w.start(ipref, first, count);
+            auto load = [&](int s, int block) {
+                // What used the slot last: an I block gives its parts back one by one.  A J block was in use until its last pair, and the
+                // pairs with an I have given their slots back by now (both others were taken since); the diagonal one is waited for here.
+                const bool was_i = (lasti >> s) & 1u;
+                if ((lastd >> s) & 1u) ok = role_wait(&ctl->ddone[s], ((dpar >> s) & 1u) ^ 1u, limit, &ctl->abort_flag, status);
+                for (int part = 1; part >= 0 && ok; --part) {             // low, high: the order in which they are given back
+                    if (was_i) ok = role_wait(&ctl->empty[s][part], ((ipar >> s) & 1u) ^ 1u, limit, &ctl->abort_flag, status);
                     if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t b_hi = smem_u32(Bt + size_t(s) * 2 * kOpBytes), b_lo = b_hi + kOpBytes;
-                    const uint32_t d = tmem_base + acc * 128;
-                    umma_tile_128x128x128(d, a_hi, b_lo, false);
-                    umma_commit(&ctl->bempty[s][1]);
-                    umma_tile_128x128x128(d, a_hi, b_hi, true);
-                    mbar_arrive(&ctl->turn[me ^ 1u]);
-                    umma_tile_128x128x128(d, a_lo, b_hi, true);
-                    umma_commit(&ctl->tfull[acc]);
-                    umma_commit(&ctl->bempty[s][0]);
+                    uint8_t* dst = slots + size_t(2 * s + part) * kOpBytes;
+                    const CUtensorMap* map = part ? &mapLo : &mapHi;
+                    const int row = w.slab * max_sent + block * 128;
+                    mbar_expect_tx(&ctl->full[s][part], kOpBytes);
+                    tma_load_2d(dst, map, 0, row, &ctl->full[s][part]);
+                    tma_load_2d(dst + kOpHalfBytes, map, 64, row, &ctl->full[s][part]);
                 }
-                if (ok) umma_commit(&ctl->aempty);                   // every MMA of this issuer that reads this i block has completed
+            };
+            bool fresh = true;
+            while (w.left > 0 && ok) {
+                if (fresh) {
+                    w.take_j();
+                    load(w.jslot, w.J);
+                    const uint32_t bit = 1u << w.jslot;
+                    lasti &= ~bit;
+                    lastd = w.t == 0 ? lastd | bit : lastd & ~bit;
+                    if (w.t == 0) dpar ^= bit;                        // parity of the next diagonal in this slot
+                }
+                if (w.t > 0 && ok) {
+                    const int s = w.take_i();
+                    load(s, w.t - 1);
+                    lasti |= 1u << s;
+                    lastd &= ~(1u << s);
+                    ipar ^= 1u << s;
+                }
+                fresh = w.next(ipref);
+            }
+            if (!ok)                                     // let the copies in flight land before the CTA exits
+                for (int s = 0; s < 3; ++s)
+                    for (int part = 0; part < 2; ++part) { mbar_wait(&ctl->full[s][part], 0u, 1u << 16); mbar_wait(&ctl->full[s][part], 1u, 1u << 16); }
+        } else if ((warp == 1 || warp == 2) && lane == 0) {
+            // A pair each in turn, so that one waits for its operands while the other's products run.  The turn is handed over a little
+            // before a pair's last instructions are issued.  It comes before the other waits: every barrier's earlier phases have been seen by then.
+            const uint32_t me = warp - 1;
+            bool ok = true, fresh = true;
+            uint32_t fpar = 0, jpar = 0;                               // parity of a slot's next use; of J's present one
+            GramWalk w;
+            w.start(ipref, first, count);
+            for (uint32_t bc = 0; w.left > 0 && ok; ++bc) {
+                if (fresh) {
+                    w.take_j();
+                    jpar = (fpar >> w.jslot) & 1u;
+                    fpar ^= 1u << w.jslot;
+                }
+                int is = w.jslot;
+                uint32_t ip = jpar;
+                const bool diag = w.t == 0;
+                if (!diag) {
+                    is = w.take_i();
+                    ip = (fpar >> is) & 1u;
+                    fpar ^= 1u << is;
+                }
+                const int js = w.jslot;
+                fresh = w.next(ipref);
+                if ((bc & 1u) != me) continue;
+                const uint32_t acc = bc % kGramAcc;
+                if (bc > 0) ok = role_wait(&ctl->turn[me], ((bc >> 1) - (me ? 0u : 1u)) & 1u, limit, &ctl->abort_flag, status);
+                for (int part = 1; part >= 0 && ok; --part) {
+                    ok = role_wait(&ctl->full[js][part], jpar, limit, &ctl->abort_flag, status);
+                    if (ok && !diag) ok = role_wait(&ctl->full[is][part], ip, limit, &ctl->abort_flag, status);
+                }
+                if (ok && bc >= kGramAcc) ok = role_wait(&ctl->tempty[acc], ((bc / kGramAcc) - 1) & 1u, limit, &ctl->abort_flag, status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t i_hi = smem_u32(slots + size_t(2 * is) * kOpBytes), j_hi = smem_u32(slots + size_t(2 * js) * kOpBytes);
+                const uint32_t d = tmem_base + acc * 128;
+                umma_tile_128x128x128(d, i_hi + kOpBytes, j_hi, false);
+                if (!diag) umma_commit(&ctl->empty[is][1]);
+                umma_tile_128x128x128(d, i_hi, j_hi + kOpBytes, true);
+                mbar_arrive(&ctl->turn[me ^ 1u]);
+                umma_tile_128x128x128(d, i_hi, j_hi, true);
+                umma_commit(&ctl->tfull[acc]);
+                umma_commit(diag ? &ctl->ddone[js] : &ctl->empty[is][0]);
             }
         }
     } else {
-        const int grp = (warp - 2) >> 2;                           // the accumulator this warpgroup drains
-        const int quarter = warp & 3, wt = (tid - 64) & 127;
-        const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + grp * 128;
-        bool ok = true;
-        int slab = 0;
-        uint32_t bc = 0, ic = 0;
-        for (int item = cta; item < n_items; item += G, ++ic) {
-            while (ipref[slab + 1] <= item) ++slab;
-            const int S = sent_of(slab), NJ = (S + 127) >> 7, rowbase = slab * max_sent;
-            const int i0 = (item - ipref[slab]) * 128;
-            const int row = quarter * 32 + lane;
-            const int i = i0 + row;
-            float accum = 0.f, mx = -INFINITY;
-            for (int jb = 0; jb < NJ; ++jb, ++bc) {
-                if (int(bc % kGramGroups) != grp) continue;        // another warpgroup's block
-                const int j0 = jb * 128;
-                float* invz_s = ctl->invz[grp][(bc / kGramGroups) & 1u];
-                if (kPass == 2) {
-                    const int j = j0 + wt;
-                    const float z = (j < S) ? sc_z[size_t(rowbase) + j] : 1.f;
-                    invz_s[wt] = (z > 0.f) ? 1.f / z : 0.f;
-                    named_bar_sync(1 + grp, 128);
-                }
-                if (ok) {
-                    ok = role_wait(&ctl->tfull[grp], (bc / kGramGroups) & 1u, limit, &ctl->abort_flag, status);
-                    ok = __all_sync(0xffffffffu, ok);
-                }
-                if (!ok) continue;                               // keeps the barrier pattern uniform
-                tc_fence_after();
-                const bool interior = (j0 + 128 <= S) && (j0 != i0);
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        const int quarter = warp & 3, c0 = ((warp - 4) >> 2) * 32;   // this warp's rows (32 * quarter + lane) and columns
+        const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + c0;
+        float* colz_s = ctl->colz[warp - 4];
+        const float2* colz = reinterpret_cast<const float2*>(colz_s);
+        float2 cs[16];
+        bool ok = true, fresh = true;
+        uint32_t acc = 0, parity = 0;
+        int done = 0;                                                // pairs of this slab in this range
+        int cslot = 0;                                               // whose partial the column sums become
+        uint32_t* lam_bits = reinterpret_cast<uint32_t*>(sent_lam);
+        GramWalk w;
+        w.start(ipref, first, count);
+        w.S = count > 0 ? sent_of(w.slab) : 0;
 #pragma unroll 1
-                for (int ch = 0; ch < 4; ++ch) {
-                    float v[32];
-                    tmem_ld32(lane_addr + ch * 32, v);
-                    const float* iz = invz_s + ch * 32;
-                    if (interior) {
-                        float e0 = 0.f, e1 = 0.f;
+        while (w.left > 0) {
+            const size_t base = size_t(w.slab) * max_sent;
+            const int j0 = w.J * 128 + c0;
+            const bool diag = w.t == 0;
+            const int ib = diag ? w.J : w.t - 1, i = ib * 128 + quarter * 32 + lane;
+            float* p_slab = parts + size_t(w.slab) * parts_slab;         // [4 * blocks][max_sent]
+            if (fresh) {
 #pragma unroll
-                        for (int jj = 0; jj < 32; jj += 2) {
-                            if (kPass == 1) {
-                                e0 += ex2f(v[jj] * kLog2e);
-                                e1 += ex2f(v[jj + 1] * kLog2e);
-                            } else {
-                                e0 = fmaf(ex2f(v[jj] * kLog2e), iz[jj], e0);
-                                e1 = fmaf(ex2f(v[jj + 1] * kLog2e), iz[jj + 1], e1);
-                            }
-                        }
-                        accum += e0 + e1;
-                        if (kPass == 1 && j0 > i0) {
-#pragma unroll
-                            for (int jj = 0; jj < 32; ++jj) mx = fmaxf(mx, v[jj]);
-                        }
-                    } else {
-#pragma unroll
-                        for (int jj = 0; jj < 32; ++jj) {
-                            const int j = j0 + ch * 32 + jj;
-                            if (j < S && j != i) {
-                                const float e = ex2f(v[jj] * kLog2e);
-                                if (kPass == 1) {
-                                    accum += e;
-                                    if (j > i) mx = fmaxf(mx, v[jj]);
-                                } else {
-                                    accum = fmaf(e, iz[jj], accum);
-                                }
-                            }
-                        }
-                    }
+                for (int k = 0; k < 16; ++k) cs[k] = make_float2(0.f, 0.f);
+                cslot = ib;
+                if (kPass == 2) {
+                    const float z = j0 + lane < w.S ? sc_z[base + j0 + lane] : 0.f;
+                    __syncwarp();
+                    colz_s[lane] = z > 0.f ? 1.f / z : 0.f;
+                    __syncwarp();
                 }
+            } else if (j0 + lane < w.S) {
+                p_slab[size_t(ib * 4 + quarter) * max_sent + j0 + lane] = 0.f;
+            }
+            float invz_i = 0.f;                                      // pass 2: 1 / Z_i, the weight of this row in column sums
+            if (kPass == 2 && i < w.S) { const float z = sc_z[base + i]; invz_i = z > 0.f ? 1.f / z : 0.f; }
+            if (ok) {
+                // (inline: a call would spill the sums)
+                bool r = mbar_try_wait(&ctl->tfull[acc], parity);
+                for (uint32_t n = 0; !r && n < limit; ++n) {
+                    if ((n & 63) == 63 && *reinterpret_cast<volatile int*>(&ctl->abort_flag)) break;
+                    r = mbar_try_wait(&ctl->tfull[acc], parity);
+                }
+                ok = __all_sync(0xffffffffu, r);
+                if (!ok) {
+                    atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
+                    *reinterpret_cast<volatile int*>(&ctl->abort_flag) = 1;
+                }
+            }
+            if (ok) {
+                tc_fence_after();
+                float v[32];
+                tmem_ld32(lane_addr + acc * 128, v);
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->tempty[grp]);
-            }
-            // the warpgroups hold the sums (and maxima) over interleaved j blocks: the others hand theirs to the first
-            if (grp > 0) {
-                ctl->part[ic & 1][grp - 1][0][row] = accum;
-                if (kPass == 1) ctl->part[ic & 1][grp - 1][1][row] = mx;
-            }
-            named_bar_sync(1 + kGramGroups, 128 * kGramGroups);
-            if (grp == 0 && ok && i < S) {
-#pragma unroll
-                for (int g = 0; g < kGramGroups - 1; ++g) {
-                    accum += ctl->part[ic & 1][g][0][row];
-                    if (kPass == 1) mx = fmaxf(mx, ctl->part[ic & 1][g][1][row]);
-                }
-                const size_t o = size_t(rowbase) + i;
-                if (kPass == 1) {
-                    sc_z[o] = accum;
-                    if (ext.table) {                             // penalty from the generation-space table through Phi
-                        const int g = ext.sent_id[o];
-                        sent_lam[o] = (g >= 0 && g < ext.table_len) ? ext.table[size_t(slab / ext.Hk) * ext.table_len + g] : 0.f;
+                if (lane == 0) mbar_arrive(&ctl->tempty[acc]);
+                float2 row = make_float2(0.f, 0.f);
+                const float2 l2 = make_float2(kLog2e, kLog2e), iz2 = make_float2(invz_i, invz_i);
+                auto add = [&](int k, float2 e) {
+                    if (kPass == 1) {
+                        row = __fadd2_rn(row, e);
+                        cs[k] = __fadd2_rn(cs[k], e);
                     } else {
-                        sent_lam[o] = (mx > tau) ? mx : 0.f;
+                        row = __ffma2_rn(e, colz[k], row);
+                        cs[k] = __ffma2_rn(e, iz2, cs[k]);
                     }
-                } else {
-                    const float red = accum / float(S);
-                    sent_red[o] = red;
-                    sent_score[o] = sigma * sent_imp[o] - (1.f - sigma) * red - sent_lam[o];
+                };
+                float mx = -INFINITY;
+                if (!diag && (w.J + 1) * 128 <= w.S) {               // (I < J: all rows are the slab's)
+                    if (kPass == 1) {
+                        float m1 = -INFINITY;
+#pragma unroll
+                        for (int k = 0; k < 32; k += 4) { mx = max3(mx, v[k], v[k + 1]); m1 = max3(m1, v[k + 2], v[k + 3]); }
+                        mx = fmaxf(mx, m1);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const float2 x = __fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), l2);
+                        add(k, make_float2(ex2f(x.x), ex2f(x.y)));
+                    }
+                } else {                                             // nothing where a row or column is none of the slab's, and for i == j
+                    const int lim = i < w.S ? w.S - j0 : 0, self = i - j0;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const bool x = 2 * k < lim, y = 2 * k + 1 < lim;
+                        if (kPass == 1) {
+                            if (x && 2 * k > self) mx = fmaxf(mx, v[2 * k]);
+                            if (y && 2 * k + 1 > self) mx = fmaxf(mx, v[2 * k + 1]);
+                        }
+                        add(k, make_float2(x && 2 * k != self ? ex2f(v[2 * k] * kLog2e) : 0.f,
+                                           y && 2 * k + 1 != self ? ex2f(v[2 * k + 1] * kLog2e) : 0.f));
+                    }
                 }
+                if (kPass == 1 && mx > tau && !ext.table) atomicMax(lam_bits + base + i, ordered_bits(mx));
+                // (the diagonal pair is symmetric: its column sums are all there is to it)
+                if (!diag && i < w.S) p_slab[size_t(w.J * 4 + (c0 >> 5)) * max_sent + i] = row.x + row.y;
+            }
+            if (++acc == kGramAcc) { acc = 0; parity ^= 1u; }
+            ++done;
+            const int slab = w.slab, S = w.S;
+            fresh = w.next(ipref);
+            if ((fresh || w.left == 0) && ok) {
+                float s[32];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) { s[2 * k] = cs[k].x; s[2 * k + 1] = cs[k].y; }
+                const float sum = col_reduce32(s, lane);
+                if (j0 + lane < S) p_slab[size_t(cslot * 4 + quarter) * max_sent + j0 + lane] = sum;
+            }
+            if (w.slab != slab || w.left == 0) {                     // the range's part of this slab is complete
+                __threadfence();
+                named_bar_sync(1, 512);
+                const int nb = (S + 127) >> 7;
+                if (warp == 4 && lane == 0) {
+                    const int all = nb * (nb + 1) / 2;
+                    const int have = ok ? int(atomicAdd(cnt + slab, uint32_t(done))) + done : 0;
+                    ctl->last = have == all;
+                    if (have == all) cnt[slab] = 0u;                 // for the next pass or call
+                    __threadfence();
+                }
+                named_bar_sync(1, 512);
+                if (*reinterpret_cast<volatile int*>(&ctl->last)) {
+                    for (int k = tid - 128; k < S; k += 512) {
+                        float sum = 0.f;
+#pragma unroll 4
+                        for (int q = 0; q < nb; ++q) {
+                            const float* p = p_slab + size_t(q * 4) * max_sent + k;
+                            sum += (__ldcg(p) + __ldcg(p + max_sent)) + (__ldcg(p + 2 * size_t(max_sent)) + __ldcg(p + 3 * size_t(max_sent)));
+                        }
+                        const size_t o = base + k;
+                        if (kPass == 1) {
+                            sc_z[o] = sum;
+                        } else {
+                            const float red = sum / float(S);
+                            float lam;
+                            if (ext.table) {                         // penalty from the generation-space table through Phi
+                                const int g = ext.sent_id[o];
+                                lam = (g >= 0 && g < ext.table_len) ? ext.table[size_t(slab / ext.Hk) * ext.table_len + g] : 0.f;
+                            } else {
+                                const uint32_t u = lam_bits[o];
+                                lam = u ? from_ordered_bits(u) : 0.f;
+                            }
+                            sent_lam[o] = lam;
+                            sent_red[o] = red;
+                            sent_score[o] = sigma * sent_imp[o] - (1.f - sigma) * red - lam;
+                        }
+                    }
+                }
+                named_bar_sync(1, 512);                              // `last` may be written again
+                done = 0;
+                w.S = w.left > 0 ? sent_of(w.slab) : 0;
             }
         }
     }
@@ -1149,7 +1269,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 128 * kGramGroups);
+        tmem_dealloc(tmem_base, 128 * kGramAcc);
     }
 }
 
@@ -1391,19 +1511,19 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         dim3 pgrid((shape->max_sent + 8 * kPoolRows - 1) / (8 * kPoolRows), L.slabs);
         SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, shape->max_cap,
                                      shape->cap, kv_len, sent_off, n_sent, params->eps, sc_tok, vsum, sent_imp, vbar_hi,
-                                     vbar_lo));
+                                     vbar_lo, sent_lam));
     }
     {
         const size_t gsmem = gram_smem_bytes(L.slabs);
         if (gsmem > 227 * 1024) return SKIPKV_ERR_UNSUPPORTED;
-        const long long max_items = (long long)L.slabs * ((shape->max_sent + 127) / 128);
+        const long long nb = (shape->max_sent + 127) / 128, max_items = L.slabs * (nb * (nb + 1) / 2);
         const int ggrid = int(max_items < (long long)grid ? max_items : (long long)grid);
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<1>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,
                                      shape->max_sent, n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
-                                     sent_score, ext, reinterpret_cast<const Header*>(w + L.header)));
+                                     sent_score, vsum, L.sc_vsum_slab, a.lse_cnt, ext, reinterpret_cast<const Header*>(w + L.header)));
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<2>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,
                                      shape->max_sent, n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
-                                     sent_score, ext, reinterpret_cast<const Header*>(w + L.header)));
+                                     sent_score, vsum, L.sc_vsum_slab, a.lse_cnt, ext, reinterpret_cast<const Header*>(w + L.header)));
     }
     return SKIPKV_OK;
 }

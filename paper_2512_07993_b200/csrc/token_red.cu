@@ -50,21 +50,6 @@ __device__ __forceinline__ int tr_count(int NB, int I) {
     const int half = NB >> 1;
     return (NB & 1) ? 1 + half : half + (I < half ? 1 : 0);
 }
-// Sum over the 32 lanes of x[c] for every c: lane c returns the sum of column c (31 exchanges).
-__device__ __forceinline__ float tr_col_reduce(const float (&x)[32], int lane) {
-    float a[16], b[8], c[4], d[2];
-    const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4, u2 = lane & 2, u1 = lane & 1;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) a[k] = (u16 ? x[k + 16] : x[k]) + __shfl_xor_sync(0xffffffffu, u16 ? x[k] : x[k + 16], 16);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) b[k] = (u8 ? a[k + 8] : a[k]) + __shfl_xor_sync(0xffffffffu, u8 ? a[k] : a[k + 8], 8);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) c[k] = (u4 ? b[k + 4] : b[k]) + __shfl_xor_sync(0xffffffffu, u4 ? b[k] : b[k + 4], 4);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) d[k] = (u2 ? c[k + 2] : c[k]) + __shfl_xor_sync(0xffffffffu, u2 ? c[k] : c[k + 2], 2);
-    return (u1 ? d[1] : d[0]) + __shfl_xor_sync(0xffffffffu, u1 ? d[0] : d[1], 1);
-}
-
 __device__ __forceinline__ float tr_ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -314,7 +299,7 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
                 float s[32];
 #pragma unroll
                 for (int k = 0; k < 16; ++k) { s[2 * k] = cs[k].x; s[2 * k + 1] = cs[k].y; }
-                const float sum = tr_col_reduce(s, lane);
+                const float sum = col_reduce32(s, lane);
                 if (j0 + lane < x.S) atomicAdd(dst + j0 + lane, kPass == 1 ? sum : sum * inv_S);
             }
         }

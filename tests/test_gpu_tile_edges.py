@@ -63,9 +63,10 @@ def check_scores(B, L, D, rtol=1e-3):
             assert (np.abs(g - r) <= rtol * np.abs(r)).all(), ("tok_imp", b, h)
 
 
-@pytest.mark.parametrize("sentences", [[1, 2, 31, 33], [63, 64, 65, 128], [127, 129, 5, 1], [256, 257, 300]])
+@pytest.mark.parametrize("sentences", [[1, 2, 31, 33], [63, 64, 65, 128], [127, 129, 5, 1], [256, 257, 300], [640, 1153], [4225]])
 def test_score_sentence_counts_around_a_tile(sentences):
-    """Up to 128 sentences per slab: one kernel behind the sweeps; more: the blocked kernels."""
+    """Up to 128 sentences per slab: one kernel behind the sweeps; more: the blocked kernels, block columns cut by the CTAs' ranges
+    or not, and partial sums that outgrow the key sums."""
     B, L, D = layer([5 * n for n in sentences], sent_lo=5, sent_hi=5, dup_rate=0.3, seed=500 + sentences[0])
     assert int(L["n_sent"].max()) == max(sentences)
     check_scores(B, L, D)
