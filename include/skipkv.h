@@ -56,7 +56,7 @@ extern "C" {
 
 #define SKIPKV_OK               0
 #define SKIPKV_ERR_INVALID_ARG (-1)  /* null pointer, negative size, inconsistent shape      */
-#define SKIPKV_ERR_UNSUPPORTED (-2)  /* head_dim != 128, Hq % Hk != 0, group or window too big */
+#define SKIPKV_ERR_UNSUPPORTED (-2)  /* head_dim != 128, Hq % Hk != 0, group or window too big, too many slabs */
 #define SKIPKV_ERR_WORKSPACE   (-3)  /* workspace null or misaligned                          */
 #define SKIPKV_ERR_CUDA        (-4)  /* a CUDA runtime call failed; see skipkv_last_cuda_error */
 #define SKIPKV_ERR_TIMEOUT     (-5)  /* reported by skipkv_status: a bounded device wait ran out */
@@ -136,8 +136,10 @@ const char* skipkv_last_cuda_error(void);
  * [batch][Hk][max_sent]; entries at i >= n_sent are not written.
  * shape->total_rows must be the exact number of rows of the K buffer (the tiled copies are bounded by
  * it).  The per-sentence sums are accumulated with floating-point atomics, so the last bits of the
- * scores may differ from run to run.  The kernels of one call, and the first kernel of a call after
- * the kernel before it on the stream, are launched as programmatic dependents: stream order holds.
+ * scores may differ from run to run.  Limit: where max_sent > 128, about 8000 slabs (batch * n_kv_heads), whatever
+ * the group size and the window; with more the call returns SKIPKV_ERR_UNSUPPORTED and skipkv_last_cuda_error() says
+ * why.  The kernels of one call, and the first kernel of a call after the kernel before it on the stream, are launched
+ * as programmatic dependents: stream order holds.
  */
 int skipkv_score(const skipkv_shape* shape, const skipkv_params* params, const void* K,
                  const void* q_win, const int32_t* kv_len, const int32_t* sent_off,

@@ -91,6 +91,7 @@ struct SweepArgs {
     const Header* hdr;
     const int32_t* block_table;         // nullable: paged cache, tile j of slab s is page block_table[s * max_pages + j]
     int max_pages;
+    int* table;                         // [2 * n_slabs + 1] tile prefix and first cache rows, where shared memory has no room for them
 };
 
 __device__ __forceinline__ float ex2f(float x) {
@@ -242,7 +243,22 @@ __device__ __forceinline__ void indicator_piece(uint8_t* ind, int j, int c, int 
     *reinterpret_cast<uint4*>(ind + (c >> 3) * (kIndBytes / 2) + j * 128 + (((c & 7) ^ (j & 7)) << 4)) = val;
 }
 
-template <int kWB>
+// The sweep's table of slabs in global memory, for calls with more slabs than shared memory has room for beside the query rows.
+__global__ void __launch_bounds__(1024) sweep_table_kernel(const SweepArgs a) {
+    __shared__ uint32_t wsum[32];
+    pdl_trigger();
+    pdl_wait();
+    for (int s = threadIdx.x; s < a.n_slabs; s += 1024)
+        a.table[a.n_slabs + 1 + s] = a.block_table ? 0 : int(slab_row0(a.slab_off, a.cap, a.Hk, s / a.Hk, s % a.Hk));
+    auto tiles = [&](int s) {
+        const int room = a.block_table ? min(a.cap[s / a.Hk], a.max_pages * 128) : a.cap[s / a.Hk];
+        return (min(max(a.kv_len[s], 0), room) + 127) >> 7;
+    };
+    cta_prefix<1024>(a.n_slabs, tiles, a.table, wsum);
+}
+
+// kTable: the table of slabs is in global memory (an instance of its own: the other one keeps its accesses to shared memory).
+template <int kWB, bool kTable>
 __global__ void __launch_bounds__(kSweepThreads, 1)
 score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapQ, const SweepArgs a) {
     extern __shared__ uint8_t sweep_smem_raw[];
@@ -255,7 +271,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     uint8_t* extb = onesb + 128 * kExtRow;                                       // pass B: the queries' side; pass A: [4 groups][RA * 128] (m, l)
     SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + size_t(a.RA) * 128 * kExtRow);
     float* tokp = reinterpret_cast<float*>(ctl + 1);                             // [4 tiles][RB - 1][128] shares of a tile's tokens
-    int* pref = reinterpret_cast<int*>(tokp + 4 * (a.RB - 1) * 128);             // [n_slabs + 1] tile prefix
+    int* pref = kTable ? a.table : reinterpret_cast<int*>(tokp + 4 * (a.RB - 1) * 128);    // [n_slabs + 1] tile prefix
     int* rowb = pref + a.n_slabs + 1;                                            // [n_slabs] cache row of a slab's first token
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -292,9 +308,13 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     pdl_wait();                                          // the lengths may come from the kernel before this call
     const uint32_t limit = load_wait_limit(a.hdr);
     tc_fence_before();
-    for (int s = tid; s < n_slabs; s += kSweepThreads)
-        rowb[s] = a.block_table ? 0 : int(slab_row0(a.slab_off, a.cap, Hk, s / Hk, s % Hk));
-    cta_prefix<kSweepThreads>(n_slabs, [&](int s) { return (live(s) + 127) >> 7; }, pref, ctl->wsum);   // also publishes the set-up
+    if (kTable) {
+        __syncthreads();
+    } else {
+        for (int s = tid; s < n_slabs; s += kSweepThreads)
+            rowb[s] = a.block_table ? 0 : int(slab_row0(a.slab_off, a.cap, Hk, s / Hk, s % Hk));
+        cta_prefix<kSweepThreads>(n_slabs, [&](int s) { return (live(s) + 127) >> 7; }, pref, ctl->wsum);   // also publishes the set-up
+    }
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     const int T = pref[n_slabs], Ge = min(G, T);         // CTA c has the tiles [c T / Ge, (c + 1) T / Ge)
@@ -1482,9 +1502,19 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     a.hdr = reinterpret_cast<const Header*>(w + L.header);
     a.block_table = block_table; a.max_pages = max_pages;
     const size_t max_smem = 227 * 1024;
-    const size_t fixed = 1024 + size_t(a.R) * kRowBytes + size_t(kIndRing) * kIndBytes + 128 * kExtRow + size_t(a.RA) * 128 * kExtRow +
-                         sizeof(SweepCtl) + size_t(a.RB - 1) * 4 * 128 * 4 + size_t(2 * L.slabs + 1) * 4;
-    if (fixed + kOpBytes > max_smem) return SKIPKV_ERR_UNSUPPORTED;
+    size_t fixed = 1024 + size_t(a.R) * kRowBytes + size_t(kIndRing) * kIndBytes + 128 * kExtRow + size_t(a.RA) * 128 * kExtRow +
+                   sizeof(SweepCtl) + size_t(a.RB - 1) * 4 * 128 * 4;
+    // The table of slabs (8 bytes each) goes into shared memory as long as one tile stage fits beside it: all but windows of some hundred
+    // query rows with a thousand slabs and more.  A 512-row window leaves room for 900 slabs; without the other form the call would end there.
+    const size_t table_bytes = size_t(2 * L.slabs + 1) * 4;
+    const bool in_global = fixed + table_bytes + kOpBytes > max_smem;
+    if (in_global) a.table = reinterpret_cast<int*>(w + L.sc_table);
+    else fixed += table_bytes;
+    const size_t gsmem = gram_smem_bytes(L.slabs);
+    if (shape->max_sent > kSmallSent && gsmem > max_smem) {          // (before anything is enqueued)
+        set_error_text("skipkv_score: more than 128 sentences per slab and batch * n_kv_heads too large for the shared-memory table of the Gram kernels");
+        return SKIPKV_ERR_UNSUPPORTED;
+    }
     a.stages = int((max_smem - fixed) / kOpBytes);
     if (a.stages > kStagesMax) a.stages = kStagesMax;
     int grid = num_sms();
@@ -1492,9 +1522,11 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     // Cooperative: the CTAs wait for one another between the passes, so they have to be resident together whatever else
     // runs on the GPU.  Where the context may use fewer SMs than the device has, a smaller grid does.
     cudaError_t le = cudaErrorCooperativeLaunchTooLarge;
+    if (in_global) SKIPKV_CUDA(launch_dependent(sweep_table_kernel, dim3(1), dim3(1024), 0, st, a));
+    const auto sweep = L.sc_wb == 32 ? (in_global ? score_sweep_kernel<32, true> : score_sweep_kernel<32, false>)
+                                     : (in_global ? score_sweep_kernel<16, true> : score_sweep_kernel<16, false>);
     for (; grid >= 1 && le == cudaErrorCooperativeLaunchTooLarge; grid /= 2) {
-        le = launch_dependent<true>(L.sc_wb == 32 ? score_sweep_kernel<32> : score_sweep_kernel<16>, dim3(grid), dim3(kSweepThreads),
-                                    fixed + size_t(a.stages) * kOpBytes, st, mapK, mapQ, a);
+        le = launch_dependent<true>(sweep, dim3(grid), dim3(kSweepThreads), fixed + size_t(a.stages) * kOpBytes, st, mapK, mapQ, a);
         if (le == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();
         else break;
     }
@@ -1514,8 +1546,6 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
                                      vbar_lo, sent_lam));
     }
     {
-        const size_t gsmem = gram_smem_bytes(L.slabs);
-        if (gsmem > 227 * 1024) return SKIPKV_ERR_UNSUPPORTED;
         const long long nb = (shape->max_sent + 127) / 128, max_items = L.slabs * (nb * (nb + 1) / 2);
         const int ggrid = int(max_items < (long long)grid ? max_items : (long long)grid);
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<1>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,

@@ -81,3 +81,39 @@ def test_score_query_blocks(group, window):
         B, L, D = layer([max(c, window) for c in ctx], n_q_heads=2 * group, n_kv_heads=2, window=window, sent_lo=8, sent_hi=40,
                         dup_rate=0.3, seed=700 + 10 * group + window % 10)
         check_scores(B, L, D)
+
+
+@pytest.mark.parametrize("group,window,batch,sent", [(1, 512, 16, (8, 40)), (5, 100, 19, (8, 40)), (1, 512, 16, (2, 4))])
+def test_score_with_more_slabs_than_shared_memory_has_room_for(group, window, batch, sent):
+    """Over a thousand slabs beside a wide window: the sweep's table of slabs is in global memory; contiguous against the oracle, paged
+    against contiguous, up to 128 sentences per slab and more."""
+    lens = [1, 2, 127, 128, 129, 255, 256, 257, 384, 40, 77, 300, 500, 9, 16, 130, 31, 64, 200][:batch]
+    B, L, D = layer(lens, n_q_heads=64 * group, n_kv_heads=64, window=window, sent_lo=sent[0], sent_hi=sent[1], dup_rate=0.3, seed=900 + group)
+    assert batch * 64 > 1000 and (int(L["n_sent"].max()) > 128) == (sent[1] < 8)
+    check_scores(B, L, D)
+    pages = -(-np.asarray(lens) // 128)
+    max_pages, n_pool = int(pages.max()), int(pages.sum()) * 64
+    ids = np.random.Generator(np.random.Philox(5)).permutation(n_pool)
+    Kp = torch.full((n_pool * 128, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    table, k = np.full((batch, 64, max_pages), -1, np.int32), 0
+    for b in range(batch):
+        for h in range(64):
+            table[b, h, :pages[b]] = ids[k:k + pages[b]]
+            k += pages[b]
+    table = torch.as_tensor(table).cuda()
+    for b, n in enumerate(lens):
+        t = torch.arange(n, device="cuda")
+        rows = table[b].long()[:, t // 128] * 128 + t % 128
+        off = int(L["slab_off"][b]) * 64
+        Kp[rows.reshape(-1)] = D.K[off:off + 64 * n]
+    shp = B.make_shape(batch, 64 * group, 64, 128, window, L["cfg"].d_model, D.max_sent, max(lens), D.slab_off, D.cap, int(Kp.shape[0]))
+    imp = torch.full((batch, 64, max_pages * 128), float("nan"), device="cuda")
+    outs = [torch.full_like(D.sent_imp, float("nan")) for _ in range(4)]
+    B.skipkv_score_paged(shp, D.params, Kp, table, max_pages, D.q_win, D.kv_len, D.sent_off, D.n_sent, imp, *outs, D.ws)
+    torch.cuda.synchronize()
+    assert D.status() == 0
+    for b, n in enumerate(lens):
+        off, S = int(L["slab_off"][b]) * 64, int(L["n_sent"][b, 0])
+        assert torch.equal(imp[b, :, :n].reshape(-1), D.tok_imp[off:off + 64 * n])
+        for got, ref in zip(outs, (D.sent_imp, D.sent_red, D.sent_lam, D.sent_score)):
+            assert torch.equal(got[b, :, :S], ref[b, :, :S])
