@@ -46,7 +46,7 @@ struct WsLayout {
     size_t sc_vbar_hi;     // bf16   [slabs][max_sent][128]  normalised mean key, high part
     size_t sc_vbar_lo;     // bf16   [slabs][max_sent][128]  and the rounding remainder
     size_t sc_z;           // float  [slabs][max_sent]
-    size_t sc_table;       // int32  [2 * slabs + 1]  tile prefix and first rows of the slabs, where shared memory has no room for them
+    size_t slab_table;       // int32  [2 * slabs + 1]  tile prefix and first rows of the slabs, where shared memory has no room for them
     size_t tr_inv;         // float  [slabs][max_cap]  token redundancy: 1 / (|K_t| + eps)
     size_t tr_z;           // float  [slabs][max_cap]  token redundancy: row sums of exp(G)
     size_t total;
@@ -102,7 +102,7 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     L.sc_vbar_hi = take(slabs * ms * kHeadDim * 2);
     L.sc_vbar_lo = take(slabs * ms * kHeadDim * 2);
     L.sc_z = take(slabs * ms * 4);
-    L.sc_table = take((2 * slabs + 1) * 4);
+    L.slab_table = take((2 * slabs + 1) * 4);
     L.tr_inv = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);
     L.tr_z = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);
     L.total = o;

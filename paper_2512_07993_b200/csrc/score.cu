@@ -1508,7 +1508,7 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     // query rows with a thousand slabs and more.  A 512-row window leaves room for 900 slabs; without the other form the call would end there.
     const size_t table_bytes = size_t(2 * L.slabs + 1) * 4;
     const bool in_global = fixed + table_bytes + kOpBytes > max_smem;
-    if (in_global) a.table = reinterpret_cast<int*>(w + L.sc_table);
+    if (in_global) a.table = reinterpret_cast<int*>(w + L.slab_table);
     else fixed += table_bytes;
     const size_t gsmem = gram_smem_bytes(L.slabs);
     if (shape->max_sent > kSmallSent && gsmem > max_smem) {          // (before anything is enqueued)

@@ -43,7 +43,7 @@ struct TrCtl {
     uint32_t wsum[32];
     alignas(16) float col[16][2][32];        // by epilogue warp: log2(e) / (|K_j| + eps) of its columns; pass 2: 1 / Z_j
 };
-static size_t tr_smem_bytes(int slabs) { return 1024 + (2 + kTrStages) * size_t(kOpBytes) + sizeof(TrCtl) + size_t(slabs + 1) * 4; }
+constexpr size_t kTrSmem = 1024 + (2 + kTrStages) * size_t(kOpBytes) + sizeof(TrCtl);          // and the table of slabs behind it
 
 // Blocks that item (slab of NB blocks, block J) multiplies block J with: J itself and the next ones, cyclically.
 __device__ __forceinline__ int tr_count(int NB, int I) {
@@ -86,17 +86,27 @@ token_norm_kernel(int Hk, int max_cap, const int64_t* slab_off, const int32_t* c
 
 struct TrItem { int slab, S, NB, J, NJ; size_t sbase; };
 
-template <int kPass>
+// Table of slabs in global memory, for calls with more slabs than shared memory has room for beside the tiles.
+__global__ void __launch_bounds__(1024)
+token_table_kernel(int n_slabs, int Hk, int max_cap, const int32_t* cap, const int32_t* kv_len, int* table) {
+    __shared__ uint32_t wsum[32];
+    pdl_trigger();
+    pdl_wait();
+    cta_prefix<1024>(n_slabs, [&](int s) { return (min(max(kv_len[s], 0), min(cap[s / Hk], max_cap)) + 127) >> 7; }, table, wsum);
+}
+
+// kTable: the table of slabs is in global memory (an instance of its own: the other one keeps its accesses to shared memory)
+template <int kPass, bool kTable>
 __global__ void __launch_bounds__(kTrThreads, 1)
 token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, int max_cap, const int64_t* slab_off,
                  const int32_t* cap, const int32_t* kv_len, const float* inv_norm, float* z, float* tok_red,
-                 const Header* hdr) {
+                 const Header* hdr, int* table) {
     extern __shared__ uint8_t tr_smem_raw[];
     const uint32_t raw = smem_u32(tr_smem_raw);
     uint8_t* Jt = tr_smem_raw + (((raw + 1023u) & ~1023u) - raw);
     uint8_t* It = Jt + 2 * kOpBytes;
     TrCtl* ctl = reinterpret_cast<TrCtl*>(It + kTrStages * kOpBytes);
-    int* ipref = reinterpret_cast<int*>(ctl + 1);                                // [n_slabs + 1] prefix of blocks
+    int* ipref = kTable ? table : reinterpret_cast<int*>(ctl + 1);               // [n_slabs + 1] prefix of blocks
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, cta = blockIdx.x;
     auto len_of = [&](int s) { return min(max(kv_len[s], 0), min(cap[s / Hk], max_cap)); };
@@ -115,7 +125,8 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
     uint32_t* status = const_cast<uint32_t*>(&hdr->status);
     const uint32_t limit = load_wait_limit(hdr);
     tc_fence_before();
-    cta_prefix<kTrThreads>(n_slabs, [&](int s) { return (len_of(s) + 127) >> 7; }, ipref, ctl->wsum);   // blocks per slab
+    if (kTable) __syncthreads();
+    else cta_prefix<kTrThreads>(n_slabs, [&](int s) { return (len_of(s) + 127) >> 7; }, ipref, ctl->wsum);   // blocks per slab
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     const int n_items = ipref[n_slabs];
@@ -330,8 +341,11 @@ extern "C" int skipkv_token_redundancy(const skipkv_shape* shape, const skipkv_p
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     CUtensorMap mapK;
     if (int rc = tmap_rows(&mapK, K, uint64_t(shape->total_rows), 128)) return rc;
-    const size_t smem = tr_smem_bytes(L.slabs);
-    if (smem > 227 * 1024) return SKIPKV_ERR_UNSUPPORTED;
+    // The table (4 bytes a slab) goes into shared memory up to about 7600 slabs, the room beside six tiles; beyond that into the workspace.
+    size_t smem = kTrSmem + size_t(L.slabs + 1) * 4;
+    const bool in_global = smem > 227 * 1024;
+    if (in_global) smem = kTrSmem;
+    int* table = in_global ? reinterpret_cast<int*>(w + L.slab_table) : nullptr;
     const int Hk = shape->n_kv_heads;
     SKIPKV_CUDA(launch_dependent(token_norm_kernel, dim3((shape->max_cap + 63) / 64, L.slabs), dim3(256), 0, st, Hk,
                                  int(shape->max_cap), shape->slab_off, shape->cap, static_cast<const __nv_bfloat16*>(K),
@@ -339,11 +353,14 @@ extern "C" int skipkv_token_redundancy(const skipkv_shape* shape, const skipkv_p
     const long long max_items = (long long)L.slabs * ((shape->max_cap + 127) / 128);
     int grid = num_sms();
     if (max_items < grid) grid = int(max_items);
-    SKIPKV_CUDA(launch_dependent(token_red_kernel<1>, dim3(grid), dim3(kTrThreads), smem, st, mapK, int(L.slabs), Hk,
-                                 int(shape->max_cap), shape->slab_off, shape->cap, kv_len, static_cast<const float*>(inv_norm),
-                                 z, tok_red, hdr));
-    SKIPKV_CUDA(launch_dependent(token_red_kernel<2>, dim3(grid), dim3(kTrThreads), smem, st, mapK, int(L.slabs), Hk,
-                                 int(shape->max_cap), shape->slab_off, shape->cap, kv_len, static_cast<const float*>(inv_norm),
-                                 z, tok_red, hdr));
+    if (in_global)
+        SKIPKV_CUDA(launch_dependent(token_table_kernel, dim3(1), dim3(1024), 0, st, int(L.slabs), Hk, int(shape->max_cap), shape->cap,
+                                     kv_len, table));
+    for (int pass = 1; pass <= 2; ++pass) {
+        const auto kernel = pass == 1 ? (in_global ? token_red_kernel<1, true> : token_red_kernel<1, false>)
+                                      : (in_global ? token_red_kernel<2, true> : token_red_kernel<2, false>);
+        SKIPKV_CUDA(launch_dependent(kernel, dim3(grid), dim3(kTrThreads), smem, st, mapK, int(L.slabs), Hk, int(shape->max_cap),
+                                     shape->slab_off, shape->cap, kv_len, static_cast<const float*>(inv_norm), z, tok_red, hdr, table));
+    }
     return SKIPKV_OK;
 }

@@ -69,3 +69,33 @@ def test_token_redundancy_empty_and_single_row_slabs():
             elif N > 1:
                 ref = oracle.token_redundancy(Kb[rows][:N], 1e-6)
                 assert (np.abs(got[:N] - ref) <= 1e-3 * np.abs(ref)).all()
+
+
+def test_token_redundancy_with_more_slabs_than_shared_memory_has_room_for():
+    """9216 slabs: the kernels' table of slabs is in global memory.  Slabs of no row, of one, of whole and partly filled tiles."""
+    from paper_2512_07993_b200 import build, binding as B
+    build.build()
+    lens = np.tile([0, 1, 2, 127, 128, 129, 300, 31, 5], 16)
+    bt, hk = len(lens), 64
+    off = np.concatenate([[0], np.cumsum(lens)])
+    g = torch.Generator(device="cuda").manual_seed(83)
+    K = torch.randn(int(off[-1]) * hk, 128, generator=g, device="cuda").bfloat16()
+    slab_off, cap = torch.as_tensor(off[:-1].copy()).cuda(), torch.as_tensor(lens.astype(np.int32)).cuda()
+    shape = B.make_shape(bt, hk, hk, 128, 8, 0, 1, int(lens.max()), slab_off, cap, K.shape[0])
+    ws = torch.empty(B.skipkv_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    B.skipkv_workspace_init(shape, ws)
+    kv_len = cap[:, None].repeat(1, hk).contiguous()
+    red = torch.full((K.shape[0],), float("nan"), device="cuda")
+    B.skipkv_token_redundancy(shape, B.make_params(), K, kv_len, red, ws)
+    torch.cuda.synchronize()
+    assert B.skipkv_status(ws) == 0
+    for b in range(bt):
+        n = int(lens[b])
+        if n == 0:
+            continue
+        got = red[off[b] * hk:off[b + 1] * hk].view(hk, n)
+        k = K[off[b] * hk:off[b + 1] * hk].view(hk, n, 128).double()
+        k = k / (k.norm(dim=-1, keepdim=True) + 1e-6)
+        e = torch.exp(k @ k.transpose(1, 2)) * (1 - torch.eye(n, device="cuda", dtype=torch.float64))
+        ref = (e / e.sum(-1, keepdim=True).clamp_min(1e-30)).sum(1) / n
+        assert ((got - ref).abs() <= 1e-3 * ref.abs()).all(), b
