@@ -13,10 +13,16 @@
 //    16-byte pieces permuted (piece c of row r at c ^ (r & 7)), which makes the matrix loads free of bank conflicts, and
 //    because rows past the slab's end are zero-filled and the row being appended can come from another pointer.
 //    Three stages of 8 KB per warp keep 64 KB in flight per SM while 32 KB are worked on.
-//  * Math on the tensor cores (mma.sync m16n8k16: one query row per head is far below a tcgen05 tile): S = Q K^T with the
-//    group's heads as the first rows of the A operand, then P V with the probabilities as bf16 high parts in rows 0..7
-//    and their remainders in rows 8..15, so that nothing is lost against fp32 probabilities to 2^-17.  The cost does not
-//    depend on the group size: 5 heads per group used to be bound by packed FMAs (768 us over the un-evicted stress cache).
+//  * Math on the tensor cores (mma.sync m16n8k16: one query row per head is far below a tcgen05 tile): S^T = K Q^T with 16
+//    tokens as rows and the group's heads as the eight columns, then (P V)^T = V^T P^T with 16 channels as rows.  The probabilities
+//    go in as three bf16 parts (transposed in registers by movmatrix), which together are the fp32 value, and the products of a
+//    tile are added to the sums over the tiles in fp32 with rounding: the tensor core's own accumulation truncates.  With two
+//    parts and sums kept in the tensor core 1 to 3 outputs in a thousand were not the exact result rounded to bf16; now 0.2 to 0.5,
+//    as with fp32 arithmetic throughout.  Any group size costs the same up to four heads, and the same from five to eight.
+//    There is one warp to a scheduler, so a tile is a chain of latencies (16 x 8 x 16 products 10 clocks apart and 30 long, exchanges
+//    24, matrix loads 16): independent chains of products, exchanges of the heads' maxima only when one of them rises.
+//    Against the two parts: 72.8 -> 74.4 us (two steps of 80 slabs x 4.1K rows), 163.2 -> 168.6 (80 slabs of 16K to 32K), 96.8 -> 104.5
+//    (128 slabs x 8.2K, five heads).
 //  * Little shared memory and few threads, so that the CTAs of the next launch are resident while this one streams: a
 //    programmatic dependent launch derives its tile schedule and starts its first tiles towards L2 before the launch
 //    ahead of it has finished, and only then waits.  What it read early is checked afterwards (see "schedule").
@@ -76,12 +82,29 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// two probabilities as bf16 high parts and as the bf16 remainders
-__device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    hi = *reinterpret_cast<const uint32_t*>(&h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(x - bf16lo(hi), y - bf16hi(hi));
-    lo = *reinterpret_cast<const uint32_t*>(&l);
+// the same without a sum to add to
+__device__ __forceinline__ void mma16816_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+// Two probabilities as three bf16 parts each, the leading, middle and last 8 bits of the fp32 values.
+__device__ __forceinline__ uint32_t top_halves(float2 x) { return __byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x7632); }
+__device__ __forceinline__ float2 without_top(float2 x) {
+    const float2 top = make_float2(__uint_as_float(__float_as_uint(x.x) & 0xffff0000u), __uint_as_float(__float_as_uint(x.y) & 0xffff0000u));
+    return __ffma2_rn(top, make_float2(-1.f, -1.f), x);
+}
+__device__ __forceinline__ void split_bf16(float2 x, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    hi = top_halves(x);
+    x = without_top(x);
+    mid = top_halves(x);
+    lo = top_halves(without_top(x));
+}
+// an 8 x 8 matrix of bf16 pairs across the warp, transposed
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
+    uint32_t y;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
 }
 
 // Optional fusion of the per-step bookkeeping into the decode launch (k_new == nullptr: plain decode attention).
@@ -103,7 +126,9 @@ struct StepArgs {
 
 // kStep: the launch also performs the per-step bookkeeping described at StepArgs (a separate instance, so that
 // plain decode attention carries none of it).
-template <bool kStep>
+// kFew: up to four heads per group.  The eight columns of an operand are then the heads twice: the high parts of the probabilities
+// in the first four, the middle ones in the others, so that two products do the work of three.
+template <bool kStep, bool kFew>
 __global__ void __launch_bounds__(kDecThreads, 2)
 decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows, const int64_t* slab_off, const int32_t* cap,
                    const __nv_bfloat16* q, const uint8_t* K, const uint8_t* V, const int32_t* kv_len,
@@ -220,12 +245,13 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
                           size_t(p_r0 % kPageRows);
                 const size_t off = (row + size_t(c_half)) * kRowBytes + size_t(c_col) * 16;
                 const uint8_t *kp = K + off, *vp = V + off;
-                const uint32_t dst = ring + p_stage * kStageBytes + c_half * kRowBytes;
+                // (row 2 i + c_half takes its pieces at c_col ^ ((2 i + c_half) & 7): four addresses and constant distances from them)
+                const uint32_t dst = ring + p_stage * kStageBytes + c_half * kRowBytes + ((c_col ^ c_half) << 4);
                 const int last = rows - 1;                // the appended row, where there is one
                 if (rows > kWarpRows || (rows == kWarpRows && !p_app)) {
 #pragma unroll
                     for (int i = 0; i < kWarpRows / 2; ++i) {
-                        const uint32_t d = dst + i * 2 * kRowBytes + ((c_col ^ ((2 * i + c_half) & 7)) << 4);
+                        const uint32_t d = (dst ^ ((i & 3) << 5)) + i * 2 * kRowBytes;
                         cp_async16(d, kp + i * 2 * kRowBytes);
                         cp_async16(d + kWarpRows * kRowBytes, vp + i * 2 * kRowBytes);
                     }
@@ -233,7 +259,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
 #pragma unroll
                     for (int i = 0; i < kWarpRows / 2; ++i) {
                         const int r = 2 * i + c_half;
-                        const uint32_t d = dst + i * 2 * kRowBytes + ((c_col ^ (r & 7)) << 4);
+                        const uint32_t d = (dst ^ ((i & 3) << 5)) + i * 2 * kRowBytes;
                         const void *ks = kp + i * 2 * kRowBytes, *vs = vp + i * 2 * kRowBytes;
                         if (kStep && p_app && r == last) {
                             ks = step.k_new + size_t(p_slab) * 16 + c_col;
@@ -295,12 +321,14 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
             for (int i = S + tid; i <= step.max_sent; i += kDecThreads) so[i] = new_len;
     };
 
-    const int g = lane >> 2, qd = lane & 3;               // mma fragments: row (head) g, columns 2 qd and 2 qd + 1
+    const int g = lane >> 2, qd = lane & 3;               // mma fragments: rows (tokens, channels) g and g + 8, columns (heads) 2 qd and 2 qd + 1
     const float qscale = 1.4426950408889634f * rsqrtf(float(kHeadDim));
+    const float2 qscale2 = make_float2(qscale, qscale);
     // this lane's row address offsets inside a stage for the matrix loads (K: token octets by the upper bit, V: by the lower)
     const int lm = lane >> 3, k_row = (lane & 7) + (lm >> 1) * 8, v_row = (lane & 7) + (lm & 1) * 8;
-    const uint32_t k_base = ring + k_row * kRowBytes, v_base = ring + (kWarpRows + v_row) * kRowBytes;
-    const int k_x = lm & 1, v_x = lm >> 1, sw = lane & 7;
+    // piece 2 ks + x of a row lies at (2 ks + x) ^ (row & 7): the addresses of steps 0 to 3 differ in two bits, steps 4 to 7 are 128 bytes on
+    const uint32_t k_base = ring + k_row * kRowBytes + (((lm & 1) ^ (lane & 7)) << 4);
+    const uint32_t v_base = ring + (kWarpRows + v_row) * kRowBytes + (((lm >> 1) ^ (lane & 7)) << 4);
 
     int slab = slab0, t = t_begin, c_stage = 0;
     while (t < t_end) {
@@ -322,17 +350,18 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
         }
         uint32_t qa[8][2];
         {
-            const uint32_t* qp = reinterpret_cast<const uint32_t*>(q + (size_t(b) * Hq + size_t(h) * n + min(g, n - 1)) * kHeadDim) + qd;
+            const int hd = kFew ? g & 3 : g;              // head of this lane's column
+            const uint32_t* qp = reinterpret_cast<const uint32_t*>(q + (size_t(b) * Hq + size_t(h) * n + min(hd, n - 1)) * kHeadDim) + qd;
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-                qa[ks][0] = g < n ? qp[ks * 8] : 0u;
-                qa[ks][1] = g < n ? qp[ks * 8 + 4] : 0u;
+                qa[ks][0] = hd < n ? qp[ks * 8] : 0u;
+                qa[ks][1] = hd < n ? qp[ks * 8 + 4] : 0u;
             }
         }
-        float acc[16][4];
+        float2 acc[8][2];                                 // channels 16 j + g and 16 j + 8 + g of the lane's two heads
 #pragma unroll
-        for (int j = 0; j < 16; ++j) { acc[j][0] = 0.f; acc[j][1] = 0.f; acc[j][2] = 0.f; acc[j][3] = 0.f; }
-        float m_run = -INFINITY, l_run = 0.f;
+        for (int j = 0; j < 8; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+        float2 m = make_float2(-INFINITY, -INFINITY), l = make_float2(0.f, 0.f);    // their running maximum, this lane's share of the sum
         int rows_left = n_rows - (t - pref[slab]) * kTileRows - warp * kWarpRows;     // of this warp's part of the tile
         for (; t < seg_end; ++t, rows_left -= kTileRows) {
             cp_async_wait<kStages - 2>();
@@ -341,60 +370,110 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
             maybe_trigger(t_end - t);
             if (rows_left > 0) {
                 const uint32_t stage = c_stage * kStageBytes;
-                float s[2][4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { s[0][k] = 0.f; s[1][k] = 0.f; }
+                float s[4][4];                            // four chains of two steps each
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
-                    uint32_t kb[4];
-                    ldmatrix4(k_base + stage + (((2 * ks + k_x) ^ sw) << 4), kb);
-                    mma16816(s[0], qa[ks][0], 0u, qa[ks][1], 0u, kb[0], kb[1]);
-                    mma16816(s[1], qa[ks][0], 0u, qa[ks][1], 0u, kb[2], kb[3]);
+                    uint32_t ka[4];
+                    ldmatrix4(((k_base + stage) ^ ((ks & 3) << 5)) + (ks >> 2) * 128, ka);
+                    if (ks < 4) mma16816_first(s[ks], ka[0], ka[2], ka[1], ka[3], qa[ks][0], qa[ks][1]);
+                    else        mma16816(s[ks - 4], ka[0], ka[2], ka[1], ka[3], qa[ks][0], qa[ks][1]);
                 }
-                // this lane's logits: head g, tokens 2 qd, 2 qd + 1, 8 + 2 qd, 9 + 2 qd
-                float x0 = s[0][0] * qscale, x1 = s[0][1] * qscale, x2 = s[1][0] * qscale, x3 = s[1][1] * qscale;
-                if (rows_left < kWarpRows) {
-                    if (2 * qd >= rows_left) x0 = -INFINITY;
-                    if (2 * qd + 1 >= rows_left) x1 = -INFINITY;
-                    if (2 * qd + 8 >= rows_left) x2 = -INFINITY;
-                    if (2 * qd + 9 >= rows_left) x3 = -INFINITY;
-                }
-                float bm = fmaxf(fmaxf(x0, x1), fmaxf(x2, x3));
-                bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
-                bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
-                const float m_new = fmaxf(m_run, bm);
-                if (__any_sync(0xffffffffu, m_new > m_run)) {
-                    const float sc = ex2(m_run - m_new);  // first rows: 2^(-inf) = 0
-                    l_run *= sc;
+                uint32_t va[8][4];
+                auto load_v = [&](int j) { ldmatrix4_trans(((v_base + stage) ^ ((j & 3) << 5)) + (j >> 2) * 128, va[j]); };
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) { acc[j][0] *= sc; acc[j][1] *= sc; acc[j][2] *= sc; acc[j][3] *= sc; }
-                    m_run = m_new;
+                for (int j = 0; j < 4; ++j) load_v(j);
+                // this lane's logits: tokens g and g + 8 of its two heads (packed fp32 arithmetic: a pair of heads per instruction)
+                auto sum = [&](int k) {
+                    return __fmul2_rn(__fadd2_rn(__fadd2_rn(make_float2(s[0][k], s[0][k + 1]), make_float2(s[1][k], s[1][k + 1])),
+                                                 __fadd2_rn(make_float2(s[2][k], s[2][k + 1]), make_float2(s[3][k], s[3][k + 1]))), qscale2);
+                };
+                float2 x = sum(0), y = sum(2);
+                if (rows_left < kWarpRows) {
+                    if (g >= rows_left) x = make_float2(-INFINITY, -INFINITY);
+                    if (g + 8 >= rows_left) y = make_float2(-INFINITY, -INFINITY);
                 }
-                const float p0 = ex2(x0 - m_run), p1 = ex2(x1 - m_run), p2 = ex2(x2 - m_run), p3 = ex2(x3 - m_run);
-                l_run += (p0 + p1) + (p2 + p3);
-                uint32_t a0, a1, a2, a3;
-                split_bf16(p0, p1, a0, a1);
-                split_bf16(p2, p3, a2, a3);
+                float2 top = make_float2(fmaxf(x.x, y.x), fmaxf(x.y, y.y)), sc = make_float2(1.f, 1.f);
+                if (__any_sync(0xffffffffu, top.x > m.x || top.y > m.y)) {
+#pragma unroll
+                    for (int d = 4; d < 32; d <<= 1) {
+                        top.x = fmaxf(top.x, __shfl_xor_sync(0xffffffffu, top.x, d));
+                        top.y = fmaxf(top.y, __shfl_xor_sync(0xffffffffu, top.y, d));
+                    }
+                    top = make_float2(fmaxf(top.x, m.x), fmaxf(top.y, m.y));
+                    sc = make_float2(ex2(m.x - top.x), ex2(m.y - top.y));   // first rows: 2^(-inf) = 0
+                    l = __fmul2_rn(l, sc);
+                    m = top;
+                }
+                const float2 neg = make_float2(-m.x, -m.y);
+                x = __fadd2_rn(x, neg); y = __fadd2_rn(y, neg);
+                x = make_float2(ex2(x.x), ex2(x.y)); y = make_float2(ex2(y.x), ex2(y.y));
+                l = __fadd2_rn(l, __fadd2_rn(x, y));
+                uint32_t hx, mx, lx, hy, my, ly;
+                split_bf16(x, hx, mx, lx);
+                split_bf16(y, hy, my, ly);
+                float d[8][4];
+                if (kFew) {
+                    const bool first = qd < 2;            // this lane's columns hold high parts (the others middle ones)
+                    const uint32_t hm0 = movmatrix_trans(first ? hx : mx), hm1 = movmatrix_trans(first ? hy : my);
+                    const uint32_t lo0 = movmatrix_trans(first ? lx : 0u), lo1 = movmatrix_trans(first ? ly : 0u);
+#pragma unroll
+                    for (int i = 0; i < 11; ++i) {
+                        if (i < 8) {
+                            mma16816_first(d[i], va[i][0], va[i][2], va[i][1], va[i][3], hm0, hm1);
+                            if (i < 4) load_v(i + 4);
+                        }
+                        if (i >= 3) { const int j = i - 3; mma16816(d[j], va[j][0], va[j][2], va[j][1], va[j][3], lo0, lo1); }
+                    }
+                } else {
+                    const uint32_t hi0 = movmatrix_trans(hx), hi1 = movmatrix_trans(hy);
+                    const uint32_t mi0 = movmatrix_trans(mx), mi1 = movmatrix_trans(my), lo0 = movmatrix_trans(lx), lo1 = movmatrix_trans(ly);
+#pragma unroll
+                    for (int i = 0; i < 12; ++i) {
+                        if (i < 8) {
+                            mma16816_first(d[i], va[i][0], va[i][2], va[i][1], va[i][3], hi0, hi1);
+                            if (i < 4) load_v(i + 4);
+                        }
+                        if (i >= 2 && i < 10) { const int j = i - 2; mma16816(d[j], va[j][0], va[j][2], va[j][1], va[j][3], mi0, mi1); }
+                        if (i >= 4) { const int j = i - 4; mma16816(d[j], va[j][0], va[j][2], va[j][1], va[j][3], lo0, lo1); }
+                    }
+                }
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    uint32_t vb[4];
-                    ldmatrix4_trans(v_base + stage + (((2 * j + v_x) ^ sw) << 4), vb);
-                    mma16816(acc[2 * j], a0, a1, a2, a3, vb[0], vb[1]);
-                    mma16816(acc[2 * j + 1], a0, a1, a2, a3, vb[2], vb[3]);
+                    acc[j][0] = __ffma2_rn(acc[j][0], sc, make_float2(d[j][0], d[j][1]));
+                    acc[j][1] = __ffma2_rn(acc[j][1], sc, make_float2(d[j][2], d[j][3]));
                 }
             }
             if (++c_stage == kStages) c_stage = 0;
         }
 
         // -------------------------------------------------------------- flush this (CTA, slab) segment
-        l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
-        l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
-        if (g < n) {
-            float* wp = wpart + (size_t(warp) * n + g) * kWpStride;
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-                *reinterpret_cast<float2*>(wp + j * 8 + 2 * qd) = make_float2(acc[j][0] + acc[j][2], acc[j][1] + acc[j][3]);
-            if (qd == 0) { wp[128] = m_run; wp[129] = l_run; }
+        for (int d = 4; d < 32; d <<= 1) {
+            l.x += __shfl_xor_sync(0xffffffffu, l.x, d);
+            l.y += __shfl_xor_sync(0xffffffffu, l.y, d);
+        }
+        if (kFew) {                                       // the same heads' middle parts
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    acc[j][k].x += __shfl_xor_sync(0xffffffffu, acc[j][k].x, 2);
+                    acc[j][k].y += __shfl_xor_sync(0xffffffffu, acc[j][k].y, 2);
+                }
+        }
+        if (!kFew || qd < 2) {
+            float* wp = wpart + (size_t(warp) * n + 2 * qd) * kWpStride;
+            if (2 * qd < n) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { wp[16 * j + g] = acc[j][0].x; wp[16 * j + 8 + g] = acc[j][1].x; }
+                if (g == 0) { wp[128] = m.x; wp[129] = l.x; }
+            }
+            wp += kWpStride;
+            if (2 * qd + 1 < n) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { wp[16 * j + g] = acc[j][0].y; wp[16 * j + 8 + g] = acc[j][1].y; }
+                if (g == 0) { wp[128] = m.y; wp[129] = l.y; }
+            }
         }
         __syncthreads();
         // merge the warps; thread -> channel
@@ -524,7 +603,8 @@ static int decode_impl(const skipkv_shape* shape, const void* q, const void* K, 
     }
     const int grid = num_sms() < kDecMaxGrid ? num_sms() : kDecMaxGrid;
     SKIPKV_CUDA(launch_dependent(
-        step.k_new ? decode_attn_kernel<true> : decode_attn_kernel<false>, dim3(grid), dim3(kDecThreads), smem,
+        L.group <= 4 ? (step.k_new ? decode_attn_kernel<true, true> : decode_attn_kernel<false, true>)
+                     : (step.k_new ? decode_attn_kernel<true, false> : decode_attn_kernel<false, false>), dim3(grid), dim3(kDecThreads), smem,
         static_cast<cudaStream_t>(stream), int(shape->batch), int(shape->n_q_heads), int(shape->n_kv_heads), int(L.slabs),
         static_cast<long long>(shape->total_rows), shape->slab_off, shape->cap, static_cast<const __nv_bfloat16*>(q),
         static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len, static_cast<__nv_bfloat16*>(out),
@@ -668,14 +748,15 @@ extern "C" int skipkv_decode_attn_static(const skipkv_shape* shape, const void* 
     const size_t smem = dec_smem_bytes(slabs, shape->n_q_heads / shape->n_kv_heads);
     unsigned char* base = nullptr;
     if (int rc = static_setup(dev, &base)) return rc;
-    SKIPKV_CUDA(allow_max_smem(reinterpret_cast<const void*>(decode_attn_kernel<false>)));
+    const auto kernel = shape->n_q_heads / shape->n_kv_heads <= 4 ? decode_attn_kernel<false, true> : decode_attn_kernel<false, false>;
+    SKIPKV_CUDA(allow_max_smem(reinterpret_cast<const void*>(kernel)));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // The array keeps whatever the previous call left: the status word and the arrival counters
     // must start at zero (the partial records are fully written before they are read).
     SKIPKV_CUDA(cudaMemsetAsync(base, 0, kStaticPartOff, st));
     const int grid = num_sms() < kStaticMaxCtas ? num_sms() : kStaticMaxCtas;
     uint32_t* status_word = status ? status : reinterpret_cast<uint32_t*>(base);
-    decode_attn_kernel<false><<<grid, kDecThreads, smem, st>>>(
+    kernel<<<grid, kDecThreads, smem, st>>>(
         shape->batch, shape->n_q_heads, shape->n_kv_heads, slabs, static_cast<long long>(shape->total_rows), shape->slab_off,
         shape->cap, static_cast<const __nv_bfloat16*>(q), static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len,
         static_cast<__nv_bfloat16*>(out), status_word, reinterpret_cast<uint32_t*>(base + kStaticCntOff),

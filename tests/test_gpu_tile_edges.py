@@ -117,3 +117,28 @@ def test_score_with_more_slabs_than_shared_memory_has_room_for(group, window, ba
         assert torch.equal(imp[b, :, :n].reshape(-1), D.tok_imp[off:off + 64 * n])
         for got, ref in zip(outs, (D.sent_imp, D.sent_red, D.sent_lam, D.sent_score)):
             assert torch.equal(got[b, :, :S], ref[b, :, :S])
+
+
+@pytest.mark.parametrize("hq,ctx", [(2, [30000, 23456]), (8, [4100, 9000, 20000]), (10, [16384, 8000]), (16, [2048, 12345])])
+def test_decode_keeps_fp32_probabilities(hq, ctx):
+    """The share of outputs that are not the exact result rounded to bf16.  A value with relative error e lies on the wrong side of
+    a rounding boundary with probability e times 2^8 (its bf16 ulps), about e * 2^10 on average over outputs that are normal
+    around zero.  Probabilities, logits and sums in fp32 (exponential 2 ulp, logits of up to 8 to 2^-22): e < 6e-7, a share of 6e-4;
+    probabilities of 16 bits: e = 2^-18, a share of 4e-3."""
+    B, L, D = layer(ctx, n_q_heads=hq, n_kv_heads=2, seed=330 + hq)
+    wrong = total = 0
+    for rep in range(8):
+        L["q"] = torch.randn(L["q"].shape, generator=torch.Generator().manual_seed(rep)).bfloat16()
+        D.q.copy_(L["q"])
+        D.decode_attn(steer=False)
+        torch.cuda.synchronize()
+        assert D.status() == 0
+        for b in range(len(ctx)):
+            for h in range(2):
+                n = int(L["kv_len"][b, h])
+                k, v = (t[W.slab_rows(L, b, h)][:n].double() for t in (D.K, D.V))
+                g = slice(h * hq // 2, (h + 1) * hq // 2)
+                ref = torch.softmax(D.q[b, g].double() @ k.T / 128 ** 0.5, -1) @ v
+                wrong += int((D.out[b, g] != ref.bfloat16()).sum())
+                total += ref.numel()
+    assert wrong <= 1e-3 * total + 3, (wrong, total)
