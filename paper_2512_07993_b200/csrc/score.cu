@@ -131,6 +131,11 @@ __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
     return uint64_t((smem_addr >> 4) & 0x3fffu) | (uint64_t(1) << 16) | (uint64_t(256 >> 4) << 32) | (uint64_t(1) << 46) | (uint64_t(6) << 61);
 }
 __device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
+// The logits of pass B are accumulated less (log-sum-exp - e), e = 1 + floor(log2 rows).  The difference lies between the row's mean
+// logit - 1 and its largest one (Jensen), so the sums keep the magnitude of the logits and stay about as often positive as negative;
+// the tensor core truncates when it adds.  With the whole log-sum-exp, 15 for 32K rows, they were ten times as large and all
+// negative, and every importance came out 9e-7 too large.  The factor 2^-e is exact and comes with the 1 / window.
+__device__ __forceinline__ int lse_shift(int rows) { return 32 - __clz(max(rows, 1)); }
 
 // ---- pass A epilogue: one accumulator (128 tokens) folded into a row's sum of 2^(logit - m).  The reference m is the
 // largest logit of the row's first 32 tokens; it stays, whatever comes later, as long as a chunk's sum is below 2^60 --
@@ -580,7 +585,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             int slab = slab_of(t_begin), lo = 0, hi = 0, N = 0;         // the slab's tiles are [lo, hi)
             uint32_t ext_no = 0;                             // slabs begun so far
             float *imp_ws = nullptr, *imp_user = nullptr;
-            const float inv_window = 1.f / float(a.window);
+            float out_scale = 0.f;                           // 2^-e / window of the slab
             int ti = 0, tk = 0;
             for (int it = 0; it < ntl * a.RB; ++it) {
                 const int t = t_begin + ti, i = ti, k = tk;
@@ -589,6 +594,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     while (pref[slab + 1] <= t) ++slab;
                     lo = pref[slab]; hi = pref[slab + 1];
                     N = live(slab);
+                    out_scale = __uint_as_float(uint32_t(127 - lse_shift(N)) << 23) / float(a.window);
                     imp_ws = a.tok_imp_ws + size_t(slab) * a.max_cap;
                     imp_user = a.tok_imp_user ? a.tok_imp_user + (a.block_table ? size_t(slab) * a.max_pages * 128 : size_t(rowb[slab])) : nullptr;
                     ++ext_no;
@@ -620,7 +626,10 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
 #pragma unroll
                                 for (int p = 0; p < 8; ++p) L += x[p].y > 0.f ? x[p].y * ex2f(x[p].x - M) : 0.f;
                             }
-                            const float v = L > 0.f ? -0.5f * (M + log2f(L)) / scale : 0.f;
+                            // (the exponent of the sum apart, so that neither its logarithm nor the total is rounded at a larger magnitude)
+                            const int ex = int(__float_as_uint(L) >> 23) - 127;
+                            const float mant = __uint_as_float((__float_as_uint(L) & 0x007fffffu) | 0x3f800000u);
+                            const float v = L > 0.f ? -0.5f * ((M + float(ex - lse_shift(N))) + log2f(mant)) / scale : 0.f;
                             const __nv_bfloat16 b0 = __float2bfloat16_rn(v);
                             const float v1 = v - __bfloat162float(b0);
                             const __nv_bfloat16 b1 = __float2bfloat16_rn(v1), b2 = __float2bfloat16_rn(v1 - __bfloat162float(b1));
@@ -657,7 +666,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 }
                 const int tok = (t - lo) * 128 + row;
                 if (k + 1 == a.RB && ok && tok < N) {
-                    const float v = total * inv_window;
+                    const float v = total * out_scale;
                     imp_ws[tok] = v;
                     if (imp_user) imp_user[tok] = v;
                 }

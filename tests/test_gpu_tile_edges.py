@@ -142,3 +142,24 @@ def test_decode_keeps_fp32_probabilities(hq, ctx):
                 wrong += int((D.out[b, g] != ref.bfloat16()).sum())
                 total += ref.numel()
     assert wrong <= 1e-3 * total + 3, (wrong, total)
+
+
+@pytest.mark.parametrize("group,window,ctx", [(4, 32, [2048, 1500]), (4, 32, [20000, 30011]), (5, 64, [40000]), (8, 16, [700, 9000])])
+def test_score_importance_keeps_fp32_logits(group, window, ctx):
+    """Error of the token importances against 64 bits (2-norm over a slab's tokens).  A probability 2^x is off by ln 2 times the error of x: a
+    logit of up to 32 raw units, truncated a few times at 2^-19, times 0.13 for base 2: 3e-7 at most; its row's log-sum-exp 2^-22; the
+    exponential 2^-22 of itself.  The mean over the window's 16 rows and more makes that 1e-7 where the errors of the rows are independent.
+    A sum that holds the whole log-sum-exp (120 raw units), or a logarithm of the whole sum (10 and more, to 2^-22 of itself), is off by the
+    same amount in all rows: 4e-7 to 9e-7."""
+    B, L, D = layer(ctx, n_q_heads=2 * group, n_kv_heads=2, window=window, sent_lo=8, sent_hi=60, seed=950 + group)
+    D.score()
+    torch.cuda.synchronize()
+    assert D.status() == 0
+    for b in range(len(ctx)):
+        for h in range(2):
+            rows, n = W.slab_rows(L, b, h), int(L["kv_len"][b, h])
+            k = D.K[rows][:n].double()
+            q = D.q_win[b, h * group:(h + 1) * group].double().reshape(group * window, 128)
+            ref = torch.softmax(q @ k.T / 128 ** 0.5, -1).view(group, window, n).amax(0).mean(0)
+            err = (D.tok_imp[rows][:n].double() - ref).norm() / ref.norm()
+            assert err <= 2e-7, (b, h, float(err))
