@@ -4,15 +4,19 @@
 //     G_ij  = K_i . K_j / ((|K_i| + eps)(|K_j| + eps))
 //     Z_j   = sum_{k != j} exp(G_jk)
 //     R_i   = (1/N') sum_{j != i} exp(G_ji) / Z_j
-// Three launches:
+// Four launches:
 //   token_norm_kernel      1 / (|K_t| + eps) of every live row (a warp per row); clears Z and R;
 //   token_red_kernel<1>    row sums Z;
-//   token_red_kernel<2>    R.
+//   token_red_kernel<2>    R, without the 1/N' and less its mean;
+//   token_mean_kernel      both.
 // G is symmetric, so every pair of 128-row blocks {I, J} is multiplied and exponentiated once: the tile gives the
 // rows of I their sums over the columns and the rows of J theirs as column sums.  A work item is block J of a slab as
 // columns against itself and the blocks after it as rows, cyclically, half-way round: every pair once, all items of a
 // slab equally long.  Z and R are accumulated with floating-point reductions: sums agree to rounding, not to the bit,
-// from run to run.
+// from run to run.  A value of R gets about N/64 contributions, each of which would be rounded at the magnitude of the sum; so every
+// contribution comes less tr_mean(N), about 1/N, for each of its terms, what is accumulated stays small, and token_mean_kernel
+// adds what was left out: error against 64 bits 8.6e-8 -> 2.3e-8 at 4224 rows, 1.27e-7 -> 3.5e-8 at 7611 (one reduction after the other
+// from zero; with half as many of them it had been 5.8e-8 and 9.0e-8), for 617 -> 628 us (80 slabs x 4224 rows).
 // The Gram kernels are persistent and warp-specialised.  Warp 0 streams the bf16 key tiles straight from the cache
 // with tiled TMA loads (the J tile once per item, the I tiles through a ring), warps 1 and 2 issue one
 // 128 x 128 x 128 tcgen05.mma group per block pair in turn into one of four tensor-memory accumulators (a single issuer
@@ -26,7 +30,7 @@
 // warp) and about one instruction of overhead; the schedulers issue on 6 clocks of 10.  Four warps per scheduler hide the latencies
 // of these short chains, two with 64 columns each do not (326 us a pass); a share of the exponentials as polynomials adds more
 // issue slots than it takes off the special-function unit.  80 slabs x 4224 keys, both passes and the norms: 804 -> 617 us
-// back to back (558 in a short burst: the clock falls under the power limit).
+// back to back (558 in a short burst: the clock falls under the power limit), before the mean was kept apart.
 #include "tc.cuh"
 
 namespace skipkv {
@@ -50,6 +54,8 @@ __device__ __forceinline__ int tr_count(int NB, int I) {
     const int half = NB >> 1;
     return (NB & 1) ? 1 + half : half + (I < half ? 1 : 0);
 }
+// 1/N to 12 bits, so that a few thousand times it is exact.
+__device__ __forceinline__ float tr_mean(int N) { return __uint_as_float(__float_as_uint(1.f / float(max(N, 1))) & 0xfffff000u); }
 __device__ __forceinline__ float tr_ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -240,7 +246,7 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
             __syncwarp();
 #pragma unroll
             for (int k = 0; k < 16; ++k) cs[k] = make_float2(0.f, 0.f);
-            const float inv_S = 1.f / float(max(x.S, 1));
+            const float row_mean = kPass == 2 ? float(min(max(x.S - x.J * 128 - c0, 0), 32)) * tr_mean(x.S) : 0.f;   // of this warp's columns
             float* dst = kPass == 1 ? z + x.sbase : tok_red + row0_of(slab);
             const int j0 = x.J * 128 + c0;
             int i = x.J * 128 + quarter * 32 + lane;
@@ -267,7 +273,7 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
                     break;
                 }
                 const bool interior = full && t > 0 && i - lane + 32 <= x.S;
-                float2 row = make_float2(0.f, 0.f);
+                float2 row = make_float2(-row_mean, 0.f);
                 float v[32];
                 tmem_ld32(lane_addr + acc * 128, v);
                 tc_fence_before();
@@ -300,7 +306,7 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
                     }
                 }
                 // (the block against itself is symmetric: its column sums are all there is to it)
-                if (t > 0 && i < x.S) atomicAdd(dst + i, kPass == 1 ? row.x + row.y : (row.x + row.y) * inv_S);
+                if (t > 0 && i < x.S) atomicAdd(dst + i, row.x + row.y);
                 i = i_next;
                 ++tfull;
                 if (++acc == kTrAcc) { acc = 0; tfull = ctl->tfull; parity ^= 1u; }
@@ -310,8 +316,12 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
                 float s[32];
 #pragma unroll
                 for (int k = 0; k < 16; ++k) { s[2 * k] = cs[k].x; s[2 * k + 1] = cs[k].y; }
-                const float sum = col_reduce32(s, lane);
-                if (j0 + lane < x.S) atomicAdd(dst + j0 + lane, kPass == 1 ? sum : sum * inv_S);
+                float sum = col_reduce32(s, lane);
+                if (kPass == 2) {                            // this warp's rows in the item's blocks, the last of which may be partly filled, less the token itself
+                    const int short_of = x.J + x.NJ >= x.NB ? 32 - min(max(x.S - (x.NB - 1) * 128 - quarter * 32, 0), 32) : 0;
+                    sum -= float(32 * x.NJ - short_of - (quarter * 32 == c0 ? 1 : 0)) * tr_mean(x.S);
+                }
+                if (j0 + lane < x.S) atomicAdd(dst + j0 + lane, sum);
             }
         }
     }
@@ -321,6 +331,20 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
         tc_fence_after();
         tmem_dealloc(tmem_base, 128 * kTrAcc);
     }
+}
+
+__global__ void __launch_bounds__(256)
+token_mean_kernel(int Hk, int max_cap, const int64_t* slab_off, const int32_t* cap, const int32_t* kv_len, float* tok_red) {
+    pdl_trigger();
+    pdl_wait();
+    const int slab = blockIdx.y, t0 = blockIdx.x * 1024 + threadIdx.x;
+    const int len = min(max(kv_len[slab], 0), min(cap[slab / Hk], max_cap));
+    float* dst = tok_red + slab_row0(slab_off, cap, Hk, slab / Hk, slab % Hk);
+    if (len == 0) return;
+    const double rest = double(len - 1) * double(tr_mean(len)), inv = 1.0 / double(len);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (t0 + k * 256 < len) dst[t0 + k * 256] = float((double(dst[t0 + k * 256]) + rest) * inv);
 }
 
 }  // namespace skipkv
@@ -362,5 +386,7 @@ extern "C" int skipkv_token_redundancy(const skipkv_shape* shape, const skipkv_p
         SKIPKV_CUDA(launch_dependent(kernel, dim3(grid), dim3(kTrThreads), smem, st, mapK, int(L.slabs), Hk, int(shape->max_cap),
                                      shape->slab_off, shape->cap, kv_len, static_cast<const float*>(inv_norm), z, tok_red, hdr, table));
     }
+    SKIPKV_CUDA(launch_dependent(token_mean_kernel, dim3((shape->max_cap + 1023) / 1024, L.slabs), dim3(256), 0, st, Hk, int(shape->max_cap),
+                                 shape->slab_off, shape->cap, kv_len, tok_red));
     return SKIPKV_OK;
 }
