@@ -214,6 +214,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
     if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(bar, parity, limit);
 }
+// Polls that a thread makes for its own copies and products in flight before its CTA gives shared and tensor memory back.  Whatever else
+// gave up, these complete by themselves, so the wait is not subject to the workspace's limit; without a failure it costs nothing.
+constexpr uint32_t kRetirePolls = 1u << 20;
 // global -> shared, completion counted in bytes on an mbarrier.  16-byte aligned, size % 16 == 0.
 __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
     asm volatile(

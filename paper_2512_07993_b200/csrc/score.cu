@@ -67,7 +67,7 @@ struct SweepCtl {                       // barriers and small shared state, afte
     // ring of indicator matrices: written by the four pooling warps -> multiplied by their issuer -> read out by the pooling warps
     uint64_t ifull[kIndRing], iempty[kIndRing];
     uint64_t pfull[2];                  // the last product of a run of tiles into accumulator i has completed
-    uint64_t issued_done[3];            // after a failed wait: every product of the MMA warps (0, 1) / the pooling issuer (2) has retired
+    uint64_t retired[3];                // every product of the MMA warps (0, 1) / the pooling issuer (2) has completed
     uint32_t tmem_base;
     int abort_flag;
     int ind_flags[kIndRing];            // 1: the tile has another matrix after this one, 2: joins the open run, 4: closes a run
@@ -299,7 +299,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         mbar_init(&ctl->extempty, 2);
         for (int i = 0; i < kIndRing; ++i) { mbar_init(&ctl->ifull[i], kPoolWarps); mbar_init(&ctl->iempty[i], 1); }
         for (int i = 0; i < 2; ++i) mbar_init(&ctl->pfull[i], 1);
-        for (int i = 0; i < 3; ++i) mbar_init(&ctl->issued_done[i], 1);
+        for (int i = 0; i < 3; ++i) mbar_init(&ctl->retired[i], 1);
         ctl->abort_flag = 0;
         mbar_fence_init();
         tmap_prefetch(&mapK);
@@ -389,12 +389,14 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     if (pass == 0 || !resident) load_tile(slab, t - lo, row0);
                 }
             }
-            if (!ok) {
-                // copies already issued must land before the CTA retires
-                for (int s = 0; s < a.stages; ++s) { mbar_wait(&ctl->full[s], 0u, 1u << 16); mbar_wait(&ctl->full[s], 1u, 1u << 16); }
-                mbar_wait(&ctl->qfull, 0u, 1u << 16);
-                mbar_wait(&ctl->qfull, 1u, 1u << 16);
+            // Whoever gave up: this warp stays until its copies have landed and the issuers' products have completed, so that the CTA gives
+            // back shared and tensor memory with nothing in flight.  Stage s was loaded lap (+ 1) times.
+            for (int s = 0; s < a.stages; ++s) {
+                const uint32_t loads = lap + (s < stage ? 1u : 0u);
+                if (loads) mbar_wait(&ctl->full[s], (loads - 1) & 1u, kRetirePolls);
             }
+            if (qlap) mbar_wait(&ctl->qfull, (qlap - 1) & 1u, kRetirePolls);
+            for (int s = 0; s < 3; ++s) mbar_wait(&ctl->retired[s], 0u, kRetirePolls);
         }
     } else if (warp == 1 || warp == 19) {
         // ------------------------------------------------------------------ MMA warps
@@ -442,7 +444,6 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 }
                 if (++stage == a.stages) { stage = 0; ++lap; }
             }
-            if (!ok) { umma_commit(&ctl->issued_done[mine]); mbar_wait(&ctl->issued_done[mine], 0u, 1u << 18); }
         }
         __syncwarp();
         tc_fence_before();
@@ -481,12 +482,8 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 if (here) umma_commit(&ctl->empty[stage]);
                 if (++stage == a.stages) { stage = 0; ++lap; }
             }
-            if (!ok) {
-                // nobody will wait for the products still in flight: let them retire before the tensor memory is released
-                umma_commit(&ctl->issued_done[mine]);
-                mbar_wait(&ctl->issued_done[mine], 0u, 1u << 18);
-            }
         }
+        if (lane == 0) umma_commit(&ctl->retired[mine]);
     } else {
         // ------------------------------------------------------------------ pass A: epilogue warpgroups (and the clearing warp)
         const int quarter = warp & 3;                        // tensor-memory lanes this warp may read
@@ -837,10 +834,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     if (++stage == a.stages) stage = 0;
                 }
                 if (ok && run >= 0) umma_commit(&ctl->pfull[run & 1]);
-                if (!ok) {
-                    umma_commit(&ctl->issued_done[2]);
-                    mbar_wait(&ctl->issued_done[2], 0u, 1u << 18);
-                }
+                umma_commit(&ctl->retired[2]);
             }
         }
     }
@@ -956,6 +950,8 @@ struct GramCtl {
     int abort_flag, last;
     uint32_t wsum[32];
     alignas(16) float colz[16][32];          // pass 2, by epilogue warp: 1 / Z_j of its columns
+    uint64_t retired[2];                     // every product of an MMA warp has completed
+    uint32_t loads[6];                       // by slot and part: copies issued (in shared memory for want of registers)
 };
 constexpr int kGramThreads = 20 * 32;        // TMA warp, two MMA warps, one idle, four epilogue warpgroups
 static size_t gram_smem_bytes(int slabs) { return 1024 + 6 * size_t(kOpBytes) + sizeof(GramCtl) + size_t(slabs + 1) * 4; }
@@ -1032,7 +1028,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
             for (int part = 0; part < 2; ++part) { mbar_init(&ctl->full[s][part], 1); mbar_init(&ctl->empty[s][part], 1); }
             mbar_init(&ctl->ddone[s], 1);
         }
-        for (int s = 0; s < 2; ++s) mbar_init(&ctl->turn[s], 1);
+        for (int s = 0; s < 2; ++s) { mbar_init(&ctl->turn[s], 1); mbar_init(&ctl->retired[s], 1); }
         for (int s = 0; s < kGramAcc; ++s) { mbar_init(&ctl->tfull[s], 1); mbar_init(&ctl->tempty[s], 16); }
         ctl->abort_flag = 0;
         mbar_fence_init();
@@ -1055,6 +1051,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
         if (warp == 0 && lane == 0) {
             bool ok = true;
             uint32_t ipar = 0, lasti = 0, dpar = 0, lastd = 0;         // bits by slot
+            ctl->loads[0] = ctl->loads[1] = ctl->loads[2] = ctl->loads[3] = ctl->loads[4] = ctl->loads[5] = 0;
             GramWalk w;
             w.start(ipref, first, count);
             auto load = [&](int s, int block) {
@@ -1071,6 +1068,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                     mbar_expect_tx(&ctl->full[s][part], kOpBytes);
                     tma_load_2d(dst, map, 0, row, &ctl->full[s][part]);
                     tma_load_2d(dst + kOpHalfBytes, map, 64, row, &ctl->full[s][part]);
+                    ++ctl->loads[2 * s + part];
                 }
             };
             bool fresh = true;
@@ -1092,9 +1090,12 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 }
                 fresh = w.next(ipref);
             }
-            if (!ok)                                     // let the copies in flight land before the CTA exits
-                for (int s = 0; s < 3; ++s)
-                    for (int part = 0; part < 2; ++part) { mbar_wait(&ctl->full[s][part], 0u, 1u << 16); mbar_wait(&ctl->full[s][part], 1u, 1u << 16); }
+            // Whoever gave up: this warp stays until its copies have landed and the issuers' products have completed, so that the CTA gives
+            // back shared and tensor memory with nothing in flight.
+            for (int s = 0; s < 3; ++s)
+                for (int part = 0; part < 2; ++part)
+                    if (ctl->loads[2 * s + part]) mbar_wait(&ctl->full[s][part], (ctl->loads[2 * s + part] - 1) & 1u, kRetirePolls);
+            for (int s = 0; s < 2; ++s) mbar_wait(&ctl->retired[s], 0u, kRetirePolls);
         } else if ((warp == 1 || warp == 2) && lane == 0) {
             // A pair each in turn, so that one waits for its operands while the other's products run.  The turn is handed over a little
             // before a pair's last instructions are issued.  It comes before the other waits: every barrier's earlier phases have been seen by then.
@@ -1139,6 +1140,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 umma_commit(&ctl->tfull[acc]);
                 umma_commit(diag ? &ctl->ddone[js] : &ctl->empty[is][0]);
             }
+            umma_commit(&ctl->retired[me]);
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
@@ -1408,7 +1410,11 @@ score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const i
         umma_commit(&ctl->done);
     }
     const bool ok = mbar_wait(&ctl->done, 0u, load_wait_limit(hdr));
-    if (!ok && lane == 0) atomicOr(const_cast<uint32_t*>(&hdr->status), SKIPKV_STATUS_COPY_TIMEOUT);
+    if (!ok) {                                           // the outputs are skipped, but the product retires before it is read or released
+        if (lane == 0) atomicOr(const_cast<uint32_t*>(&hdr->status), SKIPKV_STATUS_COPY_TIMEOUT);
+        mbar_wait(&ctl->done, 0u, kRetirePolls);
+    }
+    __syncwarp();
     tc_fence_after();
     // ---- thread: row i, 32 columns; four warps share a row
     const int part = warp >> 2, i = (warp & 3) * 32 + lane, c0 = part * 32;

@@ -105,3 +105,41 @@ def test_compaction_wait_runs_out_and_recovers():
             rows = W.slab_rows(L, b, h)
             n = int(cp["kv_len"][b, h])
             assert np.array_equal(Kg[rows][:n], cp["K"][rows][:n]) and np.array_equal(Vg[rows][:n], cp["V"][rows][:n])
+
+
+def run_out_and_recover(B, D, call, outputs):
+    """`call` under ever larger wait limits: it returns, reports what ran out or gives the default's bits, and after a fresh workspace the
+    default's bits come again.  Returns how many of the calls timed out."""
+    def result():
+        for t in outputs:
+            t.fill_(float("nan"))
+        call()
+        torch.cuda.synchronize()                            # the kernels came back
+        return B.skipkv_status(D.ws, raise_on_error=False), [t.clone() for t in outputs]
+    same = lambda x, y: all(torch.equal(a.view(torch.int32), b.view(torch.int32)) for a, b in zip(x, y))
+    bits, ref = result()
+    assert bits == 0
+    timed_out = 0
+    for limit in (1, 1, 1, 2, 4, 16, 64, 256):
+        B.skipkv_workspace_init(D.shape, D.ws)
+        B.skipkv_set_wait_limit(D.ws, limit)
+        bits, got = result()
+        assert bits in (0, COPY_TIMEOUT), hex(bits)
+        assert bits or same(got, ref), limit
+        timed_out += bits != 0
+        B.skipkv_workspace_init(D.shape, D.ws)              # (and the default limit)
+        bits, got = result()
+        assert bits == 0 and same(got, ref), limit
+    return timed_out
+
+
+@pytest.mark.parametrize("sent_lo,sent_hi,window,group", [(90, 130, 32, 4), (8, 40, 32, 4), (8, 40, 64, 5)])
+def test_score_waits_run_out_and_recover(sent_lo, sent_hi, window, group):
+    """Up to 128 sentences per slab and more (the one kernel behind the sweep, the Gram kernels), one and several query blocks: the sweep's CTAs wait for
+    one another's records, its roles and those of the kernels behind it for copies and products."""
+    cfg = W.config(1, name="timeout-score", batch=2, ctx_lo=6000, ctx_hi=9000, n_q_heads=8 * group, window=window, sent_lo=sent_lo, sent_hi=sent_hi,
+                   seed=43)
+    L, D, B = layer(cfg)
+    assert (int(L["n_sent"].max()) > 128) == (sent_hi <= 40)
+    # (one poll is less than a copy takes, and less than the sweep's slowest CTA is behind: six and seven of the eight run out)
+    assert run_out_and_recover(B, D, D.score, [D.tok_imp, D.sent_imp, D.sent_red, D.sent_lam, D.sent_score]) > 0
