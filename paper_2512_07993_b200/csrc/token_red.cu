@@ -46,6 +46,7 @@ struct TrCtl {
     int abort_flag;
     uint32_t wsum[32];
     alignas(16) float col[16][2][32];        // by epilogue warp: log2(e) / (|K_j| + eps) of its columns; pass 2: 1 / Z_j
+    uint64_t retired[2];                     // every product of an MMA warp has completed
 };
 constexpr size_t kTrSmem = 1024 + (2 + kTrStages) * size_t(kOpBytes) + sizeof(TrCtl);          // and the table of slabs behind it
 
@@ -119,7 +120,7 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
     pdl_trigger();
 
     if (tid == 0) {
-        for (int s = 0; s < 2; ++s) { mbar_init(&ctl->jfull[s], 1); mbar_init(&ctl->jempty[s], 2); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&ctl->jfull[s], 1); mbar_init(&ctl->jempty[s], 2); mbar_init(&ctl->retired[s], 1); }
         for (int s = 0; s < kTrStages; ++s) { mbar_init(&ctl->ifull[s], 1); mbar_init(&ctl->iempty[s], 1); }
         for (int s = 0; s < kTrAcc; ++s) { mbar_init(&ctl->tfull[s], 1); mbar_init(&ctl->tempty[s], 16); }
         ctl->abort_flag = 0;
@@ -176,10 +177,13 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
                     if (++I == x.NB) I = 0;
                 }
             }
-            if (!ok) {                                   // let the copies in flight land before the CTA exits
-                for (int s = 0; s < 2; ++s) { mbar_wait(&ctl->jfull[s], 0u, 1u << 16); mbar_wait(&ctl->jfull[s], 1u, 1u << 16); }
-                for (int s = 0; s < kTrStages; ++s) { mbar_wait(&ctl->ifull[s], 0u, 1u << 16); mbar_wait(&ctl->ifull[s], 1u, 1u << 16); }
-            }
+            // Whoever gave up: this warp stays until its copies have landed and the issuers' products have completed, so that the CTA gives
+            // back shared and tensor memory with nothing in flight.
+            for (uint32_t s = 0; s < 2; ++s)
+                if (ic > s) mbar_wait(&ctl->jfull[s], ((ic - 1 - s) >> 1) & 1u, kRetirePolls);
+            for (uint32_t s = 0; s < kTrStages; ++s)
+                if (bc > s) mbar_wait(&ctl->ifull[s], ((bc - 1 - s) / kTrStages) & 1u, kRetirePolls);
+            for (int s = 0; s < 2; ++s) mbar_wait(&ctl->retired[s], 0u, kRetirePolls);
         } else if ((warp == 1 || warp == 2) && lane == 0) {
             // two issuers, a tile each in turn (stages and accumulators are four: each is always the same issuer's)
             const uint32_t me = warp - 1;
@@ -204,6 +208,7 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
                 }
                 if (ok) umma_commit(&ctl->jempty[ic & 1]);           // every product of this issuer that reads the column tile has completed
             }
+            umma_commit(&ctl->retired[me]);
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");

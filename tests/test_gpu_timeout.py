@@ -143,3 +143,28 @@ def test_score_waits_run_out_and_recover(sent_lo, sent_hi, window, group):
     assert (int(L["n_sent"].max()) > 128) == (sent_hi <= 40)
     # (one poll is less than a copy takes, and less than the sweep's slowest CTA is behind: six and seven of the eight run out)
     assert run_out_and_recover(B, D, D.score, [D.tok_imp, D.sent_imp, D.sent_red, D.sent_lam, D.sent_score]) > 0
+
+
+def test_token_redundancy_waits_run_out_and_recover():
+    """The result is accumulated with reductions in no fixed order: equal to rounding."""
+    cfg = W.config(1, name="timeout-token-red", batch=2, ctx_lo=3000, ctx_hi=4224, seed=44)
+    L, D, B = layer(cfg)
+    red = torch.empty(D.K.shape[0], device="cuda")
+    def result(limit):
+        B.skipkv_workspace_init(D.shape, D.ws)
+        B.skipkv_set_wait_limit(D.ws, limit)
+        red.fill_(float("nan"))
+        B.skipkv_token_redundancy(D.shape, D.params, D.K, D.kv_len, red, D.ws)
+        torch.cuda.synchronize()                            # the kernels came back
+        return B.skipkv_status(D.ws, raise_on_error=False), red.clone()
+    bits, ref = result(0)
+    assert bits == 0 and bool(torch.isfinite(ref).all())
+    timed_out = 0
+    for limit in (1, 1, 1, 2, 4, 16, 64, 256):
+        bits, got = result(limit)
+        assert bits in (0, COPY_TIMEOUT), hex(bits)
+        timed_out += bits != 0
+        assert bits or torch.allclose(got, ref, rtol=1e-5, atol=0), limit
+        bits, got = result(0)
+        assert bits == 0 and torch.allclose(got, ref, rtol=1e-5, atol=0), limit
+    assert timed_out > 0                                    # (five of the eight run out)
