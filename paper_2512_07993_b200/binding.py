@@ -14,6 +14,8 @@ from typing import Optional
 
 import torch
 
+from .build import built_for
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libskipkv.so")
 _lib = None
@@ -73,6 +75,9 @@ def _load_native():
     spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
+    made_for = getattr(mod, "built_for", "an unknown version")
+    if made_for != built_for():
+        raise RuntimeError(f"{path} is built for {made_for}, this is {built_for()}: run `python -m paper_2512_07993_b200.build`")
     _native = mod
     return mod
 

@@ -22,10 +22,16 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def built_for() -> str:
+    """The Python and torch that ``_native.so`` is built for: it unpacks their objects, whose layout belongs to one version each."""
+    import torch
+    return f"python {sys.version_info[0]}.{sys.version_info[1]}, torch {torch.__version__}"
+
+
 def source_hash() -> str:
-    """Content hash of everything the library is built from (mtimes do not survive a copy)."""
+    """Content hash of everything the two files are built from (mtimes do not survive a copy)."""
     import hashlib
-    h = hashlib.sha256(" ".join(FLAGS[:8]).encode())
+    h = hashlib.sha256((" ".join(FLAGS[:8]) + built_for()).encode())
     deps = sources() + [EXT_SRC] + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + sorted(glob.glob(os.path.join(ROOT, "include", "*.h")))
     for p in deps:
         h.update(os.path.basename(p).encode())
@@ -48,7 +54,7 @@ def _ext_command(out: str):
            *cpp_extension.include_paths()]
     torch_lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in inc), EXT_SRC, "-o", out,
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DSKIPKV_BUILT_FOR="{built_for()}"', *(f"-I{d}" for d in inc), EXT_SRC, "-o", out,
             f"-L{HERE}", "-l:libskipkv.so", "-Wl,-rpath,$ORIGIN", f"-L{torch_lib}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 

@@ -147,4 +147,8 @@ PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_native", "Marshalling of the 
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__native(void) { return PyModule_Create(&module_def); }
+PyMODINIT_FUNC PyInit__native(void) {
+    PyObject* m = PyModule_Create(&module_def);
+    if (m && PyModule_AddStringConstant(m, "built_for", SKIPKV_BUILT_FOR) < 0) Py_CLEAR(m);      // the caller compares it with what runs
+    return m;
+}

@@ -78,3 +78,18 @@ def test_binding_fails_loudly_without_library(binding, monkeypatch):
     monkeypatch.setattr(binding, "LIB_PATH", "/nonexistent/libskipkv.so")
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         binding.lib()
+
+
+def test_extension_belongs_to_one_torch_and_python(binding, monkeypatch):
+    """After an upgrade of torch the build is stale, and an extension that was not rebuilt is refused at load."""
+    import torch
+    from paper_2512_07993_b200 import build
+    assert not build.stale()
+    monkeypatch.setattr(binding, "_native", None)
+    assert binding._load_native().built_for == build.built_for()
+    monkeypatch.setattr(torch, "__version__", "9.9.9")
+    assert build.stale()
+    monkeypatch.setattr(binding, "_native", None)
+    with pytest.raises(RuntimeError, match="built for python"):
+        binding._load_native()
+    assert binding._native is None
