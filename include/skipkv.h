@@ -100,8 +100,8 @@ int skipkv_workspace_init(const skipkv_shape* shape, void* ws, void* stream);
 /* Set how many times a bounded device wait polls before it gives up and records SKIPKV_STATUS_*_TIMEOUT in the
  * status word (every wait inside the kernels is bounded: a copy that never lands, or a hand-off another thread
  * block never makes, ends the wait instead of hanging the GPU).  polls = 0 restores the default (about four
- * million polls, seconds of waiting).  The value lives in the workspace, survives skipkv_workspace_init, and is
- * read by the kernels enqueued after this call on `stream`.  ws: device. */
+ * million polls, seconds of waiting).  The value lives in the workspace, is read by the kernels enqueued after this
+ * call on `stream`, and goes back to the default with skipkv_workspace_init.  ws: device. */
 int skipkv_set_wait_limit(void* ws, uint32_t polls, void* stream);
 
 /* Self-check of the time-out path: enqueues one warp that waits, bounded by the workspace's wait limit, for an

@@ -3,7 +3,7 @@
 //   sweeps    (one launch) pass A: log-sum-exp of every window-query row over the slab's tokens
 //             (tensor cores: logits = Q_rows x K_tile^T, one thread per query row);
 //             pass B: tok_imp[t] = (1/alpha) sum_w max_q 2^(s_q[w][t] - lse_q[w])   (max before exp: exp is monotone)
-//             (tensor cores: logits - lse = [K_tile, 1] x [Q_block, -lse]^T, one thread per token), and in the same pass
+//             (tensor cores: logits - (lse - e) = [K_tile, 1] x [Q_block, e - lse]^T, one thread per token; e: see lse_shift), and in the same pass
 //             the per-sentence sums of the key rows as a second product on the tile already in shared
 //             memory: K_tile^T x (0/1 matrix token -> sentence slot)
 //   up to 128 sentences per slab: one kernel for the rest, else
@@ -16,8 +16,8 @@
 // needs no max subtraction.
 //
 // The sweeps are a persistent, warp-specialised kernel, one CTA per SM: a TMA warp streams 128-token key tiles (and the
-// group's query rows) into shared memory, one thread issues tcgen05.mma into a ring of tensor-memory accumulators,
-// warpgroups of epilogue warps take the tiles round-robin, and (pass B) one more warpgroup writes the 0/1
+// group's query rows) into shared memory, two threads in two warps issue tcgen05.mma in turn into a ring of tensor-memory accumulators,
+// epilogue warpgroups take the products round-robin (four in pass A, three in pass B), and in pass B one more warpgroup writes the 0/1
 // matrices of the pooling product and reads out the pooled sums while one thread of a further warp issues
 // that product.  Work is the list of 128-token tiles over all slabs cut into equal contiguous ranges, so
 // ragged slabs balance.
@@ -936,9 +936,10 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const in
 // rows x 32 columns of every accumulator each, column sums in registers for as long as J stays.
 // Three shared-memory slots hold a block's high and low parts.  One is J's, the other two take the I blocks in turn; the next J takes
 // the slot that is free next and the old J's goes to the end of the queue, so a change of J costs no drain.
-// Bound by shared memory where there are many sentences: the three products of a pair stream 192 KB of operands in 1536 clocks,
-// the port's 128 bytes per clock, and the next block's 64 KB are written through the same port; under a sustained load the clock falls with the
-// power limit, and half the products is the larger gain.  128 slabs x 2K sentences, the whole scoring call: 2319 -> 2190 us against all pairs twice.
+// Bound by its epilogue: 2.3 and 2.9 us a pair (passes 1 and 2, about 130 pairs per SM) against 0.8 us for the three products, which stream
+// 192 KB of operands at the shared-memory port's 128 bytes per clock.  The four warps of a scheduler are in the same phase of the
+// same pair, and column sums leave no registers for two pairs at once.  Half the products and half the exponentials of evaluating
+// all pairs twice: 128 slabs x 2K sentences, the whole scoring call: 2319 -> 2190 us.
 // ---------------------------------------------------------------------------------------
 constexpr int kGramAcc = 4;
 struct GramCtl {
