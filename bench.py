@@ -359,8 +359,8 @@ def time_extras(cfg, B, flush, clean, peaks, reps=10):
     out["token_redundancy"] = {"us": us, "rows_per_slab": n_tok, "bound": "alu", "achieved": exps / us / 1e6,
                                "peak": mufu_peak, "unit": "T exp/s", "frac": exps / us / 1e6 / mufu_peak,
                                "matrix_elements_T_per_s": elems / us / 1e6, "tensor_tflops": exps * 256 / us / 1e6,
-                               "note": "each block pair is evaluated once; the column sums (a butterfly per 32 columns) "
-                                       "make the issue slots, not the exponentials, the limit"}
+                               "note": "each block pair is evaluated once; the issue slots of the epilogue, not the "
+                                       "exponentials, are the limit"}
     return out
 
 

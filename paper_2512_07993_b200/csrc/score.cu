@@ -936,7 +936,7 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const in
 // rows x 32 columns of every accumulator each, column sums in registers for as long as J stays.
 // Three shared-memory slots hold a block's high and low parts.  One is J's, the other two take the I blocks in turn; the next J takes
 // the slot that is free next and the old J's goes to the end of the queue, so a change of J costs no drain.
-// Bound by its epilogue: 2.3 and 2.9 us a pair (passes 1 and 2, about 130 pairs per SM) against 0.8 us for the three products, which stream
+// Bound by its epilogue: 2.4 and 2.1 us a pair (passes 1 and 2, about 130 pairs per SM) against 0.8 us for the three products, which stream
 // 192 KB of operands at the shared-memory port's 128 bytes per clock.  The four warps of a scheduler are in the same phase of the
 // same pair, and column sums leave no registers for two pairs at once.  Half the products and half the exponentials of evaluating
 // all pairs twice: 128 slabs x 2K sentences, the whole scoring call: 2319 -> 2190 us.
