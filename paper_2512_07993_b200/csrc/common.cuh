@@ -266,6 +266,10 @@ __device__ __forceinline__ bool role_wait(uint64_t* bar, uint32_t parity, uint32
     if (mbar_try_wait(bar, parity)) return true;
     return role_wait_slow(bar, parity, limit, abort_flag, status);
 }
+// The same for a whole warp, which stays converged.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint32_t limit, int* abort_flag, uint32_t* status) {
+    return __all_sync(0xffffffffu, role_wait(bar, parity, limit, abort_flag, status));
+}
 
 // Exclusive prefix of count(0..n-1) into pref[0..n] (pref[n] = total) by a whole CTA of kThreads threads; every thread
 // owns a contiguous block of indices.  wsum: kThreads / 32 words of shared memory.  Holds two CTA barriers; the

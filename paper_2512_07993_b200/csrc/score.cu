@@ -118,13 +118,13 @@ static __device__ __noinline__ bool flag_wait(const uint32_t* p, uint32_t want, 
 }
 
 // D[128 x n] (+)= A[128 x 128] * B[n x 128]^T.  Both operands are two halves of 64 channels, a_half / b_half bytes apart.
-__device__ __forceinline__ void umma_tile(uint32_t tmem_d, uint32_t a_smem, uint32_t a_half, uint32_t b_smem, uint32_t b_half, uint32_t idesc) {
+__device__ __forceinline__ void umma_tile(uint32_t tmem_d, uint32_t a_smem, uint32_t a_half, uint32_t b_smem, uint32_t b_half, uint32_t idesc, uint32_t leader) {
     const uint64_t da = umma_desc_sw128(a_smem), db = umma_desc_sw128(b_smem);
 #pragma unroll
     for (int half = 0; half < 2; ++half)
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks)
-            umma_bf16(tmem_d, da + uint64_t(half * (a_half >> 4) + ks * 2), db + uint64_t(half * (b_half >> 4) + ks * 2), idesc, (half || ks) ? 1u : 0u);
+            umma_bf16(tmem_d, da + uint64_t(half * (a_half >> 4) + ks * 2), db + uint64_t(half * (b_half >> 4) + ks * 2), idesc, (half || ks) ? 1u : 0u, leader);
 }
 // Descriptor of a K-major operand of 16 columns, rows 32 bytes apart, 32-byte swizzle (groups of 8 rows 256 bytes apart).
 __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
@@ -225,14 +225,14 @@ __device__ __forceinline__ float imp_fold(uint32_t taddr, int n, int wvalid, flo
 // B = the indicator matrix [slot][token], K-major like every other operand here.
 constexpr uint32_t kIdescPool = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t(kIndSlots) >> 3) << 17) |
                                 ((128u >> 4) << 24);
-__device__ __forceinline__ void umma_pool(uint32_t tmem_d, uint32_t tile_smem, uint32_t ind_smem, bool accumulate) {
+__device__ __forceinline__ void umma_pool(uint32_t tmem_d, uint32_t tile_smem, uint32_t ind_smem, bool accumulate, uint32_t leader) {
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {                     // 16 tokens per step
         const uint32_t a_addr = tile_smem + ks * 2048;
         const uint64_t da = uint64_t((a_addr >> 4) & 0x3fffu) | (uint64_t(kOpHalfBytes >> 4) << 16) |
                             (uint64_t(1024 >> 4) << 32) | (uint64_t(1) << 46) | (uint64_t(2) << 61);
         const uint64_t db = umma_desc_sw128(ind_smem + (ks >> 2) * (kIndBytes / 2) + (ks & 3) * 32);
-        umma_bf16(tmem_d, da, db, kIdescPool, (accumulate || ks) ? 1u : 0u);
+        umma_bf16(tmem_d, da, db, kIdescPool, (accumulate || ks) ? 1u : 0u, leader);
     }
 }
 // One 16-byte piece of an indicator matrix: tokens 8c .. 8c + 7 of slot row j; ones (bf16 1.0) for the tokens
@@ -404,10 +404,11 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         // at a barrier in between (115 cycles and more) leaves it idle; with two issuers one waits while the other's
         // product runs (measured without epilogue: 817 against 579 cycles per 128 x 128 x 128 product, 512 the least).
         const int mine = warp == 1 ? 0 : 1;
+        const uint32_t leader = elect_leader();
         bool ok = true;
         uint32_t qlap = 0;
         const uint32_t q0 = smem_u32(qbuf);
-        if (lane == 0) {
+        {
             int stage = 0, it = 0, slab = slab_of(resident ? t_begin : t_end - 1), lo = 0, hi = 0;
             uint32_t lap = 0;
             const int n_empty = a.RB > 1 ? 3 : 2;        // arrivals that free a stage
@@ -417,30 +418,30 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     while (pref[slab + 1] <= t) ++slab;
                     while (pref[slab] > t) --slab;
                     lo = pref[slab]; hi = pref[slab + 1];
-                    ok = role_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status);
+                    ok = warp_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     ++qlap;
                 }
                 // (both warps follow every tile's arrival, so that they see each phase of a stage's barrier)
-                ok = role_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
+                ok = warp_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
                 bool here = false;                       // this warp has a product of the tile
                 for (int k = 0; k < a.RA && ok; ++k, ++it) {
                     if ((it & 1) != mine) continue;
                     here = true;
                     const int buf = it & (kAGroups - 1), use = it / kAGroups;
-                    if (use > 0) ok = role_wait(&ctl->tempty_a[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
+                    if (use > 0) ok = warp_wait(&ctl->tempty_a[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     tc_fence_after();
                     const int r = k + 1 == a.RA && shifted(i) ? a.R - 128 : k * 128;       // first query row
                     umma_tile(tmem_base + buf * 128, q0 + uint32_t(r) * 128u, q_half, smem_u32(tiles + size_t(stage) * kOpBytes),
-                              kOpHalfBytes, kIdescBf16M128N128);
-                    umma_commit(&ctl->tfull_a[buf]);
+                              kOpHalfBytes, kIdescBf16M128N128, leader);
+                    umma_commit(&ctl->tfull_a[buf], leader);
                 }
                 const int t_next = resident ? t + 1 : t - 1;
-                if (i + 1 == ntl || t_next >= hi || t_next < lo) umma_commit(&ctl->qempty);
+                if (i + 1 == ntl || t_next >= hi || t_next < lo) umma_commit(&ctl->qempty, leader);
                 if (!resident && here) {                 // one warp: all arrivals; two: the second one of the tile makes up the number
                     const int c = a.RA == 1 ? n_empty : (((it - 1) & 1) == mine ? n_empty - 1 : 1);
-                    for (int e = 0; e < c; ++e) umma_commit(&ctl->empty[stage]);
+                    for (int e = 0; e < c; ++e) umma_commit(&ctl->empty[stage], leader);
                 }
                 if (++stage == a.stages) { stage = 0; ++lap; }
             }
@@ -449,7 +450,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         tc_fence_before();
         named_bar_sync(1, kSweepThreads - 32);           // every accumulator of pass A has been read
         tc_fence_after();
-        if (lane == 0 && ok) {
+        if (ok) {
             int it = 0, slab = slab_of(t_begin), hi = 0, stage = resident ? 0 : ntl % a.stages;
             uint32_t elap = 0, lap = resident ? 0u : uint32_t(ntl / a.stages);
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t(a.N) >> 3) << 17) | ((128u >> 4) << 24);
@@ -459,31 +460,31 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 if (i == 0 || t >= hi) {
                     while (pref[slab + 1] <= t) ++slab;
                     hi = pref[slab + 1];
-                    ok = role_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status) &&
-                         role_wait(&ctl->extfull, elap & 1u, limit, &ctl->abort_flag, a.status);
+                    ok = warp_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status) &&
+                         warp_wait(&ctl->extfull, elap & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     ++qlap; ++elap;
                 }
-                ok = role_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
+                ok = warp_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
                 bool here = false;
                 for (int k = 0; k < a.RB && ok; ++k, ++it) {
                     if ((it & 1) != mine) continue;
                     here = true;
                     const int buf = it % kBGroups, before = it - kBGroups;
-                    if (before >= 0) ok = role_wait(&ctl->tempty_b[before % (2 * kBGroups)], uint32_t(before / (2 * kBGroups)) & 1u, limit, &ctl->abort_flag, a.status);
+                    if (before >= 0) ok = warp_wait(&ctl->tempty_b[before % (2 * kBGroups)], uint32_t(before / (2 * kBGroups)) & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d = tmem_base + buf * kBAccCols;
-                    umma_tile(d, smem_u32(tiles + size_t(stage) * kOpBytes), kOpHalfBytes, q0 + uint32_t(k * a.N) * 128u, q_half, idesc);
-                    umma_bf16(d, d_ones, umma_desc_sw32(ext_smem + uint32_t(k * a.N) * kExtRow), idesc, 1u);      // - lse
-                    umma_commit(&ctl->tfull_b[buf]);
+                    umma_tile(d, smem_u32(tiles + size_t(stage) * kOpBytes), kOpHalfBytes, q0 + uint32_t(k * a.N) * 128u, q_half, idesc, leader);
+                    umma_bf16(d, d_ones, umma_desc_sw32(ext_smem + uint32_t(k * a.N) * kExtRow), idesc, 1u, leader);      // - lse
+                    umma_commit(&ctl->tfull_b[buf], leader);
                 }
-                if (i + 1 == ntl || hi <= t + 1) { umma_commit(&ctl->qempty); umma_commit(&ctl->extempty); }
-                if (here) umma_commit(&ctl->empty[stage]);
+                if (i + 1 == ntl || hi <= t + 1) { umma_commit(&ctl->qempty, leader); umma_commit(&ctl->extempty, leader); }
+                if (here) umma_commit(&ctl->empty[stage], leader);
                 if (++stage == a.stages) { stage = 0; ++lap; }
             }
         }
-        if (lane == 0) umma_commit(&ctl->retired[mine]);
+        umma_commit(&ctl->retired[mine], leader);
     } else {
         // ------------------------------------------------------------------ pass A: epilogue warpgroups (and the clearing warp)
         const int quarter = warp & 3;                        // tensor-memory lanes this warp may read
@@ -812,29 +813,30 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             // -------------------------------------------------------------- pass B: issuer of the pooling products
             // (its own thread: an issue blocks for the length of the product, and every look at shared memory costs the
             // thread that issues the logits a few hundred cycles)
-            if (lane == 0) {
+            {
+                const uint32_t leader = elect_leader();
                 const uint32_t indb_u32 = smem_u32(indb);
                 int pc = 0, run = -1, stage = load0 % a.stages;
                 for (int tl = 0; tl < ntl && ok; ++tl) {
                     int flags = 0;
                     do {
                         const int is = pc & (kIndRing - 1);
-                        ok = role_wait(&ctl->ifull[is], uint32_t(pc / kIndRing) & 1u, limit, &ctl->abort_flag, a.status);
+                        ok = warp_wait(&ctl->ifull[is], uint32_t(pc / kIndRing) & 1u, limit, &ctl->abort_flag, a.status);
                         if (!ok) break;
                         flags = *reinterpret_cast<volatile int*>(&ctl->ind_flags[is]);       // 1: more, 2: joins the run, 4: closes one
                         tc_fence_after();
-                        if (flags & 4) umma_commit(&ctl->pfull[run & 1]);                    // everything of the run before is issued
+                        if (flags & 4) umma_commit(&ctl->pfull[run & 1], leader);                    // everything of the run before is issued
                         if (!(flags & 2)) ++run;
                         umma_pool(tmem_base + kPoolCol + uint32_t(run & 1) * kIndSlots, smem_u32(tiles + size_t(stage) * kOpBytes),
-                                  indb_u32 + uint32_t(is) * kIndBytes, (flags & 2) != 0);
-                        umma_commit(&ctl->iempty[is]);
+                                  indb_u32 + uint32_t(is) * kIndBytes, (flags & 2) != 0, leader);
+                        umma_commit(&ctl->iempty[is], leader);
                         ++pc;
                     } while (flags & 1);
-                    if (ok) umma_commit(&ctl->empty[stage]);
+                    if (ok) umma_commit(&ctl->empty[stage], leader);
                     if (++stage == a.stages) stage = 0;
                 }
-                if (ok && run >= 0) umma_commit(&ctl->pfull[run & 1]);
-                umma_commit(&ctl->retired[2]);
+                if (ok && run >= 0) umma_commit(&ctl->pfull[run & 1], leader);
+                umma_commit(&ctl->retired[2], leader);
             }
         }
     }
@@ -1097,10 +1099,10 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 for (int part = 0; part < 2; ++part)
                     if (ctl->loads[2 * s + part]) mbar_wait(&ctl->full[s][part], (ctl->loads[2 * s + part] - 1) & 1u, kRetirePolls);
             for (int s = 0; s < 2; ++s) mbar_wait(&ctl->retired[s], 0u, kRetirePolls);
-        } else if ((warp == 1 || warp == 2) && lane == 0) {
+        } else if (warp == 1 || warp == 2) {
             // A pair each in turn, so that one waits for its operands while the other's products run.  The turn is handed over a little
             // before a pair's last instructions are issued.  It comes before the other waits: every barrier's earlier phases have been seen by then.
-            const uint32_t me = warp - 1;
+            const uint32_t me = warp - 1, leader = elect_leader();
             bool ok = true, fresh = true;
             uint32_t fpar = 0, jpar = 0;                               // parity of a slot's next use; of J's present one
             GramWalk w;
@@ -1123,25 +1125,26 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 fresh = w.next(ipref);
                 if ((bc & 1u) != me) continue;
                 const uint32_t acc = bc % kGramAcc;
-                if (bc > 0) ok = role_wait(&ctl->turn[me], ((bc >> 1) - (me ? 0u : 1u)) & 1u, limit, &ctl->abort_flag, status);
+                if (bc > 0) ok = warp_wait(&ctl->turn[me], ((bc >> 1) - (me ? 0u : 1u)) & 1u, limit, &ctl->abort_flag, status);
                 for (int part = 1; part >= 0 && ok; --part) {
-                    ok = role_wait(&ctl->full[js][part], jpar, limit, &ctl->abort_flag, status);
-                    if (ok && !diag) ok = role_wait(&ctl->full[is][part], ip, limit, &ctl->abort_flag, status);
+                    ok = warp_wait(&ctl->full[js][part], jpar, limit, &ctl->abort_flag, status);
+                    if (ok && !diag) ok = warp_wait(&ctl->full[is][part], ip, limit, &ctl->abort_flag, status);
                 }
-                if (ok && bc >= kGramAcc) ok = role_wait(&ctl->tempty[acc], ((bc / kGramAcc) - 1) & 1u, limit, &ctl->abort_flag, status);
+                if (ok && bc >= kGramAcc) ok = warp_wait(&ctl->tempty[acc], ((bc / kGramAcc) - 1) & 1u, limit, &ctl->abort_flag, status);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t i_hi = smem_u32(slots + size_t(2 * is) * kOpBytes), j_hi = smem_u32(slots + size_t(2 * js) * kOpBytes);
                 const uint32_t d = tmem_base + acc * 128;
-                umma_tile_128x128x128(d, i_hi + kOpBytes, j_hi, false);
-                if (!diag) umma_commit(&ctl->empty[is][1]);
-                umma_tile_128x128x128(d, i_hi, j_hi + kOpBytes, true);
-                mbar_arrive(&ctl->turn[me ^ 1u]);
-                umma_tile_128x128x128(d, i_hi, j_hi, true);
-                umma_commit(&ctl->tfull[acc]);
-                umma_commit(diag ? &ctl->ddone[js] : &ctl->empty[is][0]);
+                umma_tile_128x128x128(d, i_hi + kOpBytes, j_hi, false, leader);
+                if (!diag) umma_commit(&ctl->empty[is][1], leader);
+                umma_tile_128x128x128(d, i_hi, j_hi + kOpBytes, true, leader);
+                if (leader) mbar_arrive(&ctl->turn[me ^ 1u]);
+                __syncwarp();
+                umma_tile_128x128x128(d, i_hi, j_hi, true, leader);
+                umma_commit(&ctl->tfull[acc], leader);
+                umma_commit(diag ? &ctl->ddone[js] : &ctl->empty[is][0], leader);
             }
-            umma_commit(&ctl->retired[me]);
+            umma_commit(&ctl->retired[me], leader);
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
@@ -1403,12 +1406,12 @@ score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const i
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    if (tid == 0) {
-        const uint32_t a = smem_u32(hi_t), b = smem_u32(lo_t);
-        umma_tile_128x128x128(tmem_base, a, a, false);
-        umma_tile_128x128x128(tmem_base, a, b, true);
-        umma_tile_128x128x128(tmem_base, b, a, true);
-        umma_commit(&ctl->done);
+    if (warp == 0) {
+        const uint32_t a = smem_u32(hi_t), b = smem_u32(lo_t), leader = elect_leader();
+        umma_tile_128x128x128(tmem_base, a, a, false, leader);
+        umma_tile_128x128x128(tmem_base, a, b, true, leader);
+        umma_tile_128x128x128(tmem_base, b, a, true, leader);
+        umma_commit(&ctl->done, leader);
     }
     const bool ok = mbar_wait(&ctl->done, 0u, load_wait_limit(hdr));
     if (!ok) {                                           // the outputs are skipped, but the product retires before it is read or released

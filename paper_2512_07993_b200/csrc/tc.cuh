@@ -66,29 +66,44 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
 // Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = N = 128.
 constexpr uint32_t kIdescBf16M128N128 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
-// D[128 x 128] (+)= A[128 x 16] * B[128 x 16]^T, issued by one thread.
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
+// Products are issued by a whole warp, of which the thread with `leader` set executes the instruction: the warp stays converged, so
+// addresses and descriptors are uniform values and an issue takes 15 to 20 clocks.  Under a branch that one lane takes they are the
+// lane's own and every instruction first moves them: 62 clocks each, 500 for the eight of a 128 x 128 x 128 product, which itself
+// takes 512; one warp then issued a product every 721 clocks whatever its size, now every 513 (128 columns) or 372 (16).
+__device__ __forceinline__ uint32_t elect_leader() {     // 1 in one lane of a converged warp, the same one every time
+    uint32_t leader;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(leader));
+    return leader;
+}
+// D[128 x 128] (+)= A[128 x 16] * B[128 x 16]^T.
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate, uint32_t leader) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(leader)
         : "memory");
 }
 // The full K = 128 contraction of two operand tiles (8 steps of 16): 4 per 64-element half.
-__device__ __forceinline__ void umma_tile_128x128x128(uint32_t tmem_d, uint32_t a_smem, uint32_t b_smem, bool accumulate_first) {
+__device__ __forceinline__ void umma_tile_128x128x128(uint32_t tmem_d, uint32_t a_smem, uint32_t b_smem, bool accumulate_first, uint32_t leader) {
     const uint64_t da = umma_desc_sw128(a_smem), db = umma_desc_sw128(b_smem);
 #pragma unroll
     for (int half = 0; half < 2; ++half)
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
             const uint64_t off = uint64_t(half * (kOpHalfBytes >> 4) + ks * 2);      // in 16-byte units
-            umma_bf16(tmem_d, da + off, db + off, kIdescBf16M128N128, (accumulate_first || half || ks) ? 1u : 0u);
+            umma_bf16(tmem_d, da + off, db + off, kIdescBf16M128N128, (accumulate_first || half || ks) ? 1u : 0u, leader);
         }
 }
-// Arrive on an mbarrier when every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+// Arrive on an mbarrier when every MMA that the leader has issued so far has completed.
+__device__ __forceinline__ void umma_commit(uint64_t* bar, uint32_t leader) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+        ::"r"(smem_u32(bar)), "r"(leader)
+        : "memory");
 }
 
 // 32 consecutive fp32 columns of this thread's tensor-memory lane (lane = 32*(warp%4) + laneid).

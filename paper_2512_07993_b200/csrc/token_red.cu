@@ -184,31 +184,31 @@ token_red_kernel(const __grid_constant__ CUtensorMap mapK, int n_slabs, int Hk, 
             for (uint32_t s = 0; s < kTrStages; ++s)
                 if (bc > s) mbar_wait(&ctl->ifull[s], ((bc - 1 - s) / kTrStages) & 1u, kRetirePolls);
             for (int s = 0; s < 2; ++s) mbar_wait(&ctl->retired[s], 0u, kRetirePolls);
-        } else if ((warp == 1 || warp == 2) && lane == 0) {
+        } else if (warp == 1 || warp == 2) {
             // two issuers, a tile each in turn (stages and accumulators are four: each is always the same issuer's)
-            const uint32_t me = warp - 1;
+            const uint32_t me = warp - 1, leader = elect_leader();
             bool ok = true;
             int slab = 0;
             uint32_t bc = 0, ic = 0;
             for (int item = cta; item < n_items && ok; item += G, ++ic) {
                 const TrItem x = get_item(item, slab);
                 slab = x.slab;
-                ok = role_wait(&ctl->jfull[ic & 1], (ic >> 1) & 1u, limit, &ctl->abort_flag, status);
+                ok = warp_wait(&ctl->jfull[ic & 1], (ic >> 1) & 1u, limit, &ctl->abort_flag, status);
                 const uint32_t jt = smem_u32(Jt + (ic & 1) * kOpBytes);
                 for (int t = 0; t < x.NJ && ok; ++t, ++bc) {
                     if ((bc & 1u) != me) continue;
                     const int st = bc % kTrStages, s = bc % kTrAcc;
-                    ok = role_wait(&ctl->ifull[st], (bc / kTrStages) & 1u, limit, &ctl->abort_flag, status);
-                    if (ok && bc >= kTrAcc) ok = role_wait(&ctl->tempty[s], ((bc / kTrAcc) - 1) & 1u, limit, &ctl->abort_flag, status);
+                    ok = warp_wait(&ctl->ifull[st], (bc / kTrStages) & 1u, limit, &ctl->abort_flag, status);
+                    if (ok && bc >= kTrAcc) ok = warp_wait(&ctl->tempty[s], ((bc / kTrAcc) - 1) & 1u, limit, &ctl->abort_flag, status);
                     if (!ok) break;
                     tc_fence_after();
-                    umma_tile_128x128x128(tmem_base + s * 128, smem_u32(It + size_t(st) * kOpBytes), jt, false);
-                    umma_commit(&ctl->tfull[s]);
-                    umma_commit(&ctl->iempty[st]);
+                    umma_tile_128x128x128(tmem_base + s * 128, smem_u32(It + size_t(st) * kOpBytes), jt, false, leader);
+                    umma_commit(&ctl->tfull[s], leader);
+                    umma_commit(&ctl->iempty[st], leader);
                 }
-                if (ok) umma_commit(&ctl->jempty[ic & 1]);           // every product of this issuer that reads the column tile has completed
+                if (ok) umma_commit(&ctl->jempty[ic & 1], leader);           // every product of this issuer that reads the column tile has completed
             }
-            umma_commit(&ctl->retired[me]);
+            umma_commit(&ctl->retired[me], leader);
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
