@@ -37,7 +37,7 @@ struct WsLayout {
     size_t cp_run_dst;     // int32  [slabs][max_sent+1]  first destination token; [nruns] = new_len
     size_t dec_cnt;        // uint32 [slabs]              partials that arrived (self-resetting)
     size_t dec_part;       // float  [max_ctas + slabs][group][kDecPartStride]
-    size_t sc_cnt;         // uint32 [slabs]              tiles whose log-sum-exp records are written (zero between calls)
+    size_t sc_cnt;         // uint32 [2][slabs]           tiles whose log-sum-exp records / key sums are written (zero between calls)
     size_t sc_part;        // float2 [max_ctas + slabs][sc_ra * 128]  (reference, sum) of a CTA's part of a slab
     size_t sc_tokimp;      // float  [slabs][max_cap]
     size_t sc_vsum;        // float  [slabs][max_sent][128]  per-sentence sums of key rows; then partial sums of the Gram passes,
@@ -91,7 +91,7 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     L.cp_run_src = take(slabs * ms * 4);
     L.cp_run_dst = take(slabs * (ms + 1) * 4);
     L.dec_cnt = take(slabs * 4);
-    L.sc_cnt = take(slabs * 4);
+    L.sc_cnt = take(2 * slabs * 4);
     L.dec_part = take((size_t(L.dec_max_ctas) + slabs) * L.group * kDecPartStride * 4);
     L.sc_part = take((size_t(L.dec_max_ctas) + slabs) * size_t(L.sc_ra) * 128 * 8);
     L.sc_tokimp = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);

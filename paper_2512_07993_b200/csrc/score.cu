@@ -3,8 +3,8 @@
 //   sweeps    (one launch) pass A: log-sum-exp of every window-query row over the slab's tokens
 //             (tensor cores: logits = Q_rows x K_tile^T, one thread per query row);
 //             pass B: tok_imp[t] = (1/alpha) sum_w max_q 2^(s_q[w][t] - lse_q[w])   (max before exp: exp is monotone)
-//             (tensor cores: logits - (lse - e) = [K_tile, 1] x [Q_block, e - lse]^T, one thread per token; e: see lse_shift), and in the same pass
-//             the per-sentence sums of the key rows as a second product on the tile already in shared
+//             (tensor cores: logits - (lse - e) = [K_tile, 1] x [Q_block, e - lse]^T, one thread per token; e: see lse_shift);
+//             in one of them the per-sentence sums of the key rows as a second product on the tile already in shared
 //             memory: K_tile^T x (0/1 matrix token -> sentence slot)
 //   up to 128 sentences per slab: one kernel for the rest, else
 //   pool      per sentence: mean tok_imp, mean key, normalisation, split into bf16 high and low parts
@@ -16,9 +16,9 @@
 // needs no max subtraction.
 //
 // The sweeps are a persistent, warp-specialised kernel, one CTA per SM: a TMA warp streams 128-token key tiles (and the
-// group's query rows) into shared memory, two threads in two warps issue tcgen05.mma in turn into a ring of tensor-memory accumulators,
-// epilogue warpgroups take the products round-robin (four in pass A, three in pass B), and in pass B one more warpgroup writes the 0/1
-// matrices of the pooling product and reads out the pooled sums while one thread of a further warp issues
+// group's query rows) into shared memory, two warps issue tcgen05.mma in turn into a ring of tensor-memory accumulators,
+// epilogue warpgroups take the products round-robin, and in one of the passes another warpgroup writes the 0/1
+// matrices of the pooling product and reads out the pooled sums while a further warp issues
 // that product.  Work is the list of 128-token tiles over all slabs cut into equal contiguous ranges, so
 // ragged slabs balance.
 //
@@ -35,47 +35,61 @@ namespace skipkv {
 // ---------------------------------------------------------------------------------------
 // Both sweeps over the keys in one persistent launch.  A CTA goes through its range of tiles twice:
 //   pass A   log-sum-exp of every window-query row over the CTA's part of each slab -> one record per (CTA, slab)
-//   pass B   importance of every token and the per-sentence key sums
+//   pass B   importance of every token
 // Between the two it waits, slab by slab, until every CTA that shares the slab has left its record (a counter of tiles);
 // nobody waits for anything but pass A of CTAs that are all resident (one per SM), and the waits are bounded anyway.
-// As two launches the second started its first tile 6 us after the first had drained.  Pass A runs backwards through the
-// range, so that pass B finds the tiles read last in L2 -- or, where the range fits into the ring, still in shared memory.
+// As two launches the second started its first tile 6 us after the first had drained.  Pass B comes back through the range, so it begins
+// with the tiles that are still in shared memory (all of them where the range fits into the ring) and finds the next ones in L2.
+// The per-sentence key sums are a product per tile in either pass.  With one operand of query rows (up to 128) pass A waits for DRAM, and they
+// are its; with several it waits for its exponentials, wants the fourth epilogue warpgroup, and they are pass B's.  80 slabs of 16K to 32K,
+// 128 rows: pass A 112 us, pass B 75 with the sums in pass A; 97 and 105 in pass B; the whole call 315 -> 294 us.  128 slabs of 32K to 64K,
+// 320 rows: 757 and 425 against 606 and 490.
+// What bounds the passes beside that: instructions.  A tile takes about 6000 warp instructions for 1500 exponentials' worth of work a warp, and
+// the warps' different loops do not fit into the instruction caches together: a 512-instruction loop in the other warps slows
+// a warp that issues products from 570 to 2800 clocks a product.  Loops are kept short, and what can be done once for several tiles is.
 // ---------------------------------------------------------------------------------------
 constexpr int kStagesMax = 6;
-constexpr int kAGroups = 4;             // pass A: epilogue warpgroups = accumulators of 128 columns
-constexpr int kBGroups = 3;             // pass B: epilogue warpgroups = accumulators of up to 160 columns
-constexpr int kBAccCols = 160;
-constexpr int kIndRing = 2;             // indicator matrices in flight (the pooled sums have two accumulators of their own)
+constexpr int kAccB = 3;                // pass B: accumulators of up to 160 columns, an epilogue warpgroup each
+constexpr int kAccCols = 160;
+constexpr int kAccAMax = 4;             // pass A: accumulators of 128 columns, an epilogue warpgroup each; three where the fourth group has the pooling
+constexpr int kIndRingMax = 4;          // indicator matrices in flight (the pooled sums have two accumulators of their own)
 constexpr int kIndSlots = 16;           // sentence slots of one indicator matrix
 constexpr int kIndBytes = kIndSlots * 128 * 2;   // [16 slots][128 tokens] bf16 as two 64-token halves, 128-byte swizzle
-constexpr uint32_t kPoolCol = kBGroups * kBAccCols;   // tensor-memory column of the first pooled-sum accumulator (16 columns each)
+constexpr uint32_t kPoolCol = kAccB * kAccCols;   // tensor-memory column of the first pooled-sum accumulator (16 columns each)
 constexpr int kPoolWarps = 4;
-constexpr int kSweepThreads = (2 + 4 * kAGroups + 2) * 32;    // TMA warp, MMA warp, 16 epilogue warps, issuer of the pooling products, second MMA warp
-constexpr int kMaxBlocksA = 5;          // blocks of 128 query rows
+constexpr int kSweepThreads = 20 * 32;  // TMA warp, two MMA warps, issuer of the pooling products; three epilogue warpgroups; a fourth, which has the pooling
 constexpr int kExtRow = 32;             // bytes of a row of the extra K step (16 bf16)
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct SweepCtl {                       // barriers and small shared state, after the tile buffers
     uint64_t full[kStagesMax], empty[kStagesMax];
     uint64_t qfull, qempty;
-    // accumulator i belongs to epilogue warpgroup i (a product of a tile and a block of query rows goes to product number % groups)
-    uint64_t tfull_a[kAGroups], tempty_a[kAGroups], tfull_b[kBGroups];
-    uint64_t tempty_b[2 * kBGroups];    // by product number: a product waits for the one kBGroups before it, which is the other MMA warp's, and
-                                        // with twice as many barriers as accumulators each has one waiter that sees all its phases
+    // A product (of a tile and a block of query rows) goes to the accumulator of its number in the pass % accumulators; "has been read" is by
+    // product number % twice the accumulators, so that each barrier has one waiter (the MMA warp whose product is the next into that
+    // accumulator) that sees all its phases
+    uint64_t tfull_a[kAccAMax], tempty_a[2 * kAccAMax], tfull_b[kAccB], tempty_b[2 * kAccB];
     uint64_t tokfull[4];                // pass B, several blocks per tile: the shares of a tile's tokens from all blocks but the last
     uint64_t extfull, extempty;         // pass B: the rows' -lse as operand columns
     // ring of indicator matrices: written by the four pooling warps -> multiplied by their issuer -> read out by the pooling warps
-    uint64_t ifull[kIndRing], iempty[kIndRing];
+    uint64_t ifull[kIndRingMax], iempty[kIndRingMax];
     uint64_t pfull[2];                  // the last product of a run of tiles into accumulator i has completed
     uint64_t retired[3];                // every product of the MMA warps (0, 1) / the pooling issuer (2) has completed
     uint32_t tmem_base;
     int abort_flag;
-    int ind_flags[kIndRing];            // 1: the tile has another matrix after this one, 2: joins the open run, 4: closes a run
+    int ind_flags[kIndRingMax];            // 1: the tile has another matrix after this one, 2: joins the open run, 4: closes a run
     uint32_t wsum[32];
 };
 
+// The rows of pass B's extra K step; before, the sums of pass A: 8 bytes by warpgroup, row and block, and one block more where there are several.
+__host__ __device__ constexpr size_t sweep_ext_bytes(int RA) {
+    const size_t ext = size_t(RA) * 128 * kExtRow, sums = size_t(kAccAMax) * (RA + (RA > 1 ? 1 : 0)) * 128 * 8;
+    return ext > sums ? ext : sums;
+}
+
 struct SweepArgs {
     int Hq, Hk, window, n_slabs, max_cap, max_sent, stages;
+    int pool_a;                         // the pooling products are pass A's (1) or pass B's (0)
+    int ind_log;                        // log2 of the indicator matrices in flight
     int WB, RB, N, R, RA;               // window positions per block of pass B, its blocks, their rows N = WB * n; all rows R = RB * N; blocks of pass A
     const int64_t* slab_off;
     const int32_t* cap;
@@ -84,6 +98,7 @@ struct SweepArgs {
     const int32_t* n_sent;
     float2* rec;                        // [cta + slab][RA * 128] (reference, sum) of a CTA's part of a slab
     uint32_t* lse_cnt;                  // [slabs] tiles whose records are written; zero at the start
+    uint32_t* sum_cnt;                  // [slabs] four times the tiles whose key sums are stored; zero at the start
     float* tok_imp_user;
     float* tok_imp_ws;
     float* vsum;                        // [slabs][max_sent][128] sums of key rows
@@ -140,45 +155,49 @@ __device__ __forceinline__ int lse_shift(int rows) { return 32 - __clz(max(rows,
 // ---- pass A epilogue: one accumulator (128 tokens) folded into a row's sum of 2^(logit - m).  The reference m is the
 // largest logit of the row's first 32 tokens; it stays, whatever comes later, as long as a chunk's sum is below 2^60 --
 // no running maximum and no rescaling in the common case.  A chunk beyond that is folded again under a larger reference.
+// `release` gives the accumulator back once its last chunk is in registers, so that the next product runs under that chunk's exponentials.
 template <bool kMasked>
-__device__ __forceinline__ void lse_fold(uint32_t taddr, int valid, float scale, float& m, float& l) {
-    const int nch = kMasked ? (valid + 31) >> 5 : 4;
+__device__ __forceinline__ void lse_chunk(float (&v)[32], int left, float scale, float& m, float& l) {
+    if (kMasked) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            if (j >= left) v[j] = -INFINITY;
+    }
+    auto chunk_max = [&]() {
+        float c0 = fmaxf(v[0], v[1]), c1 = fmaxf(v[2], v[3]);
+#pragma unroll
+        for (int j = 4; j < 32; j += 4) { c0 = max3(c0, v[j], v[j + 1]); c1 = max3(c1, v[j + 2], v[j + 3]); }
+        return fmaxf(c0, c1) * scale;
+    };
+    auto chunk_sum = [&]() {
+        float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+        const float2 sc = make_float2(scale, scale), neg = make_float2(-m, -m);
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+            const float2 x = __ffma2_rn(make_float2(v[j], v[j + 1]), sc, neg), y = __ffma2_rn(make_float2(v[j + 2], v[j + 3]), sc, neg);
+            s0 = __fadd2_rn(s0, make_float2(ex2f(x.x), ex2f(x.y)));
+            s1 = __fadd2_rn(s1, make_float2(ex2f(y.x), ex2f(y.y)));
+        }
+        return (s0.x + s0.y) + (s1.x + s1.y);
+    };
+    if (m == -INFINITY) m = chunk_max();
+    float s = chunk_sum();
+    if (!(s < 1.15e18f)) {
+        const float m_new = fmaxf(m, chunk_max());
+        l *= ex2f(m - m_new);
+        m = m_new;
+        s = chunk_sum();
+    }
+    l += s;
+}
+template <bool kMasked, typename Release>
+__device__ __forceinline__ void lse_fold(uint32_t taddr, int valid, float scale, float& m, float& l, Release release) {
 #pragma unroll 1
-    for (int ch = 0; ch < nch; ++ch) {
+    for (int c = 0; c < 128; c += 32) {
         float v[32];
-        tmem_ld32(taddr + ch * 32, v);
-        if (kMasked && ch * 32 + 32 > valid) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (ch * 32 + j >= valid) v[j] = -INFINITY;
-        }
-        auto chunk_max = [&]() {
-            float c0 = fmaxf(v[0], v[1]), c1 = fmaxf(v[2], v[3]);
-#pragma unroll
-            for (int j = 4; j < 32; j += 4) { c0 = max3(c0, v[j], v[j + 1]); c1 = max3(c1, v[j + 2], v[j + 3]); }
-            return fmaxf(c0, c1) * scale;
-        };
-        auto chunk_sum = [&]() {
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-            const float neg = -m;
-#pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-                s0 += ex2f(fmaf(v[j + 0], scale, neg));
-                s1 += ex2f(fmaf(v[j + 1], scale, neg));
-                s2 += ex2f(fmaf(v[j + 2], scale, neg));
-                s3 += ex2f(fmaf(v[j + 3], scale, neg));
-            }
-            return (s0 + s1) + (s2 + s3);
-        };
-        if (m == -INFINITY) m = chunk_max();
-        float s = chunk_sum();
-        if (!(s < 1.15e18f)) {
-            const float m_new = fmaxf(m, chunk_max());
-            l *= ex2f(m - m_new);
-            m = m_new;
-            s = chunk_sum();
-        }
-        l += s;
+        tmem_ld32(taddr + c, v);
+        if (c == 96) release();
+        if (!kMasked || valid > c) lse_chunk<kMasked>(v, valid - c, scale, m, l);
     }
 }
 
@@ -235,17 +254,16 @@ __device__ __forceinline__ void umma_pool(uint32_t tmem_d, uint32_t tile_smem, u
         umma_bf16(tmem_d, da, db, kIdescPool, (accumulate || ks) ? 1u : 0u, leader);
     }
 }
-// One 16-byte piece of an indicator matrix: tokens 8c .. 8c + 7 of slot row j; ones (bf16 1.0) for the tokens
-// [lo, hi), zeros elsewhere.
-__device__ __forceinline__ void indicator_piece(uint8_t* ind, int j, int c, int lo, int hi) {
-    const int b0 = min(max(lo - 8 * c, 0), 8), b1 = min(max(hi - 8 * c, 0), 8);
-    const uint32_t m8 = b1 > b0 ? (((1u << b1) - 1u) & ~((1u << b0) - 1u)) : 0u;
-    uint4 val;
-    val.x = (m8 & 1u) * 0x3F80u + ((m8 >> 1) & 1u) * 0x3F800000u;
-    val.y = ((m8 >> 2) & 1u) * 0x3F80u + ((m8 >> 3) & 1u) * 0x3F800000u;
-    val.z = ((m8 >> 4) & 1u) * 0x3F80u + ((m8 >> 5) & 1u) * 0x3F800000u;
-    val.w = ((m8 >> 6) & 1u) * 0x3F80u + ((m8 >> 7) & 1u) * 0x3F800000u;
-    *reinterpret_cast<uint4*>(ind + (c >> 3) * (kIndBytes / 2) + j * 128 + (((c & 7) ^ (j & 7)) << 4)) = val;
+// Tokens 16 q .. 16 q + 15 of slot row j of an indicator matrix: ones (bf16 1.0) for the tokens [lo, hi), zeros elsewhere.
+__device__ __forceinline__ void indicator_row(uint8_t* ind, int j, int q, int lo, int hi) {
+    const uint32_t b0 = min(max(lo - 16 * q, 0), 16), b1 = min(max(hi - 16 * q, 0), 16);
+    const uint32_t m = b1 > b0 ? (1u << b1) - (1u << b0) : 0u;
+    uint32_t v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = ((((m >> (2 * i)) & 3u) * 0x8001u) & 0x10001u) * 0x3F80u;      // two bits to the low ends of two halves
+    uint8_t* row = ind + (q >> 2) * (kIndBytes / 2) + j * 128;
+    *reinterpret_cast<uint4*>(row + ((((2 * q) & 7) ^ (j & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<uint4*>(row + ((((2 * q + 1) & 7) ^ (j & 7)) << 4)) = make_uint4(v[4], v[5], v[6], v[7]);
 }
 
 // The sweep's table of slabs in global memory, for calls with more slabs than shared memory has room for beside the query rows.
@@ -272,9 +290,9 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     const uint32_t q_half = uint32_t(a.R) * 128u;
     uint8_t* tiles = qbuf + size_t(a.R) * kRowBytes;                             // (R is a multiple of 16: 1024-byte aligned)
     uint8_t* indb = tiles + size_t(a.stages) * kOpBytes;                         // pass B: the indicator matrices
-    uint8_t* onesb = indb + kIndRing * kIndBytes;                                // pass B: the keys' side of the extra K step
-    uint8_t* extb = onesb + 128 * kExtRow;                                       // pass B: the queries' side; pass A: [4 groups][RA * 128] (m, l)
-    SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + size_t(a.RA) * 128 * kExtRow);
+    uint8_t* onesb = indb + (kIndBytes << a.ind_log);                                // pass B: the keys' side of the extra K step
+    uint8_t* extb = onesb + 128 * kExtRow;                                       // pass B: the queries' side; pass A: [groups][blocks] (m, l)
+    SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + sweep_ext_bytes(a.RA));
     float* tokp = reinterpret_cast<float*>(ctl + 1);                             // [4 tiles][RB - 1][128] shares of a tile's tokens
     int* pref = kTable ? a.table : reinterpret_cast<int*>(tokp + 4 * (a.RB - 1) * 128);    // [n_slabs + 1] tile prefix
     int* rowb = pref + a.n_slabs + 1;                                            // [n_slabs] cache row of a slab's first token
@@ -289,15 +307,17 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     };
 
     if (tid == 0) {
-        for (int s = 0; s < kStagesMax; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], a.RB > 1 ? 3 : 2); }
+        for (int s = 0; s < kStagesMax; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 3); }
         mbar_init(&ctl->qfull, 1);
         mbar_init(&ctl->qempty, 2);
-        for (int g = 0; g < kAGroups; ++g) { mbar_init(&ctl->tfull_a[g], 1); mbar_init(&ctl->tempty_a[g], 4); }
-        for (int g = 0; g < kBGroups; ++g) { mbar_init(&ctl->tfull_b[g], 1); mbar_init(&ctl->tempty_b[g], 4); mbar_init(&ctl->tempty_b[kBGroups + g], 4); }
+        for (int i = 0; i < kAccAMax; ++i) mbar_init(&ctl->tfull_a[i], 1);
+        for (int i = 0; i < 2 * kAccAMax; ++i) mbar_init(&ctl->tempty_a[i], 4);
+        for (int i = 0; i < kAccB; ++i) mbar_init(&ctl->tfull_b[i], 1);
+        for (int i = 0; i < 2 * kAccB; ++i) mbar_init(&ctl->tempty_b[i], 4);
         for (int i = 0; i < 4; ++i) mbar_init(&ctl->tokfull[i], a.RB > 1 ? 4 * (a.RB - 1) : 1);
         mbar_init(&ctl->extfull, 4);
         mbar_init(&ctl->extempty, 2);
-        for (int i = 0; i < kIndRing; ++i) { mbar_init(&ctl->ifull[i], kPoolWarps); mbar_init(&ctl->iempty[i], 1); }
+        for (int i = 0; i < kIndRingMax; ++i) { mbar_init(&ctl->ifull[i], kPoolWarps); mbar_init(&ctl->iempty[i], 1); }
         for (int i = 0; i < 2; ++i) mbar_init(&ctl->pfull[i], 1);
         for (int i = 0; i < 3; ++i) mbar_init(&ctl->retired[i], 1);
         ctl->abort_flag = 0;
@@ -334,87 +354,97 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         return lo;
     };
     auto owner = [&](int t) { return int(((long long)(t + 1) * Ge - 1) / T); };
-    const bool resident = ntl <= a.stages;               // the range fits into the ring: pass B reads it where pass A left it
     const float scale = kLog2e * rsqrtf(float(kHeadDim));
     const int n = a.Hq / Hk;
     const uint32_t ext_smem = smem_u32(extb);
+    // Pass A takes the tiles of the range in the order of positions 0, 1, ..., pass B comes back from the last one.  Position p is staged at
+    // p % stages in both, so pass B begins with the tiles that are still there, and every use of a stage, the first to the last, has the
+    // parity of p / stages.  The pass that has the pooling products goes up.
+    const bool pool_a = a.pool_a != 0;
+    auto tile_at = [&](int p) { return pool_a ? t_begin + p : t_end - 1 - p; };
+    const int kept = max(ntl - a.stages, 0);             // positions from here on are not loaded again
     // Pass A, last block of at most 64 rows: on every second tile its rows take the upper tensor-memory lanes, so that the
-    // exponentials spread over all four schedulers.  (Which tiles an epilogue group gets its last block from has one parity
-    // for each group when there are 2, 3 or 5 blocks.)
-    const bool can_shift = a.RA > 1 && a.RA != 4 && a.R - (a.RA - 1) * 128 <= 64;
-    auto shifted = [&](int i) { return can_shift && (i & 1); };
+    // exponentials spread over all four schedulers.
+    const int rem = a.R - (a.RA - 1) * 128;              // rows of the last block
+    const bool can_shift = a.RA > 1 && rem <= 64;
+    const int slots = a.RA + (can_shift ? 1 : 0);        // sums a thread keeps in pass A: one by block, the last block's on shifted tiles apart
+    const int accs = pool_a ? 3 : 4;                     // accumulators and epilogue warpgroups of pass A
+    constexpr int kBarA = 1;                             // named barrier: every accumulator of pass A has been read
+    const int bar_a_threads = (accs * 4 + (pool_a ? 2 : 3)) * 32;
 
     if (ntl > 0) {
     if (warp == 0) {
-        // ------------------------------------------------------------------ TMA producer
+        // ------------------------------------------------------------------ TMA producer: key tiles
         if (lane == 0) {
             // what depends on the slab only is kept in registers: between "stage free" and the next copy's issue nothing
             // waits on shared or global memory
-            int stage = 0;
-            uint32_t lap = 0, qlap = 0;
+            int stage = 0, slab = slab_of(tile_at(0)), lo = 0, hi = 0, row0 = 0;       // tiles [lo, hi) belong to the slab
+            uint32_t lap = 0, odd = 0, used = 0;                    // position / stages; by stage: an odd number of loads, any load
             bool ok = true;
-            auto load_q = [&](int slab) {
-                if (qlap > 0) ok = role_wait(&ctl->qempty, (qlap - 1) & 1u, limit, &ctl->abort_flag, a.status);
-                if (!ok) return;
-                const int b = slab / Hk, h = slab % Hk;
-                mbar_expect_tx(&ctl->qfull, uint32_t(a.R) * kRowBytes);
-                for (int k = 0; k < a.RB; ++k)
-                    for (int half = 0; half < 2; ++half)
-                        tma_load_3d(qbuf + size_t(half) * q_half + size_t(k) * a.N * 128, &mapQ, half * 64, k * kWB, b * a.Hq + h * n, &ctl->qfull);
-                ++qlap;
-            };
-            auto load_tile = [&](int slab, int j, int row0) {
+            int p = 0, step = 1;
+            while (p >= 0 && ok) {
+                const int t = tile_at(p);
+                if (t >= hi || t < lo) {
+                    while (pref[slab + 1] <= t) ++slab;
+                    while (pref[slab] > t) --slab;
+                    lo = pref[slab]; hi = pref[slab + 1];
+                    row0 = rowb[slab];
+                }
+                const int j = t - lo;
                 const int row = a.block_table ? max(a.block_table[size_t(slab) * a.max_pages + j], 0) * 128 : row0 + j * 128;
-                if (lap > 0) ok = role_wait(&ctl->empty[stage], (lap - 1) & 1u, limit, &ctl->abort_flag, a.status);
-                if (!ok) return;
+                const uint32_t bit = 1u << stage;
+                if (used & bit) ok = role_wait(&ctl->empty[stage], (lap & 1u) ^ 1u, limit, &ctl->abort_flag, a.status);
+                if (!ok) break;
                 uint8_t* dst = tiles + size_t(stage) * kOpBytes;
                 mbar_expect_tx(&ctl->full[stage], kOpBytes);
                 tma_load_2d(dst, &mapK, 0, row, &ctl->full[stage]);
                 tma_load_2d(dst + kOpHalfBytes, &mapK, 64, row, &ctl->full[stage]);
-                if (++stage == a.stages) { stage = 0; ++lap; }
-            };
-            for (int pass = 0; pass < 2 && ok; ++pass) {
-                const int t_first = pass == 0 && !resident ? t_end - 1 : t_begin;
-                int slab = slab_of(t_first), lo = 0, hi = 0, row0 = 0;          // tiles [lo, hi) belong to the slab
-                for (int i = 0; i < ntl && ok; ++i) {
-                    const int t = pass == 0 && !resident ? t_end - 1 - i : t_begin + i;
-                    if (i == 0 || t >= hi || t < lo) {
-                        while (pref[slab + 1] <= t) ++slab;
-                        while (pref[slab] > t) --slab;
-                        lo = pref[slab]; hi = pref[slab + 1];
-                        row0 = rowb[slab];
-                        load_q(slab);
-                        if (!ok) break;
-                    }
-                    if (pass == 0 || !resident) load_tile(slab, t - lo, row0);
+                used |= bit;
+                odd ^= bit;
+                if (step > 0) {
+                    if (++stage == a.stages) { stage = 0; ++lap; }
+                    if (++p < ntl) continue;
+                    // (stage and lap stand at position ntl; position kept has the same stage a lap earlier, if any lap)
+                    step = -1;
+                    p = kept;
+                    if (ntl >= a.stages) --lap;
                 }
+                if (--stage < 0) { stage = a.stages - 1; --lap; }
+                --p;
             }
             // Whoever gave up: this warp stays until its copies have landed and the issuers' products have completed, so that the CTA gives
-            // back shared and tensor memory with nothing in flight.  Stage s was loaded lap (+ 1) times.
-            for (int s = 0; s < a.stages; ++s) {
-                const uint32_t loads = lap + (s < stage ? 1u : 0u);
-                if (loads) mbar_wait(&ctl->full[s], (loads - 1) & 1u, kRetirePolls);
-            }
-            if (qlap) mbar_wait(&ctl->qfull, (qlap - 1) & 1u, kRetirePolls);
+            // back shared and tensor memory with nothing in flight.
+            for (int s = 0; s < a.stages; ++s)
+                if ((used >> s) & 1u) mbar_wait(&ctl->full[s], ((odd >> s) & 1u) ^ 1u, kRetirePolls);
             for (int s = 0; s < 3; ++s) mbar_wait(&ctl->retired[s], 0u, kRetirePolls);
         }
-    } else if (warp == 1 || warp == 19) {
+    } else if (warp < 3) {
         // ------------------------------------------------------------------ MMA warps
-        // Two of them take the products in turn.  An issue blocks until the tensor core has taken the product, and a look
-        // at a barrier in between (115 cycles and more) leaves it idle; with two issuers one waits while the other's
-        // product runs (measured without epilogue: 817 against 579 cycles per 128 x 128 x 128 product, 512 the least).
-        const int mine = warp == 1 ? 0 : 1;
-        const uint32_t leader = elect_leader();
+        // Two of them take the products in turn, so that one looks at its barriers while the other's product runs.
+        const uint32_t mine = warp - 1, leader = elect_leader();
+        const uint32_t q0 = smem_u32(qbuf), tiles0 = smem_u32(tiles);
         bool ok = true;
-        uint32_t qlap = 0;
-        const uint32_t q0 = smem_u32(qbuf);
+        uint32_t qlap = 0, lap = 0;
+        int stage = 0;
+        // Both warps arrive on the stage of every tile, also where one has no product of it: a stage that was filled again before that one had
+        // seen it full would leave it waiting for a phase that is two back.  The third arrival is the pooling issuer's or, in the other pass, one more here.
+        auto free_stage = [&](bool has_product, bool pooled) {
+            if (has_product) umma_commit(&ctl->empty[stage], leader);
+            if (leader) {
+                if (!has_product) mbar_arrive(&ctl->empty[stage]);
+                if (!pooled && mine == 0) mbar_arrive(&ctl->empty[stage]);
+            }
+            __syncwarp();
+        };
         {
-            int stage = 0, it = 0, slab = slab_of(resident ? t_begin : t_end - 1), lo = 0, hi = 0;
-            uint32_t lap = 0;
-            const int n_empty = a.RB > 1 ? 3 : 2;        // arrivals that free a stage
-            for (int i = 0; i < ntl && ok; ++i) {
-                const int t = resident ? t_begin + i : t_end - 1 - i;
-                if (i == 0 || t >= hi || t < lo) {
+            int slab = slab_of(tile_at(0)), lo = 0, hi = 0;
+            // the next product: whose it is, its accumulator and its place in the ring of tempty
+            uint32_t turn = 0, buf = 0, ring = 0, par = 1;           // par: the parity to wait for, at the place half a ring on
+            bool first = true;                                       // nothing to wait for yet
+            const uint32_t n_acc = accs;
+            for (int p = 0; p < ntl && ok; ++p) {
+                const int t = tile_at(p);
+                if (t >= hi || t < lo) {
                     while (pref[slab + 1] <= t) ++slab;
                     while (pref[slab] > t) --slab;
                     lo = pref[slab]; hi = pref[slab + 1];
@@ -424,172 +454,240 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 }
                 // (both warps follow every tile's arrival, so that they see each phase of a stage's barrier)
                 ok = warp_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
-                bool here = false;                       // this warp has a product of the tile
-                for (int k = 0; k < a.RA && ok; ++k, ++it) {
-                    if ((it & 1) != mine) continue;
-                    here = true;
-                    const int buf = it & (kAGroups - 1), use = it / kAGroups;
-                    if (use > 0) ok = warp_wait(&ctl->tempty_a[buf], uint32_t(use - 1) & 1u, limit, &ctl->abort_flag, a.status);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const int r = k + 1 == a.RA && shifted(i) ? a.R - 128 : k * 128;       // first query row
-                    umma_tile(tmem_base + buf * 128, q0 + uint32_t(r) * 128u, q_half, smem_u32(tiles + size_t(stage) * kOpBytes),
-                              kOpHalfBytes, kIdescBf16M128N128, leader);
-                    umma_commit(&ctl->tfull_a[buf], leader);
+                for (int k = 0; k < a.RA && ok; ++k) {
+                    if (turn == mine) {
+                        // the product n_acc before this one has been read
+                        const bool upper = ring >= n_acc;
+                        if (!first || upper) ok = warp_wait(&ctl->tempty_a[upper ? ring - n_acc : ring + n_acc], upper ? par ^ 1u : par, limit, &ctl->abort_flag, a.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const int r = k + 1 == a.RA && can_shift && (p & 1) ? a.R - 128 : k * 128;     // first query row
+                        umma_tile(tmem_base + buf * 128, q0 + uint32_t(r) * 128u, q_half, tiles0 + uint32_t(stage) * kOpBytes,
+                                  kOpHalfBytes, kIdescBf16M128N128, leader);
+                        umma_commit(&ctl->tfull_a[buf], leader);
+                    }
+                    turn ^= 1u;
+                    if (++buf == n_acc) buf = 0;
+                    if (++ring == 2 * n_acc) { ring = 0; par ^= 1u; first = false; }
                 }
-                const int t_next = resident ? t + 1 : t - 1;
-                if (i + 1 == ntl || t_next >= hi || t_next < lo) umma_commit(&ctl->qempty, leader);
-                if (!resident && here) {                 // one warp: all arrivals; two: the second one of the tile makes up the number
-                    const int c = a.RA == 1 ? n_empty : (((it - 1) & 1) == mine ? n_empty - 1 : 1);
-                    for (int e = 0; e < c; ++e) umma_commit(&ctl->empty[stage], leader);
+                if (p + 1 < ntl) {                                   // (the last slab's rows stay for pass B)
+                    const int t_next = tile_at(p + 1);
+                    if (t_next >= hi || t_next < lo) umma_commit(&ctl->qempty, leader);
                 }
+                if (p < kept) free_stage(a.RA > 1 || turn != mine, pool_a);
                 if (++stage == a.stages) { stage = 0; ++lap; }
             }
         }
-        __syncwarp();
         tc_fence_before();
-        named_bar_sync(1, kSweepThreads - 32);           // every accumulator of pass A has been read
+        named_bar_sync(kBarA, bar_a_threads);
         tc_fence_after();
         if (ok) {
-            int it = 0, slab = slab_of(t_begin), hi = 0, stage = resident ? 0 : ntl % a.stages;
-            uint32_t elap = 0, lap = resident ? 0u : uint32_t(ntl / a.stages);
+            int slab = slab_of(tile_at(ntl - 1)), lo = 0, hi = 0;
+            uint32_t elap = 0, turn = 0, buf = 0, ring = 0, par = 1;
+            bool first = true;
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t(a.N) >> 3) << 17) | ((128u >> 4) << 24);
             const uint64_t d_ones = umma_desc_sw32(smem_u32(onesb));
-            for (int i = 0; i < ntl && ok; ++i) {
-                const int t = t_begin + i;
-                if (i == 0 || t >= hi) {
+            for (int p = ntl - 1; p >= 0 && ok; --p) {
+                const int t = tile_at(p);
+                if (--stage < 0) { stage = a.stages - 1; --lap; }
+                if (t >= hi || t < lo) {
                     while (pref[slab + 1] <= t) ++slab;
-                    hi = pref[slab + 1];
-                    ok = warp_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status) &&
-                         warp_wait(&ctl->extfull, elap & 1u, limit, &ctl->abort_flag, a.status);
+                    while (pref[slab] > t) --slab;
+                    lo = pref[slab]; hi = pref[slab + 1];
+                    if (elap > 0) {                                  // (the first slab's query rows are there)
+                        ok = warp_wait(&ctl->qfull, qlap & 1u, limit, &ctl->abort_flag, a.status);
+                        ++qlap;
+                    }
+                    if (ok) ok = warp_wait(&ctl->extfull, elap & 1u, limit, &ctl->abort_flag, a.status);
                     if (!ok) break;
-                    ++qlap; ++elap;
+                    ++elap;
                 }
                 ok = warp_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
-                bool here = false;
-                for (int k = 0; k < a.RB && ok; ++k, ++it) {
-                    if ((it & 1) != mine) continue;
-                    here = true;
-                    const int buf = it % kBGroups, before = it - kBGroups;
-                    if (before >= 0) ok = warp_wait(&ctl->tempty_b[before % (2 * kBGroups)], uint32_t(before / (2 * kBGroups)) & 1u, limit, &ctl->abort_flag, a.status);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t d = tmem_base + buf * kBAccCols;
-                    umma_tile(d, smem_u32(tiles + size_t(stage) * kOpBytes), kOpHalfBytes, q0 + uint32_t(k * a.N) * 128u, q_half, idesc, leader);
-                    umma_bf16(d, d_ones, umma_desc_sw32(ext_smem + uint32_t(k * a.N) * kExtRow), idesc, 1u, leader);      // - lse
-                    umma_commit(&ctl->tfull_b[buf], leader);
+                for (int k = 0; k < a.RB && ok; ++k) {
+                    if (turn == mine) {
+                        const bool upper = ring >= kAccB;
+                        if (!first || upper) ok = warp_wait(&ctl->tempty_b[upper ? ring - kAccB : ring + kAccB], upper ? par ^ 1u : par, limit, &ctl->abort_flag, a.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t d = tmem_base + buf * kAccCols;
+                        umma_tile(d, tiles0 + uint32_t(stage) * kOpBytes, kOpHalfBytes, q0 + uint32_t(k * a.N) * 128u, q_half, idesc, leader);
+                        umma_bf16(d, d_ones, umma_desc_sw32(ext_smem + uint32_t(k * a.N) * kExtRow), idesc, 1u, leader);      // - lse
+                        umma_commit(&ctl->tfull_b[buf], leader);
+                    }
+                    turn ^= 1u;
+                    if (++buf == kAccB) buf = 0;
+                    if (++ring == 2 * kAccB) { ring = 0; par ^= 1u; first = false; }
                 }
-                if (i + 1 == ntl || hi <= t + 1) { umma_commit(&ctl->qempty, leader); umma_commit(&ctl->extempty, leader); }
-                if (here) umma_commit(&ctl->empty[stage], leader);
-                if (++stage == a.stages) { stage = 0; ++lap; }
+                if (p > 0) {
+                    const int t_next = tile_at(p - 1);
+                    if (t_next >= hi || t_next < lo) { umma_commit(&ctl->qempty, leader); umma_commit(&ctl->extempty, leader); }
+                }
+                free_stage(a.RB > 1 || turn != mine, !pool_a);
             }
         }
         umma_commit(&ctl->retired[mine], leader);
-    } else {
-        // ------------------------------------------------------------------ pass A: epilogue warpgroups (and the clearing warp)
-        const int quarter = warp & 3;                        // tensor-memory lanes this warp may read
+    } else if (warp == 3) {
+        // ------------------------------------------------------------------ issuer of the pooling products, TMA producer of the query rows
+        // (not the tiles' producer: the rows of a slab wait until the slab before is done, which must not hold up the tiles)
+        const uint32_t leader = elect_leader();
+        const uint32_t indb_u32 = smem_u32(indb), tiles0 = smem_u32(tiles);
+        uint32_t laps = 0;
         bool ok = true;
-        {
-            const int g = (warp - 2) >> 2;                   // warpgroup (warp 18: 4, clears the key sums)
-            const int row = quarter * 32 + lane;
-            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + g * 128;
-            float2* part = reinterpret_cast<float2*>(extb);  // [group][RA * 128]
-            const bool g_shifted = can_shift && (a.RA == 2 ? g == 3 : (g & 1) != 0);
-            const int rem = a.R - (a.RA - 1) * 128;          // rows of the last block
-            int it = g, ti = g / a.RA, tk = g - ti * a.RA;   // this group's next product: its number, tile (in the order of the pass) and block
-            int slab = slab_of(resident ? t_begin : t_end - 1);
+        int pc = 0, run = -1, slab = slab_of(tile_at(0));
+        for (int pass = 0; pass < 2; ++pass) {           // (whoever gave up: everyone comes to the barrier)
+            const bool pooling = (pass == 0) == pool_a;
+            if (pass == 1 && !pool_a) {                  // (the pooled sums lie where the last accumulator of pass A was)
+                tc_fence_before();
+                named_bar_sync(kBarA, bar_a_threads);
+                tc_fence_after();
+            }
+            int p = pass == 0 ? 0 : ntl - 1, stage = p % a.stages;
+            uint32_t lap = uint32_t(p / a.stages);
+            while (p >= 0 && p < ntl && ok) {
+                // the part of a slab that begins at position p
+                const int t = tile_at(p);
+                while (pref[slab + 1] <= t) ++slab;
+                while (pref[slab] > t) --slab;
+                const int n_tiles = min(pref[slab + 1], t_end) - max(pref[slab], t_begin);
+                if (pass == 0 || p < ntl - 1) {          // (pass B begins with the slab that is there)
+                    if (laps > 0) ok = warp_wait(&ctl->qempty, (laps - 1) & 1u, limit, &ctl->abort_flag, a.status);
+                    if (!ok) break;
+                    if (leader) {
+                        const int b = slab / Hk, h = slab % Hk;
+                        mbar_expect_tx(&ctl->qfull, uint32_t(a.R) * kRowBytes);
+                        for (int k = 0; k < a.RB; ++k)
+                            for (int half = 0; half < 2; ++half)
+                                tma_load_3d(qbuf + size_t(half) * q_half + size_t(k) * a.N * 128, &mapQ, half * 64, k * kWB, b * a.Hq + h * n, &ctl->qfull);
+                    }
+                    __syncwarp();
+                    ++laps;
+                }
+                p += pass == 0 ? n_tiles : -n_tiles;
+                for (int j = 0; j < n_tiles && pooling; ++j) {
+                    ok = warp_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
+                    if (!ok) break;
+                    int flags = 0;
+                    do {
+                        const int is = pc & ((1 << a.ind_log) - 1);
+                        ok = warp_wait(&ctl->ifull[is], uint32_t(pc >> a.ind_log) & 1u, limit, &ctl->abort_flag, a.status);
+                        if (!ok) break;
+                        flags = *reinterpret_cast<volatile int*>(&ctl->ind_flags[is]);       // 1: more, 2: joins the run, 4: closes one
+                        tc_fence_after();
+                        if (flags & 4) umma_commit(&ctl->pfull[run & 1], leader);            // everything of the run before is issued
+                        if (!(flags & 2)) ++run;
+                        umma_pool(tmem_base + kPoolCol + uint32_t(run & 1) * kIndSlots, tiles0 + uint32_t(stage) * kOpBytes,
+                                  indb_u32 + uint32_t(is) * kIndBytes, (flags & 2) != 0, leader);
+                        umma_commit(&ctl->iempty[is], leader);
+                        ++pc;
+                    } while (flags & 1);
+                    if (!ok) break;
+                    if (pass == 1) {
+                        umma_commit(&ctl->empty[stage], leader);
+                        if (--stage < 0) { stage = a.stages - 1; --lap; }
+                    } else {
+                        if (int(lap) * a.stages + stage < kept) umma_commit(&ctl->empty[stage], leader);
+                        if (++stage == a.stages) { stage = 0; ++lap; }
+                    }
+                }
+            }
+            if (pooling && ok && run >= 0) umma_commit(&ctl->pfull[run & 1], leader);
+        }
+        umma_commit(&ctl->retired[2], leader);
+        if (laps) mbar_wait(&ctl->qfull, (laps - 1) & 1u, kRetirePolls);             // nothing in flight at the end, whoever gave up
+    } else {
+        // ------------------------------------------------------------------ epilogue warpgroups
+        const int quarter = warp & 3;                        // tensor-memory lanes this warp may read
+        const int g = (warp - 4) >> 2;
+        const int row = quarter * 32 + lane;
+        const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16);
+        bool ok = true;
+        if (g < accs) {
+            // -------------------------------------------------------------- pass A: log-sum-exp, a thread per query row
+            float2* part = reinterpret_cast<float2*>(extb);  // [group][slots][128] reference and sum
+            float2* my = part + g * slots * 128 + row;
+            const uint32_t acc = lane_addr + g * 128;
+            uint32_t turn = 0;                               // products of this group so far
+            int ti = 0, tk = g;                              // its next product: position and block
+            while (tk >= a.RA) { tk -= a.RA; ++ti; }
+            int slab = slab_of(tile_at(0));
             for (int done = 0; done < ntl;) {
                 // one segment: the tiles of a slab that this CTA has
-                const int t_cur = resident ? t_begin + done : t_end - 1 - done;
+                const int t_cur = tile_at(done);
                 while (pref[slab + 1] <= t_cur) ++slab;
                 while (pref[slab] > t_cur) --slab;
-                const int lo = max(pref[slab], t_begin), hi = min(pref[slab + 1], t_end), seg_end = done + (hi - lo);
-                const int fc = owner(pref[slab]), lc = owner(pref[slab + 1] - 1);
-                if (g < kAGroups) {
-                    const int N = live(slab);
-                    float m[kMaxBlocksA], l[kMaxBlocksA];
-#pragma unroll
-                    for (int k = 0; k < kMaxBlocksA; ++k) { m[k] = -INFINITY; l[k] = 0.f; }
-                    for (; ti < seg_end; it += kAGroups) {
-                        const int t = resident ? t_begin + ti : t_end - 1 - ti;
-                        const int valid = min(128, N - (t - pref[slab]) * 128);
-                        if (ok) {
-                            ok = role_wait(&ctl->tfull_a[g], uint32_t(it / kAGroups) & 1u, limit, &ctl->abort_flag, a.status);
-                            ok = __all_sync(0xffffffffu, ok);
-                        }
-                        if (ok) {
-                            tc_fence_after();
-                            // (the last block may hold fewer rows than lanes)
-                            if (tk + 1 < a.RA || (g_shifted ? quarter * 32 + 31 >= 128 - rem : quarter * 32 < rem)) {
-                                float mk = m[0], lk = l[0];
-#pragma unroll
-                                for (int k = 1; k < kMaxBlocksA; ++k) if (tk == k) { mk = m[k]; lk = l[k]; }
-                                if (valid == 128) lse_fold<false>(lane_addr, valid, scale, mk, lk);
-                                else              lse_fold<true>(lane_addr, valid, scale, mk, lk);
-#pragma unroll
-                                for (int k = 0; k < kMaxBlocksA; ++k) if (tk == k) { m[k] = mk; l[k] = lk; }
-                            }
+                const int lo = pref[slab], n_tiles = min(pref[slab + 1], t_end) - max(lo, t_begin), seg_end = done + n_tiles;
+                const int N = live(slab);
+                for (int k = 0; k < slots; ++k) my[k * 128] = make_float2(-INFINITY, 0.f);
+                while (ti < seg_end) {
+                    const int valid = min(128, N - (tile_at(ti) - lo) * 128);
+                    const bool sh = tk + 1 == a.RA && can_shift && (ti & 1);
+                    float2* ml = my + (sh ? a.RA : tk) * 128;
+                    float2 x = *ml;
+                    if (ok) ok = warp_wait(&ctl->tfull_a[g], turn & 1u, limit, &ctl->abort_flag, a.status);
+                    if (ok) {
+                        tc_fence_after();
+                        auto release = [&]() {               // this warp's loads of the accumulator have completed
                             tc_fence_before();
                             __syncwarp();
-                            if (lane == 0) mbar_arrive(&ctl->tempty_a[g]);
+                            if (lane == 0) mbar_arrive(&ctl->tempty_a[g + (turn & 1u) * accs]);
+                        };
+                        // (the last block may hold fewer rows than lanes)
+                        if (tk + 1 < a.RA || (sh ? quarter * 32 + 31 >= 128 - rem : quarter * 32 < rem)) {
+                            if (valid == 128) lse_fold<false>(acc, valid, scale, x.x, x.y, release);
+                            else              lse_fold<true>(acc, valid, scale, x.x, x.y, release);
+                            *ml = x;
+                        } else {
+                            release();
                         }
-                        tk += kAGroups;
-                        while (tk >= a.RA) { tk -= a.RA; ++ti; }
                     }
-#pragma unroll
-                    for (int k = 0; k < kMaxBlocksA; ++k)
-                        if (k < a.RA) part[(g * a.RA + k) * 128 + row] = make_float2(m[k], l[k]);
-                } else {
-                    // this CTA's share of the slab's key sums, which pass B accumulates
-                    const int S = min(max(a.n_sent[slab], 0), a.max_sent), P = lc - fc + 1, p = cta - fc;
-                    float4* v4 = reinterpret_cast<float4*>(a.vsum + size_t(slab) * a.max_sent * kHeadDim);
-                    const int w1 = int((long long)S * 32 * (p + 1) / P);
-                    for (int w = int((long long)S * 32 * p / P) + lane; w < w1; w += 32) v4[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    ++turn;
+                    tk += accs;
+                    while (tk >= a.RA) { tk -= a.RA; ++ti; }
                 }
-                named_bar_sync(2, (4 * kAGroups + 1) * 32);
-                if (g == 0) {                                // the four groups' parts -> one record per CTA and slab
-                    float2* rec = a.rec + size_t(cta + slab) * (size_t(a.RA) * 128);
-                    for (int k = 0; k < a.RA; ++k) {
-                        float2 x[kAGroups];
-                        float M = -INFINITY, L = 0.f;
-#pragma unroll
-                        for (int q = 0; q < kAGroups; ++q) {
-                            const bool sh = k + 1 == a.RA && can_shift && (a.RA == 2 ? q == 3 : (q & 1) != 0);
-                            x[q] = part[(q * a.RA + k) * 128 + (sh ? min(row + 128 - rem, 127) : row)];
-                            M = fmaxf(M, x[q].x);
-                        }
-#pragma unroll
-                        for (int q = 0; q < kAGroups; ++q) L += x[q].y > 0.f ? x[q].y * ex2f(x[q].x - M) : 0.f;
-                        rec[k * 128 + row] = make_float2(M, L);
+                if (seg_end == ntl) {
+                    tc_fence_before();
+                    named_bar_arrive(kBarA, bar_a_threads);          // (the issuers go on to pass B)
+                }
+                named_bar_sync(2, accs * 128);
+                float2* rec = a.rec + size_t(cta + slab) * (size_t(a.RA) * 128);
+                for (int k = g; k < a.RA; k += accs) {       // the groups' parts -> one record per CTA and slab
+                    float M = -INFINITY, L = 0.f;
+                    auto add = [&](float2 x) {
+                        const float m = fmaxf(M, x.x);
+                        L *= L > 0.f ? ex2f(M - m) : 0.f;
+                        L += x.y > 0.f ? x.y * ex2f(x.x - m) : 0.f;
+                        M = m;
+                    };
+                    for (int q = 0; q < accs; ++q) {
+                        add(part[(q * slots + k) * 128 + row]);
+                        if (can_shift && k + 1 == a.RA && row < rem) add(part[(q * slots + a.RA) * 128 + row + 128 - rem]);
                     }
-                    named_bar_sync(3, 128);
-                    if (tid == 64 && ok) { __threadfence(); atomicAdd(a.lse_cnt + slab, uint32_t(hi - lo)); }
+                    rec[k * 128 + row] = make_float2(M, L);
                 }
-                named_bar_sync(4, (4 * kAGroups + 1) * 32);  // the parts have been read
+                named_bar_sync(4, accs * 128);               // the parts have been read, the record is written
+                if (tid == 128 && ok) { __threadfence(); atomicAdd(a.lse_cnt + slab, uint32_t(n_tiles)); }
                 done = seg_end;
             }
         }
-        tc_fence_before();
-        named_bar_sync(1, kSweepThreads - 32);               // every accumulator of pass A has been read
-        tc_fence_after();
-        const int load0 = resident ? 0 : ntl;                // the ring's tiles before pass B
-        if (warp < 10 || (warp >= 14 && warp < 18)) {
+        if (g < 3) {
             // -------------------------------------------------------------- pass B: importance, a thread per token
-            const int g = warp < 10 ? (warp - 2) >> 2 : 2;
-            const int row = quarter * 32 + lane;
-            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16);
             // (what depends on the slab only is kept in registers: while the tensor core streams its operands every look at
             // shared memory takes a hundred cycles and more)
-            int slab = slab_of(t_begin), lo = 0, hi = 0, N = 0;         // the slab's tiles are [lo, hi)
+            const uint32_t acc = lane_addr + g * kAccCols;
+            uint32_t turn = 0;                               // products of this group so far
+            int slab = slab_of(tile_at(ntl - 1)), lo = 0, hi = 0, N = 0;        // the slab's tiles are [lo, hi)
             uint32_t ext_no = 0;                             // slabs begun so far
             float *imp_ws = nullptr, *imp_user = nullptr;
             float out_scale = 0.f;                           // 2^-e / window of the slab
-            int ti = 0, tk = 0;
-            for (int it = 0; it < ntl * a.RB; ++it) {
-                const int t = t_begin + ti, i = ti, k = tk;
+            int ti = 0, tk = 0, mod = 0;                     // tile in the order of the pass, block, and whose product it is
+            for (int left = ntl * a.RB; left > 0; --left) {
+                const int t = tile_at(ntl - 1 - ti), i = ti, k = tk, whose = mod;
                 if (++tk == a.RB) { tk = 0; ++ti; }
-                if (t >= hi) {
+                if (++mod == kAccB) mod = 0;
+                const bool begins = t >= hi || t < lo;
+                if (begins) {
                     while (pref[slab + 1] <= t) ++slab;
+                    while (pref[slab] > t) --slab;
                     lo = pref[slab]; hi = pref[slab + 1];
                     N = live(slab);
                     out_scale = __uint_as_float(uint32_t(127 - lse_shift(N)) << 23) / float(a.window);
@@ -597,8 +695,8 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     imp_user = a.tok_imp_user ? a.tok_imp_user + (a.block_table ? size_t(slab) * a.max_pages * 128 : size_t(rowb[slab])) : nullptr;
                     ++ext_no;
                 }
-                if (it % kBGroups != g) continue;
-                if (k == 0 && t == max(lo, t_begin)) {
+                if (whose != g) continue;
+                if (begins) {
                     // the group of a slab's first product prepares the slab: log-sum-exp of its query rows from the records of
                     // all its CTAs, negated, in units of raw logits, as three bf16 pieces of the extra K step
                     const int fc = owner(lo), lc = owner(hi - 1);
@@ -611,18 +709,18 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                         const int n_part = lc - fc + 1;
                         for (int r = row; r < a.R; r += 128) {
                             float M = -INFINITY, L = 0.f;
-                            for (int p0 = 0; p0 < n_part; p0 += 8) {         // eight records per round: their loads are in flight together
-                                float2 x[8];
+                            for (int p0 = 0; p0 < n_part; p0 += 4) {         // four records per round: their loads are in flight together
+                                float2 x[4];
 #pragma unroll
-                                for (int p = 0; p < 8; ++p)
+                                for (int p = 0; p < 4; ++p)
                                     x[p] = p0 + p < n_part ? __ldcg(r0 + size_t(p0 + p) * (a.RA * 128) + r) : make_float2(-INFINITY, 0.f);
                                 float mx = M;
 #pragma unroll
-                                for (int p = 0; p < 8; ++p) mx = fmaxf(mx, x[p].x);
+                                for (int p = 0; p < 4; ++p) mx = fmaxf(mx, x[p].x);
                                 L *= M == -INFINITY ? 0.f : ex2f(M - mx);
                                 M = mx;
 #pragma unroll
-                                for (int p = 0; p < 8; ++p) L += x[p].y > 0.f ? x[p].y * ex2f(x[p].x - M) : 0.f;
+                                for (int p = 0; p < 4; ++p) L += x[p].y > 0.f ? x[p].y * ex2f(x[p].x - M) : 0.f;
                             }
                             // (the exponent of the sum apart, so that neither its logarithm nor the total is rounded at a larger magnitude)
                             const int ex = int(__float_as_uint(L) >> 23) - 127;
@@ -641,27 +739,24 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                         if (lane == 0) mbar_arrive(&ctl->extfull);
                     }
                 }
-                if (ok) {
-                    ok = role_wait(&ctl->tfull_b[g], uint32_t(it / kBGroups) & 1u, limit, &ctl->abort_flag, a.status);
-                    ok = __all_sync(0xffffffffu, ok);
-                }
+                if (ok) ok = warp_wait(&ctl->tfull_b[g], turn & 1u, limit, &ctl->abort_flag, a.status);
                 if (!ok) continue;
                 tc_fence_after();
-                float total = imp_fold<kWB>(lane_addr + g * kBAccCols, n, min(kWB, a.window - k * kWB), scale);
+                float total = imp_fold<kWB>(acc, n, min(kWB, a.window - k * kWB), scale);
                 float* share = tokp + (i & 3) * (a.RB - 1) * 128 + row;
                 if (k + 1 < a.RB) {
                     share[k * 128] = total;                  // another group adds the shares up, in the order of the blocks
                 } else if (a.RB > 1) {
-                    ok = role_wait(&ctl->tokfull[i & 3], uint32_t(i >> 2) & 1u, limit, &ctl->abort_flag, a.status);
-                    ok = __all_sync(0xffffffffu, ok);
+                    ok = warp_wait(&ctl->tokfull[i & 3], uint32_t(i >> 2) & 1u, limit, &ctl->abort_flag, a.status);
                     for (int q = a.RB - 2; q >= 0; --q) total += share[q * 128];
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) {
                     if (k + 1 < a.RB) mbar_arrive(&ctl->tokfull[i & 3]);
-                    mbar_arrive(&ctl->tempty_b[it % (2 * kBGroups)]);
+                    mbar_arrive(&ctl->tempty_b[g + (turn & 1u) * kAccB]);
                 }
+                ++turn;
                 const int tok = (t - lo) * 128 + row;
                 if (k + 1 == a.RB && ok && tok < N) {
                     const float v = total * out_scale;
@@ -669,174 +764,144 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     if (imp_user) imp_user[tok] = v;
                 }
             }
-        } else if (warp < 14) {
-            // -------------------------------------------------------------- pass B: per-sentence sums of the key rows
+        } else {
+            // -------------------------------------------------------------- per-sentence sums of the key rows
             // The sums are a product on the tensor cores: (tile^T: channel x token) x (indicator: token x sentence slot).
             // A run of consecutive tiles whose sentences all fall among the 16 sentences B .. B + 15 shares one accumulator
-            // (slot j = sentence B + j; the products of the run accumulate), so the sums are read out and added to global
+            // (slot j = sentence B + j; the products of the run accumulate), so the sums are read out and stored to global
             // memory once per run, about every fifth tile.  Each of the four warps writes a quarter of a tile's matrix and
-            // arrives; one thread of a fifth warp issues the product; when a tile opens a new run the four warps read out the
-            // run before it (a thread owns one channel) while the new one is being multiplied.  A tile that touches more
-            // than 16 sentences (empty ones count) gets several matrices, each a run of its own.
-            // Every warp keeps, one entry per lane, the sentence offsets B .. B + 31 of the current run (entries past the
-            // table read as "never starts"), fetched from global memory when a run opens: loads from shared memory wait
-            // several hundred cycles here (the tensor core streams its operands from it), so the per-tile work touches
-            // shared memory only to write the matrix.
+            // arrives; a fifth warp issues the product.  A tile that touches more than 16 sentences (empty ones count) gets several
+            // matrices, each a run of its own.
+            // The matrices depend on the sentence offsets alone, so they run ahead of the tiles, as far as their ring goes.  Every
+            // warp keeps, one entry per lane, the offsets B .. B + 31 of the current run (entries past the table read as "never
+            // starts"), from which a run's length, its sentences and the next run's first sentence follow at once; the next run's offsets
+            // are fetched while this one's matrices are written.  (With the run worked out tile by tile, behind the tile's arrival, a tile took
+            // these warps 2260 clocks and pass A 1.15 us.)
+            // A sentence that began in an earlier run of this CTA is added to; one that began before the CTA's range belongs to the CTA in whose
+            // range it began: its part is kept until every CTA of the slab has stored its sums, and added then.  So nothing has to be cleared.
             constexpr int kNever = 0x7fffffff;
-            const int gw = warp - 10;                               // warp of the group: slots 4 gw .. 4 gw + 3 of a matrix
-            const int gtid = tid - 320;
-            const int ch = quarter * 32 + lane;
-            const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + kPoolCol;
-            int slab = slab_of(t_begin), S = 0, N = 0, first = 0;
-            int ic = 0;                                             // indicator matrices written so far
-            int run = -1, B = 0, w = kNever, w1 = kNever;           // current run: index, sentence of slot 0, offsets B + lane and B + lane + 1
-            int wj = kNever, wj1 = kNever;                          // and the offsets of this thread's slot row
-            const int sj = 4 * gw + (lane >> 3);                    // the slot row, of which this thread writes two pieces
-            int lo = 0, hi = 0, stage = load0 % a.stages;           // the slab's tiles are [lo, hi)
-            uint32_t lap = uint32_t(load0 / a.stages);
-            uint32_t run_held = 0;                                  // its slots that hold tokens so far
-            int run_slab = 0;
+            const int gw = quarter;                               // warp of the group: slots 4 gw .. 4 gw + 3 of a matrix
+            const int gtid = tid - 512;
+            const int ch = row;
+            const int sj = 4 * gw + (lane >> 3), sq = lane & 7;     // this thread writes tokens 16 sq .. 16 sq + 15 of slot row sj
+            const int ring = (1 << a.ind_log) - 1;
+            int slab = slab_of(t_begin), lo = 0, hi = 0, S = 0, N = 0;      // the slab's tiles are [lo, hi)
+            const int slab_first = slab;
             const int32_t* so = a.sent_off;
+            int t = t_begin, ic = 0, run = 0;                       // next tile, matrices written, runs opened
+            int B = 0, w = kNever;                                  // the run's first sentence, offset of sentence B + lane
+            float head = 0.f;
+            int head_sent = -1;
             // 32-way search for the last sentence that starts at or before token `tok`, one probe per lane
             auto holder = [&](int tok) {
-                int lo = 0, len = S;
+                int first = 0, len = S;
                 while (len > 32) {
                     const int stride = (len + 31) >> 5;
-                    const int pidx = lo + lane * stride;
-                    const bool le = pidx < lo + len && so[pidx] <= tok;
+                    const int pidx = first + lane * stride;
+                    const bool le = pidx < first + len && so[pidx] <= tok;
                     const int adv = max(__popc(__ballot_sync(0xffffffffu, le)) - 1, 0) * stride;
                     len = min(stride, len - adv);
-                    lo += adv;
+                    first += adv;
                 }
-                const bool le = lane < len && so[lo + lane] <= tok;
-                return lo + max(__popc(__ballot_sync(0xffffffffu, le)) - 1, 0);
+                const bool le = lane < len && so[first + lane] <= tok;
+                return first + max(__popc(__ballot_sync(0xffffffffu, le)) - 1, 0);
             };
-            // read out run r (accumulator r & 1) and add it to the sums
-            auto drain = [&](int r, int r_slab, int r_B, uint32_t r_held) {
-                ok = role_wait(&ctl->pfull[r & 1], uint32_t(r >> 1) & 1u, limit, &ctl->abort_flag, a.status);
-                ok = __all_sync(0xffffffffu, ok);
+            auto fetch = [&](int first) { return first + lane <= S ? so[first + lane] : kNever; };
+            // the run before, to be read out: its slab, first sentence, slots that hold tokens; where its first sentence began (0: in it, 1: in an
+            // earlier run, 2: before the CTA's range); where it is the last of a slab, the tiles that this CTA has of it
+            int p_slab = 0, p_B = 0, p_from = 0, p_tiles = 0;
+            uint32_t p_held = 0;
+            auto drain = [&](int r) {                               // (accumulator r & 1)
+                ok = warp_wait(&ctl->pfull[r & 1], uint32_t(r >> 1) & 1u, limit, &ctl->abort_flag, a.status);
                 if (!ok) return;
                 tc_fence_after();
                 float v[kIndSlots];
-                tmem_ld16(lane_addr + uint32_t(r & 1) * kIndSlots, v);
+                tmem_ld16(lane_addr + kPoolCol + uint32_t(r & 1) * kIndSlots, v);
                 tc_fence_before();
-                float* dst = a.vsum + (size_t(r_slab) * a.max_sent + r_B) * kHeadDim + ch;
+                float* dst = a.vsum + (size_t(p_slab) * a.max_sent + p_B) * kHeadDim + ch;
+                if (p_held & 1u) {
+                    if (p_from == 2) { head += v[0]; head_sent = p_B; }
+                    else if (p_from == 1) atomicAdd(dst, v[0]);
+                    else *dst = v[0];
+                }
 #pragma unroll
-                for (int j = 0; j < kIndSlots; ++j)
-                    if (r_held & (1u << j)) atomicAdd(dst + size_t(j) * kHeadDim, v[j]);
+                for (int j = 1; j < kIndSlots; ++j)
+                    if (p_held & (1u << j)) dst[size_t(j) * kHeadDim] = v[j];
+                if (p_tiles > 0) {
+                    __syncwarp();
+                    if (lane == 0) { __threadfence(); atomicAdd(a.sum_cnt + p_slab, uint32_t(p_tiles)); }
+                }
             };
-            for (int tl = 0; tl < ntl && ok; ++tl) {
-                const int t = t_begin + tl;
-                const bool fresh = t >= hi;
-                if (fresh) {
+            while (t < t_end && ok) {
+                if (t >= hi) {
                     while (pref[slab + 1] <= t) ++slab;
                     lo = pref[slab]; hi = pref[slab + 1];
                     so = a.sent_off + size_t(slab) * (a.max_sent + 1);
                     S = min(max(a.n_sent[slab], 0), a.max_sent);
                     N = live(slab);
-                    // every CTA of the slab has cleared its share of the sums (and left its record)
-                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(hi - lo), limit, &ctl->abort_flag, a.status);
-                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                    if (!ok) break;
+                    B = t > lo ? holder((t - lo) * 128) : 0;        // (a slab that opens with empty sentences: they get slots)
+                    w = fetch(B);
                 }
-                const int tok0 = (t - lo) * 128, valid = min(128, N - tok0), tok_end = tok0 + valid;
-                if (fresh) first = tok0 > 0 ? holder(tok0) : 0;     // (a slab that opens with empty sentences: they get slots)
-                // every warp follows every tile's arrival (in order, so it sees each phase of the stage's barrier)
-                ok = role_wait(&ctl->full[stage], lap & 1u, limit, &ctl->abort_flag, a.status);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                if (valid < 128) {
-                    // a zero in the indicator does not silence a NaN or an infinity in a dead row: clear the rows past the
-                    // slab's end in the staged tile (the logits of those rows are never read)
-                    uint8_t* tile = tiles + size_t(stage) * kOpBytes;
-                    for (int u = valid * 8 + gtid; u < 128 * 8; u += kPoolWarps * 32) {
-                        *reinterpret_cast<uint4*>(tile + u * 16) = make_uint4(0u, 0u, 0u, 0u);
-                        *reinterpret_cast<uint4*>(tile + kOpHalfBytes + u * 16) = make_uint4(0u, 0u, 0u, 0u);
-                    }
+                // the run: all tiles that end at or before sentence B + 16 begins, at least one
+                const int tok0 = (t - lo) * 128, last_tile = min(hi, t_end);
+                const int stop = B + kIndSlots < S ? __shfl_sync(0xffffffffu, w, kIndSlots) : kNever;
+                const int fit = stop >= N ? last_tile - t : min(last_tile - t, max(stop - tok0, 0) >> 7);
+                const int more = fit == 0 ? 1 : 0, n_tiles = max(fit, 1);           // more: slot 15 leaves some of the tile
+                const int tok_end = min(tok0 + n_tiles * 128, N);
+                const int w1 = __shfl_down_sync(0xffffffffu, w, 1);
+                const uint32_t held = __ballot_sync(0xffffffffu, lane < kIndSlots && B + lane < S && min(w1, tok_end) > max(w, tok0));
+                const int began = __shfl_sync(0xffffffffu, w, 0);
+                int wj = __shfl_sync(0xffffffffu, w, sj), wj1 = __shfl_sync(0xffffffffu, w, sj + 1);    // this thread's slot row
+                if (B + sj >= S) wj = wj1 = kNever;
+                // the next run: in the same tile, or in the last sentence that starts at or before the next tile's first token
+                int B_next = B + kIndSlots, w_next = kNever;
+                if (!more && t + n_tiles < last_tile) {
+                    const int n_le = __popc(__ballot_sync(0xffffffffu, B + lane < S && w <= tok_end));
+                    B_next = (n_le == 32 && B + 32 < S) ? holder(tok_end) : B + max(n_le - 1, 0);
                 }
-                int cur = first;                                    // first sentence of the tile not yet in a matrix
-                int more = 0;
-                do {
-                    // can the tile (from sentence cur on) join the open run?  its last sentence must be below B + 16
-                    bool join = false;
-                    if (run >= 0 && !fresh && cur >= B && cur - B < kIndSlots) {
-                        const int touching = __popc(__ballot_sync(0xffffffffu, lane > cur - B && B + lane < S && w < tok_end));
-                        join = cur + touching - B < kIndSlots;
-                    }
-                    const int r_prev = run, p_slab = run_slab, p_B = B;
-                    const uint32_t p_held = run_held;
-                    if (!join) {                                    // open a run at sentence cur
-                        ++run; B = cur; run_slab = slab; run_held = 0;
-                        w = (B + lane <= S) ? so[B + lane] : kNever;
-                        w1 = (B + lane + 1 <= S) ? so[B + lane + 1] : kNever;
-                        wj = (B + sj <= S) ? so[B + sj] : kNever;
-                        wj1 = (B + sj + 1 <= S) ? so[B + sj + 1] : kNever;
-                    }
-                    // tile-relative starts of sentences, clamped to the tile; slot j holds the tokens from its start to the next one's
-                    auto clamped = [&](int off) { return min(max(min(off, tok_end) - tok0, 0), valid); };
-                    const uint32_t held = __ballot_sync(0xffffffffu, lane < kIndSlots && B + lane < S && clamped(w1) > clamped(w));
-                    more = __any_sync(0xffffffffu, lane == kIndSlots && B + kIndSlots < S && w < tok_end) ? 1 : 0;    // does slot 15 leave some?
-                    const int is = ic & (kIndRing - 1);
-                    if (ic >= kIndRing) {                           // the product that read this buffer last has completed
-                        ok = role_wait(&ctl->iempty[is], uint32_t(ic / kIndRing - 1) & 1u, limit, &ctl->abort_flag, a.status);
-                        ok = __all_sync(0xffffffffu, ok);
+                if (more || t + n_tiles < last_tile) w_next = fetch(B_next);
+                for (int k = 0; k < n_tiles && ok; ++k, ++ic) {
+                    const int tok = tok0 + k * 128, valid = min(128, N - tok), is = ic & ring;
+                    if (valid < 128) {
+                        // This matrix needs its tile: a zero in the indicator does not silence a NaN or an infinity in a dead row, so the rows
+                        // past the slab's end are cleared in the staged tile (the logits of those rows are never read).  Once the last
+                        // matrix has been multiplied, all tiles before this one had arrived, so the wait is for the right phase of the stage.
+                        if (ic > 0) ok = warp_wait(&ctl->iempty[(ic - 1) & ring], uint32_t((ic - 1) >> a.ind_log) & 1u, limit, &ctl->abort_flag, a.status);
+                        const int i = pool_a ? t + k - t_begin : t_end - 1 - (t + k), stage = i % a.stages;
+                        if (ok) ok = warp_wait(&ctl->full[stage], uint32_t(i / a.stages) & 1u, limit, &ctl->abort_flag, a.status);
+                        if (!ok) break;
+                        uint8_t* tile = tiles + size_t(stage) * kOpBytes;
+                        for (int u = valid * 8 + gtid; u < 128 * 8; u += kPoolWarps * 32) {
+                            *reinterpret_cast<uint4*>(tile + u * 16) = make_uint4(0u, 0u, 0u, 0u);
+                            *reinterpret_cast<uint4*>(tile + kOpHalfBytes + u * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    } else if (ic >> a.ind_log) {                   // the product that read this buffer last has completed
+                        ok = warp_wait(&ctl->iempty[is], uint32_t((ic >> a.ind_log) - 1) & 1u, limit, &ctl->abort_flag, a.status);
                         if (!ok) break;
                     }
-                    {
-                        const bool is_sent = (held >> sj) & 1u;
-                        const int from = is_sent ? clamped(wj) : 0, to = is_sent ? clamped(wj1) : 0;
-                        indicator_piece(indb + size_t(is) * kIndBytes, sj, (lane & 7) * 2, from, to);
-                        indicator_piece(indb + size_t(is) * kIndBytes, sj, (lane & 7) * 2 + 1, from, to);
-                    }
+                    indicator_row(indb + size_t(is) * kIndBytes, sj, sq, min(max(wj - tok, 0), valid), min(max(wj1 - tok, 0), valid));
                     fence_proxy_async_smem();                       // the matrix (and cleared rows) are read by the tensor core
                     tc_fence_before();                              // and this warp's reads of the accumulators came first
                     __syncwarp();
                     if (lane == 0) {
-                        if (gw == 0) ctl->ind_flags[is] = more | (join ? 2 : 0) | ((!join && r_prev >= 0) ? 4 : 0);
+                        if (gw == 0) ctl->ind_flags[is] = more | (k > 0 ? 2 : 0) | (k == 0 && run > 0 ? 4 : 0);
                         mbar_arrive(&ctl->ifull[is]);
                     }
-                    run_held |= held;
-                    ++ic;
-                    if (!join && r_prev >= 0) {                     // the run before, while the new one is being multiplied
-                        drain(r_prev, p_slab, p_B, p_held);
-                        if (!ok) break;
-                    }
-                    cur = B + kIndSlots;
-                } while (more);
-                // the next tile starts in the last sentence of the run's window that starts at or before its first token
-                const int n_le = __popc(__ballot_sync(0xffffffffu, B + lane < S && w <= tok0 + 128));
-                first = (n_le == 32 && B + 32 < S) ? holder(tok0 + 128) : B + max(n_le - 1, 0);
-                if (++stage == a.stages) { stage = 0; ++lap; }
-            }
-            if (ok && run >= 0) drain(run, run_slab, B, run_held);  // the issuer closes the last run when its tiles are done
-        } else {
-            // -------------------------------------------------------------- pass B: issuer of the pooling products
-            // (its own thread: an issue blocks for the length of the product, and every look at shared memory costs the
-            // thread that issues the logits a few hundred cycles)
-            {
-                const uint32_t leader = elect_leader();
-                const uint32_t indb_u32 = smem_u32(indb);
-                int pc = 0, run = -1, stage = load0 % a.stages;
-                for (int tl = 0; tl < ntl && ok; ++tl) {
-                    int flags = 0;
-                    do {
-                        const int is = pc & (kIndRing - 1);
-                        ok = warp_wait(&ctl->ifull[is], uint32_t(pc / kIndRing) & 1u, limit, &ctl->abort_flag, a.status);
-                        if (!ok) break;
-                        flags = *reinterpret_cast<volatile int*>(&ctl->ind_flags[is]);       // 1: more, 2: joins the run, 4: closes one
-                        tc_fence_after();
-                        if (flags & 4) umma_commit(&ctl->pfull[run & 1], leader);                    // everything of the run before is issued
-                        if (!(flags & 2)) ++run;
-                        umma_pool(tmem_base + kPoolCol + uint32_t(run & 1) * kIndSlots, smem_u32(tiles + size_t(stage) * kOpBytes),
-                                  indb_u32 + uint32_t(is) * kIndBytes, (flags & 2) != 0, leader);
-                        umma_commit(&ctl->iempty[is], leader);
-                        ++pc;
-                    } while (flags & 1);
-                    if (ok) umma_commit(&ctl->empty[stage], leader);
-                    if (++stage == a.stages) stage = 0;
+                    if (k == (n_tiles > 1 ? 1 : 0) && run > 0) drain(run - 1);      // the run before, while this one is multiplied
                 }
-                if (ok && run >= 0) umma_commit(&ctl->pfull[run & 1], leader);
-                umma_commit(&ctl->retired[2], leader);
+                p_slab = slab; p_B = B; p_held = held;
+                p_from = began < max(t_begin - lo, 0) * 128 ? 2 : began < tok0 ? 1 : 0;
+                p_tiles = !more && t + n_tiles == last_tile ? last_tile - max(lo, t_begin) : 0;
+                ++run;
+                if (!more) t += n_tiles;
+                B = B_next; w = w_next;
+            }
+            if (ok && run > 0) drain(run - 1);                      // (the issuer closes the last run when its tiles are done)
+            if (ok && head_sent >= 0) {
+                const uint32_t all = 4u * uint32_t(pref[slab_first + 1] - pref[slab_first]);
+                if (lane == 0) ok = flag_wait(a.sum_cnt + slab_first, all, limit, &ctl->abort_flag, a.status);
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (ok) atomicAdd(a.vsum + (size_t(slab_first) * a.max_sent + head_sent) * kHeadDim + ch, head);
             }
         }
     }
@@ -856,17 +921,17 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
 // ---------------------------------------------------------------------------------------
 constexpr int kPoolRows = 4;
 __global__ void __launch_bounds__(256)
-score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len,
+score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_rows, const int32_t* cap, const int32_t* kv_len,
                   const int32_t* sent_off, const int32_t* n_sent, float eps, const float* tok_imp_ws,
                   const float* vsum, float* sent_imp, __nv_bfloat16* vbar_hi, __nv_bfloat16* vbar_lo, float* sent_lam) {
     pdl_trigger();
     pdl_wait();
     const int slab = blockIdx.y;
-    if (blockIdx.x == 0 && threadIdx.x == 0) lse_cnt[slab] = 0u;            // for the next call's sweeps
+    if (blockIdx.x == 0 && threadIdx.x < 2) lse_cnt[threadIdx.x * gridDim.y + slab] = 0u;      // both counters, for the next call's sweeps
     const int lane = threadIdx.x & 31;
     const int i0 = blockIdx.x * 8 * kPoolRows + (threadIdx.x >> 5);         // and every eighth after it
     const int S = min(n_sent[slab], max_sent);
-    const int N = min(max(kv_len[slab], 0), cap[slab / Hk]);
+    const int N = min(max(kv_len[slab], 0), min(cap[slab / Hk], max_rows));
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
     const float* imp = tok_imp_ws + size_t(slab) * max_cap;
     int b[kPoolRows], e[kPoolRows];
@@ -1328,7 +1393,7 @@ struct SmallCtl {
 constexpr size_t kSmallSmem = 1024 + 2 * size_t(kOpBytes) + sizeof(SmallCtl);
 
 __global__ void __launch_bounds__(kSmallThreads)
-score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const int32_t* cap, const int32_t* kv_len, const int32_t* sent_off,
+score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_rows, const int32_t* cap, const int32_t* kv_len, const int32_t* sent_off,
                    const int32_t* n_sent, float eps, float sigma, float tau, const float* tok_imp_ws, const float* vsum,
                    float* sent_imp, float* sent_red, float* sent_lam, float* sent_score, LamTable ext, const Header* hdr) {
     extern __shared__ uint8_t small_smem_raw[];
@@ -1342,8 +1407,8 @@ score_small_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, const i
     if (tid == 0) { mbar_init(&ctl->done, 1); mbar_fence_init(); }
     if (warp == 1) tmem_alloc(&ctl->tmem_base, 128);
     pdl_wait();
-    if (tid == 0) lse_cnt[slab] = 0u;                    // for the next call's sweeps
-    const int S = min(max(n_sent[slab], 0), max_sent), N = min(max(kv_len[slab], 0), cap[slab / Hk]);
+    if (tid < 2) lse_cnt[tid * gridDim.x + slab] = 0u;   // both counters, for the next call's sweeps
+    const int S = min(max(n_sent[slab], 0), max_sent), N = min(max(kv_len[slab], 0), min(cap[slab / Hk], max_rows));
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
     const float* ti_p = tok_imp_ws + size_t(slab) * max_cap;
     // ---- pooling: kSmallBatch rows per warp; rows past the last sentence are zeros
@@ -1516,12 +1581,13 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     a.max_sent = shape->max_sent;
     a.WB = L.sc_wb; a.RB = L.sc_rb; a.N = L.sc_wb * n; a.R = a.RB * a.N; a.RA = L.sc_ra;
     a.slab_off = shape->slab_off; a.cap = shape->cap; a.kv_len = kv_len; a.sent_off = sent_off; a.n_sent = n_sent;
-    a.rec = reinterpret_cast<float2*>(w + L.sc_part); a.lse_cnt = reinterpret_cast<uint32_t*>(w + L.sc_cnt);
+    a.rec = reinterpret_cast<float2*>(w + L.sc_part); a.lse_cnt = reinterpret_cast<uint32_t*>(w + L.sc_cnt); a.sum_cnt = a.lse_cnt + L.slabs;
     a.tok_imp_user = tok_imp; a.tok_imp_ws = sc_tok; a.vsum = vsum; a.status = status;
+    a.pool_a = a.RA == 1;                            // see the head of the sweeps
     a.hdr = reinterpret_cast<const Header*>(w + L.header);
     a.block_table = block_table; a.max_pages = max_pages;
     const size_t max_smem = 227 * 1024;
-    size_t fixed = 1024 + size_t(a.R) * kRowBytes + size_t(kIndRing) * kIndBytes + 128 * kExtRow + size_t(a.RA) * 128 * kExtRow +
+    size_t fixed = 1024 + size_t(a.R) * kRowBytes + 2 * kIndBytes + 128 * kExtRow + sweep_ext_bytes(a.RA) +
                    sizeof(SweepCtl) + size_t(a.RB - 1) * 4 * 128 * 4;
     // The table of slabs (8 bytes each) goes into shared memory as long as one tile stage fits beside it: all but windows of some hundred
     // query rows with a thousand slabs and more.  A 512-row window leaves room for 900 slabs; without the other form the call would end there.
@@ -1534,6 +1600,10 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         set_error_text("skipkv_score: more than 128 sentences per slab and batch * n_kv_heads too large for the shared-memory table of the Gram kernels");
         return SKIPKV_ERR_UNSUPPORTED;
     }
+    // Four indicator matrices in flight (two more than counted above) wherever that leaves two tile stages: with two a matrix waits for the
+    // product two tiles back, and pass A took 1.15 us a tile instead of 0.85 (80 slabs of 16K to 32K rows).
+    a.ind_log = fixed + 2 * kIndBytes + 2 * kOpBytes <= max_smem ? 2 : 1;
+    if (a.ind_log == 2) fixed += 2 * kIndBytes;
     a.stages = int((max_smem - fixed) / kOpBytes);
     if (a.stages > kStagesMax) a.stages = kStagesMax;
     int grid = num_sms();
@@ -1550,17 +1620,18 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         else break;
     }
     SKIPKV_CUDA(le);
+    const int max_rows = block_table ? max_pages * 128 : 0x7fffffff;          // rows the sweeps look at
     // one tile of sentences per slab: one kernel instead of three, with the operands in shared memory throughout
     if (shape->max_sent <= kSmallSent) {
         SKIPKV_CUDA(launch_dependent(score_small_kernel, dim3(L.slabs), dim3(kSmallThreads), kSmallSmem, st, a.lse_cnt, Hk, int(shape->max_sent),
-                                     int(shape->max_cap), shape->cap, kv_len, sent_off, n_sent, params->eps, params->sigma,
+                                     int(shape->max_cap), max_rows, shape->cap, kv_len, sent_off, n_sent, params->eps, params->sigma,
                                      params->tau, static_cast<const float*>(sc_tok), static_cast<const float*>(vsum), sent_imp,
                                      sent_red, sent_lam, sent_score, ext, reinterpret_cast<const Header*>(w + L.header)));
         return SKIPKV_OK;
     }
     {
         dim3 pgrid((shape->max_sent + 8 * kPoolRows - 1) / (8 * kPoolRows), L.slabs);
-        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, shape->max_cap,
+        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, shape->max_cap, max_rows,
                                      shape->cap, kv_len, sent_off, n_sent, params->eps, sc_tok, vsum, sent_imp, vbar_hi,
                                      vbar_lo, sent_lam));
     }

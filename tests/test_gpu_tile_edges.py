@@ -83,6 +83,33 @@ def test_score_query_blocks(group, window):
         check_scores(B, L, D)
 
 
+@pytest.mark.parametrize("group,window", [(4, 32), (5, 64), (4, 48)])
+@pytest.mark.parametrize("lo,hi", [(9000, 9000), (700, 3000), (127, 129), (3, 20000)])
+def test_score_sentences_across_the_ranges_of_several_ctas(group, window, lo, hi):
+    """A sentence's key sum comes from every CTA that has some of its tokens: sentences of one token up to whole slabs over many CTAs, empty
+    ones between them, starts on and beside tile edges; with the sums in either pass (one operand of query rows, several)."""
+    ctx = [40000, 9000, 130]
+    B, L, D = layer(ctx, n_q_heads=2 * group, n_kv_heads=2, window=window, sent_lo=8, sent_hi=12, dup_rate=0.3, seed=760 + group)
+    rng = np.random.Generator(np.random.Philox(lo))
+    for b, n in enumerate(ctx):
+        at = [0]
+        while at[-1] < n:
+            step = lo if lo == hi else int(np.exp(rng.uniform(np.log(lo), np.log(hi))))
+            at.append(min(at[-1] + step, n))
+            if rng.random() < 0.1:
+                at.append(at[-1])                         # an empty sentence
+            if len(at) > L["max_sent"]:
+                at = at[:L["max_sent"]] + [n]
+                break
+        S = len(at) - 1
+        L["sent_off"][b, :, :S + 1] = at
+        L["sent_off"][b, :, S + 1:] = n
+        L["n_sent"][b] = S
+    D.sent_off.copy_(torch.from_numpy(np.ascontiguousarray(L["sent_off"])))
+    D.n_sent.copy_(torch.from_numpy(np.ascontiguousarray(L["n_sent"])))
+    check_scores(B, L, D)
+
+
 @pytest.mark.parametrize("group,window,batch,sent", [(1, 512, 16, (8, 40)), (5, 100, 19, (8, 40)), (1, 512, 16, (2, 4))])
 def test_score_with_more_slabs_than_shared_memory_has_room_for(group, window, batch, sent):
     """Over a thousand slabs beside a wide window: the sweep's table of slabs is in global memory; contiguous against the oracle, paged
