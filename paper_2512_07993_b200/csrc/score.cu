@@ -921,7 +921,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
 // ---------------------------------------------------------------------------------------
 constexpr int kPoolRows = 4;
 __global__ void __launch_bounds__(256)
-score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_rows, const int32_t* cap, const int32_t* kv_len,
+score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int sent_rows, int max_cap, int max_rows, const int32_t* cap, const int32_t* kv_len,
                   const int32_t* sent_off, const int32_t* n_sent, float eps, const float* tok_imp_ws,
                   const float* vsum, float* sent_imp, __nv_bfloat16* vbar_hi, __nv_bfloat16* vbar_lo, float* sent_lam) {
     pdl_trigger();
@@ -930,7 +930,7 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_
     if (blockIdx.x == 0 && threadIdx.x < 2) lse_cnt[threadIdx.x * gridDim.y + slab] = 0u;      // both counters, for the next call's sweeps
     const int lane = threadIdx.x & 31;
     const int i0 = blockIdx.x * 8 * kPoolRows + (threadIdx.x >> 5);         // and every eighth after it
-    const int S = min(n_sent[slab], max_sent);
+    const int S = min(max(n_sent[slab], 0), max_sent);
     const int N = min(max(kv_len[slab], 0), min(cap[slab / Hk], max_rows));
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
     const float* imp = tok_imp_ws + size_t(slab) * max_cap;
@@ -958,7 +958,13 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_
 #pragma unroll
     for (int q = 0; q < kPoolRows; ++q) {
         const int i = i0 + q * 8;
-        if (i >= S) break;
+        if (i >= S) {                                        // the rest of the last block: zeros, whose products are finite
+            if (i < (S + 127) / 128 * 128) {
+                const size_t o = (size_t(slab) * sent_rows + i) * kHeadDim;
+                reinterpret_cast<uint2*>(vbar_hi + o)[lane] = reinterpret_cast<uint2*>(vbar_lo + o)[lane] = make_uint2(0u, 0u);
+            }
+            continue;
+        }
         float ti = first[q][0] + first[q][1] + first[q][2];
         for (int t = b[q] + 96 + lane; t < e[q]; t += 32) ti += imp[t];
         const float len = float(max(e[q] - b[q], 1));
@@ -980,7 +986,7 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_
             hi[c] = __bfloat16_as_ushort(h);
             lo[c] = __bfloat16_as_ushort(r);
         }
-        const size_t o = (size_t(slab) * max_sent + i) * kHeadDim;
+        const size_t o = (size_t(slab) * sent_rows + i) * kHeadDim;
         reinterpret_cast<uint2*>(vbar_hi + o)[lane] = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
         reinterpret_cast<uint2*>(vbar_lo + o)[lane] = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
         if (lane == 0) {
@@ -995,18 +1001,21 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_
 // Gram passes on the tensor cores.  G is symmetric: every pair of 128-sentence blocks I <= J of a slab is multiplied and
 // exponentiated once, and gives the rows of I their sums over the columns and the columns of J theirs over the rows (the
 // diagonal pair: column sums only).  Work is the list of pairs, J by J, over all slabs, cut into equal contiguous ranges.
-// Every sentence has four partial sums per block of its slab, each written by one warp: rows by the pair (the four column groups), columns by a
-// range's part of J (the four row groups; the blocks of the part's other pairs get zeros).  The CTA that completes a slab adds them up in
-// order, so the results do not depend on who was first.  They lie where the sums of the keys were, which the pooling was the last to read.
+// A column block's sums are kept for as long as a range stays with it and stored as that part's (four warps' each); a row's are stored by pair (four column
+// groups).  The CTA that completes a slab adds a sentence's parts and rows up in order, so the results do not depend on who was first.
+// They lie where the sums of the keys were, which the pooling was the last to read.
+// Rows past a slab's last sentence are zeros (every slab has whole blocks of its own), so nothing is masked but the weights of such
+// columns and, in a diagonal pair, a sentence's product with itself.
 // The penalty is the maximum over later sentences; only those beyond tau are reported, which are few (pass 1, an integer maximum).
 // Roles as in the token-level kernel: a TMA warp, two MMA warps that take the pairs in turn, sixteen epilogue warps with 32
 // rows x 32 columns of every accumulator each, column sums in registers for as long as J stays.
 // Three shared-memory slots hold a block's high and low parts.  One is J's, the other two take the I blocks in turn; the next J takes
 // the slot that is free next and the old J's goes to the end of the queue, so a change of J costs no drain.
-// Bound by its epilogue: 2.4 and 2.1 us a pair (passes 1 and 2, about 130 pairs per SM) against 0.8 us for the three products, which stream
-// 192 KB of operands at the shared-memory port's 128 bytes per clock.  The four warps of a scheduler are in the same phase of the
-// same pair, and column sums leave no registers for two pairs at once.  Half the products and half the exponentials of evaluating
-// all pairs twice: 128 slabs x 2K sentences, the whole scoring call: 2319 -> 2190 us.
+// What counts is the epilogue's instructions, 32 exponentials and about 60 others per warp and pair: with the walk over the pairs, addresses, zeros
+// for parts that a pair did not have, masks and reciprocals in the loop it was 1790 and 1380 a scheduler and pair (passes 1 and 2), now
+// 1310 and 1140, and 306 and 271 us became 230 and 227 (128 slabs x 2K sentences; whole call 1950 -> 1848).  Of the 1.75 us a pair the three products,
+// which stream 192 KB of operands at the shared-memory port's 128 bytes per clock, take 0.8; the 64 KB of a pair's I block are
+// 5.5 TB/s from L2 over all SMs.
 // ---------------------------------------------------------------------------------------
 constexpr int kGramAcc = 4;
 struct GramCtl {
@@ -1017,7 +1026,7 @@ struct GramCtl {
     uint32_t tmem_base;
     int abort_flag, last;
     uint32_t wsum[32];
-    alignas(16) float colz[16][32];          // pass 2, by epilogue warp: 1 / Z_j of its columns
+    alignas(16) float colw[16][32];          // by epilogue warp: weights of its columns, 1 or (pass 2) 1 / Z_j, 0 for none of the slab's
     uint64_t retired[2];                     // every product of an MMA warp has completed
     uint32_t loads[6];                       // by slot and part: copies issued (in shared memory for want of registers)
 };
@@ -1033,7 +1042,7 @@ __device__ __forceinline__ float from_ordered_bits(uint32_t u) { return __uint_a
 
 // A CTA's walk over its pairs, and which slot a block is in.  Every role steps through the same sequence.
 struct GramWalk {
-    int slab, S, J, t;                       // pair t of block column J: 0 is the diagonal, t > 0 multiplies block t - 1
+    int slab, J, t;                          // pair t of block column J: 0 is the diagonal, t > 0 multiplies block t - 1
     int left;                                // pairs of the range not yet walked, this one included
     int jslot, q0, q1, q2;                   // slot of J, and the others in the order in which they are taken
     bool have_j;
@@ -1055,9 +1064,12 @@ struct GramWalk {
     }
     __device__ __forceinline__ int take_i() { const int s = pop(); q1 = s; return s; }
     // on to the next pair: true if it has another J
-    __device__ __forceinline__ bool next(const int* ipref) {
-        --left;
-        if (t++ < J) return false;
+    __device__ __forceinline__ bool next(const int* ipref) { return advance(ipref, 1); }
+    // on by n pairs, at most to the next J
+    __device__ __forceinline__ bool advance(const int* ipref, int n) {
+        left -= n;
+        t += n;
+        if (t <= J) return false;
         t = 0; ++J;
         if (left > 0 && ipref[slab] + J * (J + 1) / 2 >= ipref[slab + 1]) {
             J = 0;
@@ -1080,7 +1092,7 @@ struct LamTable {
 template <int kPass>
 __global__ void __launch_bounds__(kGramThreads, 1)
 score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ CUtensorMap mapLo, int n_slabs,
-                  int max_sent, const int32_t* n_sent, float sigma, float tau, float* sc_z, const float* sent_imp,
+                  int max_sent, int sent_rows, const int32_t* n_sent, float sigma, float tau, float* sc_z, const float* sent_imp,
                   float* sent_red, float* sent_lam, float* sent_score, float* parts, size_t parts_slab, uint32_t* cnt, LamTable ext, const Header* hdr) {
     extern __shared__ uint8_t gram_smem_raw[];
     const uint32_t raw = smem_u32(gram_smem_raw);
@@ -1112,7 +1124,8 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     const long long total = ipref[n_slabs];
-    const int first = int(total * blockIdx.x / gridDim.x), count = int(total * (blockIdx.x + 1) / gridDim.x) - first;
+    const int ctas = int(min((long long)gridDim.x, total)), cta = min(int(blockIdx.x), ctas);          // none of those with work has no pair
+    const int first = ctas > 0 ? int(total * cta / ctas) : 0, count = int(blockIdx.x) < ctas ? int(total * (cta + 1) / ctas) - first : 0;
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
@@ -1132,7 +1145,7 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                     if (!ok) break;
                     uint8_t* dst = slots + size_t(2 * s + part) * kOpBytes;
                     const CUtensorMap* map = part ? &mapLo : &mapHi;
-                    const int row = w.slab * max_sent + block * 128;
+                    const int row = w.slab * sent_rows + block * 128;
                     mbar_expect_tx(&ctl->full[s][part], kOpBytes);
                     tma_load_2d(dst, map, 0, row, &ctl->full[s][part]);
                     tma_load_2d(dst + kOpHalfBytes, map, 64, row, &ctl->full[s][part]);
@@ -1213,113 +1226,119 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
-        const int quarter = warp & 3, c0 = ((warp - 4) >> 2) * 32;   // this warp's rows (32 * quarter + lane) and columns
+        const int quarter = warp & 3, cg = (warp - 4) >> 2, c0 = cg * 32;     // this warp's rows (32 * quarter + lane) and columns
         const uint32_t lane_addr = tmem_base + (uint32_t(quarter * 32) << 16) + c0;
-        float* colz_s = ctl->colz[warp - 4];
-        const float2* colz = reinterpret_cast<const float2*>(colz_s);
-        float2 cs[16];
-        bool ok = true, fresh = true;
+        float* colw_s = ctl->colw[warp - 4];
+        const float2* colw = reinterpret_cast<const float2*>(colw_s);
+        bool ok = true;
         uint32_t acc = 0, parity = 0;
-        int done = 0;                                                // pairs of this slab in this range
-        int cslot = 0;                                               // whose partial the column sums become
         uint32_t* lam_bits = reinterpret_cast<uint32_t*>(sent_lam);
+        // the CTA whose range holds a pair
+        auto owner = [&](int pair) {
+            const long long x = (long long)(pair + 1) * ctas - 1;
+            return x < (1ll << 32) ? int(uint32_t(x) / uint32_t(total)) : int(x / total);
+        };
         GramWalk w;
         w.start(ipref, first, count);
-        w.S = count > 0 ? sent_of(w.slab) : 0;
+        int slab = -1, S = 0, done = 0;                              // of the present slab: sentences, pairs of this range so far
 #pragma unroll 1
         while (w.left > 0) {
-            const size_t base = size_t(w.slab) * max_sent;
-            const int j0 = w.J * 128 + c0;
-            const bool diag = w.t == 0;
-            const int ib = diag ? w.J : w.t - 1, i = ib * 128 + quarter * 32 + lane;
-            float* p_slab = parts + size_t(w.slab) * parts_slab;         // [4 * blocks][max_sent]
-            if (fresh) {
+            // a part of column block J: m pairs from t on
+            if (w.slab != slab) { slab = w.slab; S = sent_of(slab); done = 0; }
+            const int J = w.J, m = min(J + 1 - w.t, w.left), j0 = J * 128 + c0;
+            const size_t base = size_t(slab) * max_sent;
+            float* p_slab = parts + size_t(slab) * parts_slab;           // [4 * blocks][max_sent]
+            const bool full = (J + 1) * 128 <= S;
+            const bool my_col = j0 + lane < S;
+            float2 cs[16];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) cs[k] = make_float2(0.f, 0.f);
-                cslot = ib;
-                if (kPass == 2) {
-                    const float z = j0 + lane < w.S ? sc_z[base + j0 + lane] : 0.f;
+            for (int k = 0; k < 16; ++k) cs[k] = make_float2(0.f, 0.f);
+            // weights of the columns in row sums (nothing for those that are none of the slab's, which are products of zeros)
+            const float wj = !my_col ? 0.f : kPass == 2 ? sc_z[base + j0 + lane] : 1.f;
+            __syncwarp();
+            colw_s[lane] = wj;
+            __syncwarp();
+            bool diag = w.t == 0;
+            int i = (diag ? J : w.t - 1) * 128 + quarter * 32 + lane;
+            float* rows = p_slab + size_t(J * 4 + cg) * max_sent;
+#pragma unroll 1
+            for (int left = m; left > 0; --left) {
+                // of this row in column sums (I < J: all rows are the slab's)
+                const float wi = diag && i >= S ? 0.f : kPass == 2 ? sc_z[base + i] : 1.f;
+                if (ok) {
+                    // (inline: a call would spill the sums)
+                    bool r = mbar_try_wait(&ctl->tfull[acc], parity);
+                    for (uint32_t n = 0; !r && n < limit; ++n) {
+                        if ((n & 63) == 63 && *reinterpret_cast<volatile int*>(&ctl->abort_flag)) break;
+                        r = mbar_try_wait(&ctl->tfull[acc], parity);
+                    }
+                    ok = __all_sync(0xffffffffu, r);
+                    if (!ok) {
+                        atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
+                        *reinterpret_cast<volatile int*>(&ctl->abort_flag) = 1;
+                    }
+                }
+                if (ok) {
+                    tc_fence_after();
+                    float v[32];
+                    tmem_ld32(lane_addr + acc * 128, v);
+                    tc_fence_before();
                     __syncwarp();
-                    colz_s[lane] = z > 0.f ? 1.f / z : 0.f;
-                    __syncwarp();
-                }
-            } else if (j0 + lane < w.S) {
-                p_slab[size_t(ib * 4 + quarter) * max_sent + j0 + lane] = 0.f;
-            }
-            float invz_i = 0.f;                                      // pass 2: 1 / Z_i, the weight of this row in column sums
-            if (kPass == 2 && i < w.S) { const float z = sc_z[base + i]; invz_i = z > 0.f ? 1.f / z : 0.f; }
-            if (ok) {
-                // (inline: a call would spill the sums)
-                bool r = mbar_try_wait(&ctl->tfull[acc], parity);
-                for (uint32_t n = 0; !r && n < limit; ++n) {
-                    if ((n & 63) == 63 && *reinterpret_cast<volatile int*>(&ctl->abort_flag)) break;
-                    r = mbar_try_wait(&ctl->tfull[acc], parity);
-                }
-                ok = __all_sync(0xffffffffu, r);
-                if (!ok) {
-                    atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
-                    *reinterpret_cast<volatile int*>(&ctl->abort_flag) = 1;
-                }
-            }
-            if (ok) {
-                tc_fence_after();
-                float v[32];
-                tmem_ld32(lane_addr + acc * 128, v);
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->tempty[acc]);
-                float2 row = make_float2(0.f, 0.f);
-                const float2 l2 = make_float2(kLog2e, kLog2e), iz2 = make_float2(invz_i, invz_i);
-                auto add = [&](int k, float2 e) {
-                    if (kPass == 1) {
-                        row = __fadd2_rn(row, e);
-                        cs[k] = __fadd2_rn(cs[k], e);
-                    } else {
-                        row = __ffma2_rn(e, colz[k], row);
-                        cs[k] = __ffma2_rn(e, iz2, cs[k]);
-                    }
-                };
-                float mx = -INFINITY;
-                if (!diag && (w.J + 1) * 128 <= w.S) {               // (I < J: all rows are the slab's)
-                    if (kPass == 1) {
-                        float m1 = -INFINITY;
+                    if (lane == 0) mbar_arrive(&ctl->tempty[acc]);
+                    const bool plain = !diag && full;
+                    if (kPass == 1 && !ext.table) {
+                        float mx = -INFINITY, m1 = -INFINITY;
+                        if (plain) {
 #pragma unroll
-                        for (int k = 0; k < 32; k += 4) { mx = max3(mx, v[k], v[k + 1]); m1 = max3(m1, v[k + 2], v[k + 3]); }
-                        mx = fmaxf(mx, m1);
-                    }
+                            for (int k = 0; k < 32; k += 4) { mx = max3(mx, v[k], v[k + 1]); m1 = max3(m1, v[k + 2], v[k + 3]); }
+                        } else {
+                            const int from = i - j0, to = S - j0;    // later sentences only
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float2 x = __fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), l2);
-                        add(k, make_float2(ex2f(x.x), ex2f(x.y)));
-                    }
-                } else {                                             // nothing where a row or column is none of the slab's, and for i == j
-                    const int lim = i < w.S ? w.S - j0 : 0, self = i - j0;
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const bool x = 2 * k < lim, y = 2 * k + 1 < lim;
-                        if (kPass == 1) {
-                            if (x && 2 * k > self) mx = fmaxf(mx, v[2 * k]);
-                            if (y && 2 * k + 1 > self) mx = fmaxf(mx, v[2 * k + 1]);
+                            for (int k = 0; k < 32; ++k)
+                                if (k > from && k < to) mx = fmaxf(mx, v[k]);
                         }
-                        add(k, make_float2(x && 2 * k != self ? ex2f(v[2 * k] * kLog2e) : 0.f,
-                                           y && 2 * k + 1 != self ? ex2f(v[2 * k + 1] * kLog2e) : 0.f));
+                        mx = fmaxf(mx, m1);
+                        if (mx > tau) atomicMax(lam_bits + base + i, ordered_bits(mx));
                     }
+                    if (diag && quarter == cg) {                     // a sentence and itself
+#pragma unroll
+                        for (int k = 0; k < 32; ++k)
+                            if (k == lane) v[k] = -INFINITY;
+                    }
+                    float2 row = make_float2(0.f, 0.f);
+                    const float2 l2 = make_float2(kLog2e, kLog2e), w2 = make_float2(wi, wi);
+                    if (kPass == 1 && plain) {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            const float2 x = __fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), l2), e = make_float2(ex2f(x.x), ex2f(x.y));
+                            row = __fadd2_rn(row, e);
+                            cs[k] = __fadd2_rn(cs[k], e);
+                        }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            const float2 x = __fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), l2), e = make_float2(ex2f(x.x), ex2f(x.y));
+                            row = __ffma2_rn(e, colw[k], row);
+                            cs[k] = __ffma2_rn(e, w2, cs[k]);
+                        }
+                    }
+                    // (the diagonal pair is symmetric: its column sums are all there is to it)
+                    if (!diag) rows[i] = row.x + row.y;
                 }
-                if (kPass == 1 && mx > tau && !ext.table) atomicMax(lam_bits + base + i, ordered_bits(mx));
-                // (the diagonal pair is symmetric: its column sums are all there is to it)
-                if (!diag && i < w.S) p_slab[size_t(w.J * 4 + (c0 >> 5)) * max_sent + i] = row.x + row.y;
+                if (++acc == kGramAcc) { acc = 0; parity ^= 1u; }
+                i = diag ? quarter * 32 + lane : i + 128;
+                diag = false;
             }
-            if (++acc == kGramAcc) { acc = 0; parity ^= 1u; }
-            ++done;
-            const int slab = w.slab, S = w.S;
-            fresh = w.next(ipref);
-            if ((fresh || w.left == 0) && ok) {
+            if (ok) {
                 float s[32];
 #pragma unroll
                 for (int k = 0; k < 16; ++k) { s[2 * k] = cs[k].x; s[2 * k + 1] = cs[k].y; }
                 const float sum = col_reduce32(s, lane);
-                if (j0 + lane < S) p_slab[size_t(cslot * 4 + quarter) * max_sent + j0 + lane] = sum;
+                const int part = w.t == 0 ? 0 : cta - owner(ipref[slab] + J * (J + 1) / 2);
+                if (my_col) p_slab[size_t(part * 4 + quarter) * max_sent + j0 + lane] = sum;
             }
+            done += m;
+            w.advance(ipref, m);
             if (w.slab != slab || w.left == 0) {                     // the range's part of this slab is complete
                 __threadfence();
                 named_bar_sync(1, 512);
@@ -1334,15 +1353,20 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                 named_bar_sync(1, 512);
                 if (*reinterpret_cast<volatile int*>(&ctl->last)) {
                     for (int k = tid - 128; k < S; k += 512) {
+                        // the parts of block b's columns, then its rows with the blocks after it
+                        const int b = k >> 7, x0 = ipref[slab] + b * (b + 1) / 2, n_part = owner(x0 + b) - owner(x0) + 1;
                         float sum = 0.f;
-#pragma unroll 4
-                        for (int q = 0; q < nb; ++q) {
-                            const float* p = p_slab + size_t(q * 4) * max_sent + k;
-                            sum += (__ldcg(p) + __ldcg(p + max_sent)) + (__ldcg(p + 2 * size_t(max_sent)) + __ldcg(p + 3 * size_t(max_sent)));
-                        }
+                        auto add = [&](int from, int to) {
+                            const float* x = p_slab + size_t(from) * 4 * max_sent + k;
+#pragma unroll 8
+                            for (int q = from; q < to; ++q, x += 4 * size_t(max_sent))
+                                sum += (__ldcg(x) + __ldcg(x + max_sent)) + (__ldcg(x + 2 * max_sent) + __ldcg(x + 3 * max_sent));
+                        };
+                        add(0, n_part);
+                        add(b + 1, nb);
                         const size_t o = base + k;
                         if (kPass == 1) {
-                            sc_z[o] = sum;
+                            sc_z[o] = sum > 0.f ? 1.f / sum : 0.f;
                         } else {
                             const float red = sum / float(S);
                             float lam;
@@ -1360,8 +1384,6 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                     }
                 }
                 named_bar_sync(1, 512);                              // `last` may be written again
-                done = 0;
-                w.S = w.left > 0 ? sent_of(w.slab) : 0;
             }
         }
     }
@@ -1572,7 +1594,7 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     if (int rc = tmap_rows(&mapK, K, uint64_t(shape->total_rows), 128)) return rc;
     if (int rc = tmap_qwin(&mapQ, q_win, uint64_t(shape->batch) * Hq, uint32_t(shape->window), uint32_t(L.sc_wb), uint32_t(n)))
         return rc;
-    const uint64_t vrows = uint64_t(L.slabs) * uint64_t(shape->max_sent);
+    const uint64_t vrows = uint64_t(L.slabs) * uint64_t(L.sc_sent_rows);
     if (int rc = tmap_rows(&mapHi, vbar_hi, vrows, 128)) return rc;
     if (int rc = tmap_rows(&mapLo, vbar_lo, vrows, 128)) return rc;
 
@@ -1630,8 +1652,8 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         return SKIPKV_OK;
     }
     {
-        dim3 pgrid((shape->max_sent + 8 * kPoolRows - 1) / (8 * kPoolRows), L.slabs);
-        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, shape->max_cap, max_rows,
+        dim3 pgrid(unsigned(L.sc_sent_rows) / (8 * kPoolRows), L.slabs);
+        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, int(L.sc_sent_rows), shape->max_cap, max_rows,
                                      shape->cap, kv_len, sent_off, n_sent, params->eps, sc_tok, vsum, sent_imp, vbar_hi,
                                      vbar_lo, sent_lam));
     }
@@ -1639,10 +1661,10 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         const long long nb = (shape->max_sent + 127) / 128, max_items = L.slabs * (nb * (nb + 1) / 2);
         const int ggrid = int(max_items < (long long)grid ? max_items : (long long)grid);
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<1>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,
-                                     shape->max_sent, n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
+                                     shape->max_sent, int(L.sc_sent_rows), n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
                                      sent_score, vsum, L.sc_vsum_slab, a.lse_cnt, ext, reinterpret_cast<const Header*>(w + L.header)));
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<2>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,
-                                     shape->max_sent, n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
+                                     shape->max_sent, int(L.sc_sent_rows), n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
                                      sent_score, vsum, L.sc_vsum_slab, a.lse_cnt, ext, reinterpret_cast<const Header*>(w + L.header)));
     }
     return SKIPKV_OK;
