@@ -58,6 +58,7 @@ struct FillArgs {
     int Hk, max_cap, from_rows;
 };
 
+constexpr int kSelAhead = 2;            // sentences per thread that are read before their number is known
 constexpr int kFillStage = 1024;        // tokens of a cut sentence whose order keys are staged in shared memory
 
 __global__ void __launch_bounds__(kSelThreads)
@@ -69,23 +70,46 @@ select_kernel(int max_sent, int budget, int protect_tail, const float* sent_scor
     int* lens = reinterpret_cast<int*>(keys + max_sent);               // [max_sent] length, negative - 1 if protected
     __shared__ uint32_t hist[4][256], wsum[kSelThreads / 32];
     __shared__ uint32_t s_forced;
-    __shared__ int s_cut, s_slack;
+    __shared__ int s_cut, s_slack, s_begin, s_total;
     __shared__ float s_key[kFillStage];
     pdl_trigger();
     const int slab = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     for (int i = tid; i < 4 * 256; i += kSelThreads) (&hist[0][0])[i] = 0u;
-    if (tid == 0) { s_forced = 0u; s_cut = -1; s_slack = 0; }
+    if (tid == 0) { s_forced = 0u; s_cut = -1; s_slack = 0; s_total = 0; }
     pdl_wait();                                          // inputs may come from the kernel before
     const float* score = sent_score + size_t(slab) * max_sent;
     const int32_t* so = sent_off + size_t(slab) * (max_sent + 1);
     uint8_t* kp = keep + size_t(slab) * max_sent;
     int32_t* ki = kept_idx ? kept_idx + size_t(slab) * max_sent : nullptr;
+    // The kernel is a chain of round trips to memory, so everything is requested at once where the table is small enough for a fixed share of
+    // it per thread: the shares (whatever is in them past the last sentence), the number of sentences and the slab's first row.
+    const bool ahead = max_sent <= kSelAhead * kSelThreads;
+    const int per_max = (max_sent + kSelThreads - 1) / kSelThreads;
+    int off[kSelAhead + 1];
+    float sc[kSelAhead];
+#pragma unroll
+    for (int q = 0; q <= kSelAhead; ++q) {
+        const int i = tid * per_max + q;
+        off[q] = ahead && q <= per_max && i <= max_sent ? so[i] : 0;
+        if (q < kSelAhead) sc[q] = ahead && q < per_max && i < max_sent ? score[i] : 0.f;
+    }
+    const size_t row0 = fill.tok_keep ? slab_row0(fill.slab_off, fill.cap, fill.Hk, slab / fill.Hk, slab % fill.Hk) : 0;
     int S = n_sent[slab];
     if (S < 0 || S > max_sent) {
         if (tid == 0) atomicOr(status, SKIPKV_STATUS_BAD_TABLE);
         S = 0;
     }
-    const int total = (S > 0) ? so[S] : 0;
+    const int per = ahead ? per_max : (S + kSelThreads - 1) / kSelThreads;
+    const int i0 = min(tid * per, S), i1 = min(i0 + per, S);   // this thread's sentences
+    if (ahead) {
+#pragma unroll
+        for (int q = 0; q < kSelAhead; ++q)
+            if (i0 + q == S - 1 && i0 + q < i1) s_total = off[q + 1];
+    } else if (tid == 0 && S > 0) {
+        s_total = so[S];
+    }
+    __syncthreads();                                     // the total is known, the histograms are clear
+    const int total = s_total;
 
     if (total <= budget) {                              // already fits: identity
         for (int i = tid; i < max_sent; i += kSelThreads) {
@@ -99,16 +123,20 @@ select_kernel(int max_sent, int budget, int protect_tail, const float* sent_scor
         return;
     }
 
-    __syncthreads();                                     // the histograms are clear
-    const int per = (S + kSelThreads - 1) / kSelThreads, i0 = min(tid * per, S), i1 = min(i0 + per, S);   // this thread's sentences
-    for (int i = i0; i < i1; ++i) {
-        const int b = so[i], e = so[i + 1];
+    auto take = [&](int i, int b, int e, float x) {
         const bool forced = protect_tail > 0 && e > total - protect_tail && e > b;
-        const uint32_t k = ~orderable(score[i]);
+        const uint32_t k = ~orderable(x);
         keys[i] = k;
         lens[i] = forced ? -(e - b) - 1 : e - b;
         if (forced) atomicAdd(&s_forced, uint32_t(e - b));
         else if (e > b) atomicAdd(&hist[0][k >> 24], uint32_t(e - b));
+    };
+    if (ahead) {
+#pragma unroll
+        for (int q = 0; q < kSelAhead; ++q)
+            if (i0 + q < i1) take(i0 + q, off[q], off[q + 1], sc[q]);
+    } else {
+        for (int i = i0; i < i1; ++i) take(i, so[i], so[i + 1], score[i]);
     }
     __syncthreads();
     const uint32_t forced_len = s_forced;
@@ -157,7 +185,10 @@ select_kernel(int max_sent, int budget, int protect_tail, const float* sent_scor
             const uint32_t before = run;
             run += length(i);
             k = run <= room;
-            if (!k && before < room) { s_cut = i; s_slack = int(room - before); }      // one sentence only
+            if (!k && before < room) {                   // one sentence only
+                s_cut = i; s_slack = int(room - before);
+                s_begin = !ahead ? so[i] : i == i0 ? off[0] : off[1];
+            }
         } else {
             k = !only_forced && (lens[i] < 0 || keys[i] < cross);
         }
@@ -169,9 +200,7 @@ select_kernel(int max_sent, int budget, int protect_tail, const float* sent_scor
     const bool filled = fill.tok_keep && s_cut >= 0;
     if (filled) {
         const int c = s_cut, slack = s_slack;
-        const int cb = so[c], len = so[c + 1] - cb;
-        const int b = slab / fill.Hk, h = slab % fill.Hk;
-        const size_t row0 = slab_row0(fill.slab_off, fill.cap, fill.Hk, b, h);
+        const int cb = s_begin, len = int(length(c));
         const float* imp = fill.from_rows ? fill.tok_imp + row0 + cb : fill.tok_imp + size_t(slab) * fill.max_cap + cb;
         uint8_t* tk = fill.tok_keep + row0 + cb;
         const float* red = fill.tok_red ? fill.tok_red + row0 + cb : nullptr;
@@ -189,6 +218,7 @@ select_kernel(int max_sent, int budget, int protect_tail, const float* sent_scor
             const float mine = staged ? s_key[t] : key(t);
             int rank = 0;
             if (staged) {
+#pragma unroll 8
                 for (int u = 0; u < len; ++u) { const float other = s_key[u]; rank += (other > mine || (other == mine && u < t)) ? 1 : 0; }
             } else {
                 for (int u = 0; u < len; ++u) { const float other = key(u); rank += (other > mine || (other == mine && u < t)) ? 1 : 0; }
