@@ -679,23 +679,27 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             uint32_t ext_no = 0;                             // slabs begun so far
             float *imp_ws = nullptr, *imp_user = nullptr;
             float out_scale = 0.f;                           // 2^-e / window of the slab
-            int ti = 0, tk = 0, mod = 0;                     // tile in the order of the pass, block, and whose product it is
-            for (int left = ntl * a.RB; left > 0; --left) {
-                const int t = tile_at(ntl - 1 - ti), i = ti, k = tk, whose = mod;
-                if (++tk == a.RB) { tk = 0; ++ti; }
-                if (++mod == kAccB) mod = 0;
-                const bool begins = t >= hi || t < lo;
-                if (begins) {
-                    while (pref[slab + 1] <= t) ++slab;
-                    while (pref[slab] > t) --slab;
-                    lo = pref[slab]; hi = pref[slab + 1];
+            int i = 0, k = g;                                // this group's next product: tile in the order of the pass, and block
+            auto next_product = [&](int n) {
+                for (k += n; k >= a.RB; k -= a.RB) ++i;
+            };
+            for (next_product(0); i < ntl; next_product(kAccB)) {
+                const int t = tile_at(ntl - 1 - i);
+                bool begins = false;
+                if (t >= hi || t < lo) {
+                    do {                                     // (past slabs of which this group has no product)
+                        const int at = ext_no == 0 ? tile_at(ntl - 1) : pool_a ? lo - 1 : hi;
+                        while (pref[slab + 1] <= at) ++slab;
+                        while (pref[slab] > at) --slab;
+                        lo = pref[slab]; hi = pref[slab + 1];
+                        ++ext_no;
+                    } while (t >= hi || t < lo);
                     N = live(slab);
                     out_scale = __uint_as_float(uint32_t(127 - lse_shift(N)) << 23) / float(a.window);
                     imp_ws = a.tok_imp_ws + size_t(slab) * a.max_cap;
                     imp_user = a.tok_imp_user ? a.tok_imp_user + (a.block_table ? size_t(slab) * a.max_pages * 128 : size_t(rowb[slab])) : nullptr;
-                    ++ext_no;
+                    begins = k == 0 && t == (pool_a ? min(hi, t_end) - 1 : max(lo, t_begin));
                 }
-                if (whose != g) continue;
                 if (begins) {
                     // the group of a slab's first product prepares the slab: log-sum-exp of its query rows from the records of
                     // all its CTAs, negated, in units of raw logits, as three bf16 pieces of the extra K step
