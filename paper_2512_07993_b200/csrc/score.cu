@@ -652,15 +652,19 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 float2* rec = a.rec + size_t(cta + slab) * (size_t(a.RA) * 128);
                 for (int k = g; k < a.RA; k += accs) {       // the groups' parts -> one record per CTA and slab
                     float M = -INFINITY, L = 0.f;
-                    auto add = [&](float2 x) {
-                        const float m = fmaxf(M, x.x);
-                        L *= L > 0.f ? ex2f(M - m) : 0.f;
-                        L += x.y > 0.f ? x.y * ex2f(x.x - m) : 0.f;
-                        M = m;
+                    // (the largest reference first: a sum that is rescaled on the way is rounded on the way)
+                    const int n_part = can_shift && k + 1 == a.RA ? 2 * accs : accs;       // odd ones: the last block on shifted tiles
+                    auto at = [&](int q) {
+                        const bool sh = n_part > accs && (q & 1);
+                        const int g_ = n_part > accs ? q >> 1 : q;
+                        return part[(g_ * slots + (sh ? a.RA : k)) * 128 + (sh ? min(row + 128 - rem, 127) : row)];
                     };
-                    for (int q = 0; q < accs; ++q) {
-                        add(part[(q * slots + k) * 128 + row]);
-                        if (can_shift && k + 1 == a.RA && row < rem) add(part[(q * slots + a.RA) * 128 + row + 128 - rem]);
+#pragma unroll 1
+                    for (int q = 0; q < n_part; ++q) M = fmaxf(M, at(q).x);
+#pragma unroll 1
+                    for (int q = 0; q < n_part; ++q) {
+                        const float2 x = at(q);
+                        L += x.y > 0.f ? x.y * ex2f(x.x - M) : 0.f;
                     }
                     rec[k * 128 + row] = make_float2(M, L);
                 }
