@@ -739,6 +739,15 @@ constexpr size_t kStaticBytes =
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
+// The array keeps whatever the previous call left: the status word and the arrival counters must start at zero (the partial records
+// are fully written before they are read).  A kernel and not a memset, so that decode attention, as its programmatic dependent, derives its
+// schedule meanwhile.
+__global__ void __launch_bounds__(256) static_clear_kernel(uint32_t* words) {
+    pdl_trigger();
+    pdl_wait();
+    for (int i = threadIdx.x; i < int(kStaticPartOff / 4); i += 256) words[i] = 0u;
+}
+
 constexpr int kMaxDevices = 64;
 static unsigned char* g_static_addr[kMaxDevices];      // device address of the array, per device
 static bool g_static_ready[kMaxDevices];
@@ -789,19 +798,16 @@ extern "C" int skipkv_decode_attn_static(const skipkv_shape* shape, const void* 
     unsigned char* base = nullptr;
     if (int rc = static_setup(dev, &base)) return rc;
     const auto kernel = shape->n_q_heads / shape->n_kv_heads <= 4 ? decode_attn_kernel<false, true> : decode_attn_kernel<false, false>;
-    SKIPKV_CUDA(allow_max_smem(reinterpret_cast<const void*>(kernel)));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // The array keeps whatever the previous call left: the status word and the arrival counters
-    // must start at zero (the partial records are fully written before they are read).
-    SKIPKV_CUDA(cudaMemsetAsync(base, 0, kStaticPartOff, st));
+    SKIPKV_CUDA(launch_dependent(static_clear_kernel, dim3(1), dim3(256), 0, st, reinterpret_cast<uint32_t*>(base)));
     const int grid = num_sms() < kStaticMaxCtas ? num_sms() : kStaticMaxCtas;
     uint32_t* status_word = status ? status : reinterpret_cast<uint32_t*>(base);
-    kernel<<<grid, kDecThreads, smem, st>>>(
-        shape->batch, shape->n_q_heads, shape->n_kv_heads, slabs, static_cast<long long>(shape->total_rows), shape->slab_off,
-        shape->cap, static_cast<const __nv_bfloat16*>(q), static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len,
-        static_cast<__nv_bfloat16*>(out), status_word, reinterpret_cast<uint32_t*>(base + kStaticCntOff),
-        reinterpret_cast<float*>(base + kStaticPartOff), shape->d_model, static_cast<__nv_bfloat16*>(hidden),
-        static_cast<const __nv_bfloat16*>(steer_vec), alpha, flag, static_cast<const int32_t*>(nullptr), 0, StepArgs{});
-    SKIPKV_CUDA(cudaGetLastError());
+    SKIPKV_CUDA(launch_dependent(
+        kernel, dim3(grid), dim3(kDecThreads), smem, st, int(shape->batch), int(shape->n_q_heads), int(shape->n_kv_heads), slabs,
+        static_cast<long long>(shape->total_rows), shape->slab_off, shape->cap, static_cast<const __nv_bfloat16*>(q),
+        static_cast<const uint8_t*>(K), static_cast<const uint8_t*>(V), kv_len, static_cast<__nv_bfloat16*>(out), status_word,
+        reinterpret_cast<uint32_t*>(base + kStaticCntOff), reinterpret_cast<float*>(base + kStaticPartOff), int(shape->d_model),
+        static_cast<__nv_bfloat16*>(hidden), static_cast<const __nv_bfloat16*>(steer_vec), alpha, flag,
+        static_cast<const int32_t*>(nullptr), 0, StepArgs{}));
     return SKIPKV_OK;
 }
