@@ -237,7 +237,7 @@ __device__ __forceinline__ float imp_fold(uint32_t taddr, int n, int wvalid, flo
     return t0 + t1;
 }
 
-// ---- pass B: pooled key sums on the tensor cores
+// ---- pooled key sums on the tensor cores
 // Pooling product of one staged tile: D[128 channels x 16 slots] = K_tile^T x Ind^T.  A = the tile as the TMA load
 // wrote it ([token][channel], two 64-channel halves, 128-byte swizzle) read as an MN-major operand: 64 channels x 8
 // tokens per swizzle atom, atoms 1024 bytes apart along the tokens and a half (16 KB) apart along the channels.
@@ -289,7 +289,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     uint8_t* qbuf = sweep_smem_raw + (((raw + 1023u) & ~1023u) - raw);           // [2 halves][R rows][128 bytes]
     const uint32_t q_half = uint32_t(a.R) * 128u;
     uint8_t* tiles = qbuf + size_t(a.R) * kRowBytes;                             // (R is a multiple of 16: 1024-byte aligned)
-    uint8_t* indb = tiles + size_t(a.stages) * kOpBytes;                         // pass B: the indicator matrices
+    uint8_t* indb = tiles + size_t(a.stages) * kOpBytes;                         // the indicator matrices of the pooling
     uint8_t* onesb = indb + (kIndBytes << a.ind_log);                                // pass B: the keys' side of the extra K step
     uint8_t* extb = onesb + 128 * kExtRow;                                       // pass B: the queries' side; pass A: [groups][blocks] (m, l)
     SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + sweep_ext_bytes(a.RA));
