@@ -69,7 +69,8 @@ struct SweepCtl {                       // barriers and small shared state, afte
     // accumulator) that sees all its phases
     uint64_t tfull_a[kAccAMax], tempty_a[2 * kAccAMax], tfull_b[kAccB], tempty_b[2 * kAccB];
     uint64_t tokfull[4];                // pass B, several blocks per tile: the shares of a tile's tokens from all blocks but the last
-    uint64_t extfull, extempty;         // pass B: the rows' -lse as operand columns
+    uint64_t extfull;                   // pass B: the rows' -lse as operand columns; by group that prepares them (a slab's first product's), "the
+    uint64_t extempty[kAccB];           // products of the slab before have completed", so that a group sees every phase of its barrier
     // ring of indicator matrices: written by the four pooling warps -> multiplied by their issuer -> read out by the pooling warps
     uint64_t ifull[kIndRingMax], iempty[kIndRingMax];
     uint64_t pfull[2];                  // the last product of a run of tiles into accumulator i has completed
@@ -316,7 +317,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         for (int i = 0; i < 2 * kAccB; ++i) mbar_init(&ctl->tempty_b[i], 4);
         for (int i = 0; i < 4; ++i) mbar_init(&ctl->tokfull[i], a.RB > 1 ? 4 * (a.RB - 1) : 1);
         mbar_init(&ctl->extfull, 4);
-        mbar_init(&ctl->extempty, 2);
+        for (int i = 0; i < kAccB; ++i) mbar_init(&ctl->extempty[i], 2);
         for (int i = 0; i < kIndRingMax; ++i) { mbar_init(&ctl->ifull[i], kPoolWarps); mbar_init(&ctl->iempty[i], 1); }
         for (int i = 0; i < 2; ++i) mbar_init(&ctl->pfull[i], 1);
         for (int i = 0; i < 3; ++i) mbar_init(&ctl->retired[i], 1);
@@ -520,7 +521,10 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                 }
                 if (p > 0) {
                     const int t_next = tile_at(p - 1);
-                    if (t_next >= hi || t_next < lo) { umma_commit(&ctl->qempty, leader); umma_commit(&ctl->extempty, leader); }
+                    if (t_next >= hi || t_next < lo) {                    // (the next product's group prepares the next slab)
+                        umma_commit(&ctl->qempty, leader);
+                        umma_commit(&ctl->extempty[buf], leader);
+                    }
                 }
                 free_stage(a.RB > 1 || turn != mine, !pool_a);
             }
@@ -681,6 +685,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             uint32_t turn = 0;                               // products of this group so far
             int slab = slab_of(tile_at(ntl - 1)), lo = 0, hi = 0, N = 0;        // the slab's tiles are [lo, hi)
             uint32_t ext_no = 0;                             // slabs begun so far
+            uint32_t ext_par = 0;                            // parity of this group's next phase of extempty
             float *imp_ws = nullptr, *imp_user = nullptr;
             float out_scale = 0.f;                           // 2^-e / window of the slab
             int i = 0, k = g;                                // this group's next product: tile in the order of the pass, and block
@@ -710,7 +715,10 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     const int fc = owner(lo), lc = owner(hi - 1);
                     if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(hi - lo), limit, &ctl->abort_flag, a.status);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                    if (ok && ext_no > 1) ok = role_wait(&ctl->extempty, (ext_no - 2) & 1u, limit, &ctl->abort_flag, a.status);
+                    if (ok && ext_no > 1) {
+                        ok = role_wait(&ctl->extempty[g], ext_par, limit, &ctl->abort_flag, a.status);
+                        ext_par ^= 1u;
+                    }
                     ok = __all_sync(0xffffffffu, ok);
                     if (ok) {
                         const float2* r0 = a.rec + size_t(fc + slab) * (size_t(a.RA) * 128);

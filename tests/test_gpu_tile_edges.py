@@ -146,6 +146,39 @@ def test_score_with_more_slabs_than_shared_memory_has_room_for(group, window, ba
             assert torch.equal(got[b, :, :S], ref[b, :, :S])
 
 
+@pytest.mark.parametrize("group,window", [(4, 32), (5, 20), (8, 16), (4, 48)])
+@pytest.mark.parametrize("ctx", [[1 + (37 * i) % 128 for i in range(64)], [9000, 100, 9000], [9000, 100, 128, 1, 9000]])
+def test_score_runs_of_slabs_of_one_tile(group, window, ctx):
+    """Three and more slabs of one tile one after the other in a CTA's share, each with one product of the second pass (48 positions: two): short
+    sequences throughout, and the eight heads of one or a few among long ones.  The epilogue group that prepares a slab's log-sum-exps is then
+    another one every time, and two slabs ahead of the product before.  Contiguous against the oracle, paged against contiguous."""
+    B, L, D = layer(ctx, n_q_heads=8 * group, n_kv_heads=8, window=window, sent_lo=8, sent_hi=40, dup_rate=0.3, seed=980 + group)
+    check_scores(B, L, D)
+    pages = [-(-n // 128) for n in ctx]
+    max_pages, n_pool = max(pages), 8 * sum(pages)
+    ids = torch.as_tensor(np.random.Generator(np.random.Philox(6)).permutation(n_pool).astype(np.int32)).cuda()
+    Kp = torch.full((n_pool * 128, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    table = torch.full((len(ctx), 8, max_pages), -1, dtype=torch.int32, device="cuda")
+    k = 0
+    for b, n in enumerate(ctx):
+        table[b, :, :pages[b]] = ids[k:k + 8 * pages[b]].view(8, pages[b])
+        k += 8 * pages[b]
+        t = torch.arange(n, device="cuda")
+        off = int(L["slab_off"][b]) * 8
+        Kp[(table[b].long()[:, t // 128] * 128 + t % 128).reshape(-1)] = D.K[off:off + 8 * n]
+    shp = B.make_shape(len(ctx), 8 * group, 8, 128, window, L["cfg"].d_model, D.max_sent, max(ctx), D.slab_off, D.cap, int(Kp.shape[0]))
+    imp = torch.full((len(ctx), 8, max_pages * 128), float("nan"), device="cuda")
+    outs = [torch.full_like(D.sent_imp, float("nan")) for _ in range(4)]
+    B.skipkv_score_paged(shp, D.params, Kp, table, max_pages, D.q_win, D.kv_len, D.sent_off, D.n_sent, imp, *outs, D.ws)
+    torch.cuda.synchronize()
+    assert D.status() == 0
+    for b, n in enumerate(ctx):
+        off, S = int(L["slab_off"][b]) * 8, int(L["n_sent"][b, 0])
+        assert torch.equal(imp[b, :, :n].reshape(-1), D.tok_imp[off:off + 8 * n])
+        for got, ref in zip(outs, (D.sent_imp, D.sent_red, D.sent_lam, D.sent_score)):
+            assert torch.equal(got[b, :, :S], ref[b, :, :S])
+
+
 @pytest.mark.parametrize("hq,ctx", [(2, [30000, 23456]), (8, [4100, 9000, 20000]), (10, [16384, 8000]), (16, [2048, 12345])])
 def test_decode_keeps_fp32_probabilities(hq, ctx):
     """The share of outputs that are not the exact result rounded to bf16.  A value with relative error e lies on the wrong side of
