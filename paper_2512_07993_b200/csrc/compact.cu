@@ -359,6 +359,7 @@ compact_move_kernel(int n_slabs, int Hk, int max_sent, const int64_t* slab_off, 
                 open = *flag == 0u;
             }
             __threadfence();
+            __syncwarp();                              // what one lane saw comes before every lane's stores
             ok = __all_sync(0xffffffffu, ok);
             if (ok) {
                 for (int r = r0 + lane; piece(r, ps, pe, src, mapped); r += 32)

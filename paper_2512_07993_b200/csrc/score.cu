@@ -121,7 +121,7 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// Bounded wait of one thread until *p reaches `want`; gives up like role_wait.
+// Bounded wait of one thread until *p reaches `want`; gives up like role_wait.  See warp_flag_wait for a whole warp.
 static __device__ __noinline__ bool flag_wait(const uint32_t* p, uint32_t want, uint32_t limit, int* abort_flag, uint32_t* status) {
     for (uint32_t i = 0; i < limit; ++i) {
         if (ld_acquire(p) >= want) return true;
@@ -131,6 +131,14 @@ static __device__ __noinline__ bool flag_wait(const uint32_t* p, uint32_t want, 
     atomicOr(status, SKIPKV_STATUS_COPY_TIMEOUT);
     *reinterpret_cast<volatile int*>(abort_flag) = 1;
     return false;
+}
+// The same for a converged warp: one lane polls, and all of them see what was published.  (The vote alone orders no memory accesses; the
+// barrier behind the acquire does.)
+__device__ __forceinline__ bool warp_flag_wait(const uint32_t* p, uint32_t want, uint32_t limit, int* abort_flag, uint32_t* status) {
+    bool ok = true;
+    if ((threadIdx.x & 31) == 0) ok = flag_wait(p, want, limit, abort_flag, status);
+    __syncwarp();
+    return __all_sync(0xffffffffu, ok);
 }
 
 // D[128 x n] (+)= A[128 x 128] * B[n x 128]^T.  Both operands are two halves of 64 channels, a_half / b_half bytes apart.
@@ -713,8 +721,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
                     // the group of a slab's first product prepares the slab: log-sum-exp of its query rows from the records of
                     // all its CTAs, negated, in units of raw logits, as three bf16 pieces of the extra K step
                     const int fc = owner(lo), lc = owner(hi - 1);
-                    if (lane == 0 && ok) ok = flag_wait(a.lse_cnt + slab, uint32_t(hi - lo), limit, &ctl->abort_flag, a.status);
-                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                    if (ok) ok = warp_flag_wait(a.lse_cnt + slab, uint32_t(hi - lo), limit, &ctl->abort_flag, a.status);
                     if (ok && ext_no > 1) {
                         ok = role_wait(&ctl->extempty[g], ext_par, limit, &ctl->abort_flag, a.status);
                         ext_par ^= 1u;
@@ -915,9 +922,8 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             if (ok && run > 0) drain(run - 1);                      // (the issuer closes the last run when its tiles are done)
             if (ok && head_sent >= 0) {
                 const uint32_t all = 4u * uint32_t(pref[slab_first + 1] - pref[slab_first]);
-                if (lane == 0) ok = flag_wait(a.sum_cnt + slab_first, all, limit, &ctl->abort_flag, a.status);
-                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                if (ok) atomicAdd(a.vsum + (size_t(slab_first) * a.max_sent + head_sent) * kHeadDim + ch, head);
+                if (warp_flag_wait(a.sum_cnt + slab_first, all, limit, &ctl->abort_flag, a.status))
+                    atomicAdd(a.vsum + (size_t(slab_first) * a.max_sent + head_sent) * kHeadDim + ch, head);
             }
         }
     }
