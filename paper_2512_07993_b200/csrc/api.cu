@@ -93,10 +93,10 @@ int tmap_rows(CUtensorMap* out, const void* base, uint64_t rows, uint32_t box_ro
     return encode(out, base, 2, dims, strides, box);
 }
 
-int tmap_qwin(CUtensorMap* out, const void* base, uint64_t heads, uint32_t window, uint32_t box_w, uint32_t box_heads) {
-    const cuuint64_t dims[3] = {cuuint64_t(kHeadDim), window, heads};
-    const cuuint64_t strides[2] = {cuuint64_t(kRowBytes), cuuint64_t(kRowBytes) * window};
-    const cuuint32_t box[3] = {64, box_w, box_heads};
+int tmap_groups(CUtensorMap* out, const void* base, uint64_t groups, uint32_t rows, uint32_t box_rows, uint32_t box_groups) {
+    const cuuint64_t dims[3] = {cuuint64_t(kHeadDim), rows, groups};
+    const cuuint64_t strides[2] = {cuuint64_t(kRowBytes), cuuint64_t(kRowBytes) * rows};
+    const cuuint32_t box[3] = {64, box_rows, box_groups};
     return encode(out, base, 3, dims, strides, box);
 }
 

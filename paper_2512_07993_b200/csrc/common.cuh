@@ -43,9 +43,8 @@ struct WsLayout {
     size_t sc_vsum;        // float  [slabs][max_sent][128]  per-sentence sums of key rows; then partial sums of the Gram passes,
                            //        [slabs] x sc_vsum_slab floats, of which [4 * blocks][max_sent] are used
     size_t sc_vsum_slab;
-    size_t sc_vbar_hi;     // bf16   [slabs][sc_sent_rows][128]  normalised mean key, high part
-    size_t sc_vbar_lo;     // bf16   [slabs][sc_sent_rows][128]  and the rounding remainder
-    size_t sc_sent_rows;   // max_sent in whole blocks of 128, so that a block holds rows of one slab only
+    size_t sc_vbar_hi;     // bf16   [slabs][max_sent][128]  normalised mean key, high part
+    size_t sc_vbar_lo;     // bf16   [slabs][max_sent][128]  and the rounding remainder (both empty up to kSmallSent sentences)
     size_t sc_z;           // float  [slabs][max_sent]  1 / row sum of e^G
     size_t slab_table;       // int32  [2 * slabs + 1]  tile prefix and first rows of the slabs, where shared memory has no room for them
     size_t tr_inv;         // float  [slabs][max_cap]  token redundancy: 1 / (|K_t| + eps)
@@ -62,6 +61,7 @@ constexpr int kDecPartStride = 132;    // decode partial of one head: 128 accumu
 constexpr int kDecMaxCtas = 1024;     // upper bound of the persistent grids
 constexpr int kMaxQueryBlocks = 4;
 constexpr int kSegRows = 128;         // rows per segment of the compaction
+constexpr int kSmallSent = 128;       // sentences per slab up to which the scoring call keeps the pooled keys in shared memory
 constexpr int kMaxPartial = 4;        // partly kept sentences per slab that one compaction call can carry
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -100,9 +100,9 @@ inline WsLayout make_layout(const skipkv_shape& s) {
     const size_t sums = (ms + 127) / 128 * 4;
     L.sc_vsum_slab = ms * (sums > size_t(kHeadDim) ? sums : size_t(kHeadDim));
     L.sc_vsum = take(slabs * L.sc_vsum_slab * 4);
-    L.sc_sent_rows = (ms + 127) / 128 * 128;
-    L.sc_vbar_hi = take(slabs * L.sc_sent_rows * kHeadDim * 2);
-    L.sc_vbar_lo = take(slabs * L.sc_sent_rows * kHeadDim * 2);
+    const size_t pooled = ms > size_t(kSmallSent) ? slabs * ms * kHeadDim * 2 : 0;
+    L.sc_vbar_hi = take(pooled);
+    L.sc_vbar_lo = take(pooled);
     L.sc_z = take(slabs * ms * 4);
     L.slab_table = take((2 * slabs + 1) * 4);
     L.tr_inv = take(slabs * size_t(s.max_cap > 0 ? s.max_cap : 1) * 4);

@@ -943,7 +943,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
 // ---------------------------------------------------------------------------------------
 constexpr int kPoolRows = 4;
 __global__ void __launch_bounds__(256)
-score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int sent_rows, int max_cap, int max_rows, const int32_t* cap, const int32_t* kv_len,
+score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_rows, const int32_t* cap, const int32_t* kv_len,
                   const int32_t* sent_off, const int32_t* n_sent, float eps, const float* tok_imp_ws,
                   const float* vsum, float* sent_imp, __nv_bfloat16* vbar_hi, __nv_bfloat16* vbar_lo, float* sent_lam) {
     pdl_trigger();
@@ -981,8 +981,8 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int sent_rows, int ma
     for (int q = 0; q < kPoolRows; ++q) {
         const int i = i0 + q * 8;
         if (i >= S) {                                        // the rest of the last block: zeros, whose products are finite
-            if (i < (S + 127) / 128 * 128) {
-                const size_t o = (size_t(slab) * sent_rows + i) * kHeadDim;
+            if (i < min((S + 127) / 128 * 128, max_sent)) {
+                const size_t o = (size_t(slab) * max_sent + i) * kHeadDim;
                 reinterpret_cast<uint2*>(vbar_hi + o)[lane] = reinterpret_cast<uint2*>(vbar_lo + o)[lane] = make_uint2(0u, 0u);
             }
             continue;
@@ -1008,7 +1008,7 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int sent_rows, int ma
             hi[c] = __bfloat16_as_ushort(h);
             lo[c] = __bfloat16_as_ushort(r);
         }
-        const size_t o = (size_t(slab) * sent_rows + i) * kHeadDim;
+        const size_t o = (size_t(slab) * max_sent + i) * kHeadDim;
         reinterpret_cast<uint2*>(vbar_hi + o)[lane] = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
         reinterpret_cast<uint2*>(vbar_lo + o)[lane] = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
         if (lane == 0) {
@@ -1026,7 +1026,7 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int sent_rows, int ma
 // A column block's sums are kept for as long as a range stays with it and stored as that part's (four warps' each); a row's are stored by pair (four column
 // groups).  The CTA that completes a slab adds a sentence's parts and rows up in order, so the results do not depend on who was first.
 // They lie where the sums of the keys were, which the pooling was the last to read.
-// Rows past a slab's last sentence are zeros (every slab has whole blocks of its own), so nothing is masked but the weights of such
+// Rows past a slab's last sentence are zeros (written, or beyond the table and filled in by the copy), so nothing is masked but the weights of such
 // columns and, in a diagonal pair, a sentence's product with itself.
 // The penalty is the maximum over later sentences; only those beyond tau are reported, which are few (pass 1, an integer maximum).
 // Roles as in the token-level kernel: a TMA warp, two MMA warps that take the pairs in turn, sixteen epilogue warps with 32
@@ -1114,7 +1114,7 @@ struct LamTable {
 template <int kPass>
 __global__ void __launch_bounds__(kGramThreads, 1)
 score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ CUtensorMap mapLo, int n_slabs,
-                  int max_sent, int sent_rows, const int32_t* n_sent, float sigma, float tau, float* sc_z, const float* sent_imp,
+                  int max_sent, const int32_t* n_sent, float sigma, float tau, float* sc_z, const float* sent_imp,
                   float* sent_red, float* sent_lam, float* sent_score, float* parts, size_t parts_slab, uint32_t* cnt, LamTable ext, const Header* hdr) {
     extern __shared__ uint8_t gram_smem_raw[];
     const uint32_t raw = smem_u32(gram_smem_raw);
@@ -1167,10 +1167,9 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
                     if (!ok) break;
                     uint8_t* dst = slots + size_t(2 * s + part) * kOpBytes;
                     const CUtensorMap* map = part ? &mapLo : &mapHi;
-                    const int row = w.slab * sent_rows + block * 128;
                     mbar_expect_tx(&ctl->full[s][part], kOpBytes);
-                    tma_load_2d(dst, map, 0, row, &ctl->full[s][part]);
-                    tma_load_2d(dst + kOpHalfBytes, map, 64, row, &ctl->full[s][part]);
+                    tma_load_3d(dst, map, 0, block * 128, w.slab, &ctl->full[s][part]);
+                    tma_load_3d(dst + kOpHalfBytes, map, 64, block * 128, w.slab, &ctl->full[s][part]);
                     ++ctl->loads[2 * s + part];
                 }
             };
@@ -1427,7 +1426,6 @@ score_gram_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_consta
 // wait for the sweep) against 8 warps with two.
 // ---------------------------------------------------------------------------------------
 constexpr int kSmallThreads = 512;
-constexpr int kSmallSent = 128;
 constexpr int kSmallBatch = 8;          // sentences of a warp: their loads are in flight together
 struct SmallCtl {
     uint64_t done;
@@ -1612,13 +1610,14 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int Hq = shape->n_q_heads, Hk = shape->n_kv_heads, n = L.group;
 
-    CUtensorMap mapK, mapQ, mapHi, mapLo;
+    CUtensorMap mapK, mapQ, mapHi{}, mapLo{};
     if (int rc = tmap_rows(&mapK, K, uint64_t(shape->total_rows), 128)) return rc;
-    if (int rc = tmap_qwin(&mapQ, q_win, uint64_t(shape->batch) * Hq, uint32_t(shape->window), uint32_t(L.sc_wb), uint32_t(n)))
+    if (int rc = tmap_groups(&mapQ, q_win, uint64_t(shape->batch) * Hq, uint32_t(shape->window), uint32_t(L.sc_wb), uint32_t(n)))
         return rc;
-    const uint64_t vrows = uint64_t(L.slabs) * uint64_t(L.sc_sent_rows);
-    if (int rc = tmap_rows(&mapHi, vbar_hi, vrows, 128)) return rc;
-    if (int rc = tmap_rows(&mapLo, vbar_lo, vrows, 128)) return rc;
+    if (shape->max_sent > kSmallSent) {
+        if (int rc = tmap_groups(&mapHi, vbar_hi, uint64_t(L.slabs), uint32_t(shape->max_sent), 128, 1)) return rc;
+        if (int rc = tmap_groups(&mapLo, vbar_lo, uint64_t(L.slabs), uint32_t(shape->max_sent), 128, 1)) return rc;
+    }
 
     SweepArgs a{};
     a.Hq = Hq; a.Hk = Hk; a.window = shape->window; a.n_slabs = L.slabs; a.max_cap = shape->max_cap;
@@ -1674,8 +1673,8 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         return SKIPKV_OK;
     }
     {
-        dim3 pgrid(unsigned(L.sc_sent_rows) / (8 * kPoolRows), L.slabs);
-        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, int(L.sc_sent_rows), shape->max_cap, max_rows,
+        dim3 pgrid(unsigned(shape->max_sent + 8 * kPoolRows - 1) / (8 * kPoolRows), L.slabs);
+        SKIPKV_CUDA(launch_dependent(score_pool_kernel, pgrid, dim3(256), 0, st, a.lse_cnt, Hk, shape->max_sent, shape->max_cap, max_rows,
                                      shape->cap, kv_len, sent_off, n_sent, params->eps, sc_tok, vsum, sent_imp, vbar_hi,
                                      vbar_lo, sent_lam));
     }
@@ -1683,10 +1682,10 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
         const long long nb = (shape->max_sent + 127) / 128, max_items = L.slabs * (nb * (nb + 1) / 2);
         const int ggrid = int(max_items < (long long)grid ? max_items : (long long)grid);
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<1>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,
-                                     shape->max_sent, int(L.sc_sent_rows), n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
+                                     shape->max_sent, n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
                                      sent_score, vsum, L.sc_vsum_slab, a.lse_cnt, ext, reinterpret_cast<const Header*>(w + L.header)));
         SKIPKV_CUDA(launch_dependent(score_gram_kernel<2>, dim3(ggrid), dim3(kGramThreads), gsmem, st, mapHi, mapLo, L.slabs,
-                                     shape->max_sent, int(L.sc_sent_rows), n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
+                                     shape->max_sent, n_sent, params->sigma, params->tau, sc_z, sent_imp, sent_red, sent_lam,
                                      sent_score, vsum, L.sc_vsum_slab, a.lse_cnt, ext, reinterpret_cast<const Header*>(w + L.header)));
     }
     return SKIPKV_OK;

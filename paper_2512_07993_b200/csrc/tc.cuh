@@ -21,9 +21,9 @@ constexpr int kOpBytes = 2 * kOpHalfBytes;         // 32 KB
 // ---- host: tensor maps ------------------------------------------------------------------
 // 2-D view [rows][128] bf16 of a row-major buffer, box = 64 elements x box_rows rows, 128-byte swizzle.
 int tmap_rows(CUtensorMap* out, const void* base, uint64_t rows, uint32_t box_rows);
-// 3-D view of the window queries [heads][window][128] bf16 (dims fastest first: channel, window
-// position, head), box = 64 channels x box_w window positions x box_heads heads.
-int tmap_qwin(CUtensorMap* out, const void* base, uint64_t heads, uint32_t window, uint32_t box_w, uint32_t box_heads);
+// 3-D view [groups][rows][128] bf16 (dims fastest first: channel, row, group), box = 64 channels x box_rows rows x box_groups groups, 128-byte
+// swizzle: the window queries by head, the pooled keys by slab.  What a box has beyond a group's last row comes as zeros.
+int tmap_groups(CUtensorMap* out, const void* base, uint64_t groups, uint32_t rows, uint32_t box_rows, uint32_t box_groups);
 
 #ifdef __CUDACC__
 // ---- device -------------------------------------------------------------------------------

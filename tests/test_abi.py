@@ -56,6 +56,16 @@ def test_workspace_bytes_and_shape_checks(binding):
         assert e.value.code == code
 
 
+@pytest.mark.parametrize("max_sent", [1, 64, 128, 129, 200, 256, 1000])
+def test_workspace_holds_what_a_slab_needs(binding, max_sent):
+    """Bytes per slab, one head per group and 128 rows: 12 + 512 + 2 * 256 per sentence (runs, 1 / Z, key sum, pooled key in two parts: nothing in
+    whole blocks), beside them records of 128 + 4 floats and 128 pairs, three floats a row, and under 200 bytes of counters, tables and four segments."""
+    def size(batch):
+        return binding.skipkv_workspace_bytes(binding.make_shape(batch, 1, 1, 128, 16, 0, max_sent, 128, None, None))
+    per_slab = (size(8192) - size(4096)) / 4096
+    assert per_slab <= (12 + 512 + 2 * 256) * max_sent + 132 * 4 + 128 * 8 + 3 * 128 * 4 + 200
+
+
 def test_null_arguments_are_rejected_before_any_launch(binding):
     lib = binding.lib()
     shape = binding.make_shape(1, 4, 1, 128, 8, 256, 16, 128, None, None)
