@@ -181,6 +181,8 @@ int skipkv_compact(const skipkv_shape* shape, void* K, void* V, const uint8_t* k
  * t < kv_len[b][q / n]; fp32 accumulation, bf16 result; kv_len == 0 gives zeros.
  * q, out: device bf16 [batch][Hq][128].  If hidden is non-null the steering add of
  * skipkv_steer is performed on it by the same launch (arguments as below).
+ * shape->total_rows bounds what is fetched before the lengths are confirmed; the result does not depend on it
+ * (this holds for every decode entry).
  */
 int skipkv_decode_attn(const skipkv_shape* shape, const void* q, const void* K, const void* V,
                        const int32_t* kv_len, void* out, void* hidden, const void* steer_vec,

@@ -227,6 +227,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     int p_t = t_begin, p_slab = slab0, p_end = t_begin, p_r0 = 0, p_rows = 0, p_stage = 0;
     size_t p_row0 = 0;
     bool p_app = false;
+    long long far = 0;                                    // where the farthest of the unchecked copies ends
     auto issue_next = [&](auto unchecked) {
         if (p_t < t_end) {
             if (p_end <= p_t) {
@@ -243,8 +244,9 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
                 if (block_table)
                     row = (p_t == t_begin ? row_first : size_t(max(block_table[size_t(p_slab) * max_pages + p_r0 / kPageRows], 0))) * kPageRows +
                           size_t(p_r0 % kPageRows);
-                // (never beyond the buffers, also under lengths that turn out to be old)
-                if (!decltype(unchecked)::value || (long long)row + min(rows, kWarpRows) <= total_rows) {
+                // (never beyond the buffers, also under lengths that turn out to be old; from one that is left out on all are, and count as changed)
+                if (decltype(unchecked)::value) far = max(far, (long long)row + min(rows, kWarpRows));
+                if (!decltype(unchecked)::value || far <= total_rows) {
                     const size_t off = (row + size_t(c_half)) * kRowBytes + size_t(c_col) * 16;
                     const uint8_t *kp = K + off, *vp = V + off;
                     // (row 2 i + c_half takes its pieces at c_col ^ ((2 i + c_half) & 7): four addresses and constant distances from them)
@@ -311,7 +313,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
         for (int k = 0; k < kStages - 1; ++k) issue_next(std::true_type{});
     }
     {
-        int changed = row_again != row_first;
+        int changed = row_again != row_first || far > total_rows;
         if (s_lo < s_hi && len_again != lens[s_lo]) changed = 1;
         for (int s = s_lo + 1; s < s_hi; ++s)
             if (slab_len(s) != lens[s]) changed = 1;

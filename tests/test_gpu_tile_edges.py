@@ -43,6 +43,39 @@ def test_decode_rows_around_warp_and_tile_edges(hq):
         assert np.isfinite(out).all() and err.max() <= 2e-2 and np.sqrt((err ** 2).mean()) < 2e-3
 
 
+@pytest.mark.parametrize("step", [False, True])
+def test_decode_reads_every_row_whatever_total_rows_says(step):
+    """total_rows bounds the copies that go out before the lengths are confirmed.  With one that ends behind a slab whose last tile is the first
+    of a CTA's share, that CTA's second tile lies beyond it and is copied behind the confirmation: the same bits as with the true number."""
+    ctx = [1300 + 171 * i for i in range(12)]
+    B, L, D = layer(ctx, n_q_heads=8, n_kv_heads=2, seed=340, cap_extra=1)
+    tiles = np.repeat([(n + step + 63) // 64 for n in ctx], 2)
+    ends, rows_end = np.cumsum(tiles), np.cumsum(np.repeat([n + 1 for n in ctx], 2))
+    ctas = min(torch.cuda.get_device_properties(0).multi_processor_count, 256, int(ends[-1]))
+    starts = [c * int(ends[-1]) // ctas for c in range(ctas)]
+    short = [int(rows_end[s]) for s in range(23) if ends[s] - 1 in starts]
+    assert short
+    cfg = L["cfg"]
+    row = lambda seed: torch.randn(12, 2, 128, generator=torch.Generator().manual_seed(seed)).bfloat16().cuda()
+    one = lambda dt, v: torch.full((12,), v, dtype=dt, device="cuda")
+
+    def run(total_rows):
+        shp = B.make_shape(12, 8, 2, 128, cfg.window, cfg.d_model, D.max_sent, max(ctx) + 1, D.slab_off, D.cap, total_rows)
+        out = torch.full_like(D.out, float("nan"))
+        if step:
+            B.skipkv_decode_step(shp, D.q, row(1), row(2), D.K.clone(), D.V.clone(), D.kv_len, torch.empty_like(D.kv_len), D.sent_off.clone(),
+                                 D.sent_id.clone(), D.n_sent.clone(), one(torch.uint8, 0), one(torch.int32, 0), None, 0, out, None, None, None, None, D.ws)
+        else:
+            B.skipkv_decode_attn(shp, D.q, D.K, D.V, D.kv_len, out, None, None, None, None, D.ws)
+        torch.cuda.synchronize()
+        assert D.status() == 0
+        return out
+
+    want = run(int(D.K.shape[0]))
+    for total_rows in short:
+        assert torch.equal(run(total_rows).view(torch.int16), want.view(torch.int16)), total_rows
+
+
 def check_scores(B, L, D, rtol=1e-3):
     cfg = L["cfg"]
     D.score()
