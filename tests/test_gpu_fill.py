@@ -277,3 +277,58 @@ def test_compact_fill_too_many_partial_sentences_is_reported():
     assert B.skipkv_status(D.ws, raise_on_error=False) & 0x4
     assert torch.equal(D.K[rows], K_before[rows])           # that slab was not moved
     B.skipkv_workspace_init(D.shape, D.ws)
+
+
+@pytest.mark.parametrize("max_sent", [1, 2, 511, 512, 513, 1023, 1024, 1025, 1600])
+def test_select_table_sizes_around_a_threads_share(max_sent):
+    """Tables of up to 512 sentences are one per thread, of up to 1024 two, read before their number is known, longer ones are not: lists as
+    long as the table, shorter and empty ones, junk behind them, and the cut in either half of a thread's pair, at both ends and in the middle."""
+    from paper_2512_07993_b200 import build, binding as B
+    build.build()
+    rng = np.random.Generator(np.random.Philox(max_sent))
+    count = np.array([max_sent, max_sent - 1, max(max_sent // 2, 1), min(max_sent, 3), 0, max_sent], np.int32).reshape(3, 2)
+    off = np.full((3, 2, max_sent + 1), 1 << 30, np.int32)
+    score = np.full((3, 2, max_sent), np.nan, np.float32)
+    for b in range(3):
+        for h in range(2):
+            S = count[b, h]
+            off[b, h, :S + 1] = np.concatenate([[0], np.cumsum(rng.integers(0, 9, S))])
+            score[b, h, :S] = np.round(rng.standard_normal(S), 2)              # ties among them
+    off[0, 0] = np.concatenate([[0], np.cumsum(rng.integers(2, 9, max_sent))])    # every sentence can be the cut one
+    kv = np.take_along_axis(off, count[..., None], -1)[..., 0]
+    cap = kv.max(1) + 1
+    first = np.concatenate([[0], np.cumsum(cap)[:-1]])
+    rows = int(cap.sum()) * 2
+    imp = rng.standard_normal(rows).astype(np.float32)
+    cuda = lambda x, dt: torch.as_tensor(x).to(dt).cuda()
+    d_off, d_ns, d_sc, d_imp = cuda(off, torch.int32), cuda(count, torch.int32), cuda(score, torch.float32), cuda(imp, torch.float32)
+    d_first, d_cap = cuda(first, torch.int64), cuda(cap, torch.int32)
+    shp = B.make_shape(3, 2, 2, 128, 8, 0, max_sent, int(cap.max()), d_first, d_cap, rows)
+    ws = torch.empty(B.skipkv_workspace_bytes(shp), dtype=torch.uint8, device="cuda")
+    B.skipkv_workspace_init(shp, ws)
+    keep, kept = torch.empty(3, 2, max_sent, dtype=torch.uint8, device="cuda"), torch.empty(3, 2, max_sent, dtype=torch.int32, device="cuda")
+    n_kept, new_len = torch.empty(3, 2, dtype=torch.int32, device="cuda"), torch.empty(3, 2, dtype=torch.int32, device="cuda")
+    tok = torch.empty(rows, dtype=torch.uint8, device="cuda")
+    length, order = np.diff(off[0, 0]), np.lexsort((np.arange(max_sent), -score[0, 0]))
+    before = np.empty(max_sent, np.int64)
+    before[order] = np.cumsum(length[order]) - length[order]                 # tokens of the sentences ranked above
+    cuts = sorted({c % max_sent for c in (0, 1, max_sent // 2, max_sent // 2 + 1, max_sent - 2, max_sent - 1, 511, 512, 1023)})
+    for cut in cuts:
+        for tail in (0, 16):
+            budget = int(before[cut] + 1 + length[cut] // 2 - (length[cut] == 2))
+            B.skipkv_select_fill(shp, B.make_params(0.1, 0.95, 1e-6, budget, tail), d_sc, d_imp, d_off, d_ns, keep, tok.fill_(7), kept, n_kept, new_len, ws)
+            torch.cuda.synchronize()
+            g_keep, g_kept, g_tok = keep.cpu().numpy(), kept.cpu().numpy(), tok.cpu().numpy()
+            for b in range(3):
+                for h in range(2):
+                    S, n, row = int(count[b, h]), int(kv[b, h]), int(first[b] * 2 + h * cap[b])
+                    k_ref, t_ref, nl = oracle.select_fill(score[b, h, :S], off[b, h, :S + 1], imp[row:row + n], budget, tail)
+                    assert np.array_equal(g_keep[b, h, :S], k_ref) and not g_keep[b, h, S:].any(), (cut, tail, b, h)
+                    assert int(new_len[b, h]) == nl and int(n_kept[b, h]) == np.count_nonzero(k_ref)
+                    assert np.array_equal(g_kept[b, h][g_kept[b, h] >= 0], np.nonzero(k_ref)[0])
+                    for c in np.nonzero(k_ref == 2)[0]:
+                        at = slice(off[b, h, c], off[b, h, c + 1])
+                        assert np.array_equal(g_tok[row:row + n][at], t_ref[at])
+            if tail == 0:
+                assert g_keep[0, 0, cut] == 2
+    assert B.skipkv_status(ws) == 0
