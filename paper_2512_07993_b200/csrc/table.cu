@@ -18,7 +18,7 @@ constexpr int kCloseThreads = 256;
 constexpr int kPssThreads = 256;
 constexpr int kPssRowsPerWarp = 2;
 constexpr int kPssUnroll = 4;
-constexpr int kPssEarly = 4;                                       // rows per CTA that start towards L2 before the sentence is closed
+constexpr int kPssEarlyRows = 4, kPssEarlyBytes = 64 << 10;         // what a CTA starts towards L2 before the sentence is closed, at most
 constexpr int kPssRows = (kPssThreads / 32) * kPssRowsPerWarp;     // earlier sentences per CTA
 
 __global__ void __launch_bounds__(kCloseThreads)
@@ -92,9 +92,13 @@ table_pss_kernel(int d_model, int max_gen_sent, const float* emb, const int32_t*
     const int row0 = blockIdx.x * kPssRows;
     pdl_trigger();
     // The earlier embeddings are older than the kernel before this one: while that one closes the sentence, the first of them start towards
-    // L2.  What is read here may be older still; it decides about nothing else.  Closing takes 5 us in which memory was idle: 43.2 -> 39.6 us
-    // for ten sequences with 1300 embeddings of 4096 (39.9 with two rows per CTA, 41.0 with eight, which is more than L2 holds).
-    if (tid < kPssEarly && flag[b] != 0 && row0 + tid < min(n_gen_sent[b], max_gen_sent))
+    // L2.  What is read here may be older still; it decides about nothing else.  At most eight CTAs to an SM and 64 KB each: 78 MB of the 126 of
+    // L2.  With other buffers streamed through L2 between calls, as a decode step over all layers does, without / with (us, two runs'
+    // mean): 10 x 1300 embeddings of 4096 45.1 / 43.6, 16 x 2000 of 2048 52.2 / 50.4, of 4096 93.4 / 91.8, of 5120 113.7 / 113.5, 16 x 1500 of 3584
+    // 62.5 / 60.7, 16 x 1000 of 8192 131.5 / 133, 10 x 300 of 16384 82.9 / 82.9.  (Four rows also of the last two: 136 and 84.6; eight of 4096: 42.3, but
+    // 16 x 2000 of them 95.4.)  Called again at once, as in a loop over the table alone, it finds lines of the call before: 39.4 for the first.
+    const int early = min(kPssEarlyRows, kPssEarlyBytes / (d_model * 4));
+    if (tid < early && flag[b] != 0 && row0 + tid < min(n_gen_sent[b], max_gen_sent))
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(emb + (size_t(b) * max_gen_sent + row0 + tid) * d_model), "r"(d_model * 4)
                      : "memory");
     pdl_wait();
