@@ -27,7 +27,12 @@
 //    programmatic dependent launch derives its tile schedule and starts its first tiles towards L2 before the launch
 //    ahead of it has finished, and only then waits.  Behind the wait the first copies go out under that schedule at once; what was read
 //    early is checked while they are on their way (see "schedule").  With the check, the steering operands and the queries one round trip
-//    after the other in front of the first tile a step of one sequence x 2048 rows took 9.97 us a layer, now 8.9.
+//    after the other in front of the first tile a step of one sequence x 2048 rows took 9.97 us a layer, with them together 8.9.
+//  * Straight-line code counts: a launch behind other kernels (the products of a model's layer) finds its code in no instruction cache, and
+//    all that stands before the first copies is fetched first, about eight instructions a line.  So what runs once or seldom is rolled up, and the
+//    first copies are one piece of code for both attempts.  With the loops unrolled as the compiler saw fit and two pieces, behind four matrix
+//    products: 80 slabs x 4.1K rows 48.4 -> 45.2 us, two sequences of 8K 34.3 -> 30.0, 80 slabs of 16K to 32K 166 -> 163, 128 slabs x 8.2K
+//    (five heads) 108 -> 103; a step of one sequence x 2048 rows, 32 launches back to back, 281.6 -> 271.
 //  * Softmax is online in base 2 with a warp-uniform lazy rescale.
 //  * The last CTA to deliver a partial for a slab (self-resetting counter in the workspace) merges that slab's partials.
 #include <cstdio>
@@ -172,6 +177,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     // the lengths are read once more: only if one of them changed is the schedule derived again.
     const int s_per = (n_slabs + kDecThreads - 1) / kDecThreads;
     const int s_lo = min(tid * s_per, n_slabs), s_hi = min(s_lo + s_per, n_slabs);
+#pragma unroll 1
     for (int s = s_lo; s < s_hi; ++s) lens[s] = slab_len(s);
     auto tiles_of = [&](int s) { return (int(lens[s] >> 1) + kTileRows - 1) / kTileRows; };
     cta_prefix<kDecThreads>(n_slabs, tiles_of, pref, s_wsum);
@@ -203,6 +209,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     }
     if (kStep) {                                          // the rows being appended are read in the middle of the stream
         const size_t bytes = size_t(n_slabs) * kRowBytes;
+#pragma unroll 1
         for (size_t o = size_t(cta * kDecThreads + tid) * 128; o < bytes; o += size_t(G) * kDecThreads * 128) {
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(step.k_new) + o));
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(step.v_new) + o));
@@ -227,6 +234,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     int p_t = t_begin, p_slab = slab0, p_end = t_begin, p_r0 = 0, p_rows = 0, p_stage = 0;
     size_t p_row0 = 0;
     bool p_app = false;
+    long long bound = total_rows;                         // of the unchecked copies, until the schedule is confirmed
     long long far = 0;                                    // where the farthest of the unchecked copies ends
     auto issue_next = [&](auto unchecked) {
         if (p_t < t_end) {
@@ -246,7 +254,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
                           size_t(p_r0 % kPageRows);
                 // (never beyond the buffers, also under lengths that turn out to be old; from one that is left out on all are, and count as changed)
                 if (decltype(unchecked)::value) far = max(far, (long long)row + min(rows, kWarpRows));
-                if (!decltype(unchecked)::value || far <= total_rows) {
+                if (!decltype(unchecked)::value || far <= bound) {
                     const size_t off = (row + size_t(c_half)) * kRowBytes + size_t(c_col) * 16;
                     const uint8_t *kp = K + off, *vp = V + off;
                     // (row 2 i + c_half takes its pieces at c_col ^ ((2 i + c_half) & 7): four addresses and constant distances from them)
@@ -308,17 +316,24 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     uint4 qw = make_uint4(0u, 0u, 0u, 0u);
     if (side0 < steer_total) st = steer_load(side0, vec_per_row, hidden, steer_vec, alpha, flag);
     if (side0 < qwin_total) qw = reinterpret_cast<const uint4*>(q)[side0];
-    if (early) {
-#pragma unroll
-        for (int k = 0; k < kStages - 1; ++k) issue_next(std::true_type{});
-    }
-    {
+    bool go = early;
+#pragma unroll 1
+    for (int attempt = 0;; ++attempt) {
+        if (go) {
+#pragma unroll 1
+            for (int k = 0; k < kStages - 1; ++k) issue_next(std::true_type{});
+        }
+        if (attempt > 0) break;
         int changed = row_again != row_first || far > total_rows;
         if (s_lo < s_hi && len_again != lens[s_lo]) changed = 1;
+#pragma unroll 1
         for (int s = s_lo + 1; s < s_hi; ++s)
             if (slab_len(s) != lens[s]) changed = 1;
-        if (__syncthreads_or(changed)) {                  // (no thread writes a length before all have compared theirs)
+        changed = __syncthreads_or(changed);              // (no thread writes a length before all have compared theirs)
+        if (early && !changed) break;
+        if (changed) {
             cp_async_wait<0>();
+#pragma unroll 1
             for (int s = s_lo; s < s_hi; ++s) lens[s] = slab_len(s);
             cta_prefix<kDecThreads>(n_slabs, tiles_of, pref, s_wsum);
             derive();
@@ -326,10 +341,8 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
             p_t = p_end = t_begin; p_slab = slab0; p_stage = 0;
             q_slab = -1;
         }
-        if (!early || q_slab < 0) {
-#pragma unroll
-            for (int k = 0; k < kStages - 1; ++k) issue_next(std::false_type{});
-        }
+        bound = 0x7fffffffffffffffll;
+        go = true;
     }
     // The next launch's CTAs may start when every CTA has come here: early enough to have their schedule and their first
     // tiles ready, and not so early that what they start towards L2 is evicted by this launch's stream.
@@ -341,8 +354,10 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     auto qwin_at = [&](int i) { return step.q_win + (size_t(i >> 4) * step.window + step.slot) * 16 + (i & 15); };
     if (side0 < steer_total) steer_store(side0, vec_per_row, hidden, st);
     if (side0 < qwin_total) *qwin_at(side0) = qw;
+#pragma unroll 1
     for (int i = side0 + side_step; i < steer_total; i += side_step)
         steer_store(i, vec_per_row, hidden, steer_load(i, vec_per_row, hidden, steer_vec, alpha, flag));
+#pragma unroll 1
     for (int i = side0 + side_step; i < qwin_total; i += side_step) *qwin_at(i) = reinterpret_cast<const uint4*>(q)[i];
     // fused step: new length and range list of a slab after the append (every thread has read n_sent before any calls this)
     auto step_tables = [&](int slab_, int b_, int new_len, bool appended, int S0, int starts_sentence) {
@@ -363,6 +378,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
             if (!appended || !table_ok || full_list) atomicOr(status, SKIPKV_STATUS_BAD_TABLE);
         }
         if (appended && table_ok)
+#pragma unroll 1
             for (int i = S + tid; i <= step.max_sent; i += kDecThreads) so[i] = new_len;
     };
 
@@ -519,7 +535,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
         const int n_part = lc - fc + 1;
         __nv_bfloat16* o = out + (size_t(b) * Hq + size_t(h) * n) * kHeadDim;
         float* rec = dec_part + size_t(cta + slab) * n * kPartStride;
-#pragma unroll (kFew ? 2 : 4)
+#pragma unroll 1
         for (int hl = 0; hl < n; ++hl) {
             float M = -INFINITY, L = 0.f, A = 0.f;
 #pragma unroll
@@ -556,11 +572,13 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
                 const float* r0 = dec_part + size_t(fc + slab) * n * kPartStride;
                 constexpr int kAhead = kFew ? 10 : 12;
                 const int stride = n * kPartStride;
+#pragma unroll 1
                 for (int hl = warp; hl < n; hl += kDecWarps) {
                     const float* rh = r0 + hl * kPartStride;
                     auto channels = [&](int p) { return __ldcg(reinterpret_cast<const float4*>(rh + size_t(p * stride)) + lane); };
                     float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
                     float M = -INFINITY, L = 0.f;
+#pragma unroll 1
                     for (int p0 = 0; p0 < n_part; p0 += 32) {
                         const float2 ml = __ldcg(reinterpret_cast<const float2*>(rh + size_t(min(p0 + lane, n_part - 1) * stride) + 128));
                         float4 a[kAhead];
@@ -580,6 +598,7 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
                         M = Mn;
                         A.x *= keep; A.y *= keep; A.z *= keep; A.w *= keep;
                         const int cnt = min(32, n_part - p0);
+#pragma unroll 1
                         for (int k0 = 0; k0 < cnt; k0 += kAhead) {
 #pragma unroll
                             for (int k = 0; k < kAhead; ++k) {
@@ -608,10 +627,12 @@ decode_attn_kernel(int batch, int Hq, int Hk, int n_slabs, long long total_rows,
     cp_async_wait<0>();
     if (!triggered) pdl_trigger();
     // slabs with no row to attend to: zeros (owned round-robin); in the fused step they have no room: unchanged, reported
+#pragma unroll 1
     for (int s = cta; s < n_slabs; s += G) {
         if (lens[s] >> 1) continue;
         const int b = s / Hk, h = s % Hk;
         __nv_bfloat16* o = out + (size_t(b) * Hq + size_t(h) * n) * kHeadDim;
+#pragma unroll 1
         for (int idx = tid; idx < n * kHeadDim; idx += kDecThreads) o[idx] = __float2bfloat16_rn(0.f);
         if (kStep) step_tables(s, b, 0, false, 0, 0);
     }
