@@ -47,7 +47,7 @@ def measured_peaks():
 
 
 def ncu_traffic():
-    """DRAM bytes per launch from the committed ncu summaries (None when not captured)."""
+    """DRAM bytes per launch of the headline workload from the committed ncu summaries (None when not captured)."""
     p = os.path.join(ROOT, "profiles", "dram_traffic.json")
     return json.load(open(p)) if os.path.exists(p) else {}
 
@@ -359,8 +359,8 @@ def time_extras(cfg, B, flush, clean, peaks, reps=10):
     out["token_redundancy"] = {"us": us, "rows_per_slab": n_tok, "bound": "alu", "achieved": exps / us / 1e6,
                                "peak": mufu_peak, "unit": "T exp/s", "frac": exps / us / 1e6 / mufu_peak,
                                "matrix_elements_T_per_s": elems / us / 1e6, "tensor_tflops": exps * 256 / us / 1e6,
-                               "note": "each block pair is evaluated once; the issue slots of the epilogue, not the "
-                                       "exponentials, are the limit"}
+                               "note": "each block pair is evaluated once; the epilogue is the limit, no unit of it "
+                                       "above two thirds"}
     return out
 
 
@@ -476,7 +476,7 @@ def main():
                  "decode_attn": int(kv1.sum()) * row * 2 // NL,       # live K and V rows read once
                  "decode_attn_full_ctx": int(kv0.sum()) * row * 2 // NL}
     peaks = measured_peaks()
-    traffic = ncu_traffic()
+    traffic = ncu_traffic() if args.config == 2 and not args.batch else {}
     roof = {}
     for leg in ("score", "compact", "decode_attn", "decode_attn_full_ctx"):
         gbs = bytes_alg[leg] / (us[leg] * 1e-6) / 1e9

@@ -135,10 +135,12 @@ const char* skipkv_last_cuda_error(void);
  * (then it lives in the workspace).  sent_imp, sent_red, sent_lam, sent_score: device fp32
  * [batch][Hk][max_sent]; entries at i >= n_sent are not written.
  * shape->total_rows must be the exact number of rows of the K buffer (the tiled copies are bounded by
- * it).  The per-sentence sums are accumulated with floating-point atomics, so the last bits of the
- * scores may differ from run to run.  Limit: where max_sent > 128, about 8000 slabs (batch * n_kv_heads), whatever
- * the group size and the window; with more the call returns SKIPKV_ERR_UNSUPPORTED and skipkv_last_cuda_error() says
- * why.  The kernels of one call, and the first kernel of a call after the kernel before it on the stream, are launched
+ * it).  The results are the same bits from run to run, but for a slab with a sentence that lies in the shares of
+ * three or more blocks of the grid (the call's 128-row tiles are cut into equal contiguous shares, one a block): all but
+ * the first part of such a sentence's key sum are added in no fixed order, and the last bits of that slab's scores may
+ * differ.  Limit: where max_sent > 128, about 8000 slabs (batch * n_kv_heads), whatever the group size and the window;
+ * with more the call returns SKIPKV_ERR_UNSUPPORTED and skipkv_last_cuda_error() says why.  The kernels of one call,
+ * and the first kernel of a call after the kernel before it on the stream, are launched
  * as programmatic dependents: stream order holds.
  */
 int skipkv_score(const skipkv_shape* shape, const skipkv_params* params, const void* K,

@@ -1035,7 +1035,7 @@ score_pool_kernel(uint32_t* lse_cnt, int Hk, int max_sent, int max_cap, int max_
 // the slot that is free next and the old J's goes to the end of the queue, so a change of J costs no drain.
 // What counts is the epilogue's instructions, 32 exponentials and about 60 others per warp and pair: with the walk over the pairs, addresses, zeros
 // for parts that a pair did not have, masks and reciprocals in the loop it was 1790 and 1380 a scheduler and pair (passes 1 and 2), now
-// 1310 and 1140, and 306 and 271 us became 230 and 227 (128 slabs x 2K sentences; whole call 1950 -> 1848).  Of the 1.75 us a pair the three products,
+// 1310 and 1140, and 306 and 271 us became 230 and 227 (kernel times, 128 slabs x 2K sentences).  Of the 1.75 us a pair the three products,
 // which stream 192 KB of operands at the shared-memory port's 128 bytes per clock, take 0.8; the 64 KB of a pair's I block are
 // 5.5 TB/s from L2 over all SMs.
 // ---------------------------------------------------------------------------------------
@@ -1633,7 +1633,8 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     size_t fixed = 1024 + size_t(a.R) * kRowBytes + 2 * kIndBytes + 128 * kExtRow + sweep_ext_bytes(a.RA) +
                    sizeof(SweepCtl) + size_t(a.RB - 1) * 4 * 128 * 4;
     // The table of slabs (8 bytes each) goes into shared memory as long as one tile stage fits beside it: all but windows of some hundred
-    // query rows with a thousand slabs and more.  A 512-row window leaves room for 900 slabs; without the other form the call would end there.
+    // query rows with hundreds of slabs and more.  Of 512 rows, one head x 512 positions leaves room for 436 slabs, four heads x 128 for 3500; without
+    // the other form the call would end there.
     const size_t table_bytes = size_t(2 * L.slabs + 1) * 4;
     const bool in_global = fixed + table_bytes + kOpBytes > max_smem;
     if (in_global) a.table = reinterpret_cast<int*>(w + L.slab_table);

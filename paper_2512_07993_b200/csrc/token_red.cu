@@ -26,10 +26,10 @@
 // The columns of an item stay the same from tile to tile, so a thread keeps its 32 column sums in registers and the lanes are added
 // up once per item; with the rows fixed and the columns streamed, that butterfly (31 exchanges and as many selects for 32
 // elements) came with every tile and took longer than the exponentials.
-// What bounds it: issue slots of the epilogue.  Per element 4 multiply-add lanes, one exponential (8 clocks of a scheduler for a
-// warp) and about one instruction of overhead; the schedulers issue on 6 clocks of 10.  Four warps per scheduler hide the latencies
-// of these short chains, two with 64 columns each do not (326 us a pass); a share of the exponentials as polynomials adds more
-// issue slots than it takes off the special-function unit.  80 slabs x 4224 keys, both passes and the norms: 804 -> 617 us
+// What bounds it: the epilogue, none of whose units is saturated: the schedulers issue on 6 clocks of 10, exponentials (8 clocks of a
+// scheduler for a warp) take 61 to 65 % of their unit, the tensor pipe is at 29 to 32 %.  A warp waits for an accumulator, loads it and works
+// on it in sequence; four warps per scheduler hide most of that, two with 64 columns each do not (326 us a pass).  A share of the
+// exponentials as polynomials took 10 % more.  80 slabs x 4224 keys, both passes and the norms: 804 -> 617 us
 // back to back (558 in a short burst: the clock falls under the power limit), before the mean was kept apart.
 #include "tc.cuh"
 

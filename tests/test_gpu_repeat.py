@@ -1,5 +1,5 @@
-"""Repeated calls on one input: the scoring call must return the same bits every time (its only unordered
-accumulation adds at most two terms to a zero, which commutes), the token-level redundancy the same values to
+"""Repeated calls on one input: the scoring call must return the same bits every time (a sentence's key sum is stored by
+the block in whose share it begins, and here at most one other block adds a part), the token-level redundancy the same values to
 rounding (its row and column sums are accumulated with floating-point reductions in no fixed order).  A race on a
 shared buffer inside the Gram kernels would show here as a difference between runs."""
 import numpy as np
