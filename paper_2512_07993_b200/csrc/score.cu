@@ -81,9 +81,12 @@ struct SweepCtl {                       // barriers and small shared state, afte
     uint32_t wsum[32];
 };
 
-// The rows of pass B's extra K step; before, the sums of pass A: 8 bytes by warpgroup, row and block, and one block more where there are several.
-__host__ __device__ constexpr size_t sweep_ext_bytes(int RA) {
-    const size_t ext = size_t(RA) * 128 * kExtRow, sums = size_t(kAccAMax) * (RA + (RA > 1 ? 1 : 0)) * 128 * 8;
+// Pass A, last block of at most 64 rows: on every second tile its rows take the upper tensor-memory lanes, so that the
+// exponentials spread over all four schedulers.
+__host__ __device__ constexpr bool sweep_can_shift(int R, int RA) { return RA > 1 && R - (RA - 1) * 128 <= 64; }
+// The rows of pass B's extra K step; before, the sums of pass A: 8 bytes by warpgroup, row and block, the last block's on shifted tiles apart.
+__host__ __device__ constexpr size_t sweep_ext_bytes(int R, int RA) {
+    const size_t ext = size_t(RA) * 128 * kExtRow, sums = size_t(kAccAMax) * (RA + (sweep_can_shift(R, RA) ? 1 : 0)) * 128 * 8;
     return ext > sums ? ext : sums;
 }
 
@@ -301,7 +304,7 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     uint8_t* indb = tiles + size_t(a.stages) * kOpBytes;                         // the indicator matrices of the pooling
     uint8_t* onesb = indb + (kIndBytes << a.ind_log);                                // pass B: the keys' side of the extra K step
     uint8_t* extb = onesb + 128 * kExtRow;                                       // pass B: the queries' side; pass A: [groups][blocks] (m, l)
-    SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + sweep_ext_bytes(a.RA));
+    SweepCtl* ctl = reinterpret_cast<SweepCtl*>(extb + sweep_ext_bytes(a.R, a.RA));
     float* tokp = reinterpret_cast<float*>(ctl + 1);                             // [4 tiles][RB - 1][128] shares of a tile's tokens
     int* pref = kTable ? a.table : reinterpret_cast<int*>(tokp + 4 * (a.RB - 1) * 128);    // [n_slabs + 1] tile prefix
     int* rowb = pref + a.n_slabs + 1;                                            // [n_slabs] cache row of a slab's first token
@@ -372,10 +375,8 @@ score_sweep_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
     const bool pool_a = a.pool_a != 0;
     auto tile_at = [&](int p) { return pool_a ? t_begin + p : t_end - 1 - p; };
     const int kept = max(ntl - a.stages, 0);             // positions from here on are not loaded again
-    // Pass A, last block of at most 64 rows: on every second tile its rows take the upper tensor-memory lanes, so that the
-    // exponentials spread over all four schedulers.
     const int rem = a.R - (a.RA - 1) * 128;              // rows of the last block
-    const bool can_shift = a.RA > 1 && rem <= 64;
+    const bool can_shift = sweep_can_shift(a.R, a.RA);
     const int slots = a.RA + (can_shift ? 1 : 0);        // sums a thread keeps in pass A: one by block, the last block's on shifted tiles apart
     const int accs = pool_a ? 3 : 4;                     // accumulators and epilogue warpgroups of pass A
     constexpr int kBarA = 1;                             // named barrier: every accumulator of pass A has been read
@@ -1630,11 +1631,11 @@ static int score_impl(const skipkv_shape* shape, const skipkv_params* params, co
     a.hdr = reinterpret_cast<const Header*>(w + L.header);
     a.block_table = block_table; a.max_pages = max_pages;
     const size_t max_smem = 227 * 1024;
-    size_t fixed = 1024 + size_t(a.R) * kRowBytes + 2 * kIndBytes + 128 * kExtRow + sweep_ext_bytes(a.RA) +
+    size_t fixed = 1024 + size_t(a.R) * kRowBytes + 2 * kIndBytes + 128 * kExtRow + sweep_ext_bytes(a.R, a.RA) +
                    sizeof(SweepCtl) + size_t(a.RB - 1) * 4 * 128 * 4;
     // The table of slabs (8 bytes each) goes into shared memory as long as one tile stage fits beside it: all but windows of some hundred
-    // query rows with hundreds of slabs and more.  Of 512 rows, one head x 512 positions leaves room for 436 slabs, four heads x 128 for 3500; without
-    // the other form the call would end there.
+    // query rows with hundreds of slabs and more.  Of 512 rows, one head x 512 positions leaves room for 948 slabs, four heads x 128 for 4000 (six heads x 84,
+    // padded to 576 rows, 436); without the other form the call would end there.
     const size_t table_bytes = size_t(2 * L.slabs + 1) * 4;
     const bool in_global = fixed + table_bytes + kOpBytes > max_smem;
     if (in_global) a.table = reinterpret_cast<int*>(w + L.slab_table);

@@ -179,6 +179,15 @@ def test_score_with_more_slabs_than_shared_memory_has_room_for(group, window, ba
             assert torch.equal(got[b, :, :S], ref[b, :, :S])
 
 
+@pytest.mark.parametrize("group,window,batch", [(1, 512, 14), (4, 128, 15), (6, 84, 6)])
+def test_score_with_shared_memory_nearly_full_of_slabs(group, window, batch):
+    """The table of slabs beside 512 rows of query operands and one tile stage: 896 slabs (room for 948), 960, and 384 (room for 436) with a short
+    last block of rows, whose sums of shifted tiles lie behind the others'."""
+    lens = [1, 2, 127, 128, 129, 255, 256, 257, 384, 40, 77, 300, 500, 9, 16][:batch]
+    B, L, D = layer(lens, n_q_heads=64 * group, n_kv_heads=64, window=window, sent_lo=8, sent_hi=40, dup_rate=0.3, seed=930 + group)
+    check_scores(B, L, D)
+
+
 @pytest.mark.parametrize("group,window", [(4, 32), (5, 20), (8, 16), (4, 48)])
 @pytest.mark.parametrize("ctx", [[1 + (37 * i) % 128 for i in range(64)], [9000, 100, 9000], [9000, 100, 128, 1, 9000]])
 def test_score_runs_of_slabs_of_one_tile(group, window, ctx):
